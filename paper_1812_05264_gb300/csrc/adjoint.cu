@@ -1434,13 +1434,6 @@ extern "C" int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_
 }
 
 namespace tbk {
-void fermi_enqueue(tbk_ctx* ctx, const double* moments, int order, double emin, double emax,
-                   double n_electrons, double mu_fixed, double kT, int damping, double* tab,
-                   double* rho, double* res);
-int quad_nodes(int p);
-}  // namespace tbk
-
-namespace tbk {
 // The one-call energies and forces on the doubled-moment adjoint (fused-eligible shapes): the
 // adjoint's forward sweep over y_1 .. y_{p/2} also yields the moments, so no separate moment pass
 // runs.  probe_panel / s_norm: a stored probe block and its sample count (NULL / 0: the
@@ -1473,19 +1466,17 @@ void energies_and_forces_doubled(tbk_ctx* ctx, const tbk_bsr* H, const tbk_model
   const int K = p / 2;
   const int nctas = step_grid_ctas(ctx, op, s);
   double* partials = (double*)scratch(ctx, WS_PARTIALS, sizeof(double) * 2 * (size_t)std::max(1, K) * nctas);
-  const int M_nodes = quad_nodes(p);
-  double* fbuf = (double*)scratch(ctx, WS_SEGMENT, sizeof(double) * ((size_t)2 * K + 64 + 5 * (size_t)M_nodes + 16 +
-                                                                     (size_t)p + 8));
-  double* sums = fbuf;
-  double* tab = sums + 2 * (size_t)K + 64;
-  double* rho = tab + 4 * (size_t)M_nodes;
-  double* res = rho + M_nodes;
+  // per-step sums, the solve's buffer (16-byte aligned), its result, the moments unless given
+  const size_t nsums = 2 * (size_t)K + 64, nfermi = fermi_doubles(quad_nodes(p), p);
+  double* sums = (double*)scratch(ctx, WS_SEGMENT, sizeof(double) * (nsums + nfermi + 16 + (size_t)p + 8));
+  double* fbuf = sums + nsums;
+  double* res = fbuf + nfermi;
   double* mom = moments ? moments : res + 16;
   double* dcoef = (double*)scratch(ctx, WS_COEF, sizeof(double) * (size_t)p);
   auto after_forward = [&]() {
     // moments from the doubling identities, then mu, Omega, E, N, then c_k = d_k beta_k[g](mu)
     launch_moment_reduction(ctx, partials, nctas, K, p, nrm, op.n_rows, 0, sums, mom, err + 1);
-    fermi_enqueue(ctx, mom, p, emin, emax, n_electrons, 0.0, kT, damping, tab, rho, res);
+    fermi_enqueue(ctx, mom, p, emin, emax, n_electrons, 0.0, kT, damping, fbuf, res);
     double h[5];
     int herr[2] = {0, 0};
     TBK_CUDA(cudaMemcpyAsync(h, res, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1497,7 +1488,7 @@ void energies_and_forces_doubled(tbk_ctx* ctx, const tbk_bsr* H, const tbk_model
     if (herr[1])
       throw Error(TBK_ERR_SPECTRUM, "a Chebyshev panel grew beyond ||r||: the spectrum of H is not "
                                     "inside [emin, emax]");
-    if (h[4] != 0.0) throw Error(TBK_ERR_NOCONV, "n_electrons is outside the range of the estimated N(mu)");
+    check_fermi_status(h[4], "n_electrons is outside the range of the estimated N(mu)");
     for (int i = 0; i < 4; ++i) observables[i] = h[i];
     coefficients(ctx, TBK_FN_FREE, p, emin, emax, h[0], kT, damping, dcoef);
     std::vector<double> c(p);

@@ -17,11 +17,6 @@
 
 namespace tbk {
 
-void fermi_enqueue(tbk_ctx* ctx, const double* moments, int order, double emin, double emax,
-                   double n_electrons, double mu_fixed, double kT, int damping, double* tab,
-                   double* rho, double* res);
-int quad_nodes(int p);
-
 // Copy cluster c into the merged operator: rows shifted by a_off, blocks by b_off, mapped block
 // values (column-major FP32, as the step kernels read them).
 __global__ void merge_cluster(int n, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
@@ -376,7 +371,7 @@ extern "C" int tbk_batched_fermi_level(tbk_ctx* ctx, int32_t n_clusters, const d
   std::vector<FermiJob> jobs(n_clusters);
   size_t need = 0;
   int64_t moff = 0;
-  int M_max = 1;
+  int M_max = 1, p_max = 1;
   for (int c = 0; c < n_clusters; ++c) {
     TBK_CHECK_ARG(orders[c] >= 1 && orders[c] <= (1 << 22), "order out of range");
     TBK_CHECK_ARG(kT[c] > 0.0 && std::isfinite(kT[c]) && emax[c] > emin[c], "bad kT or bounds");
@@ -386,28 +381,29 @@ extern "C" int tbk_batched_fermi_level(tbk_ctx* ctx, int32_t n_clusters, const d
     j.emin = emin[c];
     j.emax = emax[c];
     j.n_e = n_electrons[c];
+    j.mu_fixed = 0.0;
     j.kT = kT[c];
     j.mom_off = moff;
-    j.tab_off = (int64_t)need;
-    j.rho_off = j.tab_off + 4 * (int64_t)j.M;
-    need += 5 * (size_t)j.M + 8;
+    j.buf_off = (int64_t)need;
+    need += fermi_doubles(j.M, j.p);
     moff += orders[c];
     M_max = std::max(M_max, j.M);
+    p_max = std::max(p_max, j.p);
   }
   double* buf = (double*)scratch(ctx, WS_COEF, sizeof(double) * need);
   double* res = (double*)scratch(ctx, WS_NODES, sizeof(double) * 8 * (size_t)n_clusters + sizeof(FermiJob) * n_clusters + 64);
   FermiJob* d_jobs = (FermiJob*)(res + 8 * (size_t)n_clusters);
   TBK_CUDA(cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(FermiJob) * n_clusters, cudaMemcpyHostToDevice, ctx->stream));
-  fermi_enqueue_batched(ctx, n_clusters, d_jobs, M_max, moments, damping, buf, res);
+  fermi_enqueue_batched(ctx, n_clusters, d_jobs, M_max, p_max, moments, damping, buf, res);
   std::vector<double> h(8 * (size_t)n_clusters);
   TBK_CUDA(cudaMemcpyAsync(h.data(), res, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, ctx->stream));
   sync(ctx);
-  bool bad = false;
+  double bad = 0.0;
   for (int c = 0; c < n_clusters; ++c) {
     for (int i = 0; i < 4; ++i) out[4 * c + i] = h[8 * c + i];
-    bad = bad || h[8 * c + 4] != 0.0;
+    bad = std::max(bad, h[8 * c + 4]);
   }
-  if (bad) throw Error(TBK_ERR_NOCONV, "n_electrons is outside the estimated N(mu) range for some cluster");
+  check_fermi_status(bad, "n_electrons is outside the estimated N(mu) range for some cluster");
   TBK_API_END
 }
 
@@ -614,18 +610,18 @@ static void batched_adjoint(tbk_ctx* ctx, int ncl, const tbk_bsr* H, const tbk_m
         j.emin = emin[c];
         j.emax = emax[c];
         j.n_e = n_electrons[c];
+        j.mu_fixed = 0.0;
         j.kT = kT[c];
         j.mom_off = out_off_u[c];
-        j.tab_off = (int64_t)need;
-        j.rho_off = j.tab_off + 4 * (int64_t)j.M;
-        need += 5 * (size_t)j.M + 8;
+        j.buf_off = (int64_t)need;
+        need += fermi_doubles(j.M, j.p);
         M_max = std::max(M_max, j.M);
       }
       double* fbuf = (double*)scratch(ctx, WS_PANEL1, sizeof(double) * need);
       double* res = (double*)scratch(ctx, WS_PANEL2, sizeof(double) * 8 * (size_t)ncl + sizeof(FermiJob) * ncl + 64);
       FermiJob* d_jobs = (FermiJob*)(res + 8 * (size_t)ncl);
       TBK_CUDA(cudaMemcpyAsync(d_jobs, jobs.data(), sizeof(FermiJob) * ncl, cudaMemcpyHostToDevice, ctx->stream));
-      fermi_enqueue_batched(ctx, ncl, d_jobs, M_max, mom, damping, fbuf, res);
+      fermi_enqueue_batched(ctx, ncl, d_jobs, M_max, pmax, mom, damping, fbuf, res);
       std::vector<double> h(8 * (size_t)ncl);
       int herr[2] = {0, 0};
       TBK_CUDA(cudaMemcpyAsync(h.data(), res, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, ctx->stream));
@@ -638,13 +634,13 @@ static void batched_adjoint(tbk_ctx* ctx, int ncl, const tbk_bsr* H, const tbk_m
         throw Error(TBK_ERR_SPECTRUM, "a Chebyshev panel grew beyond ||r||: some cluster's spectrum is not "
                                       "inside its [emin, emax]");
       std::vector<double> mus(ncl);
-      bool bad = false;
+      double bad = 0.0;
       for (int c = 0; c < ncl; ++c) {
         for (int q = 0; q < 4; ++q) observables[4 * c + q] = h[8 * c + q];
         mus[c] = h[8 * c];
-        bad = bad || h[8 * c + 4] != 0.0;
+        bad = std::max(bad, h[8 * c + 4]);
       }
-      if (bad) throw Error(TBK_ERR_NOCONV, "n_electrons is outside the estimated N(mu) range for some cluster");
+      check_fermi_status(bad, "n_electrons is outside the estimated N(mu) range for some cluster");
       build_cft(mus.data());
       return std::vector<double>();
     };

@@ -96,16 +96,21 @@ struct KernelTimerScope {
 
 inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
-// One cluster's chemical-potential solve in a batch: M quadrature nodes, order p, moments at
-// mom_off, cosine table (4M doubles) at tab_off and node weights (M doubles) at rho_off of one
-// scratch buffer.
+// One chemical-potential solve: M quadrature nodes, order p, moments at mom_off, its scratch of
+// fermi_doubles(M, p) doubles at buf_off (even) of one buffer.  n_e < 0: mu_fixed is taken as mu.
 struct FermiJob {
   int M, p;
-  double emin, emax, n_e, kT;
-  int64_t mom_off, tab_off, rho_off;
+  double emin, emax, n_e, mu_fixed, kT;
+  int64_t mom_off, buf_off;
 };
-void fermi_enqueue_batched(tbk_ctx* ctx, int n, const FermiJob* d_jobs, int M_max, const double* moments,
+size_t fermi_doubles(int M, int p);
+void fermi_enqueue(tbk_ctx* ctx, const double* moments, int order, double emin, double emax,
+                   double n_electrons, double mu_fixed, double kT, int damping, double* buf, double* res);
+void fermi_enqueue_batched(tbk_ctx* ctx, int n, const FermiJob* d_jobs, int M_max, int p_max, const double* moments,
                            int damping, double* buf, double* res);
+// Throws for the status of a solve (res[4]): 1 = no sign change in the bracket, 2 = a wait expired.
+void check_fermi_status(double status, const char* no_bracket);
+int quad_nodes(int p);
 
 }  // namespace tbk
 
@@ -152,4 +157,32 @@ __device__ __forceinline__ double tbk_block_sum(double v, double* smem32) {
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   }
   return t;  // valid in thread 0
+}
+
+// Barrier of the CTAs of one cooperative launch that share *ctr (zero before the first use): the
+// n-th use waits for target = n * CTAs arrivals.  What a CTA wrote before is visible to the others
+// after (read it past L1).  Bounded: false in all threads of the CTA when 2 s of the global timer
+// went by, or after 2^26 polls.
+__device__ __forceinline__ bool tbk_grid_wait(unsigned* ctr, unsigned target) {
+  __syncthreads();
+  int ok = 1;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(ctr, 1u);
+    uint64_t t0 = 0, t = 0;
+    for (uint32_t i = 0;; ++i) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
+      if ((int)(v - target) >= 0) break;
+      if ((i & 1023u) == 1023u) {
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        if (!t0) t0 = t;
+        if (t - t0 > 2000000000ull || i >= (1u << 26)) {
+          ok = 0;
+          break;
+        }
+      }
+    }
+  }
+  return __syncthreads_and(ok) != 0;
 }

@@ -8,6 +8,7 @@
 //   rho_j = (1/M) sum_k (2 - delta_k0) d_k mu_k cos(k t_j).
 // The chemical-potential bisection therefore needs rho once and O(M) work per halving.
 // cos(k t_j) = cos(pi m / (2M)) with m = k (2j + 1) mod 4M, read from a table of 4M entries.
+#include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
@@ -31,14 +32,6 @@ __device__ __forceinline__ double node_energy(int j, int M, double emin, double 
   return emin * (1.0 - x) * 0.5 + emax * (1.0 + x) * 0.5;
 }
 
-__device__ __forceinline__ void cos_entry(int m, int M, double* __restrict__ tab) {
-  if (m < 4 * M) tab[m] = cospi((double)m / (2.0 * M));
-}
-
-__global__ void cos_table(int M, double* __restrict__ tab) {
-  cos_entry(blockIdx.x * blockDim.x + threadIdx.x, M, tab);
-}
-
 __device__ __forceinline__ double damp_factor(int k, int p, int damping) {
   if (damping != TBK_DAMP_JACKSON) return 1.0;
   // Jackson kernel (Weisse et al., Rev. Mod. Phys. 78, 275 (2006), Eq. 71) with N = p
@@ -46,10 +39,13 @@ __device__ __forceinline__ double damp_factor(int k, int p, int damping) {
   return ((p - k + 1) * cos(q * k) + sin(q * k) / tan(q)) / (p + 1);
 }
 
-// h_j = h(e_j) at the M quadrature nodes, once (the coefficient blocks all read them).
-__global__ void node_values(int fn, int M, double emin, double emax, double mu, double kT,
-                            double* __restrict__ hv) {
+// ---- a4: coefficients ------------------------------------------------------------------------------
+
+// The cosine table (4M entries) and h_j = h(e_j) at the M nodes, which the coefficient blocks read.
+__global__ void coeff_setup(int fn, int M, double emin, double emax, double mu, double kT,
+                            double* __restrict__ tab, double* __restrict__ hv) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < 4 * M) tab[j] = cospi((double)j / (2.0 * M));
   if (j >= M) return;
   const double e = node_energy(j, M, emin, emax);
   double h;
@@ -61,141 +57,276 @@ __global__ void node_values(int fn, int M, double emin, double emax, double mu, 
   hv[j] = h;
 }
 
-// One block per coefficient k.
+// One block per coefficient k.  The small coefficients of the tail are differences of large terms, so
+// the order of this sum decides their last bits; it is kept fixed.
 __global__ void coeff_kernel(int p, int M, int damping, const double* __restrict__ tab,
                              const double* __restrict__ hv, double* __restrict__ out) {
   __shared__ double red[32];
   const int k = blockIdx.x;
+  const int period = 4 * M, step = (int)((2 * (int64_t)k * blockDim.x) % period);
+  int m = (int)((int64_t)k * (2 * threadIdx.x + 1) % period);
   double s = 0.0, c = 0.0;
   for (int j = threadIdx.x; j < M; j += blockDim.x) {
-    const double h = hv[j];
-    const int64_t m = ((int64_t)k * (2 * j + 1)) % (4 * (int64_t)M);
-    const double y = h * tab[m] - c, t = s + y;
-    c = (t - s) - y;
-    s = t;
-  }
-  const double tot = tbk_block_sum(s, red);
-  if (threadIdx.x == 0) out[k] = (k == 0 ? 1.0 : 2.0) / M * tot * damp_factor(k, p, damping);
-}
-
-// rho_j, one thread per node, fixed order over k.
-__device__ __forceinline__ void rho_node(int j, const double* __restrict__ mom, int p, int M, int damping,
-                                         const double* __restrict__ tab, double* __restrict__ rho) {
-  if (j >= M) return;
-  double s = 0.0, c = 0.0;
-  const int64_t step = 2 * j + 1, period = 4 * (int64_t)M;
-  int64_t m = 0;
-  for (int k = 0; k < p; ++k) {
-    const double w = (k == 0 ? 1.0 : 2.0) * damp_factor(k, p, damping) * mom[k];
-    const double y = w * tab[m] - c, t = s + y;
+    const double y = hv[j] * tab[m] - c, t = s + y;
     c = (t - s) - y;
     s = t;
     m += step;
     if (m >= period) m -= period;
   }
-  rho[j] = s / M;
+  const double tot = tbk_block_sum(s, red);
+  if (threadIdx.x == 0) out[k] = (k == 0 ? 1.0 : 2.0) / M * tot * damp_factor(k, p, damping);
 }
 
-__global__ void rho_kernel(const double* __restrict__ mom, int p, int M, int damping,
-                           const double* __restrict__ tab, double* __restrict__ rho) {
-  rho_node(blockIdx.x * blockDim.x + threadIdx.x, mom, p, M, damping, tab, rho);
+// ---- a8: chemical potential and observables --------------------------------------------------------
+//
+// Every problem (FermiJob) owns one buffer of fermi_doubles(M, p) doubles.  A solve is three launches
+// for any number of problems (blockIdx.y = problem): the cosine table and the damped weights
+// w_k = (2 - delta_k0) d_k mu_k; the node weights rho_j beside the node energies; the bisection.
+struct FermiBuf {
+  double* tab;       // 4M cosines
+  double2* node;     // M pairs (e_j, rho_j)
+  double* part;      // FERMI_PART partial sums, two sets used in turn
+  unsigned* ctr;     // arrivals at the barrier of the CTAs that share the problem
+  double* w;         // p weights
+};
+constexpr int FERMI_DEPTH = 5, FERMI_MIDS = (1 << FERMI_DEPTH) - 1;  // midpoints evaluated at once
+constexpr int FERMI_THREADS = 256, FERMI_LANES = 1024, FERMI_PARTS = 16;
+constexpr int FERMI_PART = 3 * FERMI_MIDS * FERMI_PARTS;  // >= 32 FERMI_MIDS
+
+__device__ __forceinline__ FermiBuf fermi_buf(double* buf, int M) {
+  return {buf, (double2*)(buf + 4 * (size_t)M), buf + 6 * (size_t)M, (unsigned*)(buf + 6 * (size_t)M + 2 * FERMI_PART),
+          buf + 6 * (size_t)M + 2 * FERMI_PART + 2};
+}
+size_t fermi_doubles(int M, int p) { return 6 * (size_t)M + 2 * FERMI_PART + 2 + (size_t)p + (p & 1); }
+
+__global__ void fermi_setup(const FermiJob one, const FermiJob* __restrict__ jobs,
+                            const double* __restrict__ mom, int damping, double* __restrict__ buf) {
+  const FermiJob j = jobs ? jobs[blockIdx.y] : one;
+  const FermiBuf b = fermi_buf(buf + j.buf_off, j.M);
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) *b.ctr = 0;
+  if (i < 4 * j.M) b.tab[i] = cospi((double)i / (2.0 * j.M));
+  if (i < j.p) b.w[i] = (i == 0 ? 1.0 : 2.0) * damp_factor(i, j.p, damping) * mom[j.mom_off + i];
 }
 
-// One block: bisection for N(mu) = n_e (skipped when n_e < 0), then Omega, E, N.
-// out = {mu, Omega, E, N, status} with status 1 when the bracket has no sign change.
-__device__ void fermi_solve(const double* __restrict__ rho, int M, double emin, double emax,
-                            double n_e, double mu_fixed, double kT, double* __restrict__ out) {
+// The node energies, and rho_j and rho_{M-1-j} from the even and the odd part of the sum over k
+// (cos(k (pi - t)) = (-1)^k cos(k t): half the terms of two separate sums).  S lanes share a pair of
+// nodes, lane r takes k = r, r + S, ..., one parity per lane, each compensated.  The compensated chain
+// is four dependent FP64 operations of ~85 cycles a term, at 1/64 of the FP32 rate: one thread per
+// node took 432 us at p = 2476 by latency alone; S lanes cut the chain until the issue rate binds.
+__global__ void __launch_bounds__(64)
+rho_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int S, double* __restrict__ buf) {
+  const FermiJob job = jobs ? jobs[blockIdx.y] : one;
+  const FermiBuf b = fermi_buf(buf + job.buf_off, job.M);
+  const int M = job.M, p = job.p;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = i / S, r = i - j * S;
+  double s = 0.0, c = 0.0;
+  if (j < M / 2) {
+    const int period = 4 * M, step = (int)((int64_t)S * (2 * j + 1) % period);
+    int m = (int)((int64_t)r * (2 * j + 1) % period);
+#pragma unroll 4
+    for (int k = r; k < p; k += S) {
+      const double y = __ldg(b.w + k) * __ldg(b.tab + m) - c, t = s + y;
+      c = (t - s) - y;
+      s = t;
+      m += step;
+      if (m >= period) m -= period;
+    }
+  }
+  for (int o = S / 2; o >= 2; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  const double other = __shfl_xor_sync(0xffffffffu, s, 1);
+  if (j < M / 2 && r < 2) {
+    // lane 0 holds the even part, lane 1 the odd part
+    const int node = r == 0 ? j : M - 1 - j;
+    b.node[node] = make_double2(node_energy(node, M, job.emin, job.emax), (r == 0 ? s + other : other - s) / M);
+  }
+}
+
+// f(e) in a bisection sum.  Past 38 kT below mu, exp(z) < 2^-54 and f rounds to 2 exactly; past
+// 80 kT above, f < 4e-35, far below the rounding that every rho_j carries.  Only the nodes between
+// (about 1,200 whatever kT is, since M grows with W/kT) take the exponential and the division.
+__device__ __forceinline__ double count_occupation(double e, double mu, double inv_kT) {
+  const double z = (e - mu) * inv_kT;
+  if (z <= -38.0) return 2.0;
+  if (z >= 80.0) return 0.0;
+  return 2.0 / (1.0 + exp(z));
+}
+
+// Bisection for N(mu) = n_e (skipped when n_e < 0), then Omega, E, N, by gridDim.x CTAs of one
+// problem.  out = {mu, Omega, E, N, status}: status 1 when the bracket has no sign change, 2 when a
+// wait expired.  The midpoints of the next `depth` halvings (nm = 2^depth - 1 of them) are evaluated
+// at once, each by `parts` CTAs, and the halvings are then decided in order, so mu is the plain
+// bisection's; one barrier for `depth` halvings.  N(mu) is summed as FERMI_LANES strided chains and
+// a tree over them whatever the launch, so mu does not depend on it.  Latency binds: an FP64 operation
+// takes ~85 cycles and an occupation ~40 of them (45 halvings one after the other in one CTA: 0.65 ms
+// at M = 504, 9.2 ms at M = 9904; this form 0.10 and 0.17 ms).
+__global__ void __launch_bounds__(FERMI_THREADS)
+fermi_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int depth, int parts, double* __restrict__ buf,
+             double* __restrict__ res) {
   __shared__ double red[32];
-  __shared__ double bc;
-  auto count = [&](double mu) {
+  __shared__ double cnt[FERMI_MIDS + 1];
+  __shared__ double fs[FERMI_THREADS];
+  const FermiJob job = jobs ? jobs[blockIdx.y] : one;
+  const FermiBuf b = fermi_buf(buf + job.buf_off, job.M);
+  double* out = res + 8 * (int64_t)blockIdx.y;
+  const int M = job.M, ncta = gridDim.x, cta = blockIdx.x, tid = threadIdx.x;
+  const double kT = job.kT, inv_kT = 1.0 / kT, W = job.emax - job.emin;
+  int phase = 0;
+  bool ok = true;
+  // the chains of part pi (FERMI_LANES / parts of them), 32 of them summed into put[chain / 32]
+  auto chains = [&](int pi, double mu, double* put) {
+    const int span = FERMI_LANES / parts;
+    if (span >= FERMI_THREADS) {  // a thread per chain, several times
+      for (int g = 0; g < span; g += FERMI_THREADS) {
+        const int t0 = pi * span + g + tid;
+        double s = 0.0;
+        for (int j = t0; j < M; j += FERMI_LANES) {
+          const double2 n = __ldg(b.node + j);
+          s = fma(count_occupation(n.x, mu, inv_kT), n.y, s);
+        }
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((tid & 31) == 0) __stcg(put + (t0 >> 5), s);
+      }
+      return;
+    }
+    // several threads per chain take the occupations of consecutive links, the first one adds them
+    const int rows = FERMI_THREADS / span, rr = tid / span, vt = tid - rr * span, t0 = pi * span + vt;
     double s = 0.0;
-    for (int j = threadIdx.x; j < M; j += blockDim.x)
-      s += fermi_fn(node_energy(j, M, emin, emax), mu, kT) * rho[j];
-    double t = tbk_block_sum(s, red);
-    if (threadIdx.x == 0) bc = t;
-    __syncthreads();
-    t = bc;
-    __syncthreads();
-    return t;
+    for (int j0 = 0; j0 < M; j0 += rows * FERMI_LANES) {
+      const int j = j0 + rr * FERMI_LANES + t0;
+      fs[tid] = j < M ? count_occupation(__ldg(b.node + j).x, mu, inv_kT) : 0.0;
+      __syncthreads();
+      if (rr == 0)
+        for (int q = 0; q < rows; ++q) {
+          const int jj = j0 + q * FERMI_LANES + t0;
+          if (jj < M) s = fma(fs[q * span + vt], __ldg(b.node + jj).y, s);
+        }
+      __syncthreads();
+    }
+    if (rr == 0) {
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if ((tid & 31) == 0) __stcg(put + (t0 >> 5), s);
+    }
   };
-  double mu = mu_fixed;
-  double status = 0.0;
-  if (n_e >= 0.0) {
-    double lo = emin, hi = emax;
-    const double W = emax - emin;
-    if (count(lo) > n_e || count(hi) < n_e) status = 1.0;
-    for (int it = 0; it < 200; ++it) {
-      const double mid = 0.5 * (lo + hi);
-      if (count(mid) < n_e) lo = mid; else hi = mid;
-      if (hi - lo < 1e-13 * W) break;
+  // cnt[q] = N(mid of q), q = 0 .. nm - 1, in every CTA
+  auto evaluate = [&](int nm, auto mid_of) {
+    double* part = b.part + (phase & 1) * FERMI_PART;
+    if (ncta == 1) {
+      for (int q = 0; q < nm; ++q) chains(0, mid_of(q), part + 32 * q);
+      __threadfence_block();
+      __syncthreads();
+    } else {
+      const int pi = cta / nm, q = cta - pi * nm;
+      if (pi < parts) chains(pi, mid_of(q), part + 32 * q);
+      ok = ok && tbk_grid_wait(b.ctr, (unsigned)(ncta * (phase + 1)));
+    }
+    ++phase;
+    for (int q = tid >> 5; q < nm; q += FERMI_THREADS / 32) {
+      double t = __ldcg(part + 32 * q + (tid & 31));
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if ((tid & 31) == 0) cnt[q] = t;
+    }
+    __syncthreads();
+  };
+  double mu = job.mu_fixed, status = 0.0;
+  if (job.n_e >= 0.0) {
+    double lo = job.emin, hi = job.emax;
+    evaluate(2, [&](int q) { return q ? hi : lo; });
+    if (cnt[0] > job.n_e || cnt[1] < job.n_e) status = 1.0;
+    __syncthreads();
+    bool done = false;
+    for (int it = 0; it < 200 && !done && ok;) {
+      // heap order: node 1 is the midpoint of [lo, hi], node 2q that of the lower half below q
+      evaluate((1 << depth) - 1, [&](int q) {
+        double l = lo, h = hi;
+        for (int bit = 30 - __clz(q + 1); bit >= 0; --bit) {
+          const double mid = 0.5 * (l + h);
+          if (((q + 1) >> bit) & 1) l = mid; else h = mid;
+        }
+        return 0.5 * (l + h);
+      });
+      int node = 1;
+      for (int d = 0; d < depth && it < 200 && !done; ++d, ++it) {
+        const double mid = 0.5 * (lo + hi);
+        const bool up = cnt[node - 1] < job.n_e;
+        if (up) lo = mid; else hi = mid;
+        node = 2 * node + (up ? 1 : 0);
+        done = hi - lo < 1e-13 * W;
+      }
+      __syncthreads();
     }
     mu = 0.5 * (lo + hi);
   }
-  double so = 0.0, se = 0.0, sn = 0.0;
-  for (int j = threadIdx.x; j < M; j += blockDim.x) {
-    const double e = node_energy(j, M, emin, emax);
-    const double f = fermi_fn(e, mu, kT);
-    so += free_fn(e, mu, kT) * rho[j];
-    se += e * f * rho[j];
-    sn += f * rho[j];
+  double v[3] = {0.0, 0.0, 0.0};
+  for (int j = cta * blockDim.x + threadIdx.x; j < M; j += ncta * blockDim.x) {
+    const double2 n = __ldg(b.node + j);
+    const double f = fermi_fn(n.x, mu, kT);
+    v[0] += free_fn(n.x, mu, kT) * n.y;
+    v[1] += n.x * f * n.y;
+    v[2] += f * n.y;
   }
-  const double to = tbk_block_sum(so, red);
-  __syncthreads();
-  const double te = tbk_block_sum(se, red);
-  __syncthreads();
-  const double tn = tbk_block_sum(sn, red);
-  if (threadIdx.x == 0) {
-    out[0] = mu;
-    out[1] = to;
-    out[2] = te;
-    out[3] = tn;
-    out[4] = status;
+  double* part = b.part + (phase & 1) * FERMI_PART;
+  for (int q = 0; q < 3; ++q) {
+    const double t = tbk_block_sum(v[q], red);
+    if (threadIdx.x == 0) __stcg(part + 3 * cta + q, t);
   }
-}
-
-__global__ void fermi_kernel(const double* __restrict__ rho, int M, double emin, double emax,
-                             double n_e, double mu_fixed, double kT, double* __restrict__ out) {
-  fermi_solve(rho, M, emin, emax, n_e, mu_fixed, kT, out);
-}
-
-// ---- many clusters in three launches (blockIdx.y / blockIdx.x = cluster) ----
-
-__global__ void cos_table_batched(const FermiJob* __restrict__ jobs, double* __restrict__ buf) {
-  const FermiJob j = jobs[blockIdx.y];
-  cos_entry(blockIdx.x * blockDim.x + threadIdx.x, j.M, buf + j.tab_off);
-}
-
-__global__ void rho_batched(const FermiJob* __restrict__ jobs, const double* __restrict__ mom, int damping,
-                            double* __restrict__ buf) {
-  const FermiJob j = jobs[blockIdx.y];
-  rho_node(blockIdx.x * blockDim.x + threadIdx.x, mom + j.mom_off, j.p, j.M, damping, buf + j.tab_off,
-           buf + j.rho_off);
-}
-
-__global__ void fermi_batched(const FermiJob* __restrict__ jobs, const double* __restrict__ buf,
-                              double* __restrict__ res) {
-  const FermiJob j = jobs[blockIdx.x];
-  fermi_solve(buf + j.rho_off, j.M, j.emin, j.emax, j.n_e, 0.0, j.kT, res + 8 * (int64_t)blockIdx.x);
+  if (ncta > 1) ok = ok && tbk_grid_wait(b.ctr, (unsigned)(ncta * (phase + 1)));
+  else __syncthreads();
+  if (cta == 0 && threadIdx.x < 3) {
+    double t = 0.0;
+    for (int i = 0; i < ncta; ++i) t += __ldcg(part + 3 * i + threadIdx.x);
+    out[1 + threadIdx.x] = t;
+    if (threadIdx.x == 0) {
+      out[0] = mu;
+      out[4] = ok ? status : 2.0;
+    }
+  }
 }
 
 int quad_nodes(int p) { return std::max(4 * p, 256); }
 
-void fermi_enqueue_batched(tbk_ctx* ctx, int n, const FermiJob* d_jobs, int M_max, const double* moments,
-                           int damping, double* buf, double* res) {
-  cos_table_batched<<<dim3(ceil_div(4 * (int64_t)M_max, 256), n), 256, 0, ctx->stream>>>(d_jobs, buf);
-  post_launch(ctx, "cos_table_batched");
-  rho_batched<<<dim3(ceil_div(M_max, 128), n), 128, 0, ctx->stream>>>(d_jobs, moments, damping, buf);
-  post_launch(ctx, "rho_batched");
-  fermi_batched<<<n, 1024, 0, ctx->stream>>>(d_jobs, buf, res);
-  post_launch(ctx, "fermi_batched");
+// Enqueue the solves of n problems (jobs on the device, or `one` when NULL); M_max and p_max over
+// them.  res: 8 doubles per problem.
+static void fermi_launch(tbk_ctx* ctx, int n, const FermiJob& one, const FermiJob* d_jobs, int M_max, int p_max,
+                         const double* moments, int damping, double* buf, double* res) {
+  fermi_setup<<<dim3(ceil_div(std::max(4 * (int64_t)M_max, (int64_t)p_max), 256), n), 256, 0, ctx->stream>>>(
+      one, d_jobs, moments, damping, buf);
+  post_launch(ctx, "fermi_setup");
+  // lanes per pair of nodes: about eight warps per SM over all problems
+  int S = 2;
+  while (S < 32 && (int64_t)n * (M_max / 2) * S < (int64_t)ctx->num_sms * 256) S *= 2;
+  rho_kernel<<<dim3(ceil_div((int64_t)(M_max / 2) * S, 64), n), 64, 0, ctx->stream>>>(one, d_jobs, S, buf);
+  post_launch(ctx, "rho_kernel");
+  // CTAs per problem, as long as all problems fit the chip together: as many midpoints at once as
+  // there is room for, then 4 to 16 CTAs per midpoint (one CTA per problem takes its midpoints one by
+  // one).  Chains of one link are latency alone (M = 800: 121 us at depth 4, 103 us at 5); longer ones
+  // want the CTAs for more parts instead (M = 9904: 300 us at depth 5, 171 us at 4 with twice the parts)
+  int occ = 0;
+  TBK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fermi_kernel, FERMI_THREADS, 0));
+  const int room = occ * ctx->num_sms / n, links = ceil_div(M_max, FERMI_LANES);
+  int depth = 1;
+  const int depth_max = links > 1 ? FERMI_DEPTH - 1 : FERMI_DEPTH;
+  while (depth < depth_max && (2 << depth) - 1 <= room) ++depth;
+  const int nm = (1 << depth) - 1;
+  int parts = links > 4 ? FERMI_PARTS : (links > 1 ? 8 : 4);
+  while (parts > 1 && parts * nm > room) parts /= 2;
+  const dim3 grid(room < 3 ? 1 : nm * parts, n);
+  if (grid.x == 1) {
+    fermi_kernel<<<grid, FERMI_THREADS, 0, ctx->stream>>>(one, d_jobs, 1, 1, buf, res);
+  } else {
+    // the CTAs of a problem wait for one another: a cooperative launch keeps them all resident
+    FermiJob o = one;
+    int d = depth;
+    void* args[] = {&o, (void*)&d_jobs, &d, &parts, &buf, &res};
+    TBK_CUDA(cudaLaunchCooperativeKernel((const void*)fermi_kernel, grid, dim3(FERMI_THREADS), args, 0, ctx->stream));
+  }
+  post_launch(ctx, "fermi_kernel");
 }
 
-// cos table of 4M doubles in WS_NODES, followed by `extra` doubles of room for the caller.
-const double* make_cos_table(tbk_ctx* ctx, int M, size_t extra = 0) {
-  double* tab = (double*)scratch(ctx, WS_NODES, sizeof(double) * (4 * (size_t)M + extra));
-  cos_table<<<ceil_div(4 * (int64_t)M, 256), 256, 0, ctx->stream>>>(M, tab);
-  post_launch(ctx, "cos_table");
-  return tab;
+void fermi_enqueue_batched(tbk_ctx* ctx, int n, const FermiJob* d_jobs, int M_max, int p_max, const double* moments,
+                           int damping, double* buf, double* res) {
+  fermi_launch(ctx, n, FermiJob(), d_jobs, M_max, p_max, moments, damping, buf, res);
 }
 
 void coefficients(tbk_ctx* ctx, int fn, int p, double emin, double emax, double mu, double kT,
@@ -206,29 +337,30 @@ void coefficients(tbk_ctx* ctx, int fn, int p, double emin, double emax, double 
   TBK_CHECK_ARG(kT > 0.0 && std::isfinite(kT), "kT must be positive");
   TBK_CHECK_ARG(emax > emin, "need emax > emin");
   const int M = quad_nodes(p);
-  const double* tab = make_cos_table(ctx, M, (size_t)M);
-  double* hv = const_cast<double*>(tab) + 4 * (size_t)M;
-  node_values<<<ceil_div(M, 256), 256, 0, ctx->stream>>>(fn, M, emin, emax, mu, kT, hv);
-  post_launch(ctx, "node_values");
+  double* tab = (double*)scratch(ctx, WS_NODES, sizeof(double) * 5 * (size_t)M);
+  double* hv = tab + 4 * (size_t)M;
+  coeff_setup<<<ceil_div(4 * (int64_t)M, 256), 256, 0, ctx->stream>>>(fn, M, emin, emax, mu, kT, tab, hv);
+  post_launch(ctx, "coeff_setup");
   coeff_kernel<<<p, 256, 0, ctx->stream>>>(p, M, damping, tab, hv, out);
   post_launch(ctx, "coeff_kernel");
 }
 
-// Enqueue the chemical-potential solve for one moment vector without synchronising: tab (4M
-// doubles), rho (M doubles) and res (5 doubles: mu, Omega, E, N, status) are device buffers.
+// Enqueue the chemical-potential solve for one moment vector without synchronising: buf
+// (fermi_doubles(quad_nodes(order), order) doubles, 16-byte aligned) and res (8 doubles: mu, Omega,
+// E, N, status) are device buffers.
 void fermi_enqueue(tbk_ctx* ctx, const double* moments, int order, double emin, double emax,
-                   double n_electrons, double mu_fixed, double kT, int damping, double* tab,
-                   double* rho, double* res) {
+                   double n_electrons, double mu_fixed, double kT, int damping, double* buf, double* res) {
   TBK_CHECK_ARG(order >= 1 && order <= (1 << 22), "order out of range");
   TBK_CHECK_ARG(kT > 0.0 && std::isfinite(kT), "kT must be positive");
   TBK_CHECK_ARG(emax > emin, "need emax > emin");
   const int M = quad_nodes(order);
-  cos_table<<<ceil_div(4 * (int64_t)M, 256), 256, 0, ctx->stream>>>(M, tab);
-  post_launch(ctx, "cos_table");
-  rho_kernel<<<ceil_div(M, 128), 128, 0, ctx->stream>>>(moments, order, M, damping, tab, rho);
-  post_launch(ctx, "rho_kernel");
-  fermi_kernel<<<1, 1024, 0, ctx->stream>>>(rho, M, emin, emax, n_electrons, mu_fixed, kT, res);
-  post_launch(ctx, "fermi_kernel");
+  const FermiJob j{M, order, emin, emax, n_electrons, mu_fixed, kT, 0, 0};
+  fermi_launch(ctx, 1, j, nullptr, M, order, moments, damping, buf, res);
+}
+
+void check_fermi_status(double status, const char* no_bracket) {
+  if (status == 2.0) throw Error(TBK_ERR_TIMEOUT, "a bounded wait in the chemical-potential solve expired");
+  if (status != 0.0) throw Error(TBK_ERR_NOCONV, no_bracket);
 }
 
 }  // namespace tbk
@@ -256,18 +388,14 @@ extern "C" int tbk_fermi_level(tbk_ctx* ctx, const double* moments, int32_t orde
   TBK_CHECK_ARG(damping == TBK_DAMP_NONE || damping == TBK_DAMP_JACKSON, "unknown damping");
   DeviceGuard dg(ctx);
   const int M = quad_nodes(order);
-  const double* tab = make_cos_table(ctx, M);
-  double* rho = (double*)scratch(ctx, WS_COEF, sizeof(double) * ((size_t)M + 8));
-  double* res = rho + M;
-  rho_kernel<<<ceil_div(M, 128), 128, 0, ctx->stream>>>(moments, order, M, damping, tab, rho);
-  post_launch(ctx, "rho_kernel");
-  fermi_kernel<<<1, 1024, 0, ctx->stream>>>(rho, M, emin, emax, n_electrons, mu_fixed, kT, res);
-  post_launch(ctx, "fermi_kernel");
+  const size_t nbuf = fermi_doubles(M, order);
+  double* buf = (double*)scratch(ctx, WS_COEF, sizeof(double) * (nbuf + 8));
+  double* res = buf + nbuf;
+  fermi_enqueue(ctx, moments, order, emin, emax, n_electrons, mu_fixed, kT, damping, buf, res);
   double h[5];
   TBK_CUDA(cudaMemcpyAsync(h, res, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
   sync(ctx);
   for (int i = 0; i < 4; ++i) out[i] = h[i];
-  if (h[4] != 0.0)
-    throw Error(TBK_ERR_NOCONV, "n_electrons is outside the range of the estimated N(mu) on [emin, emax]");
+  check_fermi_status(h[4], "n_electrons is outside the range of the estimated N(mu) on [emin, emax]");
   TBK_API_END
 }
