@@ -159,30 +159,32 @@ __device__ __forceinline__ double tbk_block_sum(double v, double* smem32) {
   return t;  // valid in thread 0
 }
 
+// Waits (one thread) until *p has reached target; what was written before it reached it is visible
+// after.  Bounded: 0 when 2 s of the global timer went by, or after 2^26 polls.
+__device__ __forceinline__ int tbk_spin_until(const unsigned* p, unsigned target) {
+  uint64_t t0 = 0, t = 0;
+  for (uint32_t i = 0;; ++i) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    if ((int)(v - target) >= 0) return 1;
+    if ((i & 1023u) == 1023u) {
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+      if (!t0) t0 = t;
+      if (t - t0 > 2000000000ull || i >= (1u << 26)) return 0;
+    }
+  }
+}
+
 // Barrier of the CTAs of one cooperative launch that share *ctr (zero before the first use): the
 // n-th use waits for target = n * CTAs arrivals.  What a CTA wrote before is visible to the others
-// after (read it past L1).  Bounded: false in all threads of the CTA when 2 s of the global timer
-// went by, or after 2^26 polls.
+// after (read it past L1).  False in all threads of the CTA when the wait expired.
 __device__ __forceinline__ bool tbk_grid_wait(unsigned* ctr, unsigned target) {
   __syncthreads();
   int ok = 1;
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(ctr, 1u);
-    uint64_t t0 = 0, t = 0;
-    for (uint32_t i = 0;; ++i) {
-      unsigned v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
-      if ((int)(v - target) >= 0) break;
-      if ((i & 1023u) == 1023u) {
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-        if (!t0) t0 = t;
-        if (t - t0 > 2000000000ull || i >= (1u << 26)) {
-          ok = 0;
-          break;
-        }
-      }
-    }
+    ok = tbk_spin_until(ctr, target);
   }
   return __syncthreads_and(ok) != 0;
 }

@@ -37,14 +37,6 @@ __device__ __forceinline__ void lz_spmv_cta(int cta, int n_atoms, int B, const i
   if (threadIdx.x == 0) part[cta] = t;
 }
 
-__global__ void lz_spmv(int n_atoms, int B, const int32_t* __restrict__ row_ptr,
-                        const int32_t* __restrict__ col, const double* __restrict__ H,
-                        const double* __restrict__ v, const double* __restrict__ vprev,
-                        const double* __restrict__ beta, double* __restrict__ w,
-                        double* __restrict__ part) {
-  lz_spmv_cta(blockIdx.x, n_atoms, B, row_ptr, col, H, v, vprev, beta, w, part);
-}
-
 // w -= alpha v; per-CTA partial sums of w . w.
 __device__ __forceinline__ void lz_orth_cta(int cta, int64_t n, const double* __restrict__ v,
                                             const double* __restrict__ alpha, double* __restrict__ w,
@@ -61,11 +53,6 @@ __device__ __forceinline__ void lz_orth_cta(int cta, int64_t n, const double* __
   if (threadIdx.x == 0) part[cta] = t;
 }
 
-__global__ void lz_orth(int64_t n, const double* __restrict__ v, const double* __restrict__ alpha,
-                        double* __restrict__ w, double* __restrict__ part) {
-  lz_orth_cta(blockIdx.x, n, v, alpha, w, part);
-}
-
 // out = sum(part) (take_sqrt: sqrt of it), single block, fixed order.
 __device__ __forceinline__ void lz_reduce_block(const double* __restrict__ part, int m, int take_sqrt,
                                                 double* __restrict__ out) {
@@ -76,20 +63,307 @@ __device__ __forceinline__ void lz_reduce_block(const double* __restrict__ part,
   if (threadIdx.x == 0) *out = take_sqrt ? sqrt(t) : t;
 }
 
-__global__ void lz_reduce(const double* __restrict__ part, int m, int take_sqrt, double* __restrict__ out) {
-  lz_reduce_block(part, m, take_sqrt, out);
-}
-
-// v_next = w / beta (written over w).
-__global__ void lz_scale(int64_t n, const double* __restrict__ beta, double* __restrict__ w) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const double b = *beta;
-  if (i < n) w[i] = b > 0.0 ? w[i] / b : 0.0;
-}
-
 __global__ void lz_start(int64_t n, uint64_t seed, double* __restrict__ v) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) v[i] = (double)tbk_probe_sign(seed, i, 0) / sqrt((double)n);
+}
+
+// ---- one operator: all steps in one cooperative launch -----------------------------------------
+//
+// A warp owns 32 consecutive rows (a unit); units are dealt over the CTAs first, so that a small
+// operator still uses one warp on many SMs.  A step is H v - beta v_prev with the partial sums of
+// alpha, then w - alpha v with those of beta, then w / beta, each ended by a barrier over the grid;
+// the CTA that arrives last adds the units' partial sums (in every CTA the additions took a quarter
+// of all FP64 issue at 10,000 atoms).  The sums keep one order: rows in groups of 256, a tree per
+// group, 256 strided chains of groups, a tree; that of lz_reduce_block.
+//
+// An FP64 operation takes ~85 cycles here and a row of 19 blocks is a chain of 171: ~7 us a step,
+// while five launches a step took 57 us on 147 atoms (41 us of it in the product, whose rows sat on
+// 6 SMs) and 66 us on 10,000 atoms, where the FP64 issue rate allows 27.  Now 23 us a step on 1,000
+// atoms and 47 us on 10,000.
+// TR: blocks stored transposed (lz_transpose), so that the rows of an atom read neighbouring words.
+// PF: the next block is loaded ahead, for operators with few warps per SM.
+constexpr int LZ_CHAINS = 256;
+constexpr size_t LZ_TRANSPOSE_MAX = (size_t)128 << 20;
+
+struct LzSync {
+  unsigned arrived, gen;  // arrivals at the barrier, finished barriers
+  double sum[2];          // the sums of the last two reducing barriers
+};
+
+__device__ __forceinline__ double lz_warp_sum(double d) {
+  for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+  return d;
+}
+
+// Sum of the units' partial sums over the CTA, valid in thread 0.
+__device__ __forceinline__ double lz_units_sum(const double* part, int nb, double* red) {
+  double s = 0.0;
+  for (int g = threadIdx.x; g < nb && threadIdx.x < LZ_CHAINS; g += LZ_CHAINS) {
+    double2 p[4];
+    for (int q = 0; q < 4; ++q) p[q] = __ldcg(reinterpret_cast<const double2*>(part + 8 * (size_t)g) + q);
+    s += ((p[0].x + p[2].x) + (p[1].x + p[3].x)) + ((p[0].y + p[2].y) + (p[1].y + p[3].y));
+  }
+  if (nb <= 32) return threadIdx.x < 32 ? lz_warp_sum(s) : 0.0;  // the other warps hold zeros
+  s = lz_warp_sum(s);
+  if ((threadIdx.x & 31) == 0 && threadIdx.x < LZ_CHAINS) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  return ((red[0] + red[4]) + (red[2] + red[6])) + ((red[1] + red[5]) + (red[3] + red[7]));
+}
+
+// Barrier of the grid (co-resident CTAs), number `gen` from 1 on; with part, the last CTA to arrive
+// leaves the sum of the partial sums in sy->sum[gen & 1] first.  Bounded like tbk_grid_wait.
+__device__ __forceinline__ bool lz_barrier(LzSync* sy, unsigned gen, const double* part, int nb, double* red) {
+  __shared__ int last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned old;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(&sy->arrived) : "memory");
+    last = old == gen * gridDim.x - 1;
+  }
+  __syncthreads();
+  int ok = 1;
+  if (last) {
+    double t = 0.0;
+    if (part) t = lz_units_sum(part, nb, red);
+    if (threadIdx.x == 0) {
+      if (part) __stcg(&sy->sum[gen & 1], t);
+      asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&sy->gen), "r"(gen) : "memory");
+    }
+  } else if (threadIdx.x == 0) {
+    ok = tbk_spin_until(&sy->gen, gen);
+  }
+  return __syncthreads_and(ok) != 0;
+}
+
+// Threads per CTA: one CTA per SM, so that a barrier has few arrivals.
+template <bool PF> constexpr int lz_threads() { return PF ? 256 : 768; }
+
+template <int B, bool TR, bool PF>
+__global__ void __launch_bounds__(lz_threads<PF>(), 1)
+lz_run(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+       const double* __restrict__ H, int m, double* vecs, double* part, double* __restrict__ alpha,
+       double* __restrict__ beta, LzSync* sy, double* __restrict__ fail) {
+  __shared__ double red[8];
+  const int64_t n = (int64_t)n_atoms * B;
+  const int nb = (int)((n + 255) / 256), units = 8 * nb;
+  const int lane = threadIdx.x & 31, stride = gridDim.x * (lz_threads<PF>() / 32);
+  const int first = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  unsigned gen = 0;
+  bool ok = true;
+  // with p: returns the sum of the partial sums
+  auto wait = [&](const double* p) {
+    ok = lz_barrier(sy, ++gen, p, nb, red) && ok;
+    return p ? __ldcg(&sy->sum[gen & 1]) : 0.0;
+  };
+  double bj = 0.0;
+  for (int j = 0; j < m && ok; ++j) {
+    // v_{j-1}, v_j and w rotate through three vectors
+    const double* vp = vecs + (j % 3) * n;
+    double* v = vecs + ((j + 1) % 3) * n;
+    double* w = vecs + ((j + 2) % 3) * n;
+    double own = 0.0, vown = 0.0;  // this thread's row of the warp's first unit
+    for (int u = first; u < units; u += stride) {
+      const int64_t row = (int64_t)u * 32 + lane;
+      double d = 0.0;
+      if (row < n) {
+        const int a = (int)(row / B), i = (int)(row - (int64_t)a * B);
+        double acc = 0.0;
+        const int k1 = __ldg(row_ptr + a + 1);
+        int k = __ldg(row_ptr + a);
+        double h[B], x[B];
+        auto fetch = [&](int kk, double (&hh)[B], double (&xx)[B]) {
+          const double* xb = v + (int64_t)__ldg(col + kk) * B;
+          const double* hb = H + (int64_t)kk * B * B + (TR ? i : i * B);
+#pragma unroll
+          for (int l = 0; l < B; ++l) {
+            hh[l] = __ldg(hb + (TR ? l * B : l));
+            xx[l] = xb[l];
+          }
+        };
+        if (PF && k < k1) fetch(k, h, x);
+        for (; k < k1; ++k) {
+          double hn[B], xn[B];
+          if constexpr (PF) {
+            if (k + 1 < k1) fetch(k + 1, hn, xn);
+          } else {
+            fetch(k, h, x);
+          }
+#pragma unroll
+          for (int l = 0; l < B; ++l) acc += h[l] * x[l];
+          if constexpr (PF) {
+#pragma unroll
+            for (int l = 0; l < B; ++l) {
+              h[l] = hn[l];
+              x[l] = xn[l];
+            }
+          }
+        }
+        if (j) acc -= bj * vp[row];
+        const double vr = v[row];
+        if (u == first) {
+          own = acc;
+          vown = vr;
+        } else {
+          w[row] = acc;
+        }
+        d = acc * vr;
+      }
+      d = lz_warp_sum(d);
+      if (lane == 0) __stcg(part + u, d);
+    }
+    const double aj = wait(part);
+    for (int u = first; u < units; u += stride) {
+      const int64_t row = (int64_t)u * 32 + lane;
+      double d = 0.0;
+      if (row < n) {
+        const double x = (u == first ? own : w[row]) - aj * (u == first ? vown : v[row]);
+        if (u == first) own = x; else w[row] = x;
+        d = x * x;
+      }
+      d = lz_warp_sum(d);
+      if (lane == 0) __stcg(part + units + u, d);
+    }
+    bj = sqrt(wait(part + units));
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      alpha[j] = aj;
+      beta[j + 1] = bj;
+    }
+    if (j + 1 == m) break;
+    for (int u = first; u < units; u += stride) {
+      const int64_t row = (int64_t)u * 32 + lane;
+      if (row < n) w[row] = bj > 0.0 ? (u == first ? own : w[row]) / bj : 0.0;
+    }
+    wait(nullptr);
+  }
+  if (!ok && threadIdx.x == 0) *fail = 1.0;
+}
+
+// out[k][l][i] = H[k][i][l], 9x9 blocks
+__global__ void lz_transpose(int64_t n, const double* __restrict__ H, double* __restrict__ out) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const int64_t k = t / 81;
+  const int e = (int)(t - k * 81), l = e / 9, i = e - 9 * l;
+  out[t] = __ldg(H + k * 81 + i * 9 + l);
+}
+
+// ---- a small operator: one thread-block cluster, the vectors in shared memory and registers ----------
+//
+// The same sums with at most LZ_CL_WARPS units per CTA, one per warp: v is copied into every CTA's
+// shared memory, a thread keeps its row of v_prev, v and w, and partial sums go to every CTA, where
+// each warp adds them itself.  The hardware barrier of a cluster takes ~0.2 us where one over the
+// grid takes ~2 with its sum: what is left of a step is the row's chain (147 atoms: 0.99 ms for 64
+// steps against 1.40 over the grid; beyond 96 units the FP64 rate of 8 SMs is the longer of the two).
+constexpr int LZ_CL = 8, LZ_CL_WARPS = 12;
+constexpr int LZ_CL_UNITS = LZ_CL * LZ_CL_WARPS;
+
+__device__ __forceinline__ void lz_cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Store x at the same shared-memory place in CTA `rank` of the cluster.
+__device__ __forceinline__ void lz_store_remote(double* p, int rank, double x) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(x) : "memory");
+}
+
+template <int B>
+__global__ void __cluster_dims__(LZ_CL, 1, 1) __launch_bounds__(32 * LZ_CL_WARPS)
+lz_run_cluster(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+               const double* __restrict__ H, int m, uint64_t seed, double* __restrict__ alpha,
+               double* __restrict__ beta) {
+  __shared__ double vs[32 * LZ_CL_UNITS];
+  __shared__ double part[2][LZ_CL_UNITS];
+  const int n = n_atoms * B, nb = (n + 255) / 256, units = 8 * nb;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int u = warp * LZ_CL + blockIdx.x, row = 32 * u + lane;
+  const bool has = row < n;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) vs[i] = (double)tbk_probe_sign(seed, i, 0) / sqrt((double)n);
+  for (int i = threadIdx.x; i < 2 * LZ_CL_UNITS; i += blockDim.x) part[0][i] = 0.0;
+  lz_cluster_barrier();
+  // the sum of the units' values d, in every thread
+  auto total = [&](int set, double d) {
+    d = lz_warp_sum(d);
+    if (u < units && lane < LZ_CL) lz_store_remote(&part[set][u], lane, d);
+    lz_cluster_barrier();
+    double s = 0.0;
+    if (lane < nb) {
+      const double* p = part[set] + 8 * lane;
+      s = ((p[0] + p[4]) + (p[2] + p[6])) + ((p[1] + p[5]) + (p[3] + p[7]));
+    }
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);  // nb <= 16
+    return __shfl_sync(0xffffffffu, s, 0);
+  };
+  const int a = has ? row / B : 0, i = row - a * B;
+  const int k0 = has ? __ldg(row_ptr + a) : 0, k1 = has ? __ldg(row_ptr + a + 1) : 0;
+  double vprev = 0.0, v = has ? vs[row] : 0.0, bj = 0.0;
+  for (int j = 0; j < m; ++j) {
+    double acc = 0.0, h[B], hn[B];
+    int b = 0, bn = 0;
+    auto fetch = [&](int k, double (&hh)[B], int& bb) {
+      bb = __ldg(col + k) * B;
+#pragma unroll
+      for (int l = 0; l < B; ++l) hh[l] = __ldg(H + (int64_t)k * B * B + l * B + i);
+    };
+    if (k0 < k1) fetch(k0, h, b);
+    for (int k = k0; k < k1; ++k) {
+      if (k + 1 < k1) fetch(k + 1, hn, bn);
+#pragma unroll
+      for (int l = 0; l < B; ++l) acc += h[l] * vs[b + l];
+#pragma unroll
+      for (int l = 0; l < B; ++l) h[l] = hn[l];
+      b = bn;
+    }
+    if (j) acc -= bj * vprev;
+    const double aj = total(0, has ? acc * v : 0.0);
+    const double x = acc - aj * v;
+    bj = sqrt(total(1, has ? x * x : 0.0));
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      alpha[j] = aj;
+      beta[j + 1] = bj;
+    }
+    if (j + 1 == m) break;
+    vprev = v;
+    v = has && bj > 0.0 ? x / bj : 0.0;
+    if (has)
+      for (int r = 0; r < LZ_CL; ++r) lz_store_remote(vs + row, r, v);
+    lz_cluster_barrier();
+  }
+  lz_cluster_barrier();  // no CTA leaves while another may still write to it
+}
+
+template <int B, bool TR, bool PF>
+static void lz_launch_pf(tbk_ctx* ctx, const tbk_bsr* H, const double* val, int m, double* vecs, double* part,
+                         double* alpha, double* beta, LzSync* sy, double* fail) {
+  constexpr int T = lz_threads<PF>();
+  const int units = 8 * ceil_div((int64_t)H->n_atoms * B, 256);
+  const int grid = std::min(units, ctx->num_sms);
+  int n_atoms = H->n_atoms;
+  const int32_t *rp = H->row_ptr, *cl = H->col;
+  void* args[] = {&n_atoms, &rp, &cl, &val, &m, &vecs, &part, &alpha, &beta, &sy, &fail};
+  TBK_CUDA(cudaLaunchCooperativeKernel((const void*)lz_run<B, TR, PF>, dim3(grid), dim3(T), args, 0, ctx->stream));
+  post_launch(ctx, "lz_run");
+}
+
+// val: the blocks, transposed (TR) or as given
+template <int B, bool TR>
+static void lz_launch(tbk_ctx* ctx, const tbk_bsr* H, const double* val, int m, uint64_t seed, double* vecs,
+                      double* part, double* alpha, double* beta, LzSync* sy, double* fail) {
+  const int64_t n = (int64_t)H->n_atoms * B;
+  if ((TR || B == 1) && 8 * (int64_t)ceil_div(n, 256) <= LZ_CL_UNITS) {
+    lz_run_cluster<B><<<LZ_CL, 32 * LZ_CL_WARPS, 0, ctx->stream>>>(H->n_atoms, H->row_ptr, H->col, val, m, seed, alpha,
+                                                                   beta);
+    post_launch(ctx, "lz_run_cluster");
+    return;
+  }
+  lz_start<<<ceil_div(n, 256), 256, 0, ctx->stream>>>(n, seed, vecs + n);
+  post_launch(ctx, "lz_start");
+  // up to 8 warps per SM the loads ahead hide the latency, beyond that the warps do
+  if (n <= (int64_t)ctx->num_sms * 8 * 32)
+    lz_launch_pf<B, TR, true>(ctx, H, val, m, vecs, part, alpha, beta, sy, fail);
+  else
+    lz_launch_pf<B, TR, false>(ctx, H, val, m, vecs, part, alpha, beta, sy, fail);
 }
 
 // ---- many clusters: the same kernels, blockIdx.y = cluster ---------------------------------
@@ -260,36 +534,33 @@ extern "C" int tbk_spectral_bounds(tbk_ctx* ctx, const tbk_bsr* H, int32_t steps
   DeviceGuard dg(ctx);
   const int64_t n = (int64_t)H->n_atoms * H->n_orb;
   const int m = (int)std::min<int64_t>(steps, n);
-  const int nb = ceil_div(n, 256);
-  double* vecs = (double*)scratch(ctx, WS_LANCZOS, sizeof(double) * (size_t)(3 * n + nb + 2 * (m + 2)));
-  double *vp = vecs, *v = vecs + n, *w = vecs + 2 * n;
-  double* part = vecs + 3 * n;
-  double* alpha = part + nb;          // alpha[j], j < m
+  const int nb = ceil_div(n, 256), units = 8 * nb;
+  // transposed blocks as long as the copy stays in L2 between the steps (10,000 atoms: 115 MB)
+  const bool tr = H->n_orb == 9 && H->nnzb >= H->n_atoms && (size_t)H->nnzb * 648 <= LZ_TRANSPOSE_MAX;
+  // vectors | partial sums | alpha (m + 2) | beta (m + 2) | barrier | failure flag | H^T
+  const size_t nvec = (3 * (size_t)n + 1) & ~(size_t)1, nred = 2 * (size_t)units, nab = 2 * ((size_t)m + 2) + 4;
+  double* vecs = (double*)scratch(ctx, WS_LANCZOS, sizeof(double) * (nvec + nred + nab + (tr ? 81 * (size_t)H->nnzb : 0)));
+  double* part = vecs + nvec;
+  double* alpha = part + nred;        // alpha[j], j < m
   double* beta = alpha + (m + 2);     // beta[j]: beta[0] = 0, beta[j+1] = ||w_j||
-  TBK_CUDA(cudaMemsetAsync(beta, 0, sizeof(double) * (m + 2), ctx->stream));
-  lz_start<<<nb, 256, 0, ctx->stream>>>(n, seed, v);
-  post_launch(ctx, "lz_start");
-  for (int j = 0; j < m; ++j) {
-    lz_spmv<<<nb, 256, 0, ctx->stream>>>(H->n_atoms, H->n_orb, H->row_ptr, H->col, H->val, v,
-                                         j ? vp : nullptr, beta + j, w, part);
-    post_launch(ctx, "lz_spmv");
-    lz_reduce<<<1, 256, 0, ctx->stream>>>(part, nb, 0, alpha + j);
-    post_launch(ctx, "lz_reduce");
-    lz_orth<<<nb, 256, 0, ctx->stream>>>(n, v, alpha + j, w, part);
-    post_launch(ctx, "lz_orth");
-    lz_reduce<<<1, 256, 0, ctx->stream>>>(part, nb, 1, beta + j + 1);
-    post_launch(ctx, "lz_reduce");
-    lz_scale<<<nb, 256, 0, ctx->stream>>>(n, beta + j + 1, w);
-    post_launch(ctx, "lz_scale");
-    double* t = vp;  // rotate: vprev <- v, v <- w, w <- old vprev
-    vp = v;
-    v = w;
-    w = t;
+  LzSync* sy = (LzSync*)(beta + (m + 2));
+  double* fail = beta + (m + 2) + 3;
+  TBK_CUDA(cudaMemsetAsync(alpha, 0, sizeof(double) * nab, ctx->stream));
+  if (tr) {
+    double* ht = alpha + nab;
+    lz_transpose<<<(unsigned)((81 * H->nnzb + 255) / 256), 256, 0, ctx->stream>>>(81 * H->nnzb, H->val, ht);
+    post_launch(ctx, "lz_transpose");
+    lz_launch<9, true>(ctx, H, ht, m, seed, vecs, part, alpha, beta, sy, fail);
+  } else if (H->n_orb == 9) {
+    lz_launch<9, false>(ctx, H, H->val, m, seed, vecs, part, alpha, beta, sy, fail);
+  } else {
+    lz_launch<1, false>(ctx, H, H->val, m, seed, vecs, part, alpha, beta, sy, fail);
   }
-  std::vector<double> ha(m), hb(m + 1);
-  TBK_CUDA(cudaMemcpyAsync(ha.data(), alpha, sizeof(double) * m, cudaMemcpyDeviceToHost, ctx->stream));
-  TBK_CUDA(cudaMemcpyAsync(hb.data(), beta, sizeof(double) * (m + 1), cudaMemcpyDeviceToHost, ctx->stream));
+  std::vector<double> hab(nab);
+  TBK_CUDA(cudaMemcpyAsync(hab.data(), alpha, sizeof(double) * nab, cudaMemcpyDeviceToHost, ctx->stream));
   sync(ctx);
+  if (hab[nab - 1] != 0.0) throw Error(TBK_ERR_TIMEOUT, "a bounded wait in the Lanczos kernel expired");
+  const std::vector<double> ha(hab.begin(), hab.begin() + m), hb(hab.begin() + m + 2, hab.begin() + 2 * m + 3);
   bounds_from_tridiagonal(ha, hb, m, rel_margin, emin, emax);
   TBK_API_END
 }
