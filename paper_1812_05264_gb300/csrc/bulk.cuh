@@ -74,6 +74,10 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
 }
 
 
+// A kernel launched with launch_pdl may start before its predecessor in the stream has finished; it
+// reads and writes nothing in global memory before this, which returns when the predecessor has.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // One neighbour tile of the FP32 block product with packed f32x2 FMAs:
 //   acc(i, v) += H^[i][l] * x[l][v]   for l = 0..8,
 // X: 9 x P tile in shared memory, Hs: column-major block (columns padded to 12 floats), pl: the

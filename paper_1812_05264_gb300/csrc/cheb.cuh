@@ -42,7 +42,7 @@ inline void check_diagonal_flag(int herr) {
 HOp prepare_hop(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, int prec, Slot slot, int* err);
 
 // One fused step over all rows and probes:
-//   y_out = alpha * (H^ y_in) + c_r * r - y_prev
+//   y_out = alpha * (H^ y_in) + c_r * r - y_prev  (+ sum_e csrc_e * src_e)
 // where y_in is a panel or (cur_is_probe) the probe block r regenerated from the seed, and the
 // y_prev term is present only when `yprev` is not NULL.  `yout` may equal `yprev` (in-place
 // update: each element is read and then written by the same thread).
@@ -66,6 +66,9 @@ struct StepArgs {
   uint64_t seed = 0;
   int s = 0;
   int direct = 0;
+  // further own-row terms c_e E_e of y_out (E_e a panel), plain and row-split kernels only
+  const void* src[3] = {nullptr, nullptr, nullptr};
+  double csrc[3] = {0.0, 0.0, 0.0};
   double* partials = nullptr;
   int* err = nullptr;       // device flag raised (= 2) when a bounded wait expires
   int force_simple = 0;     // use the plain load/FMA kernel even where the TMA-fed one applies
@@ -74,6 +77,7 @@ struct StepArgs {
   BatchRows batch;
   int per_task = 0;
   int use_tc = 0;           // tensor-core (tcgen05) step where it applies
+  int grid = 0;             // CTAs of the launch (0: step_grid_ctas)
 };
 // Consumer warps of the TMA-fed step kernel for this operator and probe count (0 = not used).
 int bulk_consumer_warps(const HOp& op, int s);

@@ -94,6 +94,26 @@ struct KernelTimerScope {
   ~KernelTimerScope();
 };
 
+// Launch with programmatic stream serialization: the launch is prepared while its predecessor in the
+// stream runs and starts as that one's CTAs leave; the kernel must call pdl_wait() (bulk.cuh) before it
+// touches anything.  2-3 us less a step in a chain of short launches.  (A predecessor that lets the
+// next launch in while its own CTAs still run made it worse: the early CTAs double up on some SMs.
+// 1,000 atoms x 256 probes 28.6 us a step against 23.4, 200 atoms x 64 in FP64 92 against 37.)
+template <typename... P, typename... A>
+inline void launch_pdl(tbk_ctx* ctx, void (*kernel)(P...), int grid, int threads, size_t smem, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = ctx->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  TBK_CUDA(cudaLaunchKernelEx(&cfg, kernel, (P)args...));
+}
+
 inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
 // One chemical-potential solve: M quadrature nodes, order p, moments at mom_off, its scratch of

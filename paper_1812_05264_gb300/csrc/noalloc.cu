@@ -88,15 +88,23 @@ extern "C" int tbk_chebyshev_moments_noalloc(tbk_ctx* ctx, const tbk_bsr* H, dou
   shape.n_atoms = H->n_atoms;
   shape.n_rows = n_rows;    // the grid follows any tuned choice for this shape, as the steps do
   shape.nnzb = H->nnzb;
-  const int nctas = step_grid_ctas(ctx, shape, s);
+  int nctas = step_grid_ctas(ctx, shape, s);
   // layout: flag | sums | partials | mapped H | panel A | panel B, each 256-byte aligned
   const size_t o_flag = 0;
   const size_t o_sums = o_flag + 256;
   const size_t o_part = o_sums + align256(sizeof(double) * 2 * (size_t)std::max(1, K) + 64);
-  const size_t o_hhat = o_part + align256(sizeof(double) * 2 * (size_t)std::max(1, K) * nctas);
-  const size_t o_pa = o_hhat + align256(mapped_h_bytes(H, prec));
-  const size_t o_pb = o_pa + (K >= 1 ? align256(panel) : 0);
-  const size_t need = o_pb + (K >= 2 ? align256(panel) : 0);
+  size_t o_hhat, o_pa, o_pb, need;
+  auto place = [&]() {
+    o_hhat = o_part + align256(sizeof(double) * 2 * (size_t)std::max(1, K) * nctas);
+    o_pa = o_hhat + align256(mapped_h_bytes(H, prec));
+    o_pb = o_pa + (K >= 1 ? align256(panel) : 0);
+    need = o_pb + (K >= 2 ? align256(panel) : 0);
+  };
+  place();
+  if (need > kStaticScratchBytes && nctas > ctx->num_sms) {
+    nctas = ctx->num_sms;  // fewer CTAs leave fewer partial sums
+    place();
+  }
   if (need > kStaticScratchBytes)
     throw Error(TBK_ERR_ARG, "tbk_chebyshev_moments_noalloc: this problem needs " +
                                  std::to_string(need) + " bytes of scratch, above the static limit of " +
@@ -119,6 +127,7 @@ extern "C" int tbk_chebyshev_moments_noalloc(tbk_ctx* ctx, const tbk_bsr* H, dou
     a.partials = partials + (size_t)(j - 1) * nctas * 2;
     a.err = flag;
     a.force_simple = (flags & TBK_PLAIN_KERNEL) ? 1 : 0;
+    a.grid = nctas;
     if (j == 1) {
       a.cur_is_probe = 1;
       a.alpha = 1.0;

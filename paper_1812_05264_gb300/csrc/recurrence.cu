@@ -111,12 +111,19 @@ HOp prepare_hop(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, int pr
 
 constexpr int STEP_THREADS = 128;
 
+// Further own-row terms of a step: sum_e c[e] p[e] (p[e] NULL: none).
+template <typename T>
+struct StepSources {
+  const T* p[3];
+  T c[3];
+};
+
 template <typename T, int B, bool PROBE_IN>
 __global__ void __launch_bounds__(STEP_THREADS)
 cheb_step_kernel(const int n_atoms, const int32_t* __restrict__ row_ptr,
                  const int32_t* __restrict__ col, const T* __restrict__ hv,
                  const T* __restrict__ yin, const T* yprev, T* yout, const T alpha,
-                 const T c_r, const uint64_t seed, const int s, const int direct,
+                 const T c_r, const uint64_t seed, const int s, const int direct, const StepSources<T> src,
                  double* __restrict__ partials) {
   constexpr int VEC = Vec16<T>::N;
   constexpr int RS = Layout<T, B>::RS, BS = Layout<T, B>::BS;
@@ -200,6 +207,14 @@ cheb_step_kernel(const int n_atoms, const int32_t* __restrict__ row_ptr,
 #pragma unroll
           for (int v = 0; v < VEC; ++v) yo[v] -= t[v];
         }
+#pragma unroll
+        for (int e = 0; e < 3; ++e)
+          if (src.p[e]) {
+            T t[VEC];
+            ldg16(src.p[e] + off, t);
+#pragma unroll
+            for (int v = 0; v < VEC; ++v) yo[v] = fma(src.c[e], t[v], yo[v]);
+          }
         st16(yout + off, yo);
         if (partials) {
           T xin[VEC];
@@ -301,6 +316,7 @@ cheb_step_bulk(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  pdl_wait();
 
   if (warp == CW) {
     // ---------------- producer ----------------
@@ -500,7 +516,9 @@ cheb_step_bulk(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
 // R tiles in flight and, as soon as the warp has finished with a stage, refills it with the tile
 // R positions ahead in the CTA's tile sequence (its tasks' neighbour tiles, then the y_prev tile
 // of each task).  With 128 probes a task is quickly done, so a CTA that spends half its warps
-// and registers on a producer limits how many consumers an SM holds.
+// and registers on a producer limits how many consumers an SM holds.  The last chunk of a probe
+// count that is no multiple of 128 is narrower: its rows are copied as far as they go, and the
+// lanes past the end compute on what the ring holds and store nothing.
 template <int R>
 struct SelfCfg {
   static constexpr int P = 128;
@@ -510,7 +528,7 @@ struct SelfCfg {
   static constexpr int SMEM = R * SB + 8 * R;
 };
 
-template <int R>
+template <int R, bool NARROW>
 __global__ void __launch_bounds__(32)
 cheb_step_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const float* __restrict__ hv, const float* __restrict__ yin, const float* yprev,
@@ -522,7 +540,8 @@ cheb_step_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
   const uint32_t bar0 = smem_u32(smem + R * C::SB);
   auto full = [&](int i) { return bar0 + 8u * i; };
   const int lane = threadIdx.x;
-  const int n_chunks = s / C::P;
+  const int n_chunks = NARROW ? 1 : s / C::P;
+  const int P = NARROW ? s : C::P;  // floats between the rows of a tile
   const int n_tasks = n_atoms * n_chunks;
   const bool has_prev = yprev != nullptr;
   if (lane == 0) {
@@ -530,6 +549,7 @@ cheb_step_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
+  pdl_wait();
   // producer cursor (lane 0): the next tile to issue, as (task, tile index within the task)
   int p_task = blockIdx.x, p_q = 0, p_nt = 0, p_k0 = 0, issued = 0;
   auto load_task = [&]() {  // tasks with no tile (an empty row, no y_{k-1}) are skipped
@@ -549,9 +569,10 @@ cheb_step_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
     const uint32_t dst = smem_u32(smem + st * C::SB), bar = full(st);
     const float* src = (is_prev ? yprev : yin) + (int64_t)9 * b * s + (int64_t)ch * C::P;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_expect_tx(bar, C::XB + (is_prev ? 0 : C::HB));
-    if (s == C::P) {
-      bulk_g2s(dst, src, C::XB, bar);  // the 9 rows are contiguous
+    const int xb = NARROW ? 36 * s : C::XB;
+    mbar_expect_tx(bar, xb + (is_prev ? 0 : C::HB));
+    if (NARROW || s == C::P) {
+      bulk_g2s(dst, src, xb, bar);  // the 9 rows are contiguous
     } else {
       for (int l = 0; l < 9; ++l) bulk_g2s(dst + l * C::P * 4, src + (int64_t)l * s, C::P * 4, bar);
     }
@@ -594,7 +615,7 @@ cheb_step_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
       }
       rdy = mbar_test(full((it + 1) % R), ((it + 1) / R) & 1);
       const unsigned char* base = smem + st * C::SB;
-      spmm_tile_f2_pp(reinterpret_cast<const float*>(base), reinterpret_cast<const float*>(base + C::XB), C::P,
+      spmm_tile_f2_pp(reinterpret_cast<const float*>(base), reinterpret_cast<const float*>(base + C::XB), P,
                       pl, acc);
       consumed();
     }
@@ -610,12 +631,13 @@ cheb_step_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
       const float* X = reinterpret_cast<const float*>(smem + st * C::SB);
 #pragma unroll
       for (int l = 0; l < 9; ++l) {
-        const float4 t = *reinterpret_cast<const float4*>(X + l * C::P + pl);
+        const float4 t = *reinterpret_cast<const float4*>(X + l * P + pl);
         yp[l][0] = t.x; yp[l][1] = t.y; yp[l][2] = t.z; yp[l][3] = t.w;
       }
       consumed();
     }
     const int p0 = ch * C::P + pl;
+    if (NARROW && p0 >= s) continue;
     uint64_t sd = seed;
     int64_t rloc = (int64_t)9 * a;
     if (batch.atom_cl) {
@@ -698,6 +720,290 @@ cheb_step_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
   }
 }
 
+// Sum of the consumer threads' partial sums into the CTA's slot (fixed order; the producer warp has
+// returned or does not take part).
+__device__ __forceinline__ void step_partials(double* __restrict__ partials, double sum0, double sum1, int warp,
+                                              int lane, int nw) {
+  __shared__ double red[2][32];
+  for (int o = 16; o > 0; o >>= 1) {
+    sum0 += __shfl_xor_sync(0xffffffffu, sum0, o);
+    sum1 += __shfl_xor_sync(0xffffffffu, sum1, o);
+  }
+  if (lane == 0) {
+    red[0][warp] = sum0;
+    red[1][warp] = sum1;
+  }
+  asm volatile("bar.sync 1, %0;" ::"r"(32 * nw) : "memory");
+  if (threadIdx.x == 0) {
+    double a0 = 0.0, a1 = 0.0;
+    for (int w = 0; w < nw; ++w) {
+      a0 += red[0][w];
+      a1 += red[1][w];
+    }
+    partials[2 * blockIdx.x] = a0;
+    partials[2 * blockIdx.x + 1] = a1;
+  }
+}
+
+// ---- one probe per lane: FP32 steps with little work per SM ------------------------------------------
+//
+// A task is a block row and a chunk of up to 512 probes; each consumer warp takes 32 probes, one per
+// lane and all nine rows.  Where the chip is not full, a step lasts as long as one row does, and a
+// row's time is that of a warp's instructions: a quarter of the self-fed kernel's per tile, with up
+// to 8 tiles in flight instead of two.  A chunk is the whole panel width where that fits, so that a
+// tile is one contiguous copy (nine row copies a tile cost 0.3 us more).  Per element the sums are
+// the other kernels'.  The epilogue goes through shared memory to items of one row and four probes,
+// so that panels are read and written 16 bytes at a time and the moment products add the same four
+// probes as in the other kernels.  147 atoms x 128 probes: 8.3 us a step against 18.5 (self-fed
+// kernel), 333 x 100: 9.7 against 22 (plain kernel, whose loads wait one after the other).
+template <int NW>  // consumer warps at most: 4, 8 or 16
+struct LaneCfg {
+  static constexpr int R = NW == 16 ? 5 : 8;
+  static constexpr int P = 32 * NW;
+  static constexpr int XB = 9 * P * 4;
+  static constexpr int HB = Layout<float, 9>::BS * 4;
+  static constexpr int SB = ((XB + HB + 127) / 128) * 128;
+  static constexpr int EB = 9 * 32 * 4;  // epilogue buffer of a warp
+  static constexpr int SMEM = R * SB + NW * EB + 16 * R;
+};
+
+template <int NW>
+__global__ void __launch_bounds__(32 * (NW + 1))
+cheb_step_lane(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+               const float* __restrict__ hv, const float* __restrict__ yin, const float* yprev, float* yout,
+               const float alpha, const float c_r, const uint64_t seed, const int s, const int direct,
+               double* __restrict__ partials, int* __restrict__ err, const int stall) {
+  using C = LaneCfg<NW>;
+  constexpr int R = C::R;
+  extern __shared__ __align__(128) unsigned char smem[];
+  const uint32_t bar0 = smem_u32(smem + R * C::SB + NW * C::EB);
+  auto full = [&](int i) { return bar0 + 8u * i; };
+  auto empty = [&](int i) { return bar0 + 8u * (R + i); };
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (blockDim.x >> 5) - 1;
+  const int n_chunks = (s + C::P - 1) / C::P, n_tasks = n_atoms * n_chunks;
+  const int P = n_chunks == 1 ? s : C::P;  // floats between the rows of a tile
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < R; ++i) {
+      mbar_init(full(i), 1);
+      mbar_init(empty(i), nw);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  pdl_wait();
+
+  if (warp == nw) {
+    // producer: lanes fetch the column indices 32 at a time, lane 0 waits for the stage, one copy per
+    // lane (stall: a test of the bounded waits; nothing is copied, the consumers give up and report)
+    int st = 0, ph = 1, issued = 0, ok = !stall;
+    for (int task = blockIdx.x; task < n_tasks && ok; task += gridDim.x) {
+      const int a = task / n_chunks, ch = task - a * n_chunks;
+      const int k0 = __ldg(row_ptr + a), k1 = __ldg(row_ptr + a + 1);
+      const int wb = 4 * min(C::P, s - ch * C::P);  // bytes of a tile row
+      for (int kb = k0; kb < k1 && ok; kb += 32) {
+        const int mine = kb + lane < k1 ? __ldg(col + kb + lane) : 0;
+        for (int k = kb; k < min(kb + 32, k1); ++k) {
+          const int b = __shfl_sync(0xffffffffu, mine, k - kb);
+          const uint32_t dst = smem_u32(smem + st * C::SB), bar = full(st);
+          if (lane == 0) {
+            ok = mbar_wait(empty(st), ph);
+            if (ok) mbar_expect_tx(bar, 9 * wb + C::HB);
+          }
+          ok = __shfl_sync(0xffffffffu, ok, 0);
+          if (!ok) break;
+          const float* x = yin + (int64_t)9 * b * s + (int64_t)ch * C::P;
+          if (lane == 9) bulk_g2s(dst + C::XB, hv + (int64_t)k * Layout<float, 9>::BS, C::HB, bar);
+          if (n_chunks == 1) {
+            if (lane == 0) bulk_g2s(dst, x, 9 * wb, bar);  // the 9 rows are contiguous
+          } else if (lane < 9) {
+            bulk_g2s(dst + lane * 4 * C::P, x + (int64_t)lane * s, wb, bar);
+          }
+          ++issued;
+          if (++st == R) st = 0, ph ^= 1;
+        }
+      }
+    }
+    if (!ok && !stall && lane == 0) {
+      // let the copies in flight land before the CTA exits
+      atomicOr(err, 2);
+      for (int j = (issued > R ? issued - R : 0); j < issued; ++j) mbar_wait(full(j % R), (j / R) & 1);
+    }
+    return;
+  }
+
+  float* ep = reinterpret_cast<float*>(smem + R * C::SB + warp * C::EB);  // 9 x 32
+  const int pl = 32 * warp + lane;  // this lane's probe in the chunk
+  // items of the epilogue: row irow[j], probes 4 igrp .. 4 igrp + 3 of the warp's 32
+  const int igrp = lane & 7, irow = lane >> 3;  // item j: row irow + 4 j, j < 3
+  float cs0 = 0.f, cc0 = 0.f, cs1 = 0.f, cc1 = 0.f;  // compensated partial sums
+  int st = 0, ph = 0;
+  bool ok = true;
+  for (int task = blockIdx.x; task < n_tasks && ok; task += gridDim.x) {
+    const int a = task / n_chunks, ch = task - a * n_chunks;
+    const int k0 = __ldg(row_ptr + a), nb = __ldg(row_ptr + a + 1) - k0;
+    const int p0 = ch * C::P + 32 * warp + 4 * igrp;  // the items' first probe
+    // the items' y_prev and own y_in, fetched while the tiles stream
+    float4 yp[3], xo[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const bool has = irow + 4 * j < 9 && p0 < s;
+      const int64_t off = ((int64_t)9 * a + irow + 4 * j) * s + p0;
+      yp[j] = has && yprev ? *reinterpret_cast<const float4*>(yprev + off) : make_float4(0.f, 0.f, 0.f, 0.f);
+      xo[j] = has && partials && !direct ? *reinterpret_cast<const float4*>(yin + off) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float2 acc[4];  // rows (0, 1), (2, 3), (4, 5), (6, 7)
+    float acc8 = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j] = make_float2(0.f, 0.f);
+    for (int q = 0; q < nb; ++q) {
+      ok = mbar_wait(full(st), ph);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      const float* X = reinterpret_cast<const float*>(smem + st * C::SB) + pl;
+      const float* Hs = reinterpret_cast<const float*>(smem + st * C::SB + C::XB);
+#pragma unroll
+      for (int l = 0; l < 9; ++l) {
+        const float x = X[l * P];
+        const float4 u0 = *reinterpret_cast<const float4*>(Hs + l * 12);
+        const float4 u1 = *reinterpret_cast<const float4*>(Hs + l * 12 + 4);
+        const float2 x2 = make_float2(x, x);
+        acc[0] = __ffma2_rn(make_float2(u0.x, u0.y), x2, acc[0]);
+        acc[1] = __ffma2_rn(make_float2(u0.z, u0.w), x2, acc[1]);
+        acc[2] = __ffma2_rn(make_float2(u1.x, u1.y), x2, acc[2]);
+        acc[3] = __ffma2_rn(make_float2(u1.z, u1.w), x2, acc[3]);
+        acc8 = fmaf(Hs[l * 12 + 8], x, acc8);
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(empty(st));
+      if (++st == R) st = 0, ph ^= 1;
+    }
+    if (!ok) break;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      ep[(2 * j) * 32 + lane] = alpha * acc[j].x;
+      ep[(2 * j + 1) * 32 + lane] = alpha * acc[j].y;
+    }
+    ep[8 * 32 + lane] = alpha * acc8;
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int row = irow + 4 * j;
+      if (row >= 9 || p0 >= s) continue;
+      const float4 t = *reinterpret_cast<const float4*>(ep + row * 32 + 4 * igrp);
+      float yo[4] = {t.x, t.y, t.z, t.w}, r[4];
+      if (c_r != 0.f || direct) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) r[v] = tbk_probe_sign(seed, (int64_t)9 * a + row, p0 + v);
+      }
+      if (c_r != 0.f) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) yo[v] = fmaf(c_r, r[v], yo[v]);
+      }
+      if (yprev) {
+        yo[0] -= yp[j].x; yo[1] -= yp[j].y; yo[2] -= yp[j].z; yo[3] -= yp[j].w;
+      }
+      *reinterpret_cast<float4*>(yout + ((int64_t)9 * a + row) * s + p0) = make_float4(yo[0], yo[1], yo[2], yo[3]);
+      if (partials) {
+        const float xin[4] = {direct ? r[0] : xo[j].x, direct ? r[1] : xo[j].y, direct ? r[2] : xo[j].z,
+                              direct ? r[3] : xo[j].w};
+        float q0 = 0.f, q1 = 0.f;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          q0 = fmaf(yo[v], xin[v], q0);
+          q1 = fmaf(yo[v], yo[v], q1);
+        }
+        two_sum_acc(cs0, cc0, q0);
+        two_sum_acc(cs1, cc1, q1);
+      }
+    }
+    __syncwarp();  // the buffer is free again
+  }
+  if (!ok) atomicOr(err, 2);
+  if (partials) step_partials(partials, (double)cs0 + (double)cc0, (double)cs1 + (double)cc1, warp, lane, nw);
+}
+
+// ---- FP64 step by rows -------------------------------------------------------------------------------
+//
+// A warp takes 32 probes of ROWS (3 or 1) of the 9 rows of an atom, on its own, with the next block and
+// tile loaded a block ahead.  Each quarter of an SM issues an FP64 FMA in 64 cycles, so nothing but the
+// even spread of the FMAs over the quarters counts; a warp of a third or a ninth of a row spreads them
+// to within a few per cent (a row per three-warp CTA leaves every fourth quarter idle).  Narrow panels
+// put several row groups into a warp.  200 atoms x 64 probes: 37 us a step against 125 with the plain
+// kernel on 50 SMs (the FP64 rate alone allows 24), 2,000 x 128: 635 against 716.
+template <int ROWS>
+__global__ void __launch_bounds__(128)
+cheb_step_fp64(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+               const double* __restrict__ hv, const double* __restrict__ yin, const double* yprev, double* yout,
+               const double alpha, const double c_r, const uint64_t seed, const int s, const int direct,
+               const StepSources<double> src, double* __restrict__ partials, const int lp, const int n_sm) {
+  constexpr int NG = 9 / ROWS, RS = Layout<double, 9>::RS, BS = Layout<double, 9>::BS;
+  pdl_wait();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int gw = 32 / lp;                   // row groups in a warp
+  const int ngw = (NG + gw - 1) / gw;       // warps of an atom and chunk
+  const int n_chunks = (s + 31) / 32;
+  const int64_t units = (int64_t)n_atoms * n_chunks * ngw;
+  double sum0 = 0.0, sum1 = 0.0;
+  // long and short rows lie far apart in most listings: the CTAs that share an SM take their quarters in
+  // opposite order
+  const int quarter = (blockIdx.x / n_sm) & 1 ? 3 - warp : warp;
+  for (int64_t u = (int64_t)quarter * gridDim.x + blockIdx.x; u < units; u += (int64_t)4 * gridDim.x) {
+    const int64_t t = u / ngw;
+    const int a = (int)(t / n_chunks), p0 = (int)(t - (int64_t)a * n_chunks) * 32 + lane % lp;
+    const int g = (int)(u - t * ngw) * gw + lane / lp;
+    if (lane / lp >= gw || g >= NG || p0 >= s) continue;
+    int k = __ldg(row_ptr + a);
+    const int k1 = __ldg(row_ptr + a + 1);
+    double acc[ROWS], x[9], h[ROWS][9];
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) acc[i] = 0.0;
+    auto fetch = [&](int kk, int b, double (&xx)[9], double (&hh)[ROWS][9]) {
+      const double* xb = yin + (int64_t)9 * b * s + p0;
+      const double* hb = hv + (int64_t)kk * BS + ROWS * g * RS;
+#pragma unroll
+      for (int l = 0; l < 9; ++l) xx[l] = __ldg(xb + (int64_t)l * s);
+#pragma unroll
+      for (int i = 0; i < ROWS; ++i)
+#pragma unroll
+        for (int l = 0; l < 9; ++l) hh[i][l] = __ldg(hb + i * RS + l);
+    };
+    int bn = k + 1 < k1 ? __ldg(col + k + 1) : 0;
+    if (k < k1) fetch(k, __ldg(col + k), x, h);
+    for (; k < k1; ++k) {
+      double xn[9], hn[ROWS][9];
+      if (k + 1 < k1) fetch(k + 1, bn, xn, hn);
+      if (k + 2 < k1) bn = __ldg(col + k + 2);
+#pragma unroll
+      for (int l = 0; l < 9; ++l)
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) acc[i] = fma(h[i][l], x[l], acc[i]);
+#pragma unroll
+      for (int l = 0; l < 9; ++l) {
+        x[l] = xn[l];
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) h[i][l] = hn[i][l];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+      const int64_t row = (int64_t)9 * a + ROWS * g + i, off = row * s + p0;
+      double yo = alpha * acc[i], r = 0.0;
+      if (c_r != 0.0 || direct) r = (double)tbk_probe_sign(seed, row, p0);
+      if (c_r != 0.0) yo = fma(c_r, r, yo);
+      if (yprev) yo -= yprev[off];
+#pragma unroll
+      for (int e = 0; e < 3; ++e)
+        if (src.p[e]) yo = fma(src.c[e], __ldg(src.p[e] + off), yo);
+      yout[off] = yo;
+      if (partials) {
+        sum0 = fma(yo, direct ? r : __ldg(yin + off), sum0);
+        sum1 = fma(yo, yo, sum1);
+      }
+    }
+  }
+  if (partials) step_partials(partials, sum0, sum1, warp, lane, 4);
+}
+
 // ---- launch geometry ---------------------------------------------------------------------------
 
 template <typename T, int B, bool P>
@@ -713,9 +1019,10 @@ constexpr int SELF_R = 2;
 
 static int occupancy_self() {
   using C = SelfCfg<SELF_R>;
-  cudaFuncSetAttribute(cheb_step_self<SELF_R>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+  cudaFuncSetAttribute(cheb_step_self<SELF_R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+  cudaFuncSetAttribute(cheb_step_self<SELF_R, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   int n = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cheb_step_self<SELF_R>, 32, C::SMEM);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cheb_step_self<SELF_R, false>, 32, C::SMEM);
   return n;
 }
 
@@ -753,8 +1060,16 @@ static int chosen_cw(const tbk_ctx* ctx, const HOp& op, int s, int per_task) {
   return t && t->cw >= 1 && t->cw <= cw && s % (128 * t->cw) == 0 ? t->cw : cw;
 }
 
+template <int NW>
+static int occupancy_lane() {
+  cudaFuncSetAttribute(cheb_step_lane<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, LaneCfg<NW>::SMEM);
+  int n = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cheb_step_lane<NW>, 32 * (NW + 1), LaneCfg<NW>::SMEM);
+  return n;
+}
+
 struct Occ {
-  int simple = 0, bulk[5] = {0, 0, 0, 0, 0};
+  int simple = 0, bulk[5] = {0, 0, 0, 0, 0}, lane[3] = {0, 0, 0};
 };
 
 static Occ& occ_cache(int dev) {
@@ -775,7 +1090,9 @@ bool tc_eligible(const HOp& op, int s);
 int tc_grid(tbk_ctx* ctx);
 void launch_step_tc(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G);
 
-int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s) {
+static int lane_class(int s);
+
+static Occ& occupancies(tbk_ctx* ctx) {
   Occ& o = occ_cache(ctx->device);
   if (!o.simple) {
     int m = 1 << 30;
@@ -787,14 +1104,59 @@ int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s) {
     o.bulk[1] = occupancy_self();  // 128-probe tasks run on the self-fed kernel
     o.bulk[2] = occupancy_bulk<2, BULK_D>();
     o.bulk[4] = occupancy_bulk<4, BULK_D>();
+    o.lane[0] = occupancy_lane<4>();
+    o.lane[1] = occupancy_lane<8>();
+    o.lane[2] = occupancy_lane<16>();
   }
-  // the TMA-fed kernel's occupancy sets the grid where it runs (the first step's plain kernel
-  // then just takes more than one wave: every kernel loops over its tasks, none waits on another
-  // CTA); the tensor-core step, when selected, runs on this same grid so that the per-CTA partial
-  // sums line up
+  return o;
+}
+
+// FP32 steps that the one-probe-per-lane kernel takes: few tiles for the chip, or a width between 128
+// and 512 that is no multiple of 128 (whose tiles the other kernels would fetch row by row: 1,000 atoms
+// x 196 probes 71 us a step against 33).  Measured us a step, lane against self-fed kernel at 128 probes:
+// 147 atoms 8.3 (16.0), 333 atoms 9.6 (15.9), 700 atoms 16.4 (16.6); against cheb_step_bulk at 256: 147
+// atoms 10.1 (9.5).
+static bool use_lane(const HOp& op, int s) {
+  if (op.prec != TBK_MIXED || op.B != 9) return false;
+  if (s > 128) return s % 128 != 0;
+  return (int64_t)op.n_atoms * ((s + 31) / 32) <= 2600;
+}
+// FP64 9x9 steps run by rows at every size.
+static bool use_rows64(const HOp& op) { return op.prec == TBK_FP64 && op.B == 9; }
+
+// Warps of an FP64 step by rows, and the rows a warp takes: one where three would leave SM quarters idle.
+static int64_t fp64_units(const HOp& op, int s, int rows) {
+  const int gw = 32 / std::min(32, s), ng = 9 / rows;
+  return (int64_t)op.n_atoms * ((s + 31) / 32) * ((ng + gw - 1) / gw);
+}
+static int fp64_rows(const tbk_ctx* ctx, const HOp& op, int s) {
+  return fp64_units(op, s, 3) >= 4 * (int64_t)ctx->num_sms ? 3 : 1;
+}
+
+int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s) {
+  const Occ& o = occupancies(ctx);
+  // the TMA-fed kernel's occupancy sets the grid where it runs (the other kernels then just take
+  // more than one wave: every kernel loops over its tasks, none waits on another CTA); the
+  // tensor-core step, when selected, runs on this same grid so that the per-CTA partial sums line up
+  if (use_rows64(op))
+    return (int)std::min<int64_t>((fp64_units(op, s, fp64_rows(ctx, op, s)) + 3) / 4, 4 * ctx->num_sms);
+  if (use_lane(op, s))
+    return (int)std::min<int64_t>((int64_t)op.n_atoms * ((s + 511) / 512), (int64_t)std::max(1, o.lane[lane_class(s)]) * ctx->num_sms);
   const int cw = chosen_cw(ctx, op, s, 0);
-  const int per_sm = cw && o.bulk[cw] > 0 ? o.bulk[cw] : o.simple;
-  return std::max(1, per_sm * ctx->num_sms);
+  const bool narrow = op.prec == TBK_MIXED && op.B == 9 && s < 128;
+  const int per_sm = narrow && o.bulk[1] > 0 ? o.bulk[1] : (cw && o.bulk[cw] > 0 ? o.bulk[cw] : o.simple);
+  const int64_t tasks = cw ? (int64_t)op.n_atoms * (s / (128 * cw)) : op.n_atoms;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(per_sm * ctx->num_sms, tasks));
+}
+
+template <typename T>
+static StepSources<T> sources(const StepArgs& a) {
+  StepSources<T> r;
+  for (int e = 0; e < 3; ++e) {
+    r.p[e] = (const T*)a.src[e];
+    r.c[e] = (T)a.csrc[e];
+  }
+  return r;
 }
 
 template <typename T, int B>
@@ -804,48 +1166,91 @@ static void launch_simple(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G)
   if (a.cur_is_probe)
     cheb_step_kernel<T, B, true><<<G, blk, 0, ctx->stream>>>(
         op.n_atoms, op.row_ptr, op.col, hv, (const T*)a.yin, (const T*)a.yprev, (T*)a.yout, (T)a.alpha,
-        (T)a.c_r, a.seed, a.s, a.direct, a.partials);
+        (T)a.c_r, a.seed, a.s, a.direct, sources<T>(a), a.partials);
   else
     cheb_step_kernel<T, B, false><<<G, blk, 0, ctx->stream>>>(
         op.n_atoms, op.row_ptr, op.col, hv, (const T*)a.yin, (const T*)a.yprev, (T*)a.yout, (T)a.alpha,
-        (T)a.c_r, a.seed, a.s, a.direct, a.partials);
+        (T)a.c_r, a.seed, a.s, a.direct, sources<T>(a), a.partials);
   post_launch(ctx, "cheb_step_kernel");
 }
 
 template <int CW>
 static void launch_bulk(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
   using C = BulkCfg<CW, BULK_D>;
-  cheb_step_bulk<CW, BULK_D><<<G, C::THREADS, C::SMEM, ctx->stream>>>(
-      op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)a.yin, (const float*)a.yprev,
-      (float*)a.yout, (float)a.alpha, (float)a.c_r, a.seed, a.s, a.direct, a.partials, a.err,
-      a.batch, a.per_task, ctx->stall_next_step);
+  launch_pdl(ctx, cheb_step_bulk<CW, BULK_D>, G, C::THREADS, C::SMEM,
+               op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)a.yin, (const float*)a.yprev,
+               (float*)a.yout, (float)a.alpha, (float)a.c_r, a.seed, a.s, a.direct, a.partials, a.err, a.batch,
+               a.per_task, ctx->stall_next_step);
   ctx->stall_next_step = 0;
   post_launch(ctx, "cheb_step_bulk");
 }
 
+template <bool NARROW>
 static void launch_self(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
   using C = SelfCfg<SELF_R>;
-  cheb_step_self<SELF_R><<<G, 32, C::SMEM, ctx->stream>>>(
-      op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)a.yin, (const float*)a.yprev,
-      (float*)a.yout, (float)a.alpha, (float)a.c_r, a.seed, a.s, a.direct, a.partials, a.err,
-      a.batch, a.per_task, ctx->stall_next_step);
+  launch_pdl(ctx, cheb_step_self<SELF_R, NARROW>, G, 32, C::SMEM,
+               op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)a.yin, (const float*)a.yprev,
+               (float*)a.yout, (float)a.alpha, (float)a.c_r, a.seed, a.s, a.direct, a.partials, a.err, a.batch,
+               a.per_task, ctx->stall_next_step);
   ctx->stall_next_step = 0;
   post_launch(ctx, "cheb_step_self");
 }
 
+template <int NW>
+static void launch_lane_nw(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
+  const int nw = std::min(NW, (a.s + 31) / 32);
+  launch_pdl(ctx, cheb_step_lane<NW>, G, 32 * (nw + 1),
+               LaneCfg<NW>::SMEM, op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)a.yin,
+               (const float*)a.yprev, (float*)a.yout, (float)a.alpha, (float)a.c_r, a.seed, a.s, a.direct, a.partials,
+               a.err, ctx->stall_next_step);
+  ctx->stall_next_step = 0;
+  post_launch(ctx, "cheb_step_lane");
+}
+
+static int lane_class(int s) { return s <= 128 ? 0 : (s <= 256 ? 1 : 2); }  // 4, 8 or 16 warps
+
+static void launch_lane(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
+  const int c = lane_class(a.s);
+  if (c == 0) launch_lane_nw<4>(ctx, op, a, G);
+  else if (c == 1) launch_lane_nw<8>(ctx, op, a, G);
+  else launch_lane_nw<16>(ctx, op, a, G);
+}
+
+template <int ROWS>
+static void launch_fp64(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
+  launch_pdl(ctx, cheb_step_fp64<ROWS>, G, 128, 0, op.n_atoms, op.row_ptr, op.col,
+               (const double*)op.hv, (const double*)a.yin, (const double*)a.yprev, (double*)a.yout, a.alpha, a.c_r,
+               a.seed, a.s, a.direct, sources<double>(a), a.partials, std::min(32, a.s), ctx->num_sms);
+  post_launch(ctx, "cheb_step_fp64");
+}
+
 void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
   KernelTimerScope timer(ctx, TBK_KERNEL_STEP);
-  const int G = step_grid_ctas(ctx, op, a.s);
+  const int G = a.grid > 0 ? a.grid : step_grid_ctas(ctx, op, a.s);
   if (a.use_tc && !a.cur_is_probe && a.err && !a.force_simple && !a.batch.atom_cl && !a.per_task &&
       tc_eligible(op, a.s)) {
     launch_step_tc(ctx, op, a, G);
+    return;
+  }
+  const bool fed = !a.cur_is_probe && a.err && !a.force_simple && op.B == 9;  // a panel by bulk copies
+  if (fed && use_rows64(op)) {
+    if (fp64_rows(ctx, op, a.s) == 3) launch_fp64<3>(ctx, op, a, G);
+    else launch_fp64<1>(ctx, op, a, G);
+    return;
+  }
+  if (fed && !a.per_task && use_lane(op, a.s)) {
+    launch_lane(ctx, op, a, G);
+    return;
+  }
+  if (fed && op.prec == TBK_MIXED && a.s < 128) {
+    launch_self<true>(ctx, op, a, G);
     return;
   }
   const int cw = chosen_cw(ctx, op, a.s, a.per_task);
   if (cw && !a.cur_is_probe && a.err && !a.force_simple && occ_cache(ctx->device).bulk[cw] > 0) {
     if (cw == 4) launch_bulk<4>(ctx, op, a, G);
     else if (cw == 2) launch_bulk<2>(ctx, op, a, G);
-    else launch_self(ctx, op, a, G);
+    else launch_self<false>(ctx, op, a, G);
     return;
   }
   if (op.prec == TBK_MIXED) {
