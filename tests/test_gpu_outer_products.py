@@ -1,0 +1,49 @@
+"""The outer products of the general adjoint (probe counts that are no multiple of 128, FP64, the plain
+kernels) at the edges of their 32-probe runs and of the row lookup, against the oracle's gradient or,
+where the cluster is too large for it, against the fused kernel."""
+import numpy as np
+import pytest
+
+from gpu_common import blocks_of, oracle_estimator, oracle_H, small_fcc
+from oracle import chebyshev as och
+
+pytestmark = pytest.mark.gpu
+
+
+def _setup(n_atoms, s, order, mixed):
+    import torch
+    from paper_1812_05264_gb300 import api
+    wk = small_fcc(n_atoms, n_probes=s, order=order, mixed=mixed)
+    ctx = api.Context()
+    pos = torch.as_tensor(wk.positions, dtype=torch.float64, device="cuda")
+    model = api.Model.from_workload(wk, "cuda")
+    H = api.assemble_H(ctx, model, pos, api.build_neighbors(ctx, pos, wk.cutoff))
+    lo, hi = api.spectral_bounds(ctx, H)
+    return api, wk, ctx, pos, model, H, lo, hi
+
+
+# mixed: FP32 products of unit-variance panels, the kernel-against-oracle bound of the other G tests
+# (2e-5 of the largest entry); FP64: rounding of p steps, 1e-11 of it
+@pytest.mark.parametrize("n_atoms,s", [(1, 4), (2, 28), (13, 32), (13, 36), (35, 64), (13, 100), (40, 132), (13, 260)])
+@pytest.mark.parametrize("fp64", [False, True])
+def test_gradient_vs_oracle(n_atoms, s, fp64):
+    order = 14
+    api, wk, ctx, pos, model, H, lo, hi = _setup(n_atoms, s, order, not fp64)
+    rp, col, Hd = oracle_H(wk)
+    est = oracle_estimator(wk, Hd, lo, hi, order)
+    ref = blocks_of(och.estimator_gradient(est["w"], est["V"], est["R"], lo, hi, est["mu"], wk.kT, False, p=order),
+                    rp, col, 9)
+    G, _ = api.density_and_forces(ctx, H, model, pos, None, lo, hi, wk.probe_seed, s, order, est["mu"], wk.kT,
+                                  fp64=fp64, want_forces=False)
+    tol = (1e-11 if fp64 else 2e-5) * np.abs(ref).max()
+    assert np.abs(G.cpu().numpy() - ref).max() <= tol
+
+
+@pytest.mark.parametrize("n_atoms", [33, 1030])
+def test_plain_outer_products_equal_the_fused_ones(n_atoms):
+    api, wk, ctx, pos, model, H, lo, hi = _setup(n_atoms, 128, 8, True)
+    args = (ctx, H, model, pos, None, lo, hi, 7, 128, 8, 6.0, 0.5)
+    G, F = api.density_and_forces(*args)
+    Gp, Fp = api.density_and_forces(*args, plain=True)
+    assert (G - Gp).abs().max().item() <= 2e-5 * G.abs().max().item()
+    assert (F - Fp).abs().max().item() <= 1e-3
