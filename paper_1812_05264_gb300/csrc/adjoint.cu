@@ -957,6 +957,12 @@ __global__ void gather_forces(int n_atoms, const int32_t* __restrict__ row_ptr,
   F[3 * c + 2] = f2;
 }
 
+bool fused_eligible(const HOp& op, int s, int plain);
+// The adjoint of the doubled moments: mixed 9x9 at 128, 256 or 512 probes (fused kernels), FP64 always.
+static bool doubled_eligible(const HOp& op, int s, int plain) {
+  return fused_eligible(op, s, plain) || (!plain && op.prec == TBK_FP64);
+}
+
 bool fused_eligible(const HOp& op, int s, int plain) {
   return !plain && op.prec == TBK_MIXED && op.B == 9 && (s == 128 || s == 256 || s == 512);
 }
@@ -1124,14 +1130,15 @@ void launch_window(tbk_ctx* ctx, const HOp& op, const WindowPanels& wp, int nw, 
 // This needs the y_k only up to K = p/2: half the forward, replay and backward work of the
 // Clenshaw form of Eq. polynomial_response, for the same estimator and the same gradient.
 
-__global__ void ybar_init(int64_t n, int s, float ca, const float* __restrict__ yk, float cb,
-                          const float* __restrict__ ykm1, uint64_t seed, float* __restrict__ out) {
+template <typename T>
+__global__ void ybar_init(int64_t n, int s, T ca, const T* __restrict__ yk, T cb, const T* __restrict__ ykm1,
+                          uint64_t seed, T* __restrict__ out) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n * s) return;
   const int64_t row = i / s;
   const int p = (int)(i - row * s);
-  const float prev = ykm1 ? ykm1[i] : tbk_probe_sign(seed, row, p);
-  out[i] = fmaf(ca, yk[i], cb * prev);
+  const T prev = ykm1 ? ykm1[i] : (T)tbk_probe_sign(seed, row, p);
+  out[i] = fma(ca, yk[i], cb * prev);
 }
 
 // get_coefs() is called once every y_1 .. y_K has been formed for the first time (with
@@ -1142,9 +1149,12 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
                       int64_t max_panel_bytes, double* Gacc, int* err, int sched, const AdjBatch* bt,
                       const void* probe_panel, int s_norm) {
   TBK_CHECK_ARG(!(bt && probe_panel), "a batch regenerates its probes");
-  const bool windowed = sched == 1;
+  // FP64: plain backward steps, each followed by its outer products
+  const bool f64 = op.prec == TBK_FP64;
+  const size_t esz = f64 ? 8 : 4;
+  const bool windowed = sched == 1 && !f64;
   // outer products on the tensor cores after each backward step, where that kernel applies
-  const bool tensor = sched == 2 && !bt && tc_sddmm_eligible(ctx, op, s, tc_sddmm_max_row(ctx, op));
+  const bool tensor = sched == 2 && !bt && !f64 && tc_sddmm_eligible(ctx, op, s, tc_sddmm_max_row(ctx, op));
   // a stored probe block y_0 (single system): read wherever the probe enters
   const bool r_panel = probe_panel != nullptr;
   const double nrm = r_panel && s_norm > 0 ? s_norm : s;
@@ -1174,11 +1184,11 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
     v[1] = p > 1 ? c[1] : 0.0;
     for (int k = 2; 2 * k - 1 < p; ++k) v[1] -= c[2 * k - 1];
   };
-  auto ca = [&](int k) { return (float)(2.0 * w[k] / nrm); };
-  auto cb = [&](int k) { return (float)(v[k] / nrm); };
-  auto cc = [&](int k) { return (float)(v[k + 1] / nrm); };
+  auto ca = [&](int k) { return 2.0 * w[k] / nrm; };
+  auto cb = [&](int k) { return v[k] / nrm; };
+  auto cc = [&](int k) { return v[k + 1] / nrm; };
 
-  const size_t panel = (size_t)op.n_rows * s * 4;
+  const size_t panel = (size_t)op.n_rows * s * esz;
   size_t budget = max_panel_bytes > 0 ? (size_t)max_panel_bytes : panel_budget(ctx, WS_CHECKPOINTS);
   const int npan = K;  // y_1 .. y_K
   // ybar_j lives in ring slot j mod NB: the two of the recurrence, plus the window's SDW panels
@@ -1199,7 +1209,7 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
   std::vector<size_t> poff;
   size_t prefix_tail = 0;
   if (bt) {
-    const size_t row_bytes = (size_t)op.B * s * 4;
+    const size_t row_bytes = (size_t)op.B * s * esz;
     poff.resize((size_t)npan + 2);
     size_t o = 0;
     for (int i = 0; i <= npan + 1; ++i) {
@@ -1331,10 +1341,38 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
       o.n_atoms = active(std::max(k, 1));
       if (k == K && !bt) {
         // ybar_K = g_K (y_{K+1} does not enter)
-        const int64_t n = op.n_rows * s;
-        ybar_init<<<(unsigned)((n + 255) / 256), 256, 0, ctx->stream>>>(
-            op.n_rows, s, ca(K), (const float*)Y(K), cb(K), (const float*)Y(K - 1), probe_seed, (float*)YB(K));
+        const unsigned grid = (unsigned)((op.n_rows * s + 255) / 256);
+        if (f64)
+          ybar_init<double><<<grid, 256, 0, ctx->stream>>>(op.n_rows, s, ca(K), (const double*)Y(K), cb(K),
+                                                           (const double*)Y(K - 1), probe_seed, (double*)YB(K));
+        else
+          ybar_init<float><<<grid, 256, 0, ctx->stream>>>(op.n_rows, s, (float)ca(K), (const float*)Y(K), (float)cb(K),
+                                                          (const float*)Y(K - 1), probe_seed, (float*)YB(K));
         post_launch(ctx, "ybar_init");
+        continue;
+      }
+      if (f64) {
+        // G += 2 y_k ybar_{k+1}^T (y_0 ybar_1^T last), then ybar_k = g_k + 2 H^ ybar_{k+1} - ybar_{k+2}
+        launch_sddmm(ctx, o, Y(k), k == 0, probe_seed, YB(k + 1), s, k ? 2.0 : 1.0, Gacc);
+        if (k == 0) continue;
+        StepArgs a;
+        a.seed = probe_seed;
+        a.s = s;
+        a.yin = YB(k + 1);
+        a.yprev = k + 2 <= K ? YB(k + 2) : nullptr;
+        a.yout = YB(k);
+        a.src[0] = Y(k);
+        a.csrc[0] = ca(k);
+        a.src[1] = Y(k + 1);
+        a.csrc[1] = cc(k);
+        if (k == 1) {
+          a.c_r = cb(1);
+        } else {
+          a.src[2] = Y(k - 1);
+          a.csrc[2] = cb(k);
+        }
+        a.err = err;
+        launch_step(ctx, o, a);
         continue;
       }
       if (k >= 1) {
@@ -1342,7 +1380,8 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
         // (the probe coefficient .x scales the regenerated y_0; a stored y_0 streams as y_{k-1})
         const bool r_gen = k == 1 && !r_panel;
         const float4 cf = bt ? make_float4(0.f, 0.f, 0.f, 0.f)
-                             : make_float4(r_gen ? cb(1) : 0.f, ca(k), r_gen ? 0.f : cb(k), cc(k));
+                             : make_float4(r_gen ? (float)cb(1) : 0.f, (float)ca(k), r_gen ? 0.f : (float)cb(k),
+                                           (float)cc(k));
         const float4* cfk = bt ? bt->cft + (size_t)k * bt->K.size() : nullptr;
         launch_fused(ctx, o, YB(k + 1), (k + 2 <= K || bt) ? YB(k + 2) : nullptr, YB(k), Y(k), cf, probe_seed, s,
                      2.0, (windowed || tensor) ? nullptr : Gacc, err, br, cfk,
@@ -1418,7 +1457,7 @@ extern "C" int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_
   TBK_CUDA(cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
   HOp op = prepare_hop(ctx, H, emin, emax, prec, WS_HHAT, err);
   const int p = order, s = n_probes, BB = op.B * op.B;
-  const bool fused = fused_eligible(op, s, plain);
+  const bool doubled = doubled_eligible(op, s, plain);
   const double W = emax - emin;
 
   // coefficients c_k = d_k beta_k[g] (device, then host for the per-step scalars)
@@ -1439,7 +1478,7 @@ extern "C" int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_
   const size_t esz = prec == TBK_MIXED ? 4 : 8;
   const size_t panel = (size_t)op.n_rows * s * esz;
   double scale = 2.0 / (W * s);
-  if (fused) {
+  if (doubled) {
     adjoint_doubling(ctx, op, probe_seed, s, p, [&]() { return c; }, nullptr, 0, max_panel_bytes, Gacc, err,
                        outer_schedule(ctx, op, s, flags), nullptr);
     scale = 2.0 / W;  // the 1/s of the moments is inside the source terms
@@ -1635,9 +1674,7 @@ void energies_and_forces_doubled(tbk_ctx* ctx, const tbk_bsr* H, const tbk_model
   adjoint_doubling(ctx, op, probe_seed, s, p, after_forward, partials, nctas, max_panel_bytes, Gacc, err,
                    outer_schedule(ctx, op, s, flags), nullptr, probe_panel, s_norm);
   double* Gout = G ? G : Gsym;
-  const int64_t tot = op.nnzb * BB;
-  symmetrize<9><<<(unsigned)((tot + 255) / 256), 256, 0, ctx->stream>>>(op.nnzb, tr, Gacc, 2.0 / W, Gout);
-  post_launch(ctx, "symmetrize");
+  launch_symmetrize(ctx, op.nnzb, op.B, tr, Gacc, 2.0 / W, Gout);
   if (forces) {
     double* tq = (double*)scratch(ctx, WS_MISC, sizeof(double) * 3 * (size_t)op.nnzb);
     launch_forces(ctx, M, pos, op.n_atoms, op.row_ptr, op.col, tr, Gout, tq, forces);
@@ -1672,7 +1709,7 @@ extern "C" int tbk_energies_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk
   HOp shape;
   shape.B = H ? H->n_orb : 0;
   shape.prec = prec;
-  if (!H || !fused_eligible(shape, n_probes, plain)) {
+  if (!H || !doubled_eligible(shape, n_probes, plain) || (prec == TBK_FP64 && !G && !forces)) {
     // the separate calls give the same results for the other shapes and precisions
     double* mom = moments ? moments : (double*)scratch(ctx, WS_SEGMENT, sizeof(double) * (size_t)order);
     int rc = tbk_chebyshev_moments(ctx, H, emin, emax, probe_seed, n_probes, order,
