@@ -47,8 +47,8 @@ __device__ __forceinline__ int row_of_block(const int32_t* __restrict__ row_ptr,
 template <typename T>
 __global__ void __launch_bounds__(256)
 sddmm_one(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-          const T* __restrict__ y, uint64_t seed, const T* __restrict__ x, int s, double w,
-          double* __restrict__ Gacc, int64_t nnzb) {
+          const T* __restrict__ y, const T* __restrict__ x, int s, double w, double* __restrict__ Gacc,
+          int64_t nnzb) {
   pdl_wait();
   const int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -56,7 +56,7 @@ sddmm_one(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __res
   const int lo = row_of_block(row_ptr, n_atoms, (int)k, lane), b = __ldg(col + k);
   T acc = T(0);
   for (int p = lane; p < s; p += 32)
-    acc = fma(y ? y[(int64_t)lo * s + p] : (T)tbk_probe_sign(seed, lo, p), x[(int64_t)b * s + p], acc);
+    acc = fma(y[(int64_t)lo * s + p], x[(int64_t)b * s + p], acc);
   double v = (double)acc;
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if (lane == 0) Gacc[k] += w * v;
@@ -90,10 +90,9 @@ __device__ __forceinline__ void butterfly32_pair(float (&v)[32], int lane, float
 // the next 32 probes loaded ahead.  333 atoms x 100 probes: 18 us against 233 for one warp per block that
 // loaded as it went and added 81 FP64 butterflies (26 with all 81 sums in a warp, 12 warps per SM; 28 to
 // 32 with a thread per entry and the tiles in shared memory, whose bandwidth then binds).
-template <bool PROBE>
 __global__ void __launch_bounds__(128, 5)
 sddmm_rows32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t nnzb,
-             const float* __restrict__ y, uint64_t seed, const float* __restrict__ x, int s, double w,
+             const float* __restrict__ y, const float* __restrict__ x, int s, double w,
              double* __restrict__ Gacc) {
   pdl_wait();
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -101,8 +100,7 @@ sddmm_rows32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __
   if (gw >= 3 * nnzb) return;
   const int k = (int)(gw / 3), g = (int)(gw - 3 * (int64_t)k);
   const int b = __ldg(col + k), a = row_of_block(row_ptr, n_atoms, k, lane);
-  const int64_t row = (int64_t)9 * a + 3 * g;
-  const float* yp = y + row * s + lane;
+  const float* yp = y + ((int64_t)9 * a + 3 * g) * s + lane;
   const float* xp = x + (int64_t)9 * b * s + lane;
   float acc[27], yv[3], xv[9];
 #pragma unroll
@@ -111,8 +109,7 @@ sddmm_rows32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __
     // past the last probe: zeros, which leave the sums as they are
     const bool in = p < s;
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-      yy[i] = !in ? 0.f : (PROBE ? tbk_probe_sign(seed, row + i, p) : __ldg(yp + (p - lane) + (int64_t)i * s));
+    for (int i = 0; i < 3; ++i) yy[i] = in ? __ldg(yp + (p - lane) + (int64_t)i * s) : 0.f;
 #pragma unroll
     for (int l = 0; l < 9; ++l) xx[l] = in ? __ldg(xp + (p - lane) + (int64_t)l * s) : 0.f;
   };
@@ -143,7 +140,7 @@ sddmm_rows32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __
 // x 64 probes: 37 us against 161 with 81 butterflies per block.
 __global__ void __launch_bounds__(128)
 sddmm_rows64(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t nnzb,
-             const double* __restrict__ y, uint64_t seed, const double* __restrict__ x, int s, double w,
+             const double* __restrict__ y, const double* __restrict__ x, int s, double w,
              double* __restrict__ Gacc) {
   __shared__ double ysh[4][9][33], xsh[4][9][33];
   pdl_wait();
@@ -162,7 +159,7 @@ sddmm_rows64(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __
   auto fetch = [&](int p) {
 #pragma unroll
     for (int r = 0; r < 9; ++r) {
-      yv[r] = p < s ? (y ? __ldg(ya + (int64_t)r * s + p) : (double)tbk_probe_sign(seed, (int64_t)9 * a + r, p)) : 0.0;
+      yv[r] = p < s ? __ldg(ya + (int64_t)r * s + p) : 0.0;
       xv[r] = p < s ? __ldg(xb + (int64_t)r * s + p) : 0.0;
     }
   };
@@ -201,7 +198,7 @@ sddmm_rows64(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __
 //   b_j[a]   = 2 sum_b H^_ab b_{j+1}[b] + c_j r[a] - b_{j+2}[a]          (skipped when bout = 0)
 //   Gacc_ab += w sum_probes y_j[a] b_{j+1}[b]^T   for every neighbour block (a, b)
 // The neighbour tiles b_{j+1}[b] and blocks H^_ab stream through a D-stage ring as in the
-// forward step; the own-row tile y_j[a] (or the probe block when j = 0) is staged once per task.
+// forward step; the own-row tile y_j[a] is staged once per task.
 // The 9x9 outer product of each tile is split into three groups of 3 rows, each taken by one
 // consumer warp (in turn, so the load stays even): its 32 lanes cover interleaved 4-probe
 // groups, and a butterfly reduce-scatter over the lanes leaves one entry per lane, added to the
@@ -237,8 +234,7 @@ __device__ __forceinline__ void butterfly32(float (&v)[32], int lane) {
 // interleaved 4-probe groups): 27 entries, reduced over the lanes by one butterfly and added to
 // the FP64 accumulator (one lane per entry).
 template <int P>
-__device__ __forceinline__ void sddmm_rows3(int g, const float* Y, const float* X, bool y_probe,
-                                            uint64_t seed, int64_t rloc, int lane, int64_t k,
+__device__ __forceinline__ void sddmm_rows3(int g, const float* Y, const float* X, int lane, int64_t k,
                                             double w, double* __restrict__ Gacc) {
   // partial sums of entry (i - 3g) * 9 + l over this lane's probes; scalar accumulators keep the
   // kernel at 128 registers, so that three CTAs fit per SM
@@ -251,13 +247,8 @@ __device__ __forceinline__ void sddmm_rows3(int g, const float* Y, const float* 
     float yv[3][4];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      if (y_probe) {
-#pragma unroll
-        for (int t = 0; t < 4; ++t) yv[i][t] = tbk_probe_sign(seed, rloc + 3 * g + i, pb + t);
-      } else {
-        const float4 u = *reinterpret_cast<const float4*>(Y + (3 * g + i) * P + pb);
-        yv[i][0] = u.x; yv[i][1] = u.y; yv[i][2] = u.z; yv[i][3] = u.w;
-      }
+      const float4 u = *reinterpret_cast<const float4*>(Y + (3 * g + i) * P + pb);
+      yv[i][0] = u.x; yv[i][1] = u.y; yv[i][2] = u.z; yv[i][3] = u.w;
     }
 #pragma unroll
     for (int l = 0; l < 9; ++l) {
@@ -305,8 +296,7 @@ clenshaw_sddmm_bulk(const int n_atoms, const int32_t* __restrict__ row_ptr,
   const uint32_t y_full = bar0 + 8u * (2 * R), y_empty = bar0 + 8u * (2 * R + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool has_prev = bprev != nullptr, has_out = bout != nullptr;
-  // y_tile: the own-row tile y_j is staged once per task for the outer products
-  const bool y_probe = ypan == nullptr, y_tile = SD && !y_probe;
+  constexpr bool y_tile = SD;  // the own-row tile y_j is staged once per task for the outer products
   if (threadIdx.x == 0) {
     for (int i = 0; i < R; ++i) {
       mbar_init(full(i), 1);
@@ -412,7 +402,7 @@ clenshaw_sddmm_bulk(const int n_atoms, const int32_t* __restrict__ row_ptr,
         // per tile, in turn
         for (int g = 0; g < 3; ++g)
           if ((q + g + 1) % CW == warp)
-            sddmm_rows3<C::P>(g, Ys, X, y_probe, sd, rloc, lane, (int64_t)(k0 + q), w, Gacc);
+            sddmm_rows3<C::P>(g, Ys, X, lane, (int64_t)(k0 + q), w, Gacc);
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(empty(st));
@@ -492,14 +482,14 @@ clenshaw_sddmm_bulk(const int n_atoms, const int32_t* __restrict__ row_ptr,
 constexpr int SDW = 4;  // steps per window
 
 struct WindowPanels {
-  const float* y[SDW];  // y_{k_t} panels (n_rows x s); y[0] = NULL: the probe block
+  const float* y[SDW];  // y_{k_t} panels (n_rows x s)
   const float* x[SDW];  // ybar_{k_t + 1} panels
 };
 
 // One CTA task is one block row a.  Consumer warp (g, c) takes rows 3g .. 3g+2 of the block (27
 // entries, one scalar sum each per lane) over probe chunk c (128 probes, 4 per lane), for g < 3
 // and c < NC = P / 128.  The producer warp stages the window's own-row tiles y_{k_t}[a] once per
-// block row (or writes the probe block when y[0] is NULL, nw = 1) and streams the neighbour tiles
+// block row and streams the neighbour tiles
 // ybar_{k_t+1}[b] of every block through a D-stage ring read by all 3 NC warps.  Per block, each
 // warp reduces its 27 sums over the lanes (one butterfly for all the window's steps) and warp
 // (g, 0) adds the NC chunk partials in a fixed order and writes the 27 totals to the FP64
@@ -521,7 +511,7 @@ struct WinGCfg {
 template <int NC>
 __global__ void __launch_bounds__(32 * (3 * NC + 1), NC == 1 ? 5 : 1)
 sddmm_window_g(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-               const WindowPanels wp, const int nw, const uint64_t seed, const int s, const double w,
+               const WindowPanels wp, const int nw, const int s, const double w,
                double* __restrict__ Gacc, int* __restrict__ err, const BatchRows batch,
                const int32_t* __restrict__ kcl, const int k_lo) {
   using C = WinGCfg<NC>;
@@ -537,7 +527,6 @@ sddmm_window_g(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
   auto red_full = [&](int b, int g) { return bar0 + 8u * (2 * D + 2 + 3 * b + g); };
   auto red_empty = [&](int b, int g) { return bar0 + 8u * (2 * D + 8 + 3 * b + g); };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool probe = wp.y[0] == nullptr;
   if (threadIdx.x == 0) {
     for (int i = 0; i < D; ++i) {
       mbar_init(full(i), 1);
@@ -553,40 +542,22 @@ sddmm_window_g(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  auto atom_window = [&](int a, int& nwa, uint64_t& sd, int64_t& rloc) {
-    nwa = nw;
-    sd = seed;
-    rloc = (int64_t)9 * a;
-    if (batch.atom_cl) {
-      const int cl = __ldg(batch.atom_cl + a);
-      sd = __ldg(batch.seed + cl);
-      rloc = (int64_t)9 * (a - __ldg(batch.atom0 + cl));
-      if (kcl) nwa = min(nw, max(0, __ldg(kcl + cl) - k_lo));
-    }
+  // steps of the window that take part for atom a
+  auto atom_window = [&](int a) {
+    return batch.atom_cl && kcl ? min(nw, max(0, __ldg(kcl + __ldg(batch.atom_cl + a)) - k_lo)) : nw;
   };
 
   if (warp == NWARP) {
-    // producer warp: lane 0 issues the copies; in the probe case all lanes write the probe block
+    // producer warp: lane 0 issues the copies
     int it = 0, y_it = 0;
     bool ok = true;
     for (int a = blockIdx.x; a < n_atoms && ok; a += gridDim.x) {
-      int nwa;
-      uint64_t sd;
-      int64_t rloc;
-      atom_window(a, nwa, sd, rloc);
+      const int nwa = atom_window(a);
       if (nwa == 0) continue;
       if (lane == 0) ok = mbar_wait(y_empty, (y_it & 1) ^ 1);
       ok = __shfl_sync(0xffffffffu, ok, 0);
       if (!ok) break;
-      if (probe) {
-        for (int e = lane; e < 9 * P; e += 32) {
-          const int i = e / P, pr = e - i * P;
-          Yw[e] = tbk_probe_sign(sd, rloc + i, pr);
-        }
-        __threadfence_block();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(y_full);
-      } else if (lane == 0) {
+      if (lane == 0) {
         mbar_expect_tx(y_full, nwa * C::XB);
         for (int t = 0; t < nwa; ++t)
           bulk_g2s(smem_u32(Yw + t * 9 * P), wp.y[t] + (int64_t)9 * a * s, C::XB, y_full);
@@ -611,7 +582,7 @@ sddmm_window_g(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
     if (!ok && lane == 0) {
       atomicOr(err, 2);
       for (int j = (it > D ? it - D : 0); j < it; ++j) mbar_wait(full(j % D), (j / D) & 1);
-      if (y_it > 0 && !probe) mbar_wait(y_full, (y_it - 1) & 1);
+      if (y_it > 0) mbar_wait(y_full, (y_it - 1) & 1);
     }
     return;
   }
@@ -621,10 +592,7 @@ sddmm_window_g(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
   int it = 0, y_it = 0, r_it = 0;
   bool ok = true;
   for (int a = blockIdx.x; a < n_atoms && ok; a += gridDim.x) {
-    int nwa;
-    uint64_t sd;
-    int64_t rloc;
-    atom_window(a, nwa, sd, rloc);
+    const int nwa = atom_window(a);
     if (nwa == 0) continue;
     const int k0 = __ldg(row_ptr + a), k1 = __ldg(row_ptr + a + 1);
     ok = mbar_wait(y_full, y_it & 1);
@@ -1019,25 +987,22 @@ void launch_fused(tbk_ctx* ctx, const HOp& op, const void* bin, const void* bpre
   }
 }
 
-void launch_sddmm(tbk_ctx* ctx, const HOp& op, const void* y, int y_is_probe, uint64_t seed,
-                  const void* x, int s, double w, double* Gacc) {
-  if (y_is_probe) y = nullptr;
+void launch_sddmm(tbk_ctx* ctx, const HOp& op, const void* y, const void* x, int s, double w, double* Gacc) {
   const bool f32 = op.prec == TBK_MIXED;
   if (op.B == 9) {
     if (f32)
-      launch_pdl(ctx, y ? sddmm_rows32<false> : sddmm_rows32<true>, ceil_div(3 * op.nnzb, 4), 128, 0, op.n_atoms,
-                 op.row_ptr, op.col, op.nnzb, (const float*)y, seed,
-                 (const float*)x, s, w, Gacc);
+      launch_pdl(ctx, sddmm_rows32, ceil_div(3 * op.nnzb, 4), 128, 0, op.n_atoms, op.row_ptr, op.col, op.nnzb,
+                 (const float*)y, (const float*)x, s, w, Gacc);
     else
-      launch_pdl(ctx, sddmm_rows64, ceil_div(op.nnzb, 4), 128, 0, op.n_atoms, op.row_ptr, op.col, op.nnzb, (const double*)y, seed,
-                 (const double*)x, s, w, Gacc);
+      launch_pdl(ctx, sddmm_rows64, ceil_div(op.nnzb, 4), 128, 0, op.n_atoms, op.row_ptr, op.col, op.nnzb,
+                 (const double*)y, (const double*)x, s, w, Gacc);
   } else {
     const int grid = ceil_div(op.nnzb * 32, 256);
     if (f32)
-      launch_pdl(ctx, sddmm_one<float>, grid, 256, 0, op.n_atoms, op.row_ptr, op.col, (const float*)y, seed,
+      launch_pdl(ctx, sddmm_one<float>, grid, 256, 0, op.n_atoms, op.row_ptr, op.col, (const float*)y,
                  (const float*)x, s, w, Gacc, op.nnzb);
     else
-      launch_pdl(ctx, sddmm_one<double>, grid, 256, 0, op.n_atoms, op.row_ptr, op.col, (const double*)y, seed,
+      launch_pdl(ctx, sddmm_one<double>, grid, 256, 0, op.n_atoms, op.row_ptr, op.col, (const double*)y,
                  (const double*)x, s, w, Gacc, op.nnzb);
   }
   post_launch(ctx, "sddmm");
@@ -1094,8 +1059,7 @@ void launch_forces(tbk_ctx* ctx, const DevModel& M, const double* pos, int n_ato
 }
 
 template <int NC>
-static void launch_window_g(tbk_ctx* ctx, const HOp& op, const WindowPanels& wp, int nw, uint64_t seed,
-                            int s, double w, double* Gacc, int* err, const BatchRows& batch,
+static void launch_window_g(tbk_ctx* ctx, const HOp& op, const WindowPanels& wp, int nw, int s, double w, double* Gacc, int* err, const BatchRows& batch,
                             const int32_t* kcl, int k_lo) {
   using C = WinGCfg<NC>;
   TBK_CUDA(cudaFuncSetAttribute(sddmm_window_g<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
@@ -1103,18 +1067,16 @@ static void launch_window_g(tbk_ctx* ctx, const HOp& op, const WindowPanels& wp,
   TBK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sddmm_window_g<NC>, C::THREADS, C::SMEM));
   TBK_CHECK_ARG(occ > 0, "windowed outer-product kernel does not fit on this device");
   const int G = std::max(1, std::min(op.n_atoms, occ * ctx->num_sms));
-  sddmm_window_g<NC><<<G, C::THREADS, C::SMEM, ctx->stream>>>(op.n_atoms, op.row_ptr, op.col, wp, nw, seed,
-                                                               s, w, Gacc, err, batch, kcl, k_lo);
+  sddmm_window_g<NC><<<G, C::THREADS, C::SMEM, ctx->stream>>>(op.n_atoms, op.row_ptr, op.col, wp, nw, s, w, Gacc, err, batch, kcl, k_lo);
   post_launch(ctx, "sddmm_window_g");
 }
 
-void launch_window(tbk_ctx* ctx, const HOp& op, const WindowPanels& wp, int nw, uint64_t seed, int s,
-                   double w, double* Gacc, int* err, const BatchRows& batch, const int32_t* kcl, int k_lo) {
+void launch_window(tbk_ctx* ctx, const HOp& op, const WindowPanels& wp, int nw, int s, double w, double* Gacc, int* err, const BatchRows& batch, const int32_t* kcl, int k_lo) {
   KernelTimerScope timer(ctx, TBK_KERNEL_WINDOW);
-  TBK_CHECK_ARG(nw >= 1 && nw <= SDW && (wp.y[0] != nullptr || nw == 1), "bad outer-product window");
-  if (s == 512) launch_window_g<4>(ctx, op, wp, nw, seed, s, w, Gacc, err, batch, kcl, k_lo);
-  else if (s == 256) launch_window_g<2>(ctx, op, wp, nw, seed, s, w, Gacc, err, batch, kcl, k_lo);
-  else launch_window_g<1>(ctx, op, wp, nw, seed, s, w, Gacc, err, batch, kcl, k_lo);
+  TBK_CHECK_ARG(nw >= 1 && nw <= SDW && wp.y[0] != nullptr, "bad outer-product window");
+  if (s == 512) launch_window_g<4>(ctx, op, wp, nw, s, w, Gacc, err, batch, kcl, k_lo);
+  else if (s == 256) launch_window_g<2>(ctx, op, wp, nw, s, w, Gacc, err, batch, kcl, k_lo);
+  else launch_window_g<1>(ctx, op, wp, nw, s, w, Gacc, err, batch, kcl, k_lo);
 }
 
 // ---- adjoint of the doubled moments (TMA-fed fused path) ------------------------------------
@@ -1130,15 +1092,17 @@ void launch_window(tbk_ctx* ctx, const HOp& op, const WindowPanels& wp, int nw, 
 // This needs the y_k only up to K = p/2: half the forward, replay and backward work of the
 // Clenshaw form of Eq. polynomial_response, for the same estimator and the same gradient.
 
+// ybar_K = ca y_K + cb y_{K-1}, over all elements of the panels (four per thread).
 template <typename T>
-__global__ void ybar_init(int64_t n, int s, T ca, const T* __restrict__ yk, T cb, const T* __restrict__ ykm1,
-                          uint64_t seed, T* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n * s) return;
-  const int64_t row = i / s;
-  const int p = (int)(i - row * s);
-  const T prev = ykm1 ? ykm1[i] : (T)tbk_probe_sign(seed, row, p);
-  out[i] = fma(ca, yk[i], cb * prev);
+__global__ void ybar_init(int64_t n, T ca, const T* __restrict__ yk, T cb, const T* __restrict__ ykm1,
+                          T* __restrict__ out) {
+  const int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+  if (i >= n) return;
+  T v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[j] = fma(ca, yk[i + j], cb * ykm1[i + j]);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) out[i + j] = v[j];
 }
 
 // get_coefs() is called once every y_1 .. y_K has been formed for the first time (with
@@ -1264,21 +1228,21 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
     launch_batch_probe_panel(ctx, op, br, s, R0);
     for (int j = 0; j < NB; ++j) TBK_CUDA(cudaMemsetAsync(YB(j), 0, panel, ctx->stream));
   }
+  // y_0: the caller's or the batch's probe panel, else written just before the first step, in the first
+  // segment at its place P(0) (where the last backward steps find it) and before that in E
+  void* y0 = bt || r_panel ? R0 : E;
   auto forward_step = [&](int t, const void* yin, const void* yprev, void* yout, bool first_time) {
     HOp o = op;
     o.n_atoms = active(t);
     if (o.n_atoms <= 0) return;
+    if (t == 1 && !bt && !r_panel) launch_scaled_probe(ctx, op, y0, 1.0, probe_seed, s);
     StepArgs a;
     a.seed = probe_seed;
     a.s = s;
-    a.yin = t == 1 ? R0 : yin;
-    a.cur_is_probe = t == 1 && !bt && !r_panel;
+    a.yin = t == 1 ? y0 : yin;
     a.alpha = t == 1 ? 1.0 : 2.0;
-    if (t == 2) {
-      if (bt || r_panel) a.yprev = R0; else a.c_r = -1.0;
-    } else if (t >= 3) {
-      a.yprev = const_cast<void*>(yprev);
-    }
+    if (t == 2) a.yprev = y0;
+    else if (t >= 3) a.yprev = const_cast<void*>(yprev);
     a.yout = yout;
     a.err = err;
     a.batch = br;
@@ -1318,6 +1282,7 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
         TBK_CUDA(cudaMemcpyAsync(E, P(1), panel, cudaMemcpyDeviceToDevice, ctx->stream));
       }
       const bool first_time = sg == nseg - 1;  // the last segment was never formed before
+      if (sg == 0 && !bt && !r_panel) y0 = P(0);
       int t = t0;
       if (sg > 0) {
         TBK_CUDA(cudaMemcpyAsync(P(0), CK(sg, 1), panel, cudaMemcpyDeviceToDevice, ctx->stream));
@@ -1330,9 +1295,9 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
       }
     }
     if (!have_coefs) load_coefs();
-    // y_j for j in [t0 - 1, t1 + 1] (nullptr = the probe block r = y_0, regenerated in the kernels)
+    // y_j for j in [t0 - 1, t1 + 1]
     auto Y = [&](int j) -> const void* {
-      if (j == 0) return r_panel ? R0 : nullptr;
+      if (j == 0) return y0;
       if (j == t1 + 1) return E;
       return P(j - t0 + 1);
     };
@@ -1341,19 +1306,20 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
       o.n_atoms = active(std::max(k, 1));
       if (k == K && !bt) {
         // ybar_K = g_K (y_{K+1} does not enter)
-        const unsigned grid = (unsigned)((op.n_rows * s + 255) / 256);
+        const int64_t n = op.n_rows * s;
+        const unsigned grid = (unsigned)((n + 1023) / 1024);
         if (f64)
-          ybar_init<double><<<grid, 256, 0, ctx->stream>>>(op.n_rows, s, ca(K), (const double*)Y(K), cb(K),
-                                                           (const double*)Y(K - 1), probe_seed, (double*)YB(K));
+          ybar_init<double><<<grid, 256, 0, ctx->stream>>>(n, ca(K), (const double*)Y(K), cb(K), (const double*)Y(K - 1),
+                                                           (double*)YB(K));
         else
-          ybar_init<float><<<grid, 256, 0, ctx->stream>>>(op.n_rows, s, (float)ca(K), (const float*)Y(K), (float)cb(K),
-                                                          (const float*)Y(K - 1), probe_seed, (float*)YB(K));
+          ybar_init<float><<<grid, 256, 0, ctx->stream>>>(n, (float)ca(K), (const float*)Y(K), (float)cb(K),
+                                                          (const float*)Y(K - 1), (float*)YB(K));
         post_launch(ctx, "ybar_init");
         continue;
       }
       if (f64) {
         // G += 2 y_k ybar_{k+1}^T (y_0 ybar_1^T last), then ybar_k = g_k + 2 H^ ybar_{k+1} - ybar_{k+2}
-        launch_sddmm(ctx, o, Y(k), k == 0, probe_seed, YB(k + 1), s, k ? 2.0 : 1.0, Gacc);
+        launch_sddmm(ctx, o, Y(k), YB(k + 1), s, k ? 2.0 : 1.0, Gacc);
         if (k == 0) continue;
         StepArgs a;
         a.seed = probe_seed;
@@ -1396,16 +1362,16 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
             wp.y[t] = (const float*)Y(k + t);
             wp.x[t] = (const float*)YB(k + t + 1);
           }
-          launch_window(ctx, o, wp, nw, probe_seed, s, 2.0, Gacc, err, br, bt ? bt->d_K : nullptr, k);
+          launch_window(ctx, o, wp, nw, s, 2.0, Gacc, err, br, bt ? bt->d_K : nullptr, k);
         }
       } else if (windowed) {
         // G += y_0 ybar_1^T
         WindowPanels wp{};
         wp.y[0] = (const float*)Y(0);
         wp.x[0] = (const float*)YB(1);
-        launch_window(ctx, o, wp, 1, probe_seed, s, 1.0, Gacc, err, br, bt ? bt->d_K : nullptr, 0);
-      } else if (tensor && Y(0)) {
-        // G += y_0 ybar_1^T with a stored probe block
+        launch_window(ctx, o, wp, 1, s, 1.0, Gacc, err, br, bt ? bt->d_K : nullptr, 0);
+      } else if (tensor && r_panel) {
+        // G += y_0 ybar_1^T with the caller's probe block
         launch_tc_sddmm(ctx, o, Y(0), YB(1), s, 1.0, Gacc, err);
       } else {
         launch_fused(ctx, o, YB(1), nullptr, nullptr, Y(0), make_float4(0.f, 0.f, 0.f, 0.f), probe_seed, s,
@@ -1508,15 +1474,16 @@ extern "C" int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_
     void* bcur = P(n_seg_pan + n_ckpt);
     void* bprev = P(n_seg_pan + n_ckpt + 1);
 
-    // y_t from y_{t-1} (yin; the probe block when t == 1) and y_{t-2} (the probe when t == 2).
+    // y_t from y_{t-1} (yin) and y_{t-2} (yprev); y_0 is the probe block
+    void* y0 = bcur;  // the probe block, written just before the first step (P(0) in the first segment)
     auto forward_step = [&](int t, const void* yin, const void* yprev, void* yout) {
+      if (t == 1) launch_scaled_probe(ctx, op, y0, 1.0, probe_seed, s);
       StepArgs a;
       a.seed = probe_seed;
       a.s = s;
-      a.yin = yin;
-      a.cur_is_probe = t == 1;
+      a.yin = t == 1 ? y0 : yin;
       a.alpha = t == 1 ? 1.0 : 2.0;
-      if (t == 2) a.c_r = -1.0;
+      if (t == 2) a.yprev = y0;
       else if (t >= 3) a.yprev = const_cast<void*>(yprev);
       a.yout = yout;
       a.err = err;
@@ -1541,6 +1508,8 @@ extern "C" int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_
     }
     // Backward sweep: b_{p-1} = c_{p-1} r, then for j = p-2 .. 0 add the y_j b_{j+1} term and
     // form b_j = c_j r + 2 H^ b_{j+1} - b_{j+2}.
+    y0 = P(0);
+    if (nseg == 0 && p >= 2) launch_scaled_probe(ctx, op, y0, 1.0, probe_seed, s);
     if (p >= 2) {
       launch_scaled_probe(ctx, op, bcur, c[p - 1], probe_seed, s);
       bool have_bprev = false;
@@ -1561,8 +1530,7 @@ extern "C" int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_
           }
         }
         for (; j >= t0; --j) {
-          const void* yj = j == 0 ? nullptr : P(j - t0 + 1);
-          launch_sddmm(ctx, op, yj, j == 0, probe_seed, bcur, s, j == 0 ? 1.0 : 2.0, Gacc);
+          launch_sddmm(ctx, op, j == 0 ? y0 : P(j - t0 + 1), bcur, s, j == 0 ? 1.0 : 2.0, Gacc);
           if (j >= 1) {
             StepArgs a;
             a.seed = probe_seed;

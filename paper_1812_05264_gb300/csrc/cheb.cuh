@@ -129,13 +129,12 @@ bool tc_sddmm_eligible(tbk_ctx* ctx, const HOp& op, int s, int max_row);
 void launch_tc_sddmm(tbk_ctx* ctx, const HOp& op, const void* y, const void* x, int s, double w, double* Gacc,
                      int* err);
 // Pieces of the adjoint reused by the direct estimates (adjoint.cu): Chebyshev coefficients into
-// device memory; Gacc += w sum_probes y[a rows] b[b rows]^T on every stored block (y or b FP32/FP64
-// panels of the operator's precision; y_is_probe: y is the probe block regenerated from seed);
+// device memory; Gacc += w sum_probes y[a rows] x[b rows]^T on every stored block (y, x panels of the
+// operator's precision);
 // the transpose map of a symmetric pattern; G = scale (Gacc + Gacc^T) / 2 blockwise.
 void coefficients(tbk_ctx* ctx, int fn, int p, double emin, double emax, double mu, double kT,
                   int damping, double* out);
-void launch_sddmm(tbk_ctx* ctx, const HOp& op, const void* y, int y_is_probe, uint64_t seed,
-                  const void* b, int s, double w, double* Gacc);
+void launch_sddmm(tbk_ctx* ctx, const HOp& op, const void* y, const void* x, int s, double w, double* Gacc);
 void launch_transpose_map(tbk_ctx* ctx, int n_atoms, const int32_t* row_ptr, const int32_t* col,
                           int32_t* tr, int* err);
 void launch_symmetrize(tbk_ctx* ctx, int64_t nnzb, int B, const int32_t* tr, const double* Gacc, double scale,

@@ -101,7 +101,7 @@ extern "C" int tbk_direct_density(tbk_ctx* ctx, const tbk_bsr* H, const tbk_mode
   auto sampled = [&](const void* Y, double* out) {
     TBK_CUDA(cudaMemsetAsync(out, 0, sizeof(double) * (size_t)op.nnzb * BB, ctx->stream));
     if (tc) launch_tc_sddmm(ctx, op, Y, R, s, 1.0 / s, out, err);
-    else launch_sddmm(ctx, op, Y, 0, probe_seed, R, s, 1.0 / s, out);
+    else launch_sddmm(ctx, op, Y, R, s, 1.0 / s, out);
   };
   double* Pacc = P ? P : (double*)scratch(ctx, WS_GACC, sizeof(double) * (size_t)op.nnzb * BB * 2);
   if (P || forces) sampled(X, Pacc);

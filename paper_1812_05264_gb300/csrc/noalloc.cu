@@ -129,14 +129,16 @@ extern "C" int tbk_chebyshev_moments_noalloc(tbk_ctx* ctx, const tbk_bsr* H, dou
     a.force_simple = (flags & TBK_PLAIN_KERNEL) ? 1 : 0;
     a.grid = nctas;
     if (j == 1) {
-      a.cur_is_probe = 1;
+      if (Bp) launch_scaled_probe(ctx, op, Bp, 1.0, probe_seed, s);  // y_0, until y_2 takes its place
+      a.yin = Bp;
+      a.cur_is_probe = Bp ? 0 : 1;
       a.alpha = 1.0;
       a.yout = A;
       cur = A;
     } else if (j == 2) {
       a.yin = A;
       a.alpha = 2.0;
-      a.c_r = -1.0;
+      a.yprev = Bp;
       a.yout = Bp;
       prev = A;
       cur = Bp;

@@ -307,7 +307,7 @@ extern "C" int tbk_rational_density(tbk_ctx* ctx, const tbk_bsr* H, const tbk_mo
   // sampled products with the probe block
   auto sampled = [&](const double* Y, double* out) {
     TBK_CUDA(cudaMemsetAsync(out, 0, sizeof(double) * (size_t)op.nnzb * BB, ctx->stream));
-    launch_sddmm(ctx, op, Y, 0, probe_seed, R, s, 1.0 / s, out);
+    launch_sddmm(ctx, op, Y, R, s, 1.0 / s, out);
   };
   double* Pacc = P ? P : (double*)scratch(ctx, WS_GACC, sizeof(double) * (size_t)op.nnzb * BB);
   if (P || forces) sampled(X, Pacc);

@@ -1260,18 +1260,28 @@ void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
   }
 }
 
+// A thread writes four probes of a row (16-byte stores), a warp 128.
 template <typename T>
-__global__ void scaled_probe_kernel(int64_t n_rows, int s, double c, uint64_t seed, T* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_rows * s) return;
-  const int64_t row = i / s;
-  const int p = (int)(i - row * s);
-  out[i] = (T)(c * (double)tbk_probe_sign(seed, row, p));
+__global__ void __launch_bounds__(256)
+scaled_probe_kernel(int64_t n_rows, int s, double c, uint64_t seed, T* __restrict__ out) {
+  const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (row >= n_rows) return;
+  for (int p = 4 * (threadIdx.x & 31); p < s; p += 128) {
+    T v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = (T)(c * (double)tbk_probe_sign(seed, row, p + j));
+    T* o = out + row * s + p;
+    if constexpr (sizeof(T) == 4) {
+      st16(o, v);
+    } else {
+      st16(o, v);
+      st16(o + 2, v + 2);
+    }
+  }
 }
 
 void launch_scaled_probe(tbk_ctx* ctx, const HOp& op, void* panel, double c, uint64_t seed, int s) {
-  const int64_t n = op.n_rows * s;
-  const unsigned grid = (unsigned)((n + 255) / 256);
+  const int grid = ceil_div(op.n_rows, 8);
   if (op.prec == TBK_MIXED)
     scaled_probe_kernel<float><<<grid, 256, 0, ctx->stream>>>(op.n_rows, s, c, seed, (float*)panel);
   else
@@ -1511,15 +1521,18 @@ void moments_sweep(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, uin
     a.force_simple = (flags & TBK_PLAIN_KERNEL) ? 1 : 0;
     a.use_tc = (flags & TBK_TENSOR_CORES) ? 1 : 0;
     if (j == 1) {
-      a.cur_is_probe = probe_panel ? 0 : 1;
-      a.yin = probe_panel;
+      // a further step follows: its panel holds the probe block until then (a step on a panel takes a
+      // third of the time of one that regenerates every neighbour's probes)
+      if (!probe_panel && Bp) launch_scaled_probe(ctx, op, Bp, 1.0, probe_seed, s);
+      a.yin = probe_panel ? probe_panel : Bp;
+      a.cur_is_probe = a.yin ? 0 : 1;
       a.alpha = 1.0;
       a.yout = A;
       cur = A;
     } else if (j == 2) {
       a.yin = A;
       a.alpha = 2.0;
-      if (probe_panel) a.yprev = const_cast<void*>(probe_panel); else a.c_r = -1.0;
+      a.yprev = probe_panel ? const_cast<void*>(probe_panel) : Bp;
       a.yout = Bp;
       prev = A;
       cur = Bp;
