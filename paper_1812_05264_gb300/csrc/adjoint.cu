@@ -283,7 +283,8 @@ clenshaw_sddmm_bulk(const int n_atoms, const int32_t* __restrict__ row_ptr,
                     const float* __restrict__ ypan, const float4 cf, const uint64_t seed,
                     const int s, const double w, double* __restrict__ Gacc, int* __restrict__ err,
                     const BatchRows batch, const float4* __restrict__ cf_cl,
-                    const float* __restrict__ ym1, const float* __restrict__ yp1, const int stall) {
+                         const float* __restrict__ ym1, const float* __restrict__ yp1, const int y_first,
+                    const int stall) {
   using C = SdCfg<CW, SD>;
   // every tile, the diagonal one included, streams through a ring of R = D + 1 stages
   constexpr int R = C::D + 1;
@@ -307,6 +308,7 @@ clenshaw_sddmm_bulk(const int n_atoms, const int32_t* __restrict__ row_ptr,
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  pdl_wait();
 
   // own-row tiles streamed after the neighbour tiles, with the component of the (per-cluster)
   // coefficient vector that scales them: b_prev (-1), y_k (.y, when it is not staged), y_{k-1}
@@ -317,8 +319,10 @@ clenshaw_sddmm_bulk(const int n_atoms, const int32_t* __restrict__ row_ptr,
   int n_extra = 0;
   if (has_out) {
     const bool any = cf_cl != nullptr;
+    const bool y_own = !SD && ypan && (any || cf.y != 0.f);
+    if (y_own && y_first) { extra_src[n_extra] = ypan; extra_kind[n_extra++] = X_Y; }
     if (has_prev) { extra_src[n_extra] = bprev; extra_kind[n_extra++] = X_PREV; }
-    if (!SD && ypan && (any || cf.y != 0.f)) { extra_src[n_extra] = ypan; extra_kind[n_extra++] = X_Y; }
+    if (y_own && !y_first) { extra_src[n_extra] = ypan; extra_kind[n_extra++] = X_Y; }
     if (ym1 && (any || cf.z != 0.f)) { extra_src[n_extra] = ym1; extra_kind[n_extra++] = X_YM1; }
     if (yp1 && (any || cf.w != 0.f)) { extra_src[n_extra] = yp1; extra_kind[n_extra++] = X_YP1; }
   }
@@ -542,6 +546,7 @@ sddmm_window_g(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  pdl_wait();
   // steps of the window that take part for atom a
   auto atom_window = [&](int a) {
     return batch.atom_cl && kcl ? min(nw, max(0, __ldg(kcl + __ldg(batch.atom_cl + a)) - k_lo)) : nw;
@@ -684,6 +689,184 @@ sddmm_window_g(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
   if (!ok) atomicOr(err, 2);
 }
 
+// ---- outer products of one or more steps, after them (FP32, 9x9 blocks, 128 or 256 probes) --------------
+//
+// Gacc_ab += sum_t w_t sum_probes y_t[a] x_t[b]^T, t in order, for every stored block (a, b): what the
+// fused kernel adds inside its steps, with its additions (per lane over its interleaved 4-probe groups,
+// a butterfly over the lanes, FP64 over the steps), so the result has its bits.  A warp holds all 81 sums
+// of a block: 18 16-byte reads serve 324 FMAs where the fused kernel's three rows per warp read 12 for
+// 108.  The next 128 probes (or the next step or block) of x come into each register as the rows are done
+// with it: 8/9 of the FMAs cover their latency.  12 warps per SM of 168 registers; what binds is the
+// latency that these leave and, at 128 probes, the butterfly (372 of 775 instructions a block and step).
+// us per backward step with its outer products, fused -> a step kernel and these: 147 atoms x 128 probes
+// 31 -> 11, 1,000 x 128 61 -> 30, 10,000 x 128 488 -> 263, 147 x 256 27 -> 15, 1,000 x 256 66 -> 58, 10,000
+// x 256 548 -> 510.  At 512 probes both take the same (823 -> 836 at 10,000 atoms) and the fused kernel stays.
+constexpr int OUT_STEPS = 64;  // steps per launch at most
+struct OuterPanels {
+  const float* y[OUT_STEPS];  // y_k, highest k first
+  const float* x[OUT_STEPS];  // ybar_{k+1}
+};
+
+// 128 probes: a warp takes one block through all steps, the FP64 accumulator in registers; y_t[a] comes
+// from L1, where the row's other blocks use it too.
+__global__ void __launch_bounds__(128, 3)
+outer_blocks(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+             const int64_t nnzb, const __grid_constant__ OuterPanels wp, const int nt, const int last_is_y0,
+             double* __restrict__ Gacc) {
+  constexpr int S = 128;
+  pdl_wait();
+  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (gw >= nnzb) return;
+  const int k = (int)gw, b = __ldg(col + k), a = row_of_block(row_ptr, n_atoms, k, lane);
+  const int64_t offa = (int64_t)9 * a * S + 4 * lane, offb = (int64_t)9 * b * S + 4 * lane;
+  double* g = Gacc + (int64_t)k * 81 + lane;
+  double ga[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) ga[j] = lane < 27 ? g[27 * j] : 0.0;
+  float4 x[9];
+#pragma unroll
+  for (int l = 0; l < 9; ++l) x[l] = __ldg(reinterpret_cast<const float4*>(wp.x[0] + offb + l * S));
+  for (int t = 0; t < nt; ++t) {
+    const float* yt = wp.y[t] + offa;
+    const float* xn = wp.x[min(t + 1, nt - 1)] + offb;
+    float4 y[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) y[i] = __ldg(reinterpret_cast<const float4*>(yt + i * S));
+    float acc[81];
+#pragma unroll
+    for (int l = 0; l < 9; ++l) {
+      const float4 u = x[l];
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        float v = y[i].x * u.x;
+        v = fmaf(y[i].y, u.y, v);
+        v = fmaf(y[i].z, u.z, v); v = fmaf(y[i].w, u.w, v);
+        acc[i * 9 + l] = v;
+      }
+      x[l] = __ldg(reinterpret_cast<const float4*>(xn + l * S));
+    }
+    const double w = last_is_y0 && t == nt - 1 ? 1.0 : 2.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      float v[32];
+#pragma unroll
+      for (int e = 0; e < 32; ++e) v[e] = e < 27 ? acc[27 * j + e] : 0.f;
+      butterfly32(v, lane);
+      ga[j] += w * (double)v[0];
+    }
+  }
+  if (lane < 27) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) g[27 * j] = ga[j];
+  }
+}
+
+// 256 probes: a CTA of NW warps takes a block row and stages y_t[a] in shared memory, two steps
+// deep; a warp takes every NW-th block.
+template <int NW>
+__global__ void __launch_bounds__(32 * NW, 12 / NW)
+outer_rows(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+            const __grid_constant__ OuterPanels wp, const int nt, const int last_is_y0, double* __restrict__ Gacc,
+            int* __restrict__ err) {
+  constexpr int NC = 2, S = 128 * NC, XB = 9 * S * 4;
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ __align__(8) uint64_t bars[4];
+  const uint32_t full = smem_u32(bars), empty = full + 16;  // two each
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(full + 8 * i, 1);
+      mbar_init(empty + 8 * i, NW);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  pdl_wait();
+  // tiles y_t[a] of the CTA's rows and steps, in order: number it in buffer it & 1
+  const int rows = (n_atoms - blockIdx.x + gridDim.x - 1) / gridDim.x;
+  const int n_tiles = rows * nt;
+  auto issue = [&](int it) {
+    const int a = blockIdx.x + (it / nt) * gridDim.x;
+    const uint32_t bar = full + 8 * (it & 1);
+    mbar_expect_tx(bar, XB);
+    bulk_g2s(smem_u32(smem + (it & 1) * XB), wp.y[it % nt] + (int64_t)9 * a * S, XB, bar);
+  };
+  if (threadIdx.x == 0) {
+    issue(0);
+    if (n_tiles > 1) issue(1);
+  }
+  bool ok = true;
+  int it = 0;
+  for (int a = blockIdx.x; a < n_atoms && ok; a += gridDim.x) {
+    const int k0 = __ldg(row_ptr + a), nb = __ldg(row_ptr + a + 1) - k0;
+    float4 x[9];
+    if (warp < nb) {
+      const float* x0 = wp.x[0] + (int64_t)9 * __ldg(col + k0 + warp) * S + 4 * lane;
+#pragma unroll
+      for (int l = 0; l < 9; ++l) x[l] = __ldg(reinterpret_cast<const float4*>(x0 + l * S));
+    }
+    for (int t = 0; t < nt; ++t, ++it) {
+      ok = mbar_wait(full + 8 * (it & 1), (it >> 1) & 1);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      const float* Y = reinterpret_cast<const float*>(smem + (it & 1) * XB) + 4 * lane;
+      const double w = last_is_y0 && t == nt - 1 ? 1.0 : 2.0;
+      for (int q = warp; q < nb; q += NW) {
+        // where the next stage's x lies: this block's next probes, the next block, the next step
+        const float* xq = wp.x[t] + (int64_t)9 * __ldg(col + k0 + q) * S + 4 * lane;
+        const bool more = q + NW < nb;
+        const float* xn = wp.x[more || t + 1 == nt ? t : t + 1] +
+                          (int64_t)9 * __ldg(col + k0 + (more ? q + NW : warp)) * S + 4 * lane;
+        float acc[81];
+#pragma unroll
+        for (int e = 0; e < 81; ++e) acc[e] = 0.f;
+#pragma unroll 1
+        for (int m = 0; m < NC; ++m) {
+          float4 y[9];
+#pragma unroll
+          for (int i = 0; i < 9; ++i) y[i] = *reinterpret_cast<const float4*>(Y + i * S + 128 * m);
+          const float* nx = m + 1 < NC ? xq + 128 * (m + 1) : xn;
+#pragma unroll
+          for (int l = 0; l < 9; ++l) {
+            const float4 u = x[l];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+              float v = acc[i * 9 + l];
+              v = fmaf(y[i].x, u.x, v); v = fmaf(y[i].y, u.y, v);
+              v = fmaf(y[i].z, u.z, v); v = fmaf(y[i].w, u.w, v);
+              acc[i * 9 + l] = v;
+            }
+            x[l] = __ldg(reinterpret_cast<const float4*>(nx + l * S));
+          }
+        }
+        double* g = Gacc + (int64_t)(k0 + q) * 81 + lane;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          float v[32];
+#pragma unroll
+          for (int e = 0; e < 32; ++e) v[e] = e < 27 ? acc[27 * j + e] : 0.f;
+          butterfly32(v, lane);
+          // fire-and-forget: one writer per entry, its additions in program order
+          if (lane < 27) atomicAdd(g + 27 * j, w * (double)v[0]);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(empty + 8 * (it & 1));
+      if (threadIdx.x == 0 && it + 2 < n_tiles) {
+        if (mbar_wait(empty + 8 * (it & 1), (it >> 1) & 1)) issue(it + 2);
+        else atomicOr(err, 2);  // nothing is copied: the consumers give up in turn
+      }
+    }
+  }
+  if (!ok) {
+    if (lane == 0) atomicOr(err, 2);
+    // let the copies in flight land before the CTA exits
+    if (threadIdx.x == 0)
+      for (int j = it; j < it + 2 && j < n_tiles; ++j) mbar_wait(full + 8 * (j & 1), (j >> 1) & 1);
+  }
+}
+
 // ---- self-fed adjoint step for 128 probes (windowed schedule) ---------------------------------
 //
 // clenshaw_sddmm_bulk<1, false> with one warp per CTA and no producer warp: lane 0 keeps R tiles
@@ -704,7 +887,7 @@ clenshaw_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int3
               const float* __restrict__ hv, const float* __restrict__ bin, const float* bprev, float* bout,
               const float* __restrict__ ypan, const float4 cf, const uint64_t seed, const int s,
               int* __restrict__ err, const BatchRows batch, const float4* __restrict__ cf_cl,
-              const float* __restrict__ ym1, const float* __restrict__ yp1) {
+              const float* __restrict__ ym1, const float* __restrict__ yp1, const int y_first) {
   using C = ClenSelfCfg<R>;
   extern __shared__ __align__(128) unsigned char smem[];
   const uint32_t bar0 = smem_u32(smem + R * C::SB);
@@ -716,8 +899,10 @@ clenshaw_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int3
   int n_extra = 0;
   {
     const bool any = cf_cl != nullptr;
+    const bool y_own = ypan && (any || cf.y != 0.f);
+    if (y_own && y_first) { extra_src[n_extra] = ypan; extra_kind[n_extra++] = X_Y; }
     if (bprev) { extra_src[n_extra] = bprev; extra_kind[n_extra++] = X_PREV; }
-    if (ypan && (any || cf.y != 0.f)) { extra_src[n_extra] = ypan; extra_kind[n_extra++] = X_Y; }
+    if (y_own && !y_first) { extra_src[n_extra] = ypan; extra_kind[n_extra++] = X_Y; }
     if (ym1 && (any || cf.z != 0.f)) { extra_src[n_extra] = ym1; extra_kind[n_extra++] = X_YM1; }
     if (yp1 && (any || cf.w != 0.f)) { extra_src[n_extra] = yp1; extra_kind[n_extra++] = X_YP1; }
   }
@@ -726,6 +911,7 @@ clenshaw_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int3
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
+  pdl_wait();
   int p_a = blockIdx.x, p_q = 0, p_k0 = 0, p_nb = 0, issued = 0;
   auto load_row = [&]() {  // rows with no tile (no stored block, no source term) are skipped
     for (; p_a < n_atoms; p_a += gridDim.x) {
@@ -939,30 +1125,33 @@ template <int CW, bool SD>
 static void launch_fused_cw(tbk_ctx* ctx, const HOp& op, const void* bin, const void* bprev, void* bout,
                             const void* ypan, float4 cf, uint64_t seed, int s, double w, double* Gacc,
                             int* err, const BatchRows& batch, const float4* cf_cl, const void* ym1,
-                            const void* yp1) {
+                            const void* yp1, int y_first) {
   using C = SdCfg<CW, SD>;
-  TBK_CUDA(cudaFuncSetAttribute(clenshaw_sddmm_bulk<CW, SD>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-  int occ = 0;
-  TBK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, clenshaw_sddmm_bulk<CW, SD>, C::THREADS, C::SMEM));
-  TBK_CHECK_ARG(occ > 0, "fused adjoint kernel does not fit on this device");
+  static int occ_dev[64] = {0};
+  int& occ = occ_dev[ctx->device & 63];
+  if (!occ) {
+    TBK_CUDA(cudaFuncSetAttribute(clenshaw_sddmm_bulk<CW, SD>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+    TBK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, clenshaw_sddmm_bulk<CW, SD>, C::THREADS, C::SMEM));
+    TBK_CHECK_ARG(occ > 0, "fused adjoint kernel does not fit on this device");
+  }
   const int G = std::max(1, std::min(op.n_atoms, occ * ctx->num_sms));
-  clenshaw_sddmm_bulk<CW, SD><<<G, C::THREADS, C::SMEM, ctx->stream>>>(
-      op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)bin, (const float*)bprev,
-      (float*)bout, (const float*)ypan, cf, seed, s, w, Gacc, err, batch, cf_cl, (const float*)ym1,
-      (const float*)yp1, ctx->stall_next_adjoint);
+  launch_pdl(ctx, clenshaw_sddmm_bulk<CW, SD>, G, C::THREADS, C::SMEM, op.n_atoms, op.row_ptr, op.col,
+             (const float*)op.hv, (const float*)bin, (const float*)bprev, (float*)bout, (const float*)ypan, cf, seed, s, w,
+             Gacc, err, batch, cf_cl, (const float*)ym1, (const float*)yp1, y_first, ctx->stall_next_adjoint);
   ctx->stall_next_adjoint = 0;
   post_launch(ctx, "clenshaw_sddmm_bulk");
 }
 
+// A backward step, fused with its outer products (Gacc) or alone (Gacc NULL).  y_first: alone, add the
+// y_k term before y_prev as the fused kernel does.
 void launch_fused(tbk_ctx* ctx, const HOp& op, const void* bin, const void* bprev, void* bout,
                   const void* ypan, float4 cf, uint64_t seed, int s, double w, double* Gacc,
                   int* err, const BatchRows& batch, const float4* cf_cl, const void* ym1,
-                  const void* yp1) {
+                  const void* yp1, int y_first) {
   KernelTimerScope timer(ctx, TBK_KERNEL_BACKWARD);
-  // Gacc == nullptr: the Clenshaw step alone
   auto go = [&](auto cw, auto sd) {
     launch_fused_cw<decltype(cw)::value, decltype(sd)::value>(ctx, op, bin, bprev, bout, ypan, cf, seed, s, w,
-                                                              Gacc, err, batch, cf_cl, ym1, yp1);
+                                                              Gacc, err, batch, cf_cl, ym1, yp1, y_first);
   };
   using T = std::true_type;
   using F = std::false_type;
@@ -980,11 +1169,64 @@ void launch_fused(tbk_ctx* ctx, const HOp& op, const void* bin, const void* bpre
       TBK_CHECK_ARG(occ > 0, "self-fed adjoint kernel does not fit on this device");
     }
     const int G = std::max(1, std::min(op.n_atoms, occ * ctx->num_sms));
-    clenshaw_self<CLEN_SELF_R><<<G, 32, C::SMEM, ctx->stream>>>(
-        op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)bin, (const float*)bprev,
-        (float*)bout, (const float*)ypan, cf, seed, s, err, batch, cf_cl, (const float*)ym1, (const float*)yp1);
+    launch_pdl(ctx, clenshaw_self<CLEN_SELF_R>, G, 32, C::SMEM, op.n_atoms, op.row_ptr, op.col, (const float*)op.hv,
+               (const float*)bin, (const float*)bprev, (float*)bout, (const float*)ypan, cf, seed, s, err, batch, cf_cl,
+               (const float*)ym1, (const float*)yp1, y_first);
     post_launch(ctx, "clenshaw_self");
   }
+}
+
+// A backward step whose outer products run later, with the fused kernel's additions.
+static void launch_adjoint_step(tbk_ctx* ctx, const HOp& op, const void* bin, void* bprev, void* bout,
+                                const void* ypan, float4 cf, uint64_t seed, int s, int* err, const void* ym1,
+                                const void* yp1) {
+  StepArgs a;
+  a.seed = seed;
+  a.s = s;
+  a.yin = bin;
+  a.yprev = bprev;
+  a.yout = bout;
+  a.alpha = 2.0;
+  a.c_r = cf.x;
+  a.src[0] = ypan;
+  a.csrc[0] = cf.y;
+  a.src[1] = ym1;
+  a.csrc[1] = ym1 ? cf.z : 0.0;
+  a.src[2] = yp1;
+  a.csrc[2] = yp1 ? cf.w : 0.0;
+  a.err = err;
+  a.adjoint = 1;
+  if (lane_adjoint_step(ctx, op, a)) return;
+  launch_fused(ctx, op, bin, bprev, bout, ypan, cf, seed, s, 0.0, nullptr, err, BatchRows(), nullptr, ym1, yp1, 1);
+}
+
+// Gacc += the outer products of nt steps (in order; the last one that of y_0 when last_is_y0).
+template <int NW>
+static void launch_outer_rows(tbk_ctx* ctx, const HOp& op, const OuterPanels& wp, int nt, int last_is_y0, double* Gacc,
+                            int* err) {
+  constexpr int SMEM = 2 * 9 * 256 * 4;
+  static int occ_dev[64] = {0};
+  int& occ = occ_dev[ctx->device & 63];
+  if (!occ) {
+    TBK_CUDA(cudaFuncSetAttribute(outer_rows<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
+    TBK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, outer_rows<NW>, 32 * NW, SMEM));
+    TBK_CHECK_ARG(occ > 0, "outer-product kernel does not fit on this device");
+  }
+  launch_pdl(ctx, outer_rows<NW>, std::min(op.n_atoms, occ * ctx->num_sms), 32 * NW, SMEM, op.n_atoms, op.row_ptr,
+             op.col, wp, nt, last_is_y0, Gacc, err);
+}
+
+static void launch_outer(tbk_ctx* ctx, const HOp& op, const OuterPanels& wp, int nt, int last_is_y0, int s,
+                         double* Gacc, int* err) {
+  KernelTimerScope timer(ctx, TBK_KERNEL_BACKWARD);
+  if (s == 128)
+    launch_pdl(ctx, outer_blocks, ceil_div(op.nnzb, 4), 128, 0, op.n_atoms, op.row_ptr, op.col, op.nnzb, wp, nt,
+               last_is_y0, Gacc);
+  else if (op.n_atoms <= ctx->num_sms)  // few rows: all 12 warps of an SM on one row
+    launch_outer_rows<12>(ctx, op, wp, nt, last_is_y0, Gacc, err);
+  else
+    launch_outer_rows<4>(ctx, op, wp, nt, last_is_y0, Gacc, err);
+  post_launch(ctx, "outer_products");
 }
 
 void launch_sddmm(tbk_ctx* ctx, const HOp& op, const void* y, const void* x, int s, double w, double* Gacc) {
@@ -1062,12 +1304,15 @@ template <int NC>
 static void launch_window_g(tbk_ctx* ctx, const HOp& op, const WindowPanels& wp, int nw, int s, double w, double* Gacc, int* err, const BatchRows& batch,
                             const int32_t* kcl, int k_lo) {
   using C = WinGCfg<NC>;
-  TBK_CUDA(cudaFuncSetAttribute(sddmm_window_g<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-  int occ = 0;
-  TBK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sddmm_window_g<NC>, C::THREADS, C::SMEM));
-  TBK_CHECK_ARG(occ > 0, "windowed outer-product kernel does not fit on this device");
+  static int occ_dev[64] = {0};
+  int& occ = occ_dev[ctx->device & 63];
+  if (!occ) {
+    TBK_CUDA(cudaFuncSetAttribute(sddmm_window_g<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+    TBK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sddmm_window_g<NC>, C::THREADS, C::SMEM));
+    TBK_CHECK_ARG(occ > 0, "windowed outer-product kernel does not fit on this device");
+  }
   const int G = std::max(1, std::min(op.n_atoms, occ * ctx->num_sms));
-  sddmm_window_g<NC><<<G, C::THREADS, C::SMEM, ctx->stream>>>(op.n_atoms, op.row_ptr, op.col, wp, nw, s, w, Gacc, err, batch, kcl, k_lo);
+  launch_pdl(ctx, sddmm_window_g<NC>, G, C::THREADS, C::SMEM, op.n_atoms, op.row_ptr, op.col, wp, nw, s, w, Gacc, err, batch, kcl, k_lo);
   post_launch(ctx, "sddmm_window_g");
 }
 
@@ -1105,6 +1350,18 @@ __global__ void ybar_init(int64_t n, T ca, const T* __restrict__ yk, T cb, const
   for (int j = 0; j < 4; ++j) out[i + j] = v[j];
 }
 
+// Steps whose outer products run together after them (0: fused into each step).  Up to 64, as long as
+// their panels stay within half of L2, where the next kernel finds them; at 128 probes at least 8, since
+// one warp per block then also saves the additions to Gacc.  us per step pair (forward and backward), fused
+// and 1 / 2 / 4 / 8 steps: 2,000 atoms x 128 probes 120, 94 / 84 / 81 / 78; 10,000 x 128 584, 465 / 402 /
+// 375 / 365; 2,000 x 256 160, 141 / 140 / 140 / 139; 10,000 x 256 750, 704 / 704 / 707 / 710; at 512
+// probes 500 atoms 66.2 / 65.7, 1,000 atoms 119.1 / 119.4, 10,000 atoms 1147 / 1148.
+static int deferred_steps(const HOp& op, int s) {
+  if (s == 512) return 0;
+  const int64_t fit = ((int64_t)48 << 20) / (2 * op.n_rows * s * 4);
+  return (int)std::max<int64_t>(s == 128 ? 8 : 1, std::min<int64_t>(OUT_STEPS, fit));
+}
+
 // get_coefs() is called once every y_1 .. y_K has been formed for the first time (with
 // `partials` != NULL those steps also wrote their moment partial sums at partials + 2 nctas (t-1),
 // so the caller can finish the moments, solve for mu and return the coefficients c_0 .. c_{p-1}).
@@ -1117,6 +1374,8 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
   const bool f64 = op.prec == TBK_FP64;
   const size_t esz = f64 ? 8 : 4;
   const bool windowed = sched == 1 && !f64;
+  // fused schedule: steps whose outer products run after them in one launch (0: inside each step)
+  int defer = sched == 0 && !f64 && !bt ? deferred_steps(op, s) : 0;
   // outer products on the tensor cores after each backward step, where that kernel applies
   const bool tensor = sched == 2 && !bt && !f64 && tc_sddmm_eligible(ctx, op, s, tc_sddmm_max_row(ctx, op));
   // a stored probe block y_0 (single system): read wherever the probe enters
@@ -1157,7 +1416,12 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
   const int npan = K;  // y_1 .. y_K
   // ybar_j lives in ring slot j mod NB: the two of the recurrence, plus the window's SDW panels
   // when the outer products are summed over windows of steps; a batch also keeps the probe panel
-  const int NB = windowed ? SDW + 2 : 2;
+  if (defer > 0) {
+    // as many ybar panels as fit beside the all-stored plan
+    const int64_t room = (int64_t)(budget / panel) - (npan + 2) - 2;
+    defer = room < 0 ? 0 : (int)std::min<int64_t>(std::min(defer, K), room + 1);
+  }
+  const int NB = windowed ? SDW + 2 : (defer > 1 ? defer + 1 : 2);
   const int NX = NB + (bt ? 1 : 0);
   int seg = std::max(1, npan);
   auto seg_plan = [&]() {
@@ -1272,6 +1536,9 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
       }
     }
   }
+  if (!all_stored) defer = 0;  // the replay reuses the panels that waiting outer products read
+  OuterPanels wait{};
+  int n_wait = 0;
   int k = K;
   for (int sg = nseg - 1; sg >= -1 && k >= 0; --sg) {
     const int t0 = sg >= 0 ? 1 + seg * sg : 0;
@@ -1349,9 +1616,20 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
                              : make_float4(r_gen ? (float)cb(1) : 0.f, (float)ca(k), r_gen ? 0.f : (float)cb(k),
                                            (float)cc(k));
         const float4* cfk = bt ? bt->cft + (size_t)k * bt->K.size() : nullptr;
+        if (defer) {
+          launch_adjoint_step(ctx, o, YB(k + 1), k + 2 <= K ? YB(k + 2) : nullptr, YB(k), Y(k), cf, probe_seed, s, err,
+                              (k >= 2 || r_panel) ? Y(k - 1) : nullptr, Y(k + 1));
+          wait.y[n_wait] = (const float*)Y(k);
+          wait.x[n_wait++] = (const float*)YB(k + 1);
+          if (n_wait == defer) {
+            launch_outer(ctx, o, wait, n_wait, 0, s, Gacc, err);
+            n_wait = 0;
+          }
+          continue;
+        }
         launch_fused(ctx, o, YB(k + 1), (k + 2 <= K || bt) ? YB(k + 2) : nullptr, YB(k), Y(k), cf, probe_seed, s,
                      2.0, (windowed || tensor) ? nullptr : Gacc, err, br, cfk,
-                     (k >= 2 || r_panel) ? Y(k - 1) : nullptr, Y(k + 1));
+                     (k >= 2 || r_panel) ? Y(k - 1) : nullptr, Y(k + 1), 0);
         // G += 2 y_k ybar_{k+1}^T on the pattern, on the tensor cores
         if (tensor) launch_tc_sddmm(ctx, o, Y(k), YB(k + 1), s, 2.0, Gacc, err);
         if (windowed && (k - 1) % SDW == 0) {
@@ -1364,6 +1642,10 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
           }
           launch_window(ctx, o, wp, nw, s, 2.0, Gacc, err, br, bt ? bt->d_K : nullptr, k);
         }
+      } else if (defer) {
+        wait.y[n_wait] = (const float*)Y(0);
+        wait.x[n_wait++] = (const float*)YB(1);
+        launch_outer(ctx, o, wait, n_wait, 1, s, Gacc, err);
       } else if (windowed) {
         // G += y_0 ybar_1^T
         WindowPanels wp{};
@@ -1375,7 +1657,7 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
         launch_tc_sddmm(ctx, o, Y(0), YB(1), s, 1.0, Gacc, err);
       } else {
         launch_fused(ctx, o, YB(1), nullptr, nullptr, Y(0), make_float4(0.f, 0.f, 0.f, 0.f), probe_seed, s,
-                     1.0, Gacc, err, br, nullptr, nullptr, nullptr);
+                     1.0, Gacc, err, br, nullptr, nullptr, nullptr, 0);
       }
     }
   }

@@ -419,7 +419,7 @@ bool fused_eligible(const HOp& op, int s, int plain);
 void launch_fused(tbk_ctx* ctx, const HOp& op, const void* bin, const void* bprev, void* bout,
                   const void* ypan, float4 cf, uint64_t seed, int s, double w, double* Gacc,
                   int* err, const BatchRows& batch, const float4* cf_cl, const void* ym1,
-                  const void* yp1);
+                  const void* yp1, int y_first);
 void launch_transpose_map(tbk_ctx* ctx, int n_atoms, const int32_t* row_ptr, const int32_t* col,
                           int32_t* tr, int* err);
 void launch_symmetrize_batched(tbk_ctx* ctx, int n_atoms, const int32_t* row_ptr, const int32_t* tr,

@@ -66,7 +66,7 @@ struct StepArgs {
   uint64_t seed = 0;
   int s = 0;
   int direct = 0;
-  // further own-row terms c_e E_e of y_out (E_e a panel), plain and row-split kernels only
+  // further own-row terms c_e E_e of y_out (E_e a panel): plain and FP64 kernels, adjoint lane kernel
   const void* src[3] = {nullptr, nullptr, nullptr};
   double csrc[3] = {0.0, 0.0, 0.0};
   double* partials = nullptr;
@@ -78,12 +78,15 @@ struct StepArgs {
   int per_task = 0;
   int use_tc = 0;           // tensor-core (tcgen05) step where it applies
   int grid = 0;             // CTAs of the launch (0: step_grid_ctas)
+  int adjoint = 0;          // lane kernel: src[0] is added before y_prev, src[1] and src[2] after; no sums
 };
 // Consumer warps of the TMA-fed step kernel for this operator and probe count (0 = not used).
 int bulk_consumer_warps(const HOp& op, int s);
 // CTAs a step launches for this operator and probe count.
 int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s);
 void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a);
+// An adjoint step (a.adjoint) on the kernel for small operators; false where that does not apply.
+bool lane_adjoint_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a);
 // panel = c * r (probe block) for all rows.
 void launch_scaled_probe(tbk_ctx* ctx, const HOp& op, void* panel, double c, uint64_t seed, int s);
 

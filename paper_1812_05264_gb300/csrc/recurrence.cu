@@ -767,12 +767,15 @@ struct LaneCfg {
   static constexpr int SMEM = R * SB + NW * EB + 16 * R;
 };
 
-template <int NW>
+// ADJ: a step of the adjoint, with the further terms of `src` added in the fused adjoint kernel's order
+// (y_k before y_prev, the others after) and no moment sums.
+template <int NW, bool ADJ>
 __global__ void __launch_bounds__(32 * (NW + 1))
 cheb_step_lane(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const float* __restrict__ hv, const float* __restrict__ yin, const float* yprev, float* yout,
                const float alpha, const float c_r, const uint64_t seed, const int s, const int direct,
-               double* __restrict__ partials, int* __restrict__ err, const int stall) {
+               const StepSources<float> src, double* __restrict__ partials, int* __restrict__ err,
+               const int stall) {
   using C = LaneCfg<NW>;
   constexpr int R = C::R;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -842,14 +845,20 @@ cheb_step_lane(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
     const int a = task / n_chunks, ch = task - a * n_chunks;
     const int k0 = __ldg(row_ptr + a), nb = __ldg(row_ptr + a + 1) - k0;
     const int p0 = ch * C::P + 32 * warp + 4 * igrp;  // the items' first probe
-    // the items' y_prev and own y_in, fetched while the tiles stream
-    float4 yp[3], xo[3];
+    // the items' y_prev and own y_in (ADJ: the source terms), fetched while the tiles stream
+    float4 yp[3], xo[3], so[ADJ ? 3 : 1][3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       const bool has = irow + 4 * j < 9 && p0 < s;
       const int64_t off = ((int64_t)9 * a + irow + 4 * j) * s + p0;
       yp[j] = has && yprev ? *reinterpret_cast<const float4*>(yprev + off) : make_float4(0.f, 0.f, 0.f, 0.f);
-      xo[j] = has && partials && !direct ? *reinterpret_cast<const float4*>(yin + off) : make_float4(0.f, 0.f, 0.f, 0.f);
+      if constexpr (ADJ) {
+#pragma unroll
+        for (int e = 0; e < 3; ++e)
+          so[e][j] = has && src.p[e] ? __ldg(reinterpret_cast<const float4*>(src.p[e] + off)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      } else {
+        xo[j] = has && partials && !direct ? *reinterpret_cast<const float4*>(yin + off) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
     }
     float2 acc[4];  // rows (0, 1), (2, 3), (4, 5), (6, 7)
     float acc8 = 0.f;
@@ -899,11 +908,22 @@ cheb_step_lane(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
 #pragma unroll
         for (int v = 0; v < 4; ++v) yo[v] = fmaf(c_r, r[v], yo[v]);
       }
+      auto add = [&](float c, const float4& x) {
+        yo[0] = fmaf(c, x.x, yo[0]); yo[1] = fmaf(c, x.y, yo[1]);
+        yo[2] = fmaf(c, x.z, yo[2]); yo[3] = fmaf(c, x.w, yo[3]);
+      };
+      if constexpr (ADJ) {
+        if (src.c[0] != 0.f) add(src.c[0], so[0][j]);
+      }
       if (yprev) {
         yo[0] -= yp[j].x; yo[1] -= yp[j].y; yo[2] -= yp[j].z; yo[3] -= yp[j].w;
       }
+      if constexpr (ADJ) {
+        if (src.c[1] != 0.f) add(src.c[1], so[1][j]);
+        if (src.c[2] != 0.f) add(src.c[2], so[2][j]);
+      }
       *reinterpret_cast<float4*>(yout + ((int64_t)9 * a + row) * s + p0) = make_float4(yo[0], yo[1], yo[2], yo[3]);
-      if (partials) {
+      if (!ADJ && partials) {
         const float xin[4] = {direct ? r[0] : xo[j].x, direct ? r[1] : xo[j].y, direct ? r[2] : xo[j].z,
                               direct ? r[3] : xo[j].w};
         float q0 = 0.f, q1 = 0.f;
@@ -919,7 +939,7 @@ cheb_step_lane(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
     __syncwarp();  // the buffer is free again
   }
   if (!ok) atomicOr(err, 2);
-  if (partials) step_partials(partials, (double)cs0 + (double)cc0, (double)cs1 + (double)cc1, warp, lane, nw);
+  if (!ADJ && partials) step_partials(partials, (double)cs0 + (double)cc0, (double)cs1 + (double)cc1, warp, lane, nw);
 }
 
 // ---- FP64 step by rows -------------------------------------------------------------------------------
@@ -1062,9 +1082,10 @@ static int chosen_cw(const tbk_ctx* ctx, const HOp& op, int s, int per_task) {
 
 template <int NW>
 static int occupancy_lane() {
-  cudaFuncSetAttribute(cheb_step_lane<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, LaneCfg<NW>::SMEM);
+  cudaFuncSetAttribute(cheb_step_lane<NW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, LaneCfg<NW>::SMEM);
+  cudaFuncSetAttribute(cheb_step_lane<NW, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, LaneCfg<NW>::SMEM);
   int n = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cheb_step_lane<NW>, 32 * (NW + 1), LaneCfg<NW>::SMEM);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cheb_step_lane<NW, false>, 32 * (NW + 1), LaneCfg<NW>::SMEM);
   return n;
 }
 
@@ -1199,10 +1220,10 @@ static void launch_self(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
 template <int NW>
 static void launch_lane_nw(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
   const int nw = std::min(NW, (a.s + 31) / 32);
-  launch_pdl(ctx, cheb_step_lane<NW>, G, 32 * (nw + 1),
-               LaneCfg<NW>::SMEM, op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)a.yin,
-               (const float*)a.yprev, (float*)a.yout, (float)a.alpha, (float)a.c_r, a.seed, a.s, a.direct, a.partials,
-               a.err, ctx->stall_next_step);
+  launch_pdl(ctx, a.adjoint ? cheb_step_lane<NW, true> : cheb_step_lane<NW, false>, G, 32 * (nw + 1), LaneCfg<NW>::SMEM,
+             op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)a.yin, (const float*)a.yprev,
+             (float*)a.yout, (float)a.alpha, (float)a.c_r, a.seed, a.s, a.direct, sources<float>(a), a.partials, a.err,
+             ctx->stall_next_step);
   ctx->stall_next_step = 0;
   post_launch(ctx, "cheb_step_lane");
 }
@@ -1214,6 +1235,13 @@ static void launch_lane(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
   if (c == 0) launch_lane_nw<4>(ctx, op, a, G);
   else if (c == 1) launch_lane_nw<8>(ctx, op, a, G);
   else launch_lane_nw<16>(ctx, op, a, G);
+}
+
+bool lane_adjoint_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
+  if (!use_lane(op, a.s)) return false;
+  KernelTimerScope timer(ctx, TBK_KERNEL_BACKWARD);
+  launch_lane(ctx, op, a, step_grid_ctas(ctx, op, a.s));
+  return true;
 }
 
 template <int ROWS>

@@ -47,3 +47,18 @@ def test_plain_outer_products_equal_the_fused_ones(n_atoms):
     Gp, Fp = api.density_and_forces(*args, plain=True)
     assert (G - Gp).abs().max().item() <= 2e-5 * G.abs().max().item()
     assert (F - Fp).abs().max().item() <= 1e-3
+
+
+# Outer products after several steps against the ones fused into each step (a plan with too few panels to
+# store every y_k): the same additions in the same order, so the same bits.  Orders around a full window.
+@pytest.mark.parametrize("n_atoms,s,orders", [(1, 128, (36, 150)), (13, 128, (37, 129, 130, 131)), (153, 128, (41,)),
+                                              (700, 128, (38,)), (1, 256, (36,)), (13, 256, (37, 131)),
+                                              (152, 256, (36,)), (153, 256, (37,)), (1030, 256, (37,))])
+def test_deferred_outer_products_have_the_fused_bits(n_atoms, s, orders):
+    import torch
+    api, wk, ctx, pos, model, H, lo, hi = _setup(n_atoms, s, orders[0], True)
+    for order in orders:
+        args = (ctx, H, model, pos, None, lo, hi, wk.probe_seed, s, order, 6.0, 0.5)
+        G0, F0 = api.density_and_forces(*args)
+        G1, F1 = api.density_and_forces(*args, max_panel_bytes=(order // 2 + 3) * 9 * n_atoms * s * 4)
+        assert torch.equal(G0, G1) and torch.equal(F0, F1)
