@@ -18,6 +18,11 @@
 // p_f(H^_loc) E is formed by the backward (Clenshaw) form of the sum on the recurrence kernels,
 // with the unit-vector source added by a scatter after each step; H X is one more product with
 // the local copies of H itself.
+//
+// FP32 with 9 orbitals: local_clenshaw runs all steps of a region inside one CTA (below).  FP64, one
+// orbital, or a region whose panels exceed shared memory: one recurrence launch per step over all regions.
+#include <algorithm>
+#include <numeric>
 #include <vector>
 
 #include "cheb.cuh"
@@ -51,8 +56,8 @@ __device__ __forceinline__ int region_of(const int32_t* __restrict__ rs, int n_a
 template <bool FILL>
 __global__ void local_pattern(int n_atoms, int64_t n_loc, const int32_t* __restrict__ rs, const int32_t* __restrict__ rcol,
                               const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
-                              int32_t* __restrict__ cnt, const int64_t* __restrict__ lrp, int32_t* __restrict__ lcol,
-                              int32_t* __restrict__ lblk) {
+                              int32_t* __restrict__ cnt, const int64_t* __restrict__ lrp, int32_t* __restrict__ lrow,
+                              int32_t* __restrict__ lcol, int32_t* __restrict__ lblk) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n_loc) return;
   const int a = region_of(rs, n_atoms, t);
@@ -60,6 +65,10 @@ __global__ void local_pattern(int n_atoms, int64_t n_loc, const int32_t* __restr
   const int g = rcol[t];
   int n = 0;
   int64_t o = FILL ? lrp[t] : 0;
+  if (FILL) {
+    lrow[t] = (int32_t)o;
+    if (t == n_loc - 1) lrow[n_loc] = (int32_t)lrp[n_loc];
+  }
   for (int k = rp[g]; k < rp[g + 1]; ++k) {
     const int j = find_in(rcol, r0, r1, col[k]);
     if (j < 0) continue;
@@ -71,6 +80,185 @@ __global__ void local_pattern(int n_atoms, int64_t n_loc, const int32_t* __restr
     ++n;
   }
   if (!FILL) cnt[t] = n;
+}
+
+// size[a] = (atoms, stored blocks) of region a.
+__global__ void region_sizes(int n_atoms, const int32_t* __restrict__ rs, const int64_t* __restrict__ lrp,
+                             int64_t* __restrict__ size) {
+  const int a = blockIdx.x * blockDim.x + threadIdx.x;
+  if (a >= n_atoms) return;
+  size[2 * a] = rs[a + 1] - rs[a];
+  size[2 * a + 1] = lrp[rs[a + 1]] - lrp[rs[a]];
+}
+
+// ---- all steps of a region in one CTA (FP32, 9 orbitals) ------------------------------------------
+//
+// b_k = 2 H^ b_{k+1} - b_{k+2} + c_k E, X = H^ b_1 - b_2 + c_0 E, Y = H X for one region after another:
+// the two panels and as many mapped blocks as fit stay in shared memory, the other blocks come from L2 (the
+// same share of every row, so that all warps read both; the longest rows first, so that a warp's three have
+// about one length).  Nine lanes form an atom's 9 x 9 tile, 3 x 3 entries each: with rows and columns stored
+// as three groups of three in 12 floats, two 16-byte reads serve 9 FMAs.  What binds are these reads: L1
+// delivers 32 floats a cycle and SM, whatever lanes they go to.  Each entry adds its blocks in the order of
+// the step kernel and rounds where it does.  One launch per step reads copies of the blocks (140 MB) and the
+// panels of all regions instead.  500 atoms, 6 A, 126 terms: 10.9 ms so, 5.5 ms here; other tiles: a row of 9
+// entries per lane 7.1 ms, a row of 3 (one atom per warp) 8.0 ms, 5 x 3 7.1 ms.
+constexpr int LC_THREADS = 640, LC_ATOMS = 3, LC_BS = Layout<float, 9>::BS, LC_ROW = 12;
+
+struct LocalArgs {
+  int n_atoms, p, max_m, max_nnz, n_stage;  // n_stage: blocks in shared memory
+  const int32_t *order, *rs, *lrow, *lcol, *lblk, *own;
+  const float *hv, *h1;                     // mapped blocks; H itself (NULL: no Y)
+  const double* coef;
+  float *X, *Y;
+  int* next;
+};
+
+// Position of row (or column) e of 9 among 12: three groups of three.
+__device__ __forceinline__ int lc_pos(int e) { return e + e / 3; }
+
+// Mapped blocks with each column's rows at those positions.
+__global__ void local_blocks(int64_t n, const float* __restrict__ hv, float* __restrict__ dst) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n) return;
+  const int j = (int)(e % 12);
+  dst[e] = (j & 3) < 3 ? hv[e - j + j - j / 4] : 0.f;
+}
+
+__device__ __forceinline__ void local_stage(const LocalArgs& A, const float* __restrict__ hv, float* hs, const int2* stage,
+                                            int r0, int m) {
+  float4* dst = reinterpret_cast<float4*>(hs);
+  const float4* src = reinterpret_cast<const float4*>(hv);
+  for (int t = threadIdx.x >> 5; t < m; t += LC_THREADS / 32) {
+    const int kb = A.lrow[r0 + t];
+    for (int e = threadIdx.x & 31; e < stage[t].y * (LC_BS / 4); e += 32) {
+      const int k = e / (LC_BS / 4), j = e - k * (LC_BS / 4);
+      dst[stage[t].x * (LC_BS / 4) + e] = __ldg(src + (int64_t)__ldg(A.lblk + kb + k) * (LC_BS / 4) + j);
+    }
+  }
+}
+
+// out = alpha h in - out (SUB) or alpha h in, + c at the unit vectors of the atom at position o.
+template <bool SUB>
+__device__ __forceinline__ void local_step(const LocalArgs& A, const float* __restrict__ hv, const float* hs,
+                                           const int* idx, const int* perm, const int2* stage, int r0, int m,
+                                           int k0, const float* in, float* out, float alpha, double c, int o) {
+  const int lane = threadIdx.x & 31, sub = lane / 9, gi = (lane - 9 * sub) / 3, gc = lane % 3;  // 9 % 3 = 0
+  for (int q = LC_ATOMS * (threadIdx.x >> 5) + sub; q < m && sub < LC_ATOMS; q += LC_ATOMS * (LC_THREADS / 32)) {
+    const int t = perm[q];
+    const int kb = __ldg(A.lrow + r0 + t) - k0, ke = __ldg(A.lrow + r0 + t + 1) - k0;
+    float acc[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int v = 0; v < 3; ++v) acc[i][v] = 0.f;
+    auto block = [&](const float* x, auto&& column) {
+#pragma unroll
+      for (int l = 0; l < 9; ++l) {
+        const float4 u = *reinterpret_cast<const float4*>(x + l * LC_ROW), h = column(l * 12);
+        acc[0][0] = fmaf(h.x, u.x, acc[0][0]);
+        acc[0][1] = fmaf(h.x, u.y, acc[0][1]);
+        acc[0][2] = fmaf(h.x, u.z, acc[0][2]);
+        acc[1][0] = fmaf(h.y, u.x, acc[1][0]);
+        acc[1][1] = fmaf(h.y, u.y, acc[1][1]);
+        acc[1][2] = fmaf(h.y, u.z, acc[1][2]);
+        acc[2][0] = fmaf(h.z, u.x, acc[2][0]);
+        acc[2][1] = fmaf(h.z, u.y, acc[2][1]);
+        acc[2][2] = fmaf(h.z, u.z, acc[2][2]);
+      }
+    };
+    int k = kb;
+    const int2 st = stage[t];  // its blocks in shared memory: first slot, number
+    const float* p = hs + st.x * LC_BS + 4 * gi;
+    for (const int ks = kb + st.y; k < ks; ++k, p += LC_BS)
+      block(in + idx[k] + 4 * gc, [&](int e) { return *reinterpret_cast<const float4*>(p + e); });
+    for (; k < ke; ++k) {
+      const float* g = hv + (int64_t)__ldg(A.lblk + k0 + k) * LC_BS + 4 * gi;
+      block(in + idx[k] + 4 * gc, [&](int e) { return __ldg(reinterpret_cast<const float4*>(g + e)); });
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      float4* y = reinterpret_cast<float4*>(out + (t * 9 + 3 * gi + j) * LC_ROW + 4 * gc);
+      const float4 old = *y;
+      const float q3[3] = {old.x, old.y, old.z};
+      float r[3];
+#pragma unroll
+      for (int v = 0; v < 3; ++v) {
+        r[v] = alpha * acc[j][v];
+        if (SUB) r[v] -= q3[v];
+        if (t == o && gi == gc && v == j && c != 0.0) r[v] = (float)((double)r[v] + c);
+      }
+      *y = make_float4(r[0], r[1], r[2], 0.f);
+    }
+  }
+  __syncthreads();
+}
+
+__global__ void __launch_bounds__(LC_THREADS, 1) local_clenshaw(const __grid_constant__ LocalArgs A) {
+  extern __shared__ __align__(16) float lsm[];
+  float* pa = lsm;
+  float* pb = pa + A.max_m * 9 * LC_ROW;
+  float* hs = pb + A.max_m * 9 * LC_ROW;
+  int2* stage = reinterpret_cast<int2*>(hs + (int64_t)A.n_stage * LC_BS);
+  int* perm = reinterpret_cast<int*>(stage + A.max_m);
+  int* idx = perm + A.max_m;
+  __shared__ int job, slots;
+  for (;;) {
+    if (threadIdx.x == 0) {
+      job = atomicAdd(A.next, 1);
+      slots = 0;
+    }
+    __syncthreads();
+    const int q = job;
+    if (q >= A.n_atoms) return;
+    const int r = A.order[q], r0 = A.rs[r], m = A.rs[r + 1] - r0;
+    const int k0 = A.lrow[r0], nnz = A.lrow[r0 + m] - k0, o = A.own[r] - r0;
+    const int n_el = m * 9 * LC_ROW;
+    // idx: a block's column offset in the panels; perm: the rows, the longest first; stage: the share of
+    // a row's blocks that lies in shared memory (the same for every row: all warps read both spaces)
+    const int64_t share = (int64_t)min(A.n_stage, nnz) * 65536 / max(nnz, 1);
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x; k < nnz; k += LC_THREADS) idx[k] = (A.lcol[k0 + k] - r0) * 9 * LC_ROW;
+    for (int t = threadIdx.x >> 5; t < m; t += LC_THREADS / 32) {
+      const int len = A.lrow[r0 + t + 1] - A.lrow[r0 + t];
+      int rank = 0;
+      if (lane == 0) {
+        const int n = (int)(len * share >> 16);
+        stage[t] = make_int2(atomicAdd(&slots, n), n);
+      }
+      for (int u = lane; u < m; u += 32) {
+        const int lu = A.lrow[r0 + u + 1] - A.lrow[r0 + u];
+        rank += lu > len || (lu == len && u < t);
+      }
+      rank = __reduce_add_sync(0xffffffffu, rank);
+      if (lane == 0) perm[rank] = t;
+    }
+    for (int e = threadIdx.x; e < n_el; e += LC_THREADS) pa[e] = pb[e] = 0.f;
+    __syncthreads();
+    local_stage(A, A.hv, hs, stage, r0, m);
+    if (threadIdx.x < 9) pa[(o * 9 + threadIdx.x) * LC_ROW + lc_pos(threadIdx.x)] = (float)A.coef[A.p - 1];
+    __syncthreads();
+    float *b1 = pa, *b2 = pb;
+    for (int k = A.p - 2; k >= 0; --k) {
+      local_step<true>(A, A.hv, hs, idx, perm, stage, r0, m, k0, b1, b2, k ? 2.f : 1.f, A.coef[k], o);
+      float* t = b1;
+      b1 = b2;
+      b2 = t;
+    }
+    auto store = [&](const float* v, float* dst) {
+      for (int e = threadIdx.x; e < m * 81; e += LC_THREADS) {
+        const int row = e / 9, c = e - 9 * row;
+        dst[((int64_t)r0 * 9 + row) * LC_ROW + c] = v[row * LC_ROW + lc_pos(c)];
+      }
+    };
+    store(b1, A.X);
+    if (A.h1) {
+      local_stage(A, A.h1, hs, stage, r0, m);
+      __syncthreads();
+      local_step<false>(A, A.h1, hs, idx, perm, stage, r0, m, k0, b1, b2, 1.f, 0.0, o);
+      store(b2, A.Y);
+    }
+    __syncthreads();  // the next region overwrites the panels
+  }
 }
 
 // The local copy of every mapped block: dst[k] = src[blk[k]] (BS elements each).
@@ -160,37 +348,100 @@ extern "C" int tbk_local_density(tbk_ctx* ctx, const tbk_bsr* H, const double* p
   int* err = (int*)scratch(ctx, WS_FLAGS, 64);
   TBK_CUDA(cudaMemsetAsync(err, 0, sizeof(int), ctx->stream));
   // 2. the local pattern: M restricted to each region, merged
-  int32_t* cnt = (int32_t*)scratch(ctx, WS_LOCAL2, sizeof(int32_t) * (size_t)n_loc + sizeof(int32_t) * n + 64);
+  int32_t* cnt = (int32_t*)scratch(ctx, WS_LOCAL2, sizeof(int32_t) * ((size_t)n_loc + 2 * (size_t)n) + 64);
   int32_t* own = cnt + n_loc;
+  int32_t* d_order = own + n;  // and the counter of regions taken
   local_pattern<false><<<ceil_div(n_loc, 256), 256, 0, ctx->stream>>>(n, n_loc, rs, rcol, H->row_ptr, H->col, cnt,
-                                                                       nullptr, nullptr, nullptr);
+                                                                       nullptr, nullptr, nullptr, nullptr);
   post_launch(ctx, "local_pattern");
-  int64_t* lrp = (int64_t*)scratch(ctx, WS_LOCAL3, sizeof(int64_t) * ((size_t)n_loc + 1 + scan_tmp_elems(n_loc)));
+  const size_t scan_n = (size_t)n_loc + 1 + scan_tmp_elems(n_loc);
+  int64_t* lrp = (int64_t*)scratch(ctx, WS_LOCAL3, sizeof(int64_t) * (scan_n + 2 * (size_t)n));
+  int64_t* d_size = lrp + scan_n;
   exclusive_scan_i32(ctx, cnt, lrp, n_loc, lrp + n_loc + 1);
+  region_sizes<<<ceil_div(n, 256), 256, 0, ctx->stream>>>(n, rs, lrp, d_size);
+  post_launch(ctx, "region_sizes");
   int64_t nnz_loc = 0;
+  std::vector<int64_t> size(2 * (size_t)n);
   TBK_CUDA(cudaMemcpyAsync(&nnz_loc, lrp + n_loc, sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->stream));
+  TBK_CUDA(cudaMemcpyAsync(size.data(), d_size, sizeof(int64_t) * size.size(), cudaMemcpyDeviceToHost, ctx->stream));
   sync(ctx);
   TBK_CHECK_ARG(nnz_loc < INT32_MAX, "the local operators hold too many blocks");
   int32_t* lrow = (int32_t*)scratch(ctx, WS_LOCAL4, sizeof(int32_t) * ((size_t)n_loc + 1 + 2 * (size_t)nnz_loc));
   int32_t* lcol = lrow + n_loc + 1;
   int32_t* lblk = lcol + nnz_loc;
   local_pattern<true><<<ceil_div(n_loc, 256), 256, 0, ctx->stream>>>(n, n_loc, rs, rcol, H->row_ptr, H->col, nullptr,
-                                                                      lrp, lcol, lblk);
+                                                                      lrp, lrow, lcol, lblk);
   post_launch(ctx, "local_pattern");
-  {
-    // the int32 row pointer of the merged operator
-    std::vector<int64_t> h((size_t)n_loc + 1);
-    TBK_CUDA(cudaMemcpyAsync(h.data(), lrp, sizeof(int64_t) * h.size(), cudaMemcpyDeviceToHost, ctx->stream));
-    sync(ctx);
-    std::vector<int32_t> h32(h.begin(), h.end());
-    TBK_CUDA(cudaMemcpyAsync(lrow, h32.data(), sizeof(int32_t) * h32.size(), cudaMemcpyHostToDevice, ctx->stream));
-    sync(ctx);
-  }
   own_index<<<ceil_div(n, 256), 256, 0, ctx->stream>>>(n, rs, rcol, own, err);
   post_launch(ctx, "own_index");
 
-  // 3. local copies of the mapped blocks (H^ for X; H itself, the bounds [-1, 1], for H X)
+  const dim3 eb(32, 8);
+  auto extract = [&](const void* Y, double* out) {
+    if (prec == TBK_MIXED)
+      local_extract<float><<<ceil_div(n, 8), eb, 0, ctx->stream>>>(n, B, S, H->row_ptr, H->col, rs, rcol,
+                                                                   (const float*)Y, out, err);
+    else
+      local_extract<double><<<ceil_div(n, 8), eb, 0, ctx->stream>>>(n, B, S, H->row_ptr, H->col, rs, rcol,
+                                                                    (const double*)Y, out, err);
+    post_launch(ctx, "local_extract");
+  };
+  double* dcoef = (double*)scratch(ctx, WS_COEF, sizeof(double) * (size_t)p);
+  coefficients(ctx, TBK_FN_FERMI, p, emin, emax, mu, kT, damping, dcoef);
   const size_t esz = prec == TBK_MIXED ? 4 : 8;
+  const size_t panel = (size_t)n_loc * B * S * esz;
+
+  // 3a. FP32, 9 orbitals, panels and block list in shared memory: whole regions per CTA, the largest first
+  LocalArgs la{};
+  for (int a = 0; a < n; ++a) {
+    la.max_m = std::max(la.max_m, (int)std::min<int64_t>(size[2 * a], 1 << 20));
+    la.max_nnz = std::max(la.max_nnz, (int)std::min<int64_t>(size[2 * a + 1], 1 << 24));
+  }
+  const int64_t smem_fix = 2 * (int64_t)la.max_m * 9 * LC_ROW * 4 + ((int64_t)la.max_nnz + 3 * (int64_t)la.max_m) * 4;
+  const int64_t smem_max = 226 << 10;
+  if (prec == TBK_MIXED && B == 9 && smem_fix <= smem_max) {
+    std::vector<int32_t> ord((size_t)n + 1);
+    std::iota(ord.begin(), ord.end() - 1, 0);
+    std::stable_sort(ord.begin(), ord.end() - 1, [&](int a, int b) { return size[2 * a + 1] > size[2 * b + 1]; });
+    ord[n] = 0;
+    TBK_CUDA(cudaMemcpyAsync(d_order, ord.data(), sizeof(int32_t) * ord.size(), cudaMemcpyHostToDevice, ctx->stream));
+    la.n_atoms = n;
+    la.p = p;
+    la.n_stage = (int)std::min<int64_t>(la.max_nnz, (smem_max - smem_fix) / (LC_BS * 4));
+    la.order = d_order;
+    la.next = d_order + n;
+    la.rs = rs;
+    la.lrow = lrow;
+    la.lcol = lcol;
+    la.lblk = lblk;
+    la.own = own;
+    float* blocks = (float*)scratch(ctx, WS_SEGMENT, 2 * sizeof(float) * (size_t)H->nnzb * LC_BS);
+    auto mapped = [&](double lo, double hi, float* dst) {
+      const HOp g = prepare_hop(ctx, H, lo, hi, prec, WS_HHAT, err);
+      const int64_t tot = g.nnzb * LC_BS;
+      local_blocks<<<(unsigned)((tot + 255) / 256), 256, 0, ctx->stream>>>(tot, (const float*)g.hv, dst);
+      post_launch(ctx, "local_blocks");
+      return dst;
+    };
+    la.hv = mapped(emin, emax, blocks);
+    la.h1 = Q ? mapped(-1.0, 1.0, blocks + (size_t)H->nnzb * LC_BS) : nullptr;
+    la.coef = dcoef;
+    la.X = (float*)scratch(ctx, WS_CHECKPOINTS, 2 * panel);
+    la.Y = la.X + panel / 4;
+    const int smem = (int)(smem_fix + (int64_t)la.n_stage * LC_BS * 4);
+    TBK_CUDA(cudaFuncSetAttribute(local_clenshaw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
+    local_clenshaw<<<std::min(n, ctx->num_sms), LC_THREADS, smem, ctx->stream>>>(la);
+    post_launch(ctx, "local_clenshaw");
+    if (P) extract(la.X, P);
+    if (Q) extract(la.Y, Q);
+    int herr = 0;
+    TBK_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    sync(ctx);  // also: ord stays until its copy is done
+    check_diagonal_flag(herr);
+    TBK_CHECK_ARG(herr == 0, "a stored block of H joins atoms farther apart than r_max");
+    return TBK_OK;
+  }
+
+  // 3b. local copies of the mapped blocks (H^ for X; H itself, the bounds [-1, 1], for H X)
   const int BS = prec == TBK_MIXED ? (B == 1 ? Layout<float, 1>::BS : Layout<float, 9>::BS)
                                    : (B == 1 ? Layout<double, 1>::BS : Layout<double, 9>::BS);
   void* hv_loc = scratch(ctx, WS_SEGMENT, (size_t)nnz_loc * BS * esz);
@@ -218,12 +469,9 @@ extern "C" int tbk_local_density(tbk_ctx* ctx, const tbk_bsr* H, const double* p
   HOp op = local_operator(emin, emax);
 
   // 4. coefficients of p_f, then X = p_f(H^) E by the Clenshaw form with unit-vector sources
-  double* dcoef = (double*)scratch(ctx, WS_COEF, sizeof(double) * (size_t)p);
-  coefficients(ctx, TBK_FN_FERMI, p, emin, emax, mu, kT, damping, dcoef);
   std::vector<double> c(p);
   TBK_CUDA(cudaMemcpyAsync(c.data(), dcoef, sizeof(double) * p, cudaMemcpyDeviceToHost, ctx->stream));
   sync(ctx);
-  const size_t panel = (size_t)op.n_rows * S * esz;
   char* base = (char*)scratch(ctx, WS_CHECKPOINTS, 3 * panel);
   void* B1 = base;
   void* B2 = base + panel;
@@ -265,16 +513,6 @@ extern "C" int tbk_local_density(tbk_ctx* ctx, const tbk_bsr* H, const double* p
     step(op, bk1, bk2, X, 1.0);                    // X = H^ b_1 - b_2 + alpha_0 E
     add_e(X, c[0]);
   }
-  const dim3 eb(32, 8);
-  auto extract = [&](const void* Y, double* out) {
-    if (prec == TBK_MIXED)
-      local_extract<float><<<ceil_div(n, 8), eb, 0, ctx->stream>>>(n, B, S, H->row_ptr, H->col, rs, rcol,
-                                                                   (const float*)Y, out, err);
-    else
-      local_extract<double><<<ceil_div(n, 8), eb, 0, ctx->stream>>>(n, B, S, H->row_ptr, H->col, rs, rcol,
-                                                                    (const double*)Y, out, err);
-    post_launch(ctx, "local_extract");
-  };
   if (P) extract(X, P);
   if (Q) {
     HOp h1 = local_operator(-1.0, 1.0);

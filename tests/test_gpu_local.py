@@ -122,3 +122,20 @@ def test_local_density_single_atom(api, ctx):
     Pref = (V * pf) @ V.T
     assert np.abs(P.cpu().numpy()[0] - Pref).max() < 1e-12
     assert np.abs(Q.cpu().numpy()[0] - Hd @ Pref).max() < 1e-11
+
+
+# The FP32 region kernel at the edges of its warp passes (5 atoms a warp, 80 a pass) and with blocks beyond
+# shared memory (120 to 300 atoms in one region), and the step kernels where the panels do not fit (360),
+# against the FP64 path: FP32 products of p steps, the 2e-5 of the oracle comparison above.
+@pytest.mark.parametrize("n,r_max,p", [(1, 5.0, 1), (2, 5.0, 2), (3, 5.0, 3), (13, 4.0, 40), (80, 100.0, 41),
+                                       (81, 100.0, 40), (120, 100.0, 40), (200, 7.0, 40), (300, 100.0, 12),
+                                       (360, 100.0, 12)])
+def test_local_density_region_kernel_vs_fp64(api, ctx, n, r_max, p):
+    wk = wl.fcc_cu(n, kT=0.5, n_probes=8, seed=5264, probe_seed=1, jitter=0.05)
+    model, pos, H, emin, emax = _operator(api, ctx, wk)
+    ref = api.local_density(ctx, H, pos, None, r_max, emin, emax, p, 3.0, wk.kT, fp64=True)
+    got = api.local_density(ctx, H, pos, None, r_max, emin, emax, p, 3.0, wk.kT)
+    for g, r in zip(got, ref):
+        assert (g - r).abs().max().item() <= 2e-5 * r.abs().max().item()
+    only = api.local_density(ctx, H, pos, None, r_max, emin, emax, p, 3.0, wk.kT, want_Q=False)[0]
+    assert torch.equal(only, got[0])
