@@ -43,32 +43,48 @@ __device__ __forceinline__ void st16(T* p, const T* x) {
 
 // ---- H^ in the padded kernel layout --------------------------------------------------------
 
+// One warp per block row, element by element (lanes over a block's 81 or, for 1 x 1 blocks, over the row):
+// reads are coalesced and the FP64 product and conversion, the two that bind (an SM quarter takes 64
+// cycles for a warp's), run for stored elements only.  One thread per block: 34 us at 1,000 atoms, 188 at
+// 10,000; so 18 and 99.
+constexpr int MAP_THREADS = 128;
+
 template <typename T, int B>
-__global__ void map_h_kernel(int n_atoms, const int32_t* __restrict__ row_ptr,
-                             const int32_t* __restrict__ col, const double* __restrict__ H,
-                             double shift, double inv_half_w, T* __restrict__ out, int* __restrict__ err) {
+__global__ void __launch_bounds__(MAP_THREADS)
+map_h_kernel(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+             const double* __restrict__ H, double shift, double inv_half_w, T* __restrict__ out, int* __restrict__ err) {
   constexpr int RS = Layout<T, B>::RS, BS = Layout<T, B>::BS;
-  // blockDim (8, 16): the 8 lanes of a row are 8 consecutive lanes of one warp
-  const int a = blockIdx.x * blockDim.y + threadIdx.y;
+  const int a = blockIdx.x * (MAP_THREADS / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (a >= n_atoms) return;
   bool has_diag = false;
-  for (int k = row_ptr[a] + threadIdx.x; k < row_ptr[a + 1]; k += blockDim.x) {
-    const bool diag = col[k] == a;
-    has_diag |= diag;
-    for (int i = 0; i < B; ++i)
-      for (int j = 0; j < RS; ++j) {
-        // stored element (major index i, minor index j): H^[i][j] row-major, H^[j][i] column-major
-        const int r = Layout<T, B>::COLMAJOR ? j : i, c = Layout<T, B>::COLMAJOR ? i : j;
-        double v = 0.0;
-        if (j < B) {
-          v = H[(int64_t)k * B * B + r * B + c];
-          if (diag && r == c) v -= shift;
-          v *= inv_half_w;
-        }
-        out[(int64_t)k * BS + i * RS + j] = (T)v;
+  const int k1 = row_ptr[a + 1];
+  if constexpr (B == 1) {
+    for (int k = row_ptr[a] + lane; k < k1; k += 32) {
+      const bool diag = col[k] == a;
+      has_diag |= diag;
+      double v = H[k];
+      if (diag) v -= shift;
+      out[k] = (T)(v * inv_half_w);
+    }
+  } else {
+#pragma unroll 4
+    for (int k = row_ptr[a]; k < k1; ++k) {
+      const bool diag = col[k] == a;
+      has_diag |= diag;
+      T* o = out + (int64_t)k * BS;
+#pragma unroll
+      for (int e = lane; e < 96; e += 32) {
+        if (e >= B * B) continue;
+        const int i = e / B, j = e - i * B;
+        double v = H[(int64_t)k * (B * B) + e];
+        if (diag && i == j) v -= shift;
+        // H^[i][j] row-major, or column-major
+        o[Layout<T, B>::COLMAJOR ? j * RS + i : i * RS + j] = (T)(v * inv_half_w);
       }
+      if (lane < B * (RS - B)) o[lane / (RS - B) * RS + B + lane % (RS - B)] = T(0);
+    }
   }
-  if (!__any_sync(0xFFu << (8 * (threadIdx.y & 3)), has_diag) && threadIdx.x == 0) atomicOr(err, ERR_NO_DIAGONAL);
+  if (!__any_sync(0xffffffffu, has_diag) && lane == 0) atomicOr(err, ERR_NO_DIAGONAL);
 }
 
 HOp prepare_hop(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, int prec, Slot slot, int* err) {
@@ -88,8 +104,7 @@ HOp prepare_hop(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, int pr
   op.row_ptr = H->row_ptr;
   op.col = H->col;
   const double shift = 0.5 * (emax + emin), inv = 2.0 / (emax - emin);
-  dim3 blk(8, 16);
-  const int grid = ceil_div(op.n_atoms, 16);
+  const int blk = MAP_THREADS, grid = ceil_div(op.n_atoms, MAP_THREADS / 32);
 #define TBK_MAP(TT, BB)                                                                        \
   {                                                                                            \
     TT* out = (TT*)scratch(ctx, slot, sizeof(TT) * (size_t)op.nnzb * Layout<TT, BB>::BS);      \
@@ -1474,8 +1489,7 @@ HOp prepare_hop_into(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, i
   op.col = H->col;
   op.hv = dst;
   const double shift = 0.5 * (emax + emin), inv = 2.0 / (emax - emin);
-  const dim3 blk(8, 16);
-  const int grid = ceil_div(op.n_atoms, 16);
+  const int blk = MAP_THREADS, grid = ceil_div(op.n_atoms, MAP_THREADS / 32);
   if (prec == TBK_MIXED) {
     if (op.B == 9)
       map_h_kernel<float, 9><<<grid, blk, 0, ctx->stream>>>(op.n_atoms, op.row_ptr, op.col, H->val, shift, inv, (float*)dst, err);
