@@ -37,7 +37,7 @@ __global__ void assemble_kernel(DevModel M, const double* __restrict__ pos, int 
     for (int c = 0; c < 3; ++c) d[c] = min_image(pos[3 * b + c] - pos[3 * a + c], M.box[c]);
     if (M.kind == TBK_MODEL_SK) {
       double E[81];
-      sk_block<double>(d, M.V, M.r0, M.decay, E);
+      sk_block(d, M.V, M.r0, M.decay, E);
       for (int i = 0; i < 81; ++i) out[i] = E[i];
     } else {
       int hit = -1;

@@ -62,3 +62,19 @@ def test_deferred_outer_products_have_the_fused_bits(n_atoms, s, orders):
         G0, F0 = api.density_and_forces(*args)
         G1, F1 = api.density_and_forces(*args, max_panel_bytes=(order // 2 + 3) * 9 * n_atoms * s * 4)
         assert torch.equal(G0, G1) and torch.equal(F0, F1)
+
+
+# Forces from G: the directional derivative sum_k G_k : dH_k against central differences of the assembled
+# blocks (error h^2 H'''/6, below 1e-7 of the sum of magnitudes at h = 1e-4), at the edges of the rows that
+# a warp takes (one row up to 608 atoms, two, eight), open and with a single pair.
+@pytest.mark.parametrize("n_atoms", [2, 35, 608, 609, 1250, 5000])
+def test_forces_are_the_derivative_of_the_blocks(n_atoms):
+    import torch
+    from paper_1812_05264_gb300 import api as A
+    api, wk, ctx, pos, model, H, lo, hi = _setup(n_atoms, 128, 6, True)
+    G, F = api.density_and_forces(ctx, H, model, pos, None, lo, hi, 7, 128, 6, 6.0, 0.5)
+    v = torch.randn(pos.shape, generator=torch.Generator(device="cuda").manual_seed(1), dtype=torch.float64, device="cuda")
+    h = 1e-4
+    dH = (A.assemble_H(ctx, model, pos + h * v, H.graph).val - A.assemble_H(ctx, model, pos - h * v, H.graph).val) / (2 * h)
+    got, ref = -(F * v).sum().item(), (G * dH).sum().item()
+    assert abs(got - ref) <= 1e-6 * (G * dH).abs().sum().item()
