@@ -1464,6 +1464,124 @@ __global__ void probe_moments_finish(const double* __restrict__ dots, int K, int
   }
 }
 
+// ---- all steps of a small 1x1 operator in one launch (FP64) ----------------------------------------
+//
+// The probes do not meet until the moments are summed: a cluster of CTAs takes one probe through all steps,
+// each with its share of the rows and the whole of y_j and y_{j-1} in shared memory; a new entry is stored in
+// every CTA of the cluster, and a step ends with the cluster's barrier.  Rows are summed in the order of the
+// step kernel.  A warp's FP64 instruction takes an SM 19 cycles: 10 per row and probe are the bound (0.6 us a
+// step at 1,000 sites and 32 probes), then the chain of a row and the barrier.  Microseconds per step,
+// a launch each -> so: 216 sites x 32 probes 6.2 -> 1.4, 1,000 x 32 8.2 -> 1.9, 1,000 x 512 22.5 -> 17.3,
+// 2,744 x 64 12.4 -> 5.3, 5,832 x 64 18.6 -> 10.3, 10,648 x 4 8.2 -> 6.5, 10,648 x 512 166 -> 126.
+constexpr int SWEEP_THREADS = 512;
+constexpr int64_t SWEEP_ROWS = 11000;                   // two panels in shared memory
+constexpr size_t SWEEP_PARTIALS = (size_t)256 << 20;    // bytes of partial sums
+
+__device__ __forceinline__ void store_cluster(double* p, int rank, double x) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(x) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// probe_panel: y_0, or NULL for the +-1 probes of the seed.  partials: two per warp and step.  cap: blocks of
+// the operator that fit in shared memory beside the panels (the cluster's barrier drops what L1 holds, so
+// blocks left in global memory come from L2 in every step; a share of the rows with more blocks does that).
+__global__ void __launch_bounds__(SWEEP_THREADS)
+moments_sweep_b1(int n, int C, int cap, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+                 const double* __restrict__ hv, const double* __restrict__ probe_panel, uint64_t seed, int s, int K,
+                 double* __restrict__ partials) {
+  extern __shared__ double ysm[];
+  const int rank = blockIdx.x % C, probe = blockIdx.x / C;
+  const int r0 = (int)((int64_t)n * rank / C), rows = (int)((int64_t)n * (rank + 1) / C) - r0;
+  const int lane = threadIdx.x & 31, warps = blockDim.x / 32, n_part = gridDim.x * warps;
+  double* part = partials + 2 * ((int64_t)blockIdx.x * warps + (threadIdx.x >> 5));
+  double* hs = ysm + 2 * n;
+  int* cs = reinterpret_cast<int*>(hs + cap);
+  int* rp = cs + cap;
+  for (int i = threadIdx.x; i < n; i += blockDim.x)
+    ysm[i] = probe_panel ? probe_panel[(int64_t)i * s + probe] : (double)tbk_probe_sign(seed, i, probe);
+  const int k0 = __ldg(row_ptr + r0), nz = __ldg(row_ptr + r0 + rows) - k0;
+  for (int i = threadIdx.x; i <= rows; i += blockDim.x) rp[i] = __ldg(row_ptr + r0 + i) - k0;
+  const bool staged = nz <= cap;
+  for (int k = threadIdx.x; k < nz && staged; k += blockDim.x) {
+    hs[k] = __ldg(hv + k0 + k);
+    cs[k] = __ldg(col + k0 + k);
+  }
+  cluster_barrier();
+  for (int j = 1; j <= K; ++j) {
+    const double* in = ysm + ((j - 1) & 1) * n;
+    double* out = ysm + (j & 1) * n;
+    double s0 = 0.0, s1 = 0.0;
+    for (int i = threadIdx.x; i < rows; i += blockDim.x) {
+      double acc = 0.0;
+      const int k1 = rp[i + 1];
+      if (staged) {
+#pragma unroll 4
+        for (int k = rp[i]; k < k1; ++k) acc = fma(hs[k], in[cs[k]], acc);
+      } else {
+        for (int k = rp[i]; k < k1; ++k) acc = fma(__ldg(hv + k0 + k), in[__ldg(col + k0 + k)], acc);
+      }
+      const double y = j == 1 ? acc : 2.0 * acc - out[r0 + i];
+      for (int c = 0; c < C; ++c) store_cluster(out + r0 + i, c, y);
+      s0 = fma(y, in[r0 + i], s0);
+      s1 = fma(y, y, s1);
+    }
+    // lanes 0..15 sum s0, lanes 16..31 s1
+    double a = lane < 16 ? s0 : s1;
+    a += __shfl_xor_sync(0xffffffffu, lane < 16 ? s1 : s0, 16);
+    for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if ((lane & 15) == 0) part[2 * (int64_t)(j - 1) * n_part + (lane >> 4)] = a;
+    cluster_barrier();
+  }
+}
+
+// CTAs per probe (enough for the chip, at most a portable cluster) and threads per CTA (a row each).
+static int sweep_cluster(const tbk_ctx* ctx, int s) {
+  int c = 1;
+  while (c < 8 && s * c < ctx->num_sms * 4 / 5) c *= 2;
+  return c;
+}
+static int sweep_warps(const tbk_ctx* ctx, const HOp& op, int s) {
+  return std::min(SWEEP_THREADS / 32, ceil_div(op.n_rows, 32 * sweep_cluster(ctx, s)));
+}
+
+static int sweep_partials(const tbk_ctx* ctx, const HOp& op, int s) {
+  return s * sweep_cluster(ctx, s) * sweep_warps(ctx, op, s);
+}
+
+static bool use_sweep(const tbk_ctx* ctx, const HOp& op, int s, int K, int direct, const void* per_probe, int flags) {
+  return op.B == 1 && op.prec == TBK_FP64 && K >= 1 && !direct && !per_probe && !(flags & TBK_PLAIN_KERNEL) &&
+         op.n_rows <= SWEEP_ROWS && s <= 512 && 16 * (size_t)K * sweep_partials(ctx, op, s) <= SWEEP_PARTIALS;
+}
+
+static void launch_sweep(tbk_ctx* ctx, const HOp& op, const void* probe_panel, uint64_t seed, int s, int K,
+                         double* partials) {
+  KernelTimerScope timer(ctx, TBK_KERNEL_STEP);
+  const int C = sweep_cluster(ctx, s), n = (int)op.n_rows;
+  // panels, row pointers, and a quarter more blocks than the average share
+  const int64_t fix = 16 * (int64_t)n + 4 * (n / C + 2), most = 220 << 10;
+  const int cap = (int)std::max<int64_t>(0, std::min((most - fix) / 12 - 1, op.nnzb / C * 5 / 4 + 32)) & ~1;
+  const size_t smem = fix + 12 * (size_t)cap;
+  TBK_CUDA(cudaFuncSetAttribute(moments_sweep_b1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(s * C);
+  cfg.blockDim = dim3(32 * sweep_warps(ctx, op, s));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = ctx->stream;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = C;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  TBK_CUDA(cudaLaunchKernelEx(&cfg, moments_sweep_b1, n, C, cap, op.row_ptr, op.col, (const double*)op.hv,
+                              (const double*)probe_panel, seed, s, K, partials));
+  post_launch(ctx, "moments_sweep_b1");
+}
+
 // ---- building blocks that allocate nothing (for the static-scratch entry point) --------------
 
 size_t mapped_h_bytes(const tbk_bsr* H, int prec) {
@@ -1541,11 +1659,13 @@ void moments_sweep(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, uin
   const size_t esz = prec == TBK_MIXED ? 4 : 8;
   const size_t panel = (size_t)op.n_rows * s * esz;
   const int K = direct ? order - 1 : order / 2;   // steps: largest moment index 2K >= order - 1
-  const int nctas = step_grid_ctas(ctx, op, s);
+  const bool sweep = use_sweep(ctx, op, s, K, direct, per_probe, flags);
+  const int nctas = sweep ? sweep_partials(ctx, op, s) : step_grid_ctas(ctx, op, s);
   double* partials = (double*)scratch(ctx, WS_PARTIALS, sizeof(double) * 2 * (size_t)std::max(1, K) * nctas);
   double* sums = (double*)scratch(ctx, WS_MISC, sizeof(double) * 2 * (size_t)std::max(1, K) + 64);
-  void* A = K >= 1 ? scratch(ctx, WS_PANEL0, panel) : nullptr;
-  void* Bp = K >= 2 ? scratch(ctx, WS_PANEL1, panel) : nullptr;
+  if (sweep) launch_sweep(ctx, op, probe_panel, probe_seed, s, K, partials);
+  void* A = K >= 1 && !sweep ? scratch(ctx, WS_PANEL0, panel) : nullptr;
+  void* Bp = K >= 2 && !sweep ? scratch(ctx, WS_PANEL1, panel) : nullptr;
   // per-probe dots: row-block partials of one step, then K x s x 2 reduced dots
   const int64_t rpb = (op.n_rows + PD_BLOCKS - 1) / PD_BLOCKS;
   const int nrb = (int)((op.n_rows + rpb - 1) / rpb);
@@ -1553,7 +1673,7 @@ void moments_sweep(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, uin
   double* pd_dots = per_probe ? (double*)scratch(ctx, WS_SEGMENT, sizeof(double) * 2 * (size_t)std::max(1, K) * s)
                               : nullptr;
   void *cur = nullptr, *prev = nullptr;
-  for (int j = 1; j <= K; ++j) {
+  for (int j = 1; j <= K && !sweep; ++j) {
     StepArgs a;
     a.seed = probe_seed;
     a.s = s;

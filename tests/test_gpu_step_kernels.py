@@ -45,3 +45,22 @@ def test_fp32_steps_equal_the_plain_kernel(n_atoms, s, direct):
                                        (700, 12), (300, 64)])
 def test_fp64_steps_equal_the_plain_kernel(n_atoms, s, direct):
     _check(n_atoms, s, True, direct)
+
+
+# All steps in one launch (1x1 blocks, FP64) against a launch per step: one site, rows that do not divide over
+# the cluster, a share of the blocks beyond shared memory (22^3 at 64 probes) and a cluster beyond the rule
+# (23^3).  FP64 rounding of the sums: 1e-12 of mu_0.
+@pytest.mark.parametrize("L,s,orders", [(1, 4, (2, 3, 8)), (2, 4, (7,)), (3, 36, (2, 3, 4, 41)), (7, 32, (40,)),
+                                        (10, 100, (41,)), (13, 512, (20,)), (22, 64, (12,)), (23, 4, (12,))])
+def test_one_launch_sweep_equals_the_steps(L, s, orders):
+    import torch
+    from paper_1812_05264_gb300 import api
+    wk = wl.sc_disorder(L=L, n_probes=s)
+    ctx = api.Context()
+    pos = torch.as_tensor(wk.positions, dtype=torch.float64, device="cuda")
+    model = api.Model.from_workload(wk, "cuda")
+    H = api.assemble_H(ctx, model, pos, api.build_neighbors(ctx, pos, wk.cutoff))
+    for order in orders:
+        got = api.chebyshev_moments(ctx, H, -9.0, 9.0, 5, s, order, fp64=True)
+        ref = api.chebyshev_moments(ctx, H, -9.0, 9.0, 5, s, order, fp64=True, plain=True)
+        assert (got - ref).abs().max().item() <= 1e-12 * L ** 3
