@@ -250,13 +250,16 @@ __global__ void lz_transpose(int64_t n, const double* __restrict__ H, double* __
 
 // ---- a small operator: one thread-block cluster, the vectors in shared memory and registers ----------
 //
-// The same sums with at most LZ_CL_WARPS units per CTA, one per warp: v is copied into every CTA's
-// shared memory, a thread keeps its row of v_prev, v and w, and partial sums go to every CTA, where
-// each warp adds them itself.  The hardware barrier of a cluster takes ~0.2 us where one over the
-// grid takes ~2 with its sum: what is left of a step is the row's chain (147 atoms: 0.99 ms for 64
-// steps against 1.40 over the grid; beyond 96 units the FP64 rate of 8 SMs is the longer of the two).
-constexpr int LZ_CL = 8, LZ_CL_WARPS = 12;
-constexpr int LZ_CL_UNITS = LZ_CL * LZ_CL_WARPS;
+// The same sums with a cluster of CL CTAs, one unit per warp: v is copied into every CTA's shared memory, a
+// thread keeps its row of v_prev, v and w (and of H, as far as shared memory goes), and partial sums go to
+// every CTA, where each warp adds them itself.  The hardware barrier of a cluster takes ~0.2 us where one over
+// the grid takes ~2 with its sum: what is left of a step is the row's chain of 171 operations, 64 cycles each
+// up to three warps per SM and 19 per warp beyond (the SM's FP64 units are shared), and about 6 us of sums,
+// square root, division and barriers.  147 atoms: 21.9 us a step over the grid,
+// 15.5 with 8 CTAs, 11.7 with 16 (where the device takes such clusters).  With 16: 340 atoms 14.1, 455 atoms
+// 17.4; the grid takes 21.1 at 456 atoms and 22.6 at 1,000, most of it its barriers (with H and the gathered v
+// in shared memory there the same).
+constexpr int LZ_CL_UNITS = 128;
 
 __device__ __forceinline__ void lz_cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -268,24 +271,28 @@ __device__ __forceinline__ void lz_store_remote(double* p, int rank, double x) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(x) : "memory");
 }
 
-template <int B>
-__global__ void __cluster_dims__(LZ_CL, 1, 1) __launch_bounds__(32 * LZ_CL_WARPS)
-lz_run_cluster(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+template <int B, int CL>
+__global__ void __launch_bounds__(32 * LZ_CL_UNITS / CL)
+lz_run_cluster(int n_atoms, int cap, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const double* __restrict__ H, int m, uint64_t seed, double* __restrict__ alpha,
                double* __restrict__ beta) {
   __shared__ double vs[32 * LZ_CL_UNITS];
   __shared__ double part[2][LZ_CL_UNITS];
   const int n = n_atoms * B, nb = (n + 255) / 256, units = 8 * nb;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int u = warp * LZ_CL + blockIdx.x, row = 32 * u + lane;
+  const int u = warp * CL + blockIdx.x, row = 32 * u + lane, T = blockDim.x;
   const bool has = row < n;
+  // the thread's row of the first `cap` blocks, and where their v lies
+  extern __shared__ double lz_smem[];
+  double* hs = lz_smem + threadIdx.x;
+  int* cs = reinterpret_cast<int*>(lz_smem + (int64_t)cap * B * T) + threadIdx.x;
   for (int i = threadIdx.x; i < n; i += blockDim.x) vs[i] = (double)tbk_probe_sign(seed, i, 0) / sqrt((double)n);
   for (int i = threadIdx.x; i < 2 * LZ_CL_UNITS; i += blockDim.x) part[0][i] = 0.0;
   lz_cluster_barrier();
   // the sum of the units' values d, in every thread
   auto total = [&](int set, double d) {
     d = lz_warp_sum(d);
-    if (u < units && lane < LZ_CL) lz_store_remote(&part[set][u], lane, d);
+    if (u < units && lane < CL) lz_store_remote(&part[set][u], lane, d);
     lz_cluster_barrier();
     double s = 0.0;
     if (lane < nb) {
@@ -297,23 +304,25 @@ lz_run_cluster(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* 
   };
   const int a = has ? row / B : 0, i = row - a * B;
   const int k0 = has ? __ldg(row_ptr + a) : 0, k1 = has ? __ldg(row_ptr + a + 1) : 0;
+  const int ks = min(k1 - k0, cap);
+  for (int k = 0; k < ks; ++k) {
+    cs[k * T] = __ldg(col + k0 + k) * B;
+#pragma unroll
+    for (int l = 0; l < B; ++l) hs[(int64_t)(k * B + l) * T] = __ldg(H + (int64_t)(k0 + k) * B * B + l * B + i);
+  }
   double vprev = 0.0, v = has ? vs[row] : 0.0, bj = 0.0;
   for (int j = 0; j < m; ++j) {
-    double acc = 0.0, h[B], hn[B];
-    int b = 0, bn = 0;
-    auto fetch = [&](int k, double (&hh)[B], int& bb) {
-      bb = __ldg(col + k) * B;
+    double acc = 0.0;
+#pragma unroll 2
+    for (int k = 0; k < ks; ++k) {
+      const double *h = hs + (int64_t)k * B * T, *x = vs + cs[k * T];
 #pragma unroll
-      for (int l = 0; l < B; ++l) hh[l] = __ldg(H + (int64_t)k * B * B + l * B + i);
-    };
-    if (k0 < k1) fetch(k0, h, b);
-    for (int k = k0; k < k1; ++k) {
-      if (k + 1 < k1) fetch(k + 1, hn, bn);
+      for (int l = 0; l < B; ++l) acc += h[l * T] * x[l];
+    }
+    for (int k = k0 + ks; k < k1; ++k) {
+      const double *h = H + (int64_t)k * B * B + i, *x = vs + __ldg(col + k) * B;
 #pragma unroll
-      for (int l = 0; l < B; ++l) acc += h[l] * vs[b + l];
-#pragma unroll
-      for (int l = 0; l < B; ++l) h[l] = hn[l];
-      b = bn;
+      for (int l = 0; l < B; ++l) acc += __ldg(h + l * B) * x[l];
     }
     if (j) acc -= bj * vprev;
     const double aj = total(0, has ? acc * v : 0.0);
@@ -327,7 +336,7 @@ lz_run_cluster(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* 
     vprev = v;
     v = has && bj > 0.0 ? x / bj : 0.0;
     if (has)
-      for (int r = 0; r < LZ_CL; ++r) lz_store_remote(vs + row, r, v);
+      for (int r = 0; r < CL; ++r) lz_store_remote(vs + row, r, v);
     lz_cluster_barrier();
   }
   lz_cluster_barrier();  // no CTA leaves while another may still write to it
@@ -346,15 +355,73 @@ static void lz_launch_pf(tbk_ctx* ctx, const tbk_bsr* H, const double* val, int 
   post_launch(ctx, "lz_run");
 }
 
+template <int B, int CL>
+static cudaLaunchConfig_t lz_cluster_config(tbk_ctx* ctx, int units, int64_t blocks, cudaLaunchAttribute* at, int* cap) {
+  cudaLaunchConfig_t cfg{};
+  const int T = 32 * ceil_div(units, CL);
+  const int64_t most = 180 << 10;  // beside 34 KB of vectors
+  *cap = (int)std::min<int64_t>(blocks, most / ((8 * B + 4) * T));
+  cfg.gridDim = dim3(CL);
+  cfg.blockDim = dim3(T);
+  cfg.dynamicSmemBytes = (size_t)(8 * B + 4) * T * *cap;
+  cfg.stream = ctx->stream;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = CL;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+template <int B, int CL>
+static void lz_cluster_attributes() {
+  TBK_CUDA(cudaFuncSetAttribute(lz_run_cluster<B, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 180 << 10));
+  if (CL > 8) TBK_CUDA(cudaFuncSetAttribute(lz_run_cluster<B, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+}
+
+// Whether the device takes clusters of 16 with the largest shared memory and block used.
+template <int B>
+static bool lz_wide_clusters(tbk_ctx* ctx) {
+  static int known[64] = {0};
+  int& k = known[ctx->device & 63];
+  if (!k) {
+    lz_cluster_attributes<B, 16>();
+    cudaLaunchAttribute at{};
+    int cap, clusters = 0;
+    const cudaLaunchConfig_t cfg = lz_cluster_config<B, 16>(ctx, LZ_CL_UNITS, 1 << 20, &at, &cap);
+    if (cudaOccupancyMaxActiveClusters(&clusters, lz_run_cluster<B, 16>, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      clusters = 0;
+    }
+    k = clusters > 0 ? 1 : 2;
+  }
+  return k == 1;
+}
+
+template <int B, int CL>
+static void lz_launch_cluster(tbk_ctx* ctx, const tbk_bsr* H, const double* val, int m, uint64_t seed, double* alpha,
+                              double* beta) {
+  const int units = 8 * ceil_div((int64_t)H->n_atoms * B, 256);
+  lz_cluster_attributes<B, CL>();
+  cudaLaunchAttribute at{};
+  int cap;
+  // up to four times the average row in shared memory
+  const cudaLaunchConfig_t cfg =
+      lz_cluster_config<B, CL>(ctx, units, 4 * (int64_t)ceil_div(H->nnzb, H->n_atoms), &at, &cap);
+  TBK_CUDA(cudaLaunchKernelEx(&cfg, lz_run_cluster<B, CL>, (int)H->n_atoms, cap, H->row_ptr, H->col, val, m, seed, alpha,
+                              beta));
+  post_launch(ctx, "lz_run_cluster");
+}
+
 // val: the blocks, transposed (TR) or as given
 template <int B, bool TR>
 static void lz_launch(tbk_ctx* ctx, const tbk_bsr* H, const double* val, int m, uint64_t seed, double* vecs,
                       double* part, double* alpha, double* beta, LzSync* sy, double* fail) {
   const int64_t n = (int64_t)H->n_atoms * B;
-  if ((TR || B == 1) && 8 * (int64_t)ceil_div(n, 256) <= LZ_CL_UNITS) {
-    lz_run_cluster<B><<<LZ_CL, 32 * LZ_CL_WARPS, 0, ctx->stream>>>(H->n_atoms, H->row_ptr, H->col, val, m, seed, alpha,
-                                                                   beta);
-    post_launch(ctx, "lz_run_cluster");
+  const int64_t units = 8 * (int64_t)ceil_div(n, 256);
+  if ((TR || B == 1) && units <= LZ_CL_UNITS) {
+    if (lz_wide_clusters<B>(ctx)) lz_launch_cluster<B, 16>(ctx, H, val, m, seed, alpha, beta);
+    else lz_launch_cluster<B, 8>(ctx, H, val, m, seed, alpha, beta);
     return;
   }
   lz_start<<<ceil_div(n, 256), 256, 0, ctx->stream>>>(n, seed, vecs + n);

@@ -40,3 +40,16 @@ def test_periodic_bounds_equal_the_batched_ones():
     one, ref = _both(wl.sc9_periodic(L=8, n_probes=8), 32)
     assert one == ref
     assert np.isfinite(one).all() and one[0] < one[1]
+
+
+# the last operator of a cluster (455 atoms) and the first of the grid after it, one to four 32-row units per
+# SM, and rows longer than the shared memory that a thread's row of H gets (cutoff 7)
+@pytest.mark.parametrize("n_atoms,cutoff,steps", [(147, None, 64), (455, None, 40), (456, None, 40), (541, None, 20),
+                                                  (1081, None, 20), (1300, None, 20), (2161, None, 12),
+                                                  (2162, None, 12), (200, 7.0, 20), (700, 7.0, 20), (1500, 7.0, 10)])
+def test_bounds_equal_the_batched_ones_between_cluster_and_grid(n_atoms, cutoff, steps):
+    wk = wl.fcc_cu(n_atoms, kT=0.5, n_probes=8, jitter=0.05)
+    if cutoff:
+        wk.cutoff = cutoff
+    one, ref = _both(wk, steps)
+    assert one == ref
