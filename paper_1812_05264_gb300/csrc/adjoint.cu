@@ -134,6 +134,99 @@ sddmm_rows32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __
   if (lane < 27) atomicAdd(Gacc + (int64_t)k * 81 + 27 * g + lane, w * ((double)hi + (double)lo));
 }
 
+constexpr int OUT_STEPS = 64;  // steps per launch at most
+struct OuterPanels {
+  const float* y[OUT_STEPS];  // y_k, highest k first
+  const float* x[OUT_STEPS];  // ybar_{k+1} (or b_{k+1})
+};
+
+// hi + lo += a, the rounding error of the addition kept in lo.
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float a) {
+  const float t = __fadd_rn(hi, a), z = __fsub_rn(t, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(a, z)));
+  hi = t;
+}
+
+// The same for several steps after them, as long as their panels stay in L2: a lane adds its 27 sums of each
+// step to pairs (7 operations an entry where the butterfly takes 14), and one butterfly per launch adds the
+// pairs of the lanes.  A CTA is one block, so that its three warps find x in L1.  333 atoms x 100 probes: 14.6
+// us a step against 18; the loads' latency (12 warps per SM) and 630 instructions a step bind.
+__global__ void __launch_bounds__(96, 4)
+sddmm_steps32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t nnzb,
+              const __grid_constant__ OuterPanels wp, int nt, int last_is_y0, int s, double* __restrict__ Gacc) {
+  pdl_wait();
+  const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (gw >= 3 * nnzb) return;
+  const int k = (int)(gw / 3), g = (int)(gw - 3 * (int64_t)k);
+  const int b = __ldg(col + k), a = row_of_block(row_ptr, n_atoms, k, lane);
+  // byte offsets of the rows (panels of a window are a few MB), so that a load needs no 64-bit arithmetic
+  uint32_t oy[3], ox[9];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) oy[i] = 4u * ((9u * a + 3u * g + i) * s + lane);
+#pragma unroll
+  for (int l = 0; l < 9; ++l) ox[l] = 4u * ((9u * b + l) * s + lane);
+  float acc[27], hi[32], lo[32], yv[4][3], xv[4][9];  // 128 probes ahead
+#pragma unroll
+  for (int e = 0; e < 32; ++e) hi[e] = lo[e] = 0.f;
+  // probes p0 + 32 c + lane of step t; past the last probe zeros, which leave the sums as they are
+  auto fetch = [&](int t, int p0, int c) {
+    const char* Y = reinterpret_cast<const char*>(wp.y[t] + p0) + 128 * c;
+    const char* X = reinterpret_cast<const char*>(wp.x[t] + p0) + 128 * c;
+    auto at = [](const char* p, uint32_t o) { return __ldg(reinterpret_cast<const float*>(p + o)); };
+    if (p0 + 32 * c + 32 <= s) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i) yv[c][i] = at(Y, oy[i]);
+#pragma unroll
+      for (int l = 0; l < 9; ++l) xv[c][l] = at(X, ox[l]);
+    } else {
+      const bool in = p0 + 32 * c + lane < s;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) yv[c][i] = in ? at(Y, oy[i]) : 0.f;
+#pragma unroll
+      for (int l = 0; l < 9; ++l) xv[c][l] = in ? at(X, ox[l]) : 0.f;
+    }
+  };
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    if (32 * c < s) fetch(0, 0, c);
+  for (int t = 0; t < nt; ++t) {
+#pragma unroll
+    for (int e = 0; e < 27; ++e) acc[e] = 0.f;
+    for (int p0 = 0; p0 < s; p0 += 128) {
+      const bool more = p0 + 128 < s;
+      const int tn = more ? t : t + 1, pn = more ? p0 + 128 : 0;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (p0 + 32 * c < s)
+#pragma unroll
+          for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int l = 0; l < 9; ++l) acc[i * 9 + l] = fmaf(yv[c][i], xv[c][l], acc[i * 9 + l]);
+        if (tn < nt && pn + 32 * c < s) fetch(tn, pn, c);
+      }
+    }
+    // the weight 2 is exact at any point: pairs hold half of what the launch adds, and y_0 enters with half
+    const float w = last_is_y0 && t == nt - 1 ? 0.5f : 1.f;
+#pragma unroll
+    for (int e = 0; e < 27; ++e) pair_add(hi[e], lo[e], w * acc[e]);
+  }
+  // lane e: the lanes' sum of entry e
+#pragma unroll
+  for (int off = 16, n = 32; off >= 1; off >>= 1, n >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int e = 0; e < n / 2; ++e) {
+      const float x = __shfl_xor_sync(0xffffffffu, up ? hi[e] : hi[e + n / 2], off);
+      const float c = __shfl_xor_sync(0xffffffffu, up ? lo[e] : lo[e + n / 2], off);
+      hi[e] = up ? hi[e + n / 2] : hi[e];
+      lo[e] = __fadd_rn(up ? lo[e + n / 2] : lo[e], c);
+      pair_add(hi[e], lo[e], x);
+    }
+  }
+  if (lane < 27) atomicAdd(Gacc + (int64_t)k * 81 + 27 * g + lane, 2.0 * ((double)hi[0] + (double)lo[0]));
+}
+
 // FP64 9x9 blocks: a warp takes a block, 27 of its lanes three entries each over all probes (no sums
 // across lanes), 32 probes of both tiles at a time through shared memory and the next 32 loaded ahead.
 // Four sums per entry, over every fourth probe.  The FP64 rate binds (27 of 32 lanes at work); 200 atoms
@@ -701,12 +794,6 @@ sddmm_window_g(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
 // us per backward step with its outer products, fused -> a step kernel and these: 147 atoms x 128 probes
 // 31 -> 11, 1,000 x 128 61 -> 30, 10,000 x 128 488 -> 263, 147 x 256 27 -> 15, 1,000 x 256 66 -> 58, 10,000
 // x 256 548 -> 510.  At 512 probes both take the same (823 -> 836 at 10,000 atoms) and the fused kernel stays.
-constexpr int OUT_STEPS = 64;  // steps per launch at most
-struct OuterPanels {
-  const float* y[OUT_STEPS];  // y_k, highest k first
-  const float* x[OUT_STEPS];  // ybar_{k+1}
-};
-
 // 128 probes: a warp takes one block through all steps, the FP64 accumulator in registers; y_t[a] comes
 // from L1, where the row's other blocks use it too.
 __global__ void __launch_bounds__(128, 3)
@@ -1285,6 +1372,23 @@ void launch_sddmm(tbk_ctx* ctx, const HOp& op, const void* y, const void* x, int
   post_launch(ctx, "sddmm");
 }
 
+// Steps of the general adjoint whose outer products run together (0: after each step), as many as stay in
+// half of L2.  us per order of a whole call, after each step -> 16 together: 147 atoms x 36 probes 21.6 ->
+// 19.5, 333 x 36 29.0 -> 25.3, 2,000 x 64 131 -> 107, 4,000 x 64 250 -> 202; 55 x 100 19.8 -> 18.8, 333 x 100
+// 34.0 -> 32.4, 700 x 100 61.2 -> 60.3, 1,000 x 100 78.0 -> 78.6, 333 x 124 34.3 -> 33.4.  Beyond, the butterfly
+// is a small part and the registers of the sums cost warps: 147 x 200 27.2 -> 28.2, 333 x 384 69.7 -> 95.8.
+static int general_deferred_steps(const HOp& op, int s) {
+  if (op.prec != TBK_MIXED || op.B != 9 || s > (op.n_atoms <= 500 ? 128 : 64)) return 0;
+  return (int)std::min<int64_t>(16, ((int64_t)48 << 20) / (2 * op.n_rows * s * 4));
+}
+
+static void launch_sddmm_steps(tbk_ctx* ctx, const HOp& op, const OuterPanels& wp, int nt, int last_is_y0, int s,
+                               double* Gacc) {
+  launch_pdl(ctx, sddmm_steps32, (unsigned)op.nnzb, 96, 0, op.n_atoms, op.row_ptr, op.col, op.nnzb, wp, nt,
+             last_is_y0, s, Gacc);
+  post_launch(ctx, "sddmm_steps32");
+}
+
 // ---- pieces shared with the batched driver -------------------------------------------------
 
 void launch_symmetrize(tbk_ctx* ctx, int64_t nnzb, int B, const int32_t* tr, const double* Gacc, double scale,
@@ -1787,11 +1891,17 @@ extern "C" int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_
     // and holds y_{t0 - 1 + i} at P(i).  Checkpoint sg (sg >= 1) is (y_{t0-2}, y_{t0-1}).
     const size_t n_seg_pan = (size_t)seg + 1;
     const size_t n_ckpt = all_stored ? 0 : 2 * (size_t)nseg;
-    char* base = (char*)scratch(ctx, WS_CHECKPOINTS, panel * (n_seg_pan + n_ckpt + 2));
+    // b panels in a ring: two, or those of the steps whose outer products wait, as far as they fit
+    int defer = all_stored && !plain && npan > 0 ? general_deferred_steps(op, s) : 0;
+    defer = (int)std::max<int64_t>(0, std::min<int64_t>(std::min(defer, p - 1), (int64_t)(budget / panel) - (npan + 2)));
+    if (defer < 8) defer = 0;
+    const size_t n_ring = defer ? (size_t)defer + 1 : 2;
+    char* base = (char*)scratch(ctx, WS_CHECKPOINTS, panel * (n_seg_pan + n_ckpt + n_ring));
     auto P = [&](size_t i) { return (void*)(base + i * panel); };
     auto CK = [&](int sg, int which) { return P(n_seg_pan + 2 * (size_t)sg + which); };
-    void* bcur = P(n_seg_pan + n_ckpt);
-    void* bprev = P(n_seg_pan + n_ckpt + 1);
+    auto ring = [&](int i) { return P(n_seg_pan + n_ckpt + (size_t)((i + (int)n_ring) % (int)n_ring)); };
+    int ib = 0;
+    void* bcur = ring(ib);
 
     // y_t from y_{t-1} (yin) and y_{t-2} (yprev); y_0 is the probe block
     void* y0 = bcur;  // the probe block, written just before the first step (P(0) in the first segment)
@@ -1832,6 +1942,8 @@ extern "C" int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_
     if (p >= 2) {
       launch_scaled_probe(ctx, op, bcur, c[p - 1], probe_seed, s);
       bool have_bprev = false;
+      OuterPanels wait{};
+      int n_wait = 0;
       int j = p - 2;
       for (int sg = nseg - 1; sg >= -1 && j >= 0; --sg) {
         const int t0 = sg >= 0 ? 1 + seg * sg : 0;
@@ -1849,20 +1961,30 @@ extern "C" int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_
           }
         }
         for (; j >= t0; --j) {
-          launch_sddmm(ctx, op, j == 0 ? y0 : P(j - t0 + 1), bcur, s, j == 0 ? 1.0 : 2.0, Gacc);
+          const void* yj = j == 0 ? y0 : P(j - t0 + 1);
+          if (defer) {
+            wait.y[n_wait] = (const float*)yj;
+            wait.x[n_wait++] = (const float*)ring(ib);
+            if (n_wait == defer || j == 0) {
+              launch_sddmm_steps(ctx, op, wait, n_wait, j == 0, s, Gacc);
+              n_wait = 0;
+            }
+          } else {
+            launch_sddmm(ctx, op, yj, ring(ib), s, j == 0 ? 1.0 : 2.0, Gacc);
+          }
           if (j >= 1) {
             StepArgs a;
             a.seed = probe_seed;
             a.s = s;
-            a.yin = bcur;
+            a.yin = ring(ib);
             a.alpha = 2.0;
             a.c_r = c[j];
-            a.yprev = have_bprev ? bprev : nullptr;
-            a.yout = bprev;
+            a.yprev = have_bprev ? ring(ib - 1) : nullptr;
+            a.yout = ring(ib + 1);
             a.err = err;
             a.force_simple = plain;
             launch_step(ctx, op, a);
-            std::swap(bcur, bprev);
+            ib = (ib + 1) % (int)n_ring;
             have_bprev = true;
           }
         }

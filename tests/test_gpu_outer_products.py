@@ -78,3 +78,18 @@ def test_forces_are_the_derivative_of_the_blocks(n_atoms):
     dH = (A.assemble_H(ctx, model, pos + h * v, H.graph).val - A.assemble_H(ctx, model, pos - h * v, H.graph).val) / (2 * h)
     got, ref = -(F * v).sum().item(), (G * dH).sum().item()
     assert abs(got - ref) <= 1e-6 * (G * dH).abs().sum().item()
+
+
+# The general adjoint's outer products after several steps against one launch per step (a plan with too few
+# panels to store every y_k): sums kept to 2^-47 of their magnitudes either way, which cancel by less than
+# 10^3 here: 1e-10 of the largest entry.  Whole windows of 16 and a rest, windows ended by the size (2,500
+# atoms), the last probe count of each rule and the first beyond.
+@pytest.mark.parametrize("n_atoms,s,order", [(1, 4, 40), (13, 36, 32), (13, 36, 33), (13, 36, 34), (35, 100, 150),
+                                             (200, 28, 40), (501, 64, 30), (501, 68, 30), (2500, 36, 30),
+                                             (13, 124, 40), (13, 132, 40)])
+def test_general_deferred_outer_products(n_atoms, s, order):
+    api, wk, ctx, pos, model, H, lo, hi = _setup(n_atoms, s, order, True)
+    args = (ctx, H, model, pos, None, lo, hi, wk.probe_seed, s, order, 6.0, 0.5)
+    G0, _ = api.density_and_forces(*args)
+    G1, _ = api.density_and_forces(*args, max_panel_bytes=(order - 1) * 9 * n_atoms * s * 4)
+    assert (G0 - G1).abs().max().item() <= 1e-10 * G0.abs().max().item()
