@@ -95,14 +95,14 @@ __global__ void region_sizes(int n_atoms, const int32_t* __restrict__ rs, const 
 //
 // b_k = 2 H^ b_{k+1} - b_{k+2} + c_k E, X = H^ b_1 - b_2 + c_0 E, Y = H X for one region after another:
 // the two panels and as many mapped blocks as fit stay in shared memory, the other blocks come from L2 (the
-// same share of every row, so that all warps read both; the longest rows first, so that a warp's three have
-// about one length).  Nine lanes form an atom's 9 x 9 tile, 3 x 3 entries each: with rows and columns stored
-// as three groups of three in 12 floats, two 16-byte reads serve 9 FMAs.  What binds are these reads: L1
-// delivers 32 floats a cycle and SM, whatever lanes they go to.  Each entry adds its blocks in the order of
-// the step kernel and rounds where it does.  One launch per step reads copies of the blocks (140 MB) and the
-// panels of all regions instead.  500 atoms, 6 A, 126 terms: 10.9 ms so, 5.5 ms here; other tiles: a row of 9
-// entries per lane 7.1 ms, a row of 3 (one atom per warp) 8.0 ms, 5 x 3 7.1 ms.
-constexpr int LC_THREADS = 640, LC_ATOMS = 3, LC_BS = Layout<float, 9>::BS, LC_ROW = 12;
+// same share of every row, so that all warps read both; the longest rows first, so that a warp's ten have
+// about one length).  Three lanes form an atom's 9 x 9 tile, 9 x 3 entries each: 12 reads serve 27 FMAs.
+// What binds are these reads: L1 delivers 32 floats a cycle and SM, whatever lanes they go to, and looks up
+// ten atoms' blocks one after the other.  Each entry adds its blocks in the order of the step kernel and
+// rounds where it does.  One launch per step reads copies of the blocks (140 MB) and the panels of all
+// regions instead.  500 atoms, 6 A, 126 terms: 10.9 ms so, 4.9 ms here; other tiles: 3 x 3 entries per lane
+// 5.5 ms, 1 x 9 7.1 ms, 5 x 3 7.1 ms, 1 x 3 (one atom per warp) 8.0 ms.
+constexpr int LC_THREADS = 256, LC_ATOMS = 10, LC_HB = Layout<float, 9>::BS, LC_BS = 81, LC_ROW = 9;
 
 struct LocalArgs {
   int n_atoms, p, max_m, max_nnz, n_stage;  // n_stage: blocks in shared memory
@@ -113,26 +113,13 @@ struct LocalArgs {
   int* next;
 };
 
-// Position of row (or column) e of 9 among 12: three groups of three.
-__device__ __forceinline__ int lc_pos(int e) { return e + e / 3; }
-
-// Mapped blocks with each column's rows at those positions.
-__global__ void local_blocks(int64_t n, const float* __restrict__ hv, float* __restrict__ dst) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n) return;
-  const int j = (int)(e % 12);
-  dst[e] = (j & 3) < 3 ? hv[e - j + j - j / 4] : 0.f;
-}
-
 __device__ __forceinline__ void local_stage(const LocalArgs& A, const float* __restrict__ hv, float* hs, const int2* stage,
                                             int r0, int m) {
-  float4* dst = reinterpret_cast<float4*>(hs);
-  const float4* src = reinterpret_cast<const float4*>(hv);
   for (int t = threadIdx.x >> 5; t < m; t += LC_THREADS / 32) {
     const int kb = A.lrow[r0 + t];
-    for (int e = threadIdx.x & 31; e < stage[t].y * (LC_BS / 4); e += 32) {
-      const int k = e / (LC_BS / 4), j = e - k * (LC_BS / 4);
-      dst[stage[t].x * (LC_BS / 4) + e] = __ldg(src + (int64_t)__ldg(A.lblk + kb + k) * (LC_BS / 4) + j);
+    for (int e = threadIdx.x & 31; e < stage[t].y * LC_BS; e += 32) {
+      const int k = e / LC_BS, j = e - k * LC_BS, l = j / 9;
+      hs[stage[t].x * LC_BS + e] = __ldg(hv + (int64_t)__ldg(A.lblk + kb + k) * LC_HB + j + 3 * l);
     }
   }
 }
@@ -142,63 +129,64 @@ template <bool SUB>
 __device__ __forceinline__ void local_step(const LocalArgs& A, const float* __restrict__ hv, const float* hs,
                                            const int* idx, const int* perm, const int2* stage, int r0, int m,
                                            int k0, const float* in, float* out, float alpha, double c, int o) {
-  const int lane = threadIdx.x & 31, sub = lane / 9, gi = (lane - 9 * sub) / 3, gc = lane % 3;  // 9 % 3 = 0
+  const int lane = threadIdx.x & 31, sub = lane / 3, gc = lane - 3 * sub;
   for (int q = LC_ATOMS * (threadIdx.x >> 5) + sub; q < m && sub < LC_ATOMS; q += LC_ATOMS * (LC_THREADS / 32)) {
     const int t = perm[q];
     const int kb = __ldg(A.lrow + r0 + t) - k0, ke = __ldg(A.lrow + r0 + t + 1) - k0;
-    float acc[3][3];
+    float acc[9][3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < 9; ++i)
 #pragma unroll
       for (int v = 0; v < 3; ++v) acc[i][v] = 0.f;
     auto block = [&](const float* x, auto&& column) {
 #pragma unroll
       for (int l = 0; l < 9; ++l) {
-        const float4 u = *reinterpret_cast<const float4*>(x + l * LC_ROW), h = column(l * 12);
-        acc[0][0] = fmaf(h.x, u.x, acc[0][0]);
-        acc[0][1] = fmaf(h.x, u.y, acc[0][1]);
-        acc[0][2] = fmaf(h.x, u.z, acc[0][2]);
-        acc[1][0] = fmaf(h.y, u.x, acc[1][0]);
-        acc[1][1] = fmaf(h.y, u.y, acc[1][1]);
-        acc[1][2] = fmaf(h.y, u.z, acc[1][2]);
-        acc[2][0] = fmaf(h.z, u.x, acc[2][0]);
-        acc[2][1] = fmaf(h.z, u.y, acc[2][1]);
-        acc[2][2] = fmaf(h.z, u.z, acc[2][2]);
+        const float u[3] = {x[l * 9], x[l * 9 + 1], x[l * 9 + 2]};
+        float h[9];
+        column(l, h);
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+#pragma unroll
+          for (int v = 0; v < 3; ++v) acc[i][v] = fmaf(h[i], u[v], acc[i][v]);
       }
     };
     int k = kb;
     const int2 st = stage[t];  // its blocks in shared memory: first slot, number
-    const float* p = hs + st.x * LC_BS + 4 * gi;
+    const float* p = hs + st.x * LC_BS;
     for (const int ks = kb + st.y; k < ks; ++k, p += LC_BS)
-      block(in + idx[k] + 4 * gc, [&](int e) { return *reinterpret_cast<const float4*>(p + e); });
-    for (; k < ke; ++k) {
-      const float* g = hv + (int64_t)__ldg(A.lblk + k0 + k) * LC_BS + 4 * gi;
-      block(in + idx[k] + 4 * gc, [&](int e) { return __ldg(reinterpret_cast<const float4*>(g + e)); });
-    }
+      block(in + idx[k] + 3 * gc, [&](int l, float (&h)[9]) {
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      float4* y = reinterpret_cast<float4*>(out + (t * 9 + 3 * gi + j) * LC_ROW + 4 * gc);
-      const float4 old = *y;
-      const float q3[3] = {old.x, old.y, old.z};
-      float r[3];
+        for (int i = 0; i < 9; ++i) h[i] = p[l * 9 + i];
+      });
+    for (; k < ke; ++k) {
+      const float* g = hv + (int64_t)__ldg(A.lblk + k0 + k) * LC_HB;
+      block(in + idx[k] + 3 * gc, [&](int l, float (&h)[9]) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(g + l * 12)), b = __ldg(reinterpret_cast<const float4*>(g + l * 12 + 4));
+        h[0] = a.x; h[1] = a.y; h[2] = a.z; h[3] = a.w;
+        h[4] = b.x; h[5] = b.y; h[6] = b.z; h[7] = b.w;
+        h[8] = __ldg(g + l * 12 + 8);
+      });
+    }
+    float* y = out + t * 81 + 3 * gc;
+#pragma unroll
+    for (int j = 0; j < 9; ++j)
 #pragma unroll
       for (int v = 0; v < 3; ++v) {
-        r[v] = alpha * acc[j][v];
-        if (SUB) r[v] -= q3[v];
-        if (t == o && gi == gc && v == j && c != 0.0) r[v] = (float)((double)r[v] + c);
+        float r = alpha * acc[j][v];
+        if (SUB) r -= y[j * 9 + v];
+        if (t == o && j == 3 * gc + v && c != 0.0) r = (float)((double)r + c);
+        y[j * 9 + v] = r;
       }
-      *y = make_float4(r[0], r[1], r[2], 0.f);
-    }
   }
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(LC_THREADS, 1) local_clenshaw(const __grid_constant__ LocalArgs A) {
+__global__ void __launch_bounds__(LC_THREADS, 2) local_clenshaw(const __grid_constant__ LocalArgs A) {
   extern __shared__ __align__(16) float lsm[];
   float* pa = lsm;
   float* pb = pa + A.max_m * 9 * LC_ROW;
   float* hs = pb + A.max_m * 9 * LC_ROW;
-  int2* stage = reinterpret_cast<int2*>(hs + (int64_t)A.n_stage * LC_BS);
+  int2* stage = reinterpret_cast<int2*>(hs + (((int64_t)A.n_stage * LC_BS + 1) & ~(int64_t)1));
   int* perm = reinterpret_cast<int*>(stage + A.max_m);
   int* idx = perm + A.max_m;
   __shared__ int job, slots;
@@ -235,7 +223,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) local_clenshaw(const __grid_con
     for (int e = threadIdx.x; e < n_el; e += LC_THREADS) pa[e] = pb[e] = 0.f;
     __syncthreads();
     local_stage(A, A.hv, hs, stage, r0, m);
-    if (threadIdx.x < 9) pa[(o * 9 + threadIdx.x) * LC_ROW + lc_pos(threadIdx.x)] = (float)A.coef[A.p - 1];
+    if (threadIdx.x < 9) pa[(o * 9 + threadIdx.x) * LC_ROW + threadIdx.x] = (float)A.coef[A.p - 1];
     __syncthreads();
     float *b1 = pa, *b2 = pb;
     for (int k = A.p - 2; k >= 0; --k) {
@@ -245,10 +233,8 @@ __global__ void __launch_bounds__(LC_THREADS, 1) local_clenshaw(const __grid_con
       b2 = t;
     }
     auto store = [&](const float* v, float* dst) {
-      for (int e = threadIdx.x; e < m * 81; e += LC_THREADS) {
-        const int row = e / 9, c = e - 9 * row;
-        dst[((int64_t)r0 * 9 + row) * LC_ROW + c] = v[row * LC_ROW + lc_pos(c)];
-      }
+      for (int e = threadIdx.x; e < n_el; e += LC_THREADS)
+        dst[((int64_t)r0 * 9 + e / 9) * 12 + e % 9] = v[e];  // panel rows of 12
     };
     store(b1, A.X);
     if (A.h1) {
@@ -397,7 +383,9 @@ extern "C" int tbk_local_density(tbk_ctx* ctx, const tbk_bsr* H, const double* p
     la.max_nnz = std::max(la.max_nnz, (int)std::min<int64_t>(size[2 * a + 1], 1 << 24));
   }
   const int64_t smem_fix = 2 * (int64_t)la.max_m * 9 * LC_ROW * 4 + ((int64_t)la.max_nnz + 3 * (int64_t)la.max_m) * 4;
-  const int64_t smem_max = 226 << 10;
+  // two CTAs per SM where their panels fit (500 atoms, 6 A: 4.9 ms; one with more blocks in shared memory 5.7)
+  const int per_sm = smem_fix <= (110 << 10) ? 2 : 1;
+  const int64_t smem_max = per_sm == 2 ? 110 << 10 : 226 << 10;
   if (prec == TBK_MIXED && B == 9 && smem_fix <= smem_max) {
     std::vector<int32_t> ord((size_t)n + 1);
     std::iota(ord.begin(), ord.end() - 1, 0);
@@ -414,22 +402,14 @@ extern "C" int tbk_local_density(tbk_ctx* ctx, const tbk_bsr* H, const double* p
     la.lcol = lcol;
     la.lblk = lblk;
     la.own = own;
-    float* blocks = (float*)scratch(ctx, WS_SEGMENT, 2 * sizeof(float) * (size_t)H->nnzb * LC_BS);
-    auto mapped = [&](double lo, double hi, float* dst) {
-      const HOp g = prepare_hop(ctx, H, lo, hi, prec, WS_HHAT, err);
-      const int64_t tot = g.nnzb * LC_BS;
-      local_blocks<<<(unsigned)((tot + 255) / 256), 256, 0, ctx->stream>>>(tot, (const float*)g.hv, dst);
-      post_launch(ctx, "local_blocks");
-      return dst;
-    };
-    la.hv = mapped(emin, emax, blocks);
-    la.h1 = Q ? mapped(-1.0, 1.0, blocks + (size_t)H->nnzb * LC_BS) : nullptr;
+    la.hv = (const float*)prepare_hop(ctx, H, emin, emax, prec, WS_HHAT, err).hv;
+    la.h1 = Q ? (const float*)prepare_hop(ctx, H, -1.0, 1.0, prec, WS_SEGMENT, err).hv : nullptr;
     la.coef = dcoef;
     la.X = (float*)scratch(ctx, WS_CHECKPOINTS, 2 * panel);
     la.Y = la.X + panel / 4;
-    const int smem = (int)(smem_fix + (int64_t)la.n_stage * LC_BS * 4);
-    TBK_CUDA(cudaFuncSetAttribute(local_clenshaw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
-    local_clenshaw<<<std::min(n, ctx->num_sms), LC_THREADS, smem, ctx->stream>>>(la);
+    const int smem = (int)(smem_fix + (int64_t)la.n_stage * LC_BS * 4) + 16;
+    TBK_CUDA(cudaFuncSetAttribute(local_clenshaw, cudaFuncAttributeMaxDynamicSharedMemorySize, (226 << 10) + 16));
+    local_clenshaw<<<std::min(n, per_sm * ctx->num_sms), LC_THREADS, smem, ctx->stream>>>(la);
     post_launch(ctx, "local_clenshaw");
     if (P) extract(la.X, P);
     if (Q) extract(la.Y, Q);

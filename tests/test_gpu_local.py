@@ -124,8 +124,8 @@ def test_local_density_single_atom(api, ctx):
     assert np.abs(Q.cpu().numpy()[0] - Hd @ Pref).max() < 1e-11
 
 
-# The FP32 region kernel at the edges of its warp passes (5 atoms a warp, 80 a pass) and with blocks beyond
-# shared memory (120 to 300 atoms in one region), and the step kernels where the panels do not fit (360),
+# The FP32 region kernel at the edges of its warp passes (10 atoms a warp, 80 a pass), with blocks beyond shared
+# memory (120 to 300 atoms in one region, one CTA per SM), and the step kernels where the panels do not fit (360),
 # against the FP64 path: FP32 products of p steps, the 2e-5 of the oracle comparison above.
 @pytest.mark.parametrize("n,r_max,p", [(1, 5.0, 1), (2, 5.0, 2), (3, 5.0, 3), (13, 4.0, 40), (80, 100.0, 41),
                                        (81, 100.0, 40), (120, 100.0, 40), (200, 7.0, 40), (300, 100.0, 12),
