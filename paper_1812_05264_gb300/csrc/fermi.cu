@@ -160,12 +160,16 @@ __device__ __forceinline__ double count_occupation(double e, double mu, double i
 // bisection's; one barrier for `depth` halvings.  N(mu) is summed as FERMI_LANES strided chains and
 // a tree over them whatever the launch, so mu does not depend on it.  Latency binds: an FP64 operation
 // takes ~85 cycles and an occupation ~40 of them (45 halvings one after the other in one CTA: 0.65 ms
-// at M = 504, 9.2 ms at M = 9904; this form 0.10 and 0.17 ms).
+// at M = 504, 9.2 ms at M = 9904; this form 0.084 and 0.119 ms, of which the sums over 32 parts and the
+// decisions were 0.02 and 0.05 more with every warp of every CTA at them).
 __global__ void __launch_bounds__(FERMI_THREADS)
 fermi_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int depth, int parts, double* __restrict__ buf,
              double* __restrict__ res) {
   __shared__ double red[32];
   __shared__ double cnt[FERMI_MIDS + 1];
+  __shared__ double tree[16 * FERMI_MIDS];
+  __shared__ double state[3];  // the bracket, and whether it is done
+  __shared__ double my_mid;
   __shared__ double fs[FERMI_THREADS];
   const FermiJob job = jobs ? jobs[blockIdx.y] : one;
   const FermiBuf b = fermi_buf(buf + job.buf_off, job.M);
@@ -218,16 +222,27 @@ fermi_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int depth, i
       __syncthreads();
     } else {
       const int pi = cta / nm, q = cta - pi * nm;
-      if (pi < parts) chains(pi, mid_of(q), part + 32 * q);
+      if (tid == 0) my_mid = mid_of(q);
+      __syncthreads();
+      if (pi < parts) chains(pi, my_mid, part + 32 * q);
       ok = ok && tbk_grid_wait(b.ctr, (unsigned)(ncta * (phase + 1)));
     }
     ++phase;
-    for (int q = tid >> 5; q < nm; q += FERMI_THREADS / 32) {
-      double t = __ldcg(part + 32 * q + (tid & 31));
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if ((tid & 31) == 0) cnt[q] = t;
+    // the tree over a midpoint's 32 sums, with all lanes at work on all midpoints: an SM takes 19 cycles for
+    // a warp's FP64 addition
+    for (int e = tid; e < 16 * nm; e += FERMI_THREADS) {
+      const double* p = part + 2 * e - (e & 15);  // 32 (e / 16) + e % 16
+      tree[e] = __ldcg(p) + __ldcg(p + 16);
     }
     __syncthreads();
+    for (int o = 8; o > 0; o >>= 1) {
+      for (int e = tid; e < o * nm; e += FERMI_THREADS) {
+        const int q = e / o, i = e - q * o;
+        const double t = tree[16 * q + i] + tree[16 * q + i + o];
+        (o == 1 ? cnt[q] : tree[16 * q + i]) = t;
+      }
+      __syncthreads();
+    }
   };
   double mu = job.mu_fixed, status = 0.0;
   if (job.n_e >= 0.0) {
@@ -236,7 +251,7 @@ fermi_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int depth, i
     if (cnt[0] > job.n_e || cnt[1] < job.n_e) status = 1.0;
     __syncthreads();
     bool done = false;
-    for (int it = 0; it < 200 && !done && ok;) {
+    for (int it = 0; it < 200 && !done && ok; it += depth) {
       // heap order: node 1 is the midpoint of [lo, hi], node 2q that of the lower half below q
       evaluate((1 << depth) - 1, [&](int q) {
         double l = lo, h = hi;
@@ -246,15 +261,23 @@ fermi_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int depth, i
         }
         return 0.5 * (l + h);
       });
-      int node = 1;
-      for (int d = 0; d < depth && it < 200 && !done; ++d, ++it) {
-        const double mid = 0.5 * (lo + hi);
-        const bool up = cnt[node - 1] < job.n_e;
-        if (up) lo = mid; else hi = mid;
-        node = 2 * node + (up ? 1 : 0);
-        done = hi - lo < 1e-13 * W;
+      if (tid == 0) {
+        int node = 1;
+        for (int d = 0; d < depth && it + d < 200 && !done; ++d) {
+          const double mid = 0.5 * (lo + hi);
+          const bool up = cnt[node - 1] < job.n_e;
+          if (up) lo = mid; else hi = mid;
+          node = 2 * node + (up ? 1 : 0);
+          done = hi - lo < 1e-13 * W;
+        }
+        state[0] = lo;
+        state[1] = hi;
+        state[2] = done;
       }
       __syncthreads();
+      lo = state[0];
+      hi = state[1];
+      done = state[2] != 0.0;
     }
     mu = 0.5 * (lo + hi);
   }
@@ -273,11 +296,13 @@ fermi_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int depth, i
   }
   if (ncta > 1) ok = ok && tbk_grid_wait(b.ctr, (unsigned)(ncta * (phase + 1)));
   else __syncthreads();
-  if (cta == 0 && threadIdx.x < 3) {
+  if (cta == 0 && tid < 96) {
+    const int q = tid >> 5, lane = tid & 31;
     double t = 0.0;
-    for (int i = 0; i < ncta; ++i) t += __ldcg(part + 3 * i + threadIdx.x);
-    out[1 + threadIdx.x] = t;
-    if (threadIdx.x == 0) {
+    for (int i = lane; i < ncta; i += 32) t += __ldcg(part + 3 * i + q);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) out[1 + q] = t;
+    if (tid == 0) {
       out[0] = mu;
       out[4] = ok ? status : 2.0;
     }
@@ -300,8 +325,9 @@ static void fermi_launch(tbk_ctx* ctx, int n, const FermiJob& one, const FermiJo
   post_launch(ctx, "rho_kernel");
   // CTAs per problem, as long as all problems fit the chip together: as many midpoints at once as
   // there is room for, then 4 to 16 CTAs per midpoint (one CTA per problem takes its midpoints one by
-  // one).  Chains of one link are latency alone (M = 800: 121 us at depth 4, 103 us at 5); longer ones
-  // want the CTAs for more parts instead (M = 9904: 300 us at depth 5, 171 us at 4 with twice the parts)
+  // one).  Chains of one link are latency alone (M = 800: the call 120 us at depth 5 with 4 parts, 120 at
+  // depth 4 and 124 at depth 5 with 8); longer ones want the CTAs for more parts instead (M = 9904, before the
+  // sums were shared out: 300 us at depth 5, 171 us at 4 with twice the parts)
   int occ = 0;
   TBK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fermi_kernel, FERMI_THREADS, 0));
   const int room = occ * ctx->num_sms / n, links = ceil_div(M_max, FERMI_LANES);
