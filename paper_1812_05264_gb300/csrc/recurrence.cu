@@ -300,8 +300,9 @@ struct BulkCfg {
   static constexpr int THREADS = 32 * (CW + 1);
 };
 
-template <int CW, int D>
-__global__ void __launch_bounds__(32 * (CW + 1), 4)
+// DENSE: seven CTAs per SM (80 registers).
+template <int CW, int D, bool DENSE = false>
+__global__ void __launch_bounds__(32 * (CW + 1), DENSE ? 7 : 4)
 cheb_step_bulk(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const float* __restrict__ hv, const float* __restrict__ yin, const float* yprev,
                float* yout, const float alpha, const float c_r, const uint64_t seed, const int s,
@@ -1061,12 +1062,12 @@ static int occupancy_self() {
   return n;
 }
 
-template <int CW, int D>
+template <int CW, int D, bool DENSE = false>
 static int occupancy_bulk() {
   using C = BulkCfg<CW, D>;
-  cudaFuncSetAttribute(cheb_step_bulk<CW, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+  cudaFuncSetAttribute(cheb_step_bulk<CW, D, DENSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   int n = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cheb_step_bulk<CW, D>, C::THREADS, C::SMEM);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cheb_step_bulk<CW, D, DENSE>, C::THREADS, C::SMEM);
   return n;
 }
 
@@ -1105,7 +1106,7 @@ static int occupancy_lane() {
 }
 
 struct Occ {
-  int simple = 0, bulk[5] = {0, 0, 0, 0, 0}, lane[3] = {0, 0, 0};
+  int simple = 0, bulk[5] = {0, 0, 0, 0, 0}, dense = 0, lane[3] = {0, 0, 0};
 };
 
 static Occ& occ_cache(int dev) {
@@ -1139,6 +1140,7 @@ static Occ& occupancies(tbk_ctx* ctx) {
     o.simple = std::max(1, m);
     o.bulk[1] = occupancy_self();  // 128-probe tasks run on the self-fed kernel
     o.bulk[2] = occupancy_bulk<2, BULK_D>();
+    o.dense = occupancy_bulk<2, BULK_D, true>();
     o.bulk[4] = occupancy_bulk<4, BULK_D>();
     o.lane[0] = occupancy_lane<4>();
     o.lane[1] = occupancy_lane<8>();
@@ -1169,6 +1171,14 @@ static int fp64_rows(const tbk_ctx* ctx, const HOp& op, int s) {
   return fp64_units(op, s, 3) >= 4 * (int64_t)ctx->num_sms ? 3 : 1;
 }
 
+// 256-probe tasks with 80 instead of 108 registers, so that seven CTAs per SM run instead of five: faster once
+// there are several tasks for each, slower (8 bytes of spills) as long as five take them all at once or nearly.
+// us a step, five -> seven: 700 atoms 15.7 -> 16.7, 850 19.6 -> 20.5, 1,000 23.1 -> 22.9, 1,300 30.6 -> 28.9,
+// 3,000 64.4 -> 61.1, 10,000 215 -> 195.
+static bool dense_bulk(const tbk_ctx* ctx, const HOp& op, int s, int cw) {
+  return cw == 2 && (int64_t)op.n_atoms * (s / 256) > 8 * ctx->num_sms;
+}
+
 int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s) {
   const Occ& o = occupancies(ctx);
   // the TMA-fed kernel's occupancy sets the grid where it runs (the other kernels then just take
@@ -1180,7 +1190,8 @@ int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s) {
     return (int)std::min<int64_t>((int64_t)op.n_atoms * ((s + 511) / 512), (int64_t)std::max(1, o.lane[lane_class(s)]) * ctx->num_sms);
   const int cw = chosen_cw(ctx, op, s, 0);
   const bool narrow = op.prec == TBK_MIXED && op.B == 9 && s < 128;
-  const int per_sm = narrow && o.bulk[1] > 0 ? o.bulk[1] : (cw && o.bulk[cw] > 0 ? o.bulk[cw] : o.simple);
+  const int fed = cw && dense_bulk(ctx, op, s, cw) ? o.dense : (cw ? o.bulk[cw] : 0);
+  const int per_sm = narrow && o.bulk[1] > 0 ? o.bulk[1] : (fed > 0 ? fed : o.simple);
   const int64_t tasks = cw ? (int64_t)op.n_atoms * (s / (128 * cw)) : op.n_atoms;
   return (int)std::max<int64_t>(1, std::min<int64_t>(per_sm * ctx->num_sms, tasks));
 }
@@ -1210,10 +1221,10 @@ static void launch_simple(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G)
   post_launch(ctx, "cheb_step_kernel");
 }
 
-template <int CW>
+template <int CW, bool DENSE = false>
 static void launch_bulk(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
   using C = BulkCfg<CW, BULK_D>;
-  launch_pdl(ctx, cheb_step_bulk<CW, BULK_D>, G, C::THREADS, C::SMEM,
+  launch_pdl(ctx, cheb_step_bulk<CW, BULK_D, DENSE>, G, C::THREADS, C::SMEM,
                op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)a.yin, (const float*)a.yprev,
                (float*)a.yout, (float)a.alpha, (float)a.c_r, a.seed, a.s, a.direct, a.partials, a.err, a.batch,
                a.per_task, ctx->stall_next_step);
@@ -1292,6 +1303,7 @@ void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
   const int cw = chosen_cw(ctx, op, a.s, a.per_task);
   if (cw && !a.cur_is_probe && a.err && !a.force_simple && occ_cache(ctx->device).bulk[cw] > 0) {
     if (cw == 4) launch_bulk<4>(ctx, op, a, G);
+    else if (cw == 2 && dense_bulk(ctx, op, a.s, cw) && occ_cache(ctx->device).dense > 0) launch_bulk<2, true>(ctx, op, a, G);
     else if (cw == 2) launch_bulk<2>(ctx, op, a, G);
     else launch_self<false>(ctx, op, a, G);
     return;

@@ -64,3 +64,9 @@ def test_one_launch_sweep_equals_the_steps(L, s, orders):
         got = api.chebyshev_moments(ctx, H, -9.0, 9.0, 5, s, order, fp64=True)
         ref = api.chebyshev_moments(ctx, H, -9.0, 9.0, 5, s, order, fp64=True, plain=True)
         assert (got - ref).abs().max().item() <= 1e-12 * L ** 3
+
+
+# 256-probe tasks around the line of the denser kernel (more than eight tasks per SM: 1,217 atoms on 152 SMs)
+@pytest.mark.parametrize("n_atoms,direct", [(1216, False), (1217, False), (1217, True), (1530, False)])
+def test_256_probe_steps_equal_the_plain_kernel(n_atoms, direct):
+    _check(n_atoms, 256, False, direct, order=5)
