@@ -1257,7 +1257,7 @@ static void launch_fused_cw(tbk_ctx* ctx, const HOp& op, const void* bin, const 
     TBK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, clenshaw_sddmm_bulk<CW, SD>, C::THREADS, C::SMEM));
     TBK_CHECK_ARG(occ > 0, "fused adjoint kernel does not fit on this device");
   }
-  const int G = std::max(1, std::min(op.n_atoms, occ * ctx->num_sms));
+  const int G = task_grid(op.n_atoms, (int64_t)occ * ctx->num_sms);
   launch_pdl(ctx, clenshaw_sddmm_bulk<CW, SD>, G, C::THREADS, C::SMEM, op.n_atoms, op.row_ptr, op.col,
              (const float*)op.hv, (const float*)bin, (const float*)bprev, (float*)bout, (const float*)ypan, cf, seed, s, w,
              Gacc, err, batch, cf_cl, (const float*)ym1, (const float*)yp1, y_first, ctx->stall_next_adjoint);
@@ -1291,7 +1291,7 @@ void launch_fused(tbk_ctx* ctx, const HOp& op, const void* bin, const void* bpre
       TBK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, clenshaw_self<CLEN_SELF_R>, 32, C::SMEM));
       TBK_CHECK_ARG(occ > 0, "self-fed adjoint kernel does not fit on this device");
     }
-    const int G = std::max(1, std::min(op.n_atoms, occ * ctx->num_sms));
+    const int G = task_grid(op.n_atoms, (int64_t)occ * ctx->num_sms);
     launch_pdl(ctx, clenshaw_self<CLEN_SELF_R>, G, 32, C::SMEM, op.n_atoms, op.row_ptr, op.col, (const float*)op.hv,
                (const float*)bin, (const float*)bprev, (float*)bout, (const float*)ypan, cf, seed, s, err, batch, cf_cl,
                (const float*)ym1, (const float*)yp1, y_first);
@@ -1335,7 +1335,7 @@ static void launch_outer_rows(tbk_ctx* ctx, const HOp& op, const OuterPanels& wp
     TBK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, outer_rows<NW>, 32 * NW, SMEM));
     TBK_CHECK_ARG(occ > 0, "outer-product kernel does not fit on this device");
   }
-  launch_pdl(ctx, outer_rows<NW>, std::min(op.n_atoms, occ * ctx->num_sms), 32 * NW, SMEM, op.n_atoms, op.row_ptr,
+  launch_pdl(ctx, outer_rows<NW>, task_grid(op.n_atoms, (int64_t)occ * ctx->num_sms), 32 * NW, SMEM, op.n_atoms, op.row_ptr,
              op.col, wp, nt, last_is_y0, Gacc, err);
 }
 
@@ -1453,7 +1453,7 @@ static void launch_window_g(tbk_ctx* ctx, const HOp& op, const WindowPanels& wp,
     TBK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sddmm_window_g<NC>, C::THREADS, C::SMEM));
     TBK_CHECK_ARG(occ > 0, "windowed outer-product kernel does not fit on this device");
   }
-  const int G = std::max(1, std::min(op.n_atoms, occ * ctx->num_sms));
+  const int G = task_grid(op.n_atoms, (int64_t)occ * ctx->num_sms);
   launch_pdl(ctx, sddmm_window_g<NC>, G, C::THREADS, C::SMEM, op.n_atoms, op.row_ptr, op.col, wp, nw, s, w, Gacc, err, batch, kcl, k_lo);
   post_launch(ctx, "sddmm_window_g");
 }
@@ -1466,7 +1466,7 @@ void launch_window(tbk_ctx* ctx, const HOp& op, const WindowPanels& wp, int nw, 
   else launch_window_g<1>(ctx, op, wp, nw, s, w, Gacc, err, batch, kcl, k_lo);
 }
 
-// ---- adjoint of the doubled moments (TMA-fed fused path) ------------------------------------
+// ---- adjoint of the doubled moments (FP32 at 128, 256 and 512 probes, FP64) ---------------------
 //
 // The moments come from the doubling identities (C_m C_n = (C_{m+n} + C_{|m-n|})/2):
 //   mu_2k = 2 e_k - mu_0,  mu_2k-1 = 2 o_k - mu_1,  e_k = <y_k, y_k>/s,  o_k = <y_k, y_{k-1}>/s,
@@ -1659,6 +1659,7 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
         a.per_task = 1;
       } else {
         a.partials = partials + (size_t)(t - 1) * nctas * 2;
+        a.grid = nctas;
       }
     }
     launch_step(ctx, o, a);
@@ -2044,7 +2045,7 @@ void energies_and_forces_doubled(tbk_ctx* ctx, const tbk_bsr* H, const tbk_model
   double* Gsym = Gacc + (size_t)op.nnzb * BB;
   TBK_CUDA(cudaMemsetAsync(Gacc, 0, sizeof(double) * (size_t)op.nnzb * BB, ctx->stream));
   const int K = p / 2;
-  const int nctas = step_grid_ctas(ctx, op, s);
+  const int nctas = step_grid_ctas(ctx, op, s, K);
   double* partials = (double*)scratch(ctx, WS_PARTIALS, sizeof(double) * 2 * (size_t)std::max(1, K) * nctas);
   // per-step sums, the solve's buffer (16-byte aligned), its result, the moments unless given
   const size_t nsums = 2 * (size_t)K + 64, nfermi = fermi_doubles(quad_nodes(p), p);

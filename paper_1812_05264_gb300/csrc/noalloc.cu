@@ -88,7 +88,7 @@ extern "C" int tbk_chebyshev_moments_noalloc(tbk_ctx* ctx, const tbk_bsr* H, dou
   shape.n_atoms = H->n_atoms;
   shape.n_rows = n_rows;    // the grid follows any tuned choice for this shape, as the steps do
   shape.nnzb = H->nnzb;
-  int nctas = step_grid_ctas(ctx, shape, s);
+  int nctas = step_grid_ctas(ctx, shape, s, K, (flags & TBK_PLAIN_KERNEL) != 0);
   // layout: flag | sums | partials | mapped H | panel A | panel B, each 256-byte aligned
   const size_t o_flag = 0;
   const size_t o_sums = o_flag + 256;
@@ -101,6 +101,10 @@ extern "C" int tbk_chebyshev_moments_noalloc(tbk_ctx* ctx, const tbk_bsr* H, dou
     need = o_pb + (K >= 2 ? align256(panel) : 0);
   };
   place();
+  if (need > kStaticScratchBytes) {
+    nctas = step_grid_ctas(ctx, shape, s, K, true);
+    place();
+  }
   if (need > kStaticScratchBytes && nctas > ctx->num_sms) {
     nctas = ctx->num_sms;  // fewer CTAs leave fewer partial sums
     place();

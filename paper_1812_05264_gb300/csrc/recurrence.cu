@@ -1173,17 +1173,16 @@ static int fp64_rows(const tbk_ctx* ctx, const HOp& op, int s) {
 
 // 256-probe tasks with 80 instead of 108 registers, so that seven CTAs per SM run instead of five: faster once
 // there are several tasks for each, slower (8 bytes of spills) as long as five take them all at once or nearly.
-// us a step, five -> seven: 700 atoms 15.7 -> 16.7, 850 19.6 -> 20.5, 1,000 23.1 -> 22.9, 1,300 30.6 -> 28.9,
+// us a step, five -> seven (CTAs that stay): 700 atoms 15.7 -> 16.7, 850 19.6 -> 20.5, 1,000 23.1 -> 22.9, 1,300 30.6 -> 28.9,
 // 3,000 64.4 -> 61.1, 10,000 215 -> 195.
 static bool dense_bulk(const tbk_ctx* ctx, const HOp& op, int s, int cw) {
   return cw == 2 && (int64_t)op.n_atoms * (s / 256) > 8 * ctx->num_sms;
 }
 
-int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s) {
+int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s, int K, bool resident) {
   const Occ& o = occupancies(ctx);
-  // the TMA-fed kernel's occupancy sets the grid where it runs (the other kernels then just take
-  // more than one wave: every kernel loops over its tasks, none waits on another CTA); the
-  // tensor-core step, when selected, runs on this same grid so that the per-CTA partial sums line up
+  // every kernel loops over its tasks and none waits on another CTA, so any grid will do; the
+  // tensor-core step and the plain kernel run on the resident one (CTAs that set up their TMEM once; fewer tasks)
   if (use_rows64(op))
     return (int)std::min<int64_t>((fp64_units(op, s, fp64_rows(ctx, op, s)) + 3) / 4, 4 * ctx->num_sms);
   if (use_lane(op, s))
@@ -1192,8 +1191,10 @@ int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s) {
   const bool narrow = op.prec == TBK_MIXED && op.B == 9 && s < 128;
   const int fed = cw && dense_bulk(ctx, op, s, cw) ? o.dense : (cw ? o.bulk[cw] : 0);
   const int per_sm = narrow && o.bulk[1] > 0 ? o.bulk[1] : (fed > 0 ? fed : o.simple);
-  const int64_t tasks = cw ? (int64_t)op.n_atoms * (s / (128 * cw)) : op.n_atoms;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(per_sm * ctx->num_sms, tasks));
+  const int64_t tasks = cw ? (int64_t)op.n_atoms * (s / (128 * cw)) : op.n_atoms, held = (int64_t)per_sm * ctx->num_sms;
+  if (resident || (!cw && !narrow)) return (int)std::max<int64_t>(1, std::min(held, tasks));
+  // at most 256 MB of partial sums
+  return (int)std::min<int64_t>(task_grid(tasks, held), std::max<int64_t>(held, ((int64_t)1 << 24) / std::max(1, K)));
 }
 
 template <typename T>
@@ -1280,7 +1281,7 @@ static void launch_fp64(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
 
 void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
   KernelTimerScope timer(ctx, TBK_KERNEL_STEP);
-  const int G = a.grid > 0 ? a.grid : step_grid_ctas(ctx, op, a.s);
+  const int G = a.grid > 0 ? a.grid : step_grid_ctas(ctx, op, a.s, 0, a.force_simple || a.use_tc);
   if (a.use_tc && !a.cur_is_probe && a.err && !a.force_simple && !a.batch.atom_cl && !a.per_task &&
       tc_eligible(op, a.s)) {
     launch_step_tc(ctx, op, a, G);
@@ -1672,7 +1673,8 @@ void moments_sweep(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, uin
   const size_t panel = (size_t)op.n_rows * s * esz;
   const int K = direct ? order - 1 : order / 2;   // steps: largest moment index 2K >= order - 1
   const bool sweep = use_sweep(ctx, op, s, K, direct, per_probe, flags);
-  const int nctas = sweep ? sweep_partials(ctx, op, s) : step_grid_ctas(ctx, op, s);
+  const int nctas = sweep ? sweep_partials(ctx, op, s)
+                          : step_grid_ctas(ctx, op, s, K, (flags & (TBK_TENSOR_CORES | TBK_PLAIN_KERNEL)) != 0);
   double* partials = (double*)scratch(ctx, WS_PARTIALS, sizeof(double) * 2 * (size_t)std::max(1, K) * nctas);
   double* sums = (double*)scratch(ctx, WS_MISC, sizeof(double) * 2 * (size_t)std::max(1, K) + 64);
   if (sweep) launch_sweep(ctx, op, probe_panel, probe_seed, s, K, partials);
@@ -1694,6 +1696,7 @@ void moments_sweep(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, uin
     a.err = flag;
     a.force_simple = (flags & TBK_PLAIN_KERNEL) ? 1 : 0;
     a.use_tc = (flags & TBK_TENSOR_CORES) ? 1 : 0;
+    a.grid = nctas;
     if (j == 1) {
       // a further step follows: its panel holds the probe block until then (a step on a panel takes a
       // third of the time of one that regenerates every neighbour's probes)
