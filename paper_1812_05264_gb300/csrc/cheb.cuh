@@ -90,12 +90,10 @@ int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s, int K = 0, bool resident 
 // starts where one ends, while CTAs that stay and take every held-th task wait for the longest sum of rows at
 // the end, and hold a warp set between tasks.  us a step, staying -> one task each: 512 probes 1,000 atoms 38.2 ->
 // 33.1, 10,000 atoms 337 -> 299; 256 probes 3,000 atoms 61.2 -> 52.3, 10,000 atoms 194 -> 169; 128 probes 10,000
-// atoms 104 -> 98.7; fused adjoint 10,000 x 512 823 -> 782.  Up to a third more than fit stay with CTAs that take
-// two (126 stored steps on 1,000 atoms x 256 probes, 760 held: 3.43 ms so, 3.53 with 1,000 CTAs), and up to half
-// a round more than two rounds follow in CTAs that are there instead of filling a third round (fused adjoint
+// atoms 104 -> 98.7; fused adjoint 10,000 x 512 823 -> 782.  Up to half a
+// round more than two rounds follow in CTAs that are there instead of filling a third round (fused adjoint
 // 1,000 x 512, 2.2 rounds: 87.6 staying, 83.9 so, 89.7 with one task each).
 inline int task_grid(int64_t tasks, int64_t held) {
-  if (20 * tasks < 27 * held) return (int)(tasks < held ? tasks : held);
   return (int)(tasks > 2 * held && 2 * tasks < 5 * held ? 2 * held : tasks);
 }
 void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a);

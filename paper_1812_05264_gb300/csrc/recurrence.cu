@@ -1171,12 +1171,12 @@ static int fp64_rows(const tbk_ctx* ctx, const HOp& op, int s) {
   return fp64_units(op, s, 3) >= 4 * (int64_t)ctx->num_sms ? 3 : 1;
 }
 
-// 256-probe tasks with 80 instead of 108 registers, so that seven CTAs per SM run instead of five: faster once
-// there are several tasks for each, slower (8 bytes of spills) as long as five take them all at once or nearly.
-// us a step, five -> seven (CTAs that stay): 700 atoms 15.7 -> 16.7, 850 19.6 -> 20.5, 1,000 23.1 -> 22.9, 1,300 30.6 -> 28.9,
-// 3,000 64.4 -> 61.1, 10,000 215 -> 195.
+// 256-probe tasks with 80 instead of 108 registers, so that seven CTAs per SM run instead of five: where five
+// leave a second round.  us a step, five -> seven: 700 atoms 15.7 -> 16.7 and 850 19.6 -> 20.5 (8 bytes of
+// spills), 1,000 23.2 -> 22.8, 1,200 28.3 -> 23.7, 3,000 64.4 -> 61.1 and 10,000 215 -> 195 (both with CTAs that
+// stay); 126 stored steps on 1,000 atoms 3.45 -> 3.37 ms.
 static bool dense_bulk(const tbk_ctx* ctx, const HOp& op, int s, int cw) {
-  return cw == 2 && (int64_t)op.n_atoms * (s / 256) > 8 * ctx->num_sms;
+  return cw == 2 && (int64_t)op.n_atoms * (s / 256) > 6 * ctx->num_sms;
 }
 
 int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s, int K, bool resident) {

@@ -66,7 +66,9 @@ def test_one_launch_sweep_equals_the_steps(L, s, orders):
         assert (got - ref).abs().max().item() <= 1e-12 * L ** 3
 
 
-# 256-probe tasks around the line of the denser kernel (more than eight tasks per SM: 1,217 atoms on 152 SMs)
-@pytest.mark.parametrize("n_atoms,direct", [(1216, False), (1217, False), (1217, True), (1530, False)])
+# 256-probe tasks around the line of the denser kernel (more than six tasks per SM: 913 atoms on 152 SMs), and
+# grids of less and more than two rounds
+@pytest.mark.parametrize("n_atoms,direct", [(912, False), (913, False), (913, True), (1217, True), (1530, False),
+                                            (2300, False), (2700, False)])
 def test_256_probe_steps_equal_the_plain_kernel(n_atoms, direct):
     _check(n_atoms, 256, False, direct, order=5)
