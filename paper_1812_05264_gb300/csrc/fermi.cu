@@ -111,7 +111,8 @@ __global__ void fermi_setup(const FermiJob one, const FermiJob* __restrict__ job
 
 // The node energies, and rho_j and rho_{M-1-j} from the even and the odd part of the sum over k
 // (cos(k (pi - t)) = (-1)^k cos(k t): half the terms of two separate sums).  S lanes share a pair of
-// nodes, lane r takes k = r, r + S, ..., one parity per lane, each compensated.  The compensated chain
+// nodes, lane r takes k = r, r + S, ..., one parity per lane, each compensated, and so are the sums of the
+// lanes.  The compensated chain
 // is four dependent FP64 operations of ~85 cycles a term, at 1/64 of the FP32 rate: one thread per
 // node took 432 us at p = 2476 by latency alone; S lanes cut the chain until the issue rate binds.
 __global__ void __launch_bounds__(64)
@@ -134,12 +135,24 @@ rho_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int S, double*
       if (m >= period) m -= period;
     }
   }
-  for (int o = S / 2; o >= 2; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  const double other = __shfl_xor_sync(0xffffffffu, s, 1);
+  // the lanes' sums, each s - c, are added as pairs too (TwoSum): rho_j carries one rounding of a sum
+  double e = -c;
+  auto pair_sum = [&](double s2, double e2) {
+    const double t = s + s2, z = t - s;
+    e = (e + e2) + ((s - (t - z)) + (s2 - z));
+    s = t;
+  };
+  for (int o = S / 2; o >= 2; o >>= 1) pair_sum(__shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, e, o));
+  // lane 0 holds the even part, lane 1 the odd part
+  const double so = __shfl_xor_sync(0xffffffffu, s, 1), eo = __shfl_xor_sync(0xffffffffu, e, 1);
+  if (r == 1) {
+    s = -s;
+    e = -e;
+  }
+  pair_sum(so, eo);
   if (j < M / 2 && r < 2) {
-    // lane 0 holds the even part, lane 1 the odd part
     const int node = r == 0 ? j : M - 1 - j;
-    b.node[node] = make_double2(node_energy(node, M, job.emin, job.emax), (r == 0 ? s + other : other - s) / M);
+    b.node[node] = make_double2(node_energy(node, M, job.emin, job.emax), (s + e) / M);
   }
 }
 
