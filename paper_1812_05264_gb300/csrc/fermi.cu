@@ -109,50 +109,87 @@ __global__ void fermi_setup(const FermiJob one, const FermiJob* __restrict__ job
   if (i < j.p) b.w[i] = (i == 0 ? 1.0 : 2.0) * damp_factor(i, j.p, damping) * mom[j.mom_off + i];
 }
 
+// Lanes that share two pairs of nodes: enough for `lanes` lanes in all if the problem were alone.  From its own
+// size only, so that its sums do not depend on the problems that are solved with it.
+__host__ __device__ inline int rho_groups(int M) { return (M / 2 + 1) / 2; }
+__host__ __device__ inline int rho_lanes(int M, int lanes) {
+  int S = 2;
+  while (S < 32 && (int64_t)rho_groups(M) * S < lanes) S *= 2;
+  return S;
+}
+
 // The node energies, and rho_j and rho_{M-1-j} from the even and the odd part of the sum over k
-// (cos(k (pi - t)) = (-1)^k cos(k t): half the terms of two separate sums).  S lanes share a pair of
-// nodes, lane r takes k = r, r + S, ..., one parity per lane, each compensated, and so are the sums of the
-// lanes.  The compensated chain
+// (cos(k (pi - t)) = (-1)^k cos(k t): half the terms of two separate sums).  S lanes share the sums of
+// two pairs of nodes, lane r takes k = r, r + S, ..., one parity per lane, each sum compensated, and so
+// are the sums of the lanes.  The compensated chain
 // is four dependent FP64 operations of ~85 cycles a term, at 1/64 of the FP32 rate: one thread per
-// node took 432 us at p = 2476 by latency alone; S lanes cut the chain until the issue rate binds.
-__global__ void __launch_bounds__(64)
-rho_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int S, double* __restrict__ buf) {
+// node took 432 us at p = 2476 by latency alone; S lanes cut the chain until the issue rate binds.  Two pairs
+// per lane: two chains in flight, and after the first exchange between lanes each has one pair to add.
+__global__ void __launch_bounds__(32)
+rho_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int lanes, double* __restrict__ buf) {
   const FermiJob job = jobs ? jobs[blockIdx.y] : one;
   const FermiBuf b = fermi_buf(buf + job.buf_off, job.M);
-  const int M = job.M, p = job.p;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = i / S, r = i - j * S;
-  double s = 0.0, c = 0.0;
-  if (j < M / 2) {
-    const int period = 4 * M, step = (int)((int64_t)S * (2 * j + 1) % period);
-    int m = (int)((int64_t)r * (2 * j + 1) % period);
+  const int M = job.M, p = job.p, S = rho_lanes(M, lanes);
+  if (blockIdx.x * 32 / S >= rho_groups(M)) return;
+  const int group = (blockIdx.x * 32 + threadIdx.x) / S, r = threadIdx.x % S;
+  double s[2], e[2];
+  unsigned m[2], step[2];
+  const unsigned period = 4 * M;  // at most 2^26
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const unsigned odd = 2 * (2 * group + q) + 1;  // 2 j + 1; past the last pair: sums that are not used
+    s[q] = e[q] = 0.0;
+    step[q] = S * odd % period;
+    m[q] = r * odd % period;
+  }
 #pragma unroll 4
-    for (int k = r; k < p; k += S) {
-      const double y = __ldg(b.w + k) * __ldg(b.tab + m) - c, t = s + y;
-      c = (t - s) - y;
-      s = t;
-      m += step;
-      if (m >= period) m -= period;
+  for (int k = r; k < p; k += S) {
+    const double w = __ldg(b.w + k);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const double y = w * __ldg(b.tab + m[q]) - e[q], t = s[q] + y;
+      e[q] = (t - s[q]) - y;
+      s[q] = t;
+      m[q] += step[q];
+      if (m[q] >= period) m[q] -= period;
     }
   }
-  // the lanes' sums, each s - c, are added as pairs too (TwoSum): rho_j carries one rounding of a sum
-  double e = -c;
-  auto pair_sum = [&](double s2, double e2) {
-    const double t = s + s2, z = t - s;
-    e = (e + e2) + ((s - (t - z)) + (s2 - z));
-    s = t;
+  e[0] = -e[0];  // the sums are s + e
+  e[1] = -e[1];
+  // (s, e)[q] += (s2, e2) with the rounding error of s + s2 (TwoSum): rho_j carries one rounding of a sum
+  auto add = [&](int q, double s2, double e2) {
+    const double t = s[q] + s2, z = t - s[q];
+    e[q] = (e[q] + e2) + ((s[q] - (t - z)) + (s2 - z));
+    s[q] = t;
   };
-  for (int o = S / 2; o >= 2; o >>= 1) pair_sum(__shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, e, o));
-  // lane 0 holds the even part, lane 1 the odd part
-  const double so = __shfl_xor_sync(0xffffffffu, s, 1), eo = __shfl_xor_sync(0xffffffffu, e, 1);
-  if (r == 1) {
-    s = -s;
-    e = -e;
+  // lanes o apart add their sums; the first exchange leaves each with one of the two pairs
+  int o = S / 2, pair = 2 * group;
+  if (o >= 2) {
+    const bool up = (r & o) != 0;
+    const double s2 = __shfl_xor_sync(0xffffffffu, up ? s[0] : s[1], o), e2 = __shfl_xor_sync(0xffffffffu, up ? e[0] : e[1], o);
+    if (up) {
+      s[0] = s[1];
+      e[0] = e[1];
+      ++pair;
+    }
+    add(0, s2, e2);
+    o >>= 1;
   }
-  pair_sum(so, eo);
-  if (j < M / 2 && r < 2) {
-    const int node = r == 0 ? j : M - 1 - j;
-    b.node[node] = make_double2(node_energy(node, M, job.emin, job.emax), (s + e) / M);
+  for (; o >= 2; o >>= 1) add(0, __shfl_xor_sync(0xffffffffu, s[0], o), __shfl_xor_sync(0xffffffffu, e[0], o));
+  // an even lane holds the even part, the next the odd part; of those that hold the same pair one writes
+  const bool writes = S == 2 || (r & ~1 & (S / 2 - 1)) == 0;
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    if (q && S > 2) break;
+    const double so = __shfl_xor_sync(0xffffffffu, s[q], 1), eo = __shfl_xor_sync(0xffffffffu, e[q], 1);
+    if (r & 1) {
+      s[q] = -s[q];
+      e[q] = -e[q];
+    }
+    add(q, so, eo);
+    const int j = pair + q, node = r & 1 ? M - 1 - j : j;
+    if (j < M / 2 && writes)
+      b.node[node] = make_double2(node_energy(node, M, job.emin, job.emax), (s[q] + e[q]) / M);
   }
 }
 
@@ -171,7 +208,8 @@ __device__ __forceinline__ double count_occupation(double e, double mu, double i
 // wait expired.  The midpoints of the next `depth` halvings (nm = 2^depth - 1 of them) are evaluated
 // at once, each by `parts` CTAs, and the halvings are then decided in order, so mu is the plain
 // bisection's; one barrier for `depth` halvings.  N(mu) is summed as FERMI_LANES strided chains and
-// a tree over them whatever the launch, so mu does not depend on it.  Latency binds: an FP64 operation
+// a tree over them whatever the launch, and the observables over fixed runs of nodes, so that the results of a
+// problem do not depend on the launch.  Latency binds: an FP64 operation
 // takes ~85 cycles and an occupation ~40 of them (45 halvings one after the other in one CTA: 0.65 ms
 // at M = 504, 9.2 ms at M = 9904; this form 0.084 and 0.119 ms, of which the sums over 32 parts and the
 // decisions were 0.02 and 0.05 more with every warp of every CTA at them).
@@ -294,25 +332,30 @@ fermi_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int depth, i
     }
     mu = 0.5 * (lo + hi);
   }
-  double v[3] = {0.0, 0.0, 0.0};
-  for (int j = cta * blockDim.x + threadIdx.x; j < M; j += ncta * blockDim.x) {
-    const double2 n = __ldg(b.node + j);
-    const double f = fermi_fn(n.x, mu, kT);
-    v[0] += free_fn(n.x, mu, kT) * n.y;
-    v[1] += n.x * f * n.y;
-    v[2] += f * n.y;
-  }
+  // observables: runs of FERMI_THREADS nodes, of which a CTA takes every ncta-th; their number, and so the
+  // order of the sums, follows from M alone
+  const int runs = min((M + FERMI_THREADS - 1) / FERMI_THREADS, FERMI_PART / 3);
   double* part = b.part + (phase & 1) * FERMI_PART;
-  for (int q = 0; q < 3; ++q) {
-    const double t = tbk_block_sum(v[q], red);
-    if (threadIdx.x == 0) __stcg(part + 3 * cta + q, t);
+  for (int g = cta; g < runs; g += ncta) {
+    double v[3] = {0.0, 0.0, 0.0};
+    for (int j = g * FERMI_THREADS + tid; j < M; j += runs * FERMI_THREADS) {
+      const double2 n = __ldg(b.node + j);
+      const double f = fermi_fn(n.x, mu, kT);
+      v[0] += free_fn(n.x, mu, kT) * n.y;
+      v[1] += n.x * f * n.y;
+      v[2] += f * n.y;
+    }
+    for (int q = 0; q < 3; ++q) {
+      const double t = tbk_block_sum(v[q], red);
+      if (tid == 0) __stcg(part + 3 * g + q, t);
+    }
   }
   if (ncta > 1) ok = ok && tbk_grid_wait(b.ctr, (unsigned)(ncta * (phase + 1)));
   else __syncthreads();
   if (cta == 0 && tid < 96) {
     const int q = tid >> 5, lane = tid & 31;
     double t = 0.0;
-    for (int i = lane; i < ncta; i += 32) t += __ldcg(part + 3 * i + q);
+    for (int i = lane; i < runs; i += 32) t += __ldcg(part + 3 * i + q);
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     if (lane == 0) out[1 + q] = t;
     if (tid == 0) {
@@ -331,10 +374,10 @@ static void fermi_launch(tbk_ctx* ctx, int n, const FermiJob& one, const FermiJo
   fermi_setup<<<dim3(ceil_div(std::max(4 * (int64_t)M_max, (int64_t)p_max), 256), n), 256, 0, ctx->stream>>>(
       one, d_jobs, moments, damping, buf);
   post_launch(ctx, "fermi_setup");
-  // lanes per pair of nodes: about eight warps per SM over all problems
-  int S = 2;
-  while (S < 32 && (int64_t)n * (M_max / 2) * S < (int64_t)ctx->num_sms * 256) S *= 2;
-  rho_kernel<<<dim3(ceil_div((int64_t)(M_max / 2) * S, 64), n), 64, 0, ctx->stream>>>(one, d_jobs, S, buf);
+  // lanes of a problem: about eight warps per SM (the largest has fewer than twice that, or two per group)
+  const int lanes = ctx->num_sms * 256, groups = rho_groups(M_max);
+  const int64_t most = std::max<int64_t>(std::min<int64_t>((int64_t)groups * 32, 2 * (int64_t)lanes), 2 * (int64_t)groups);
+  rho_kernel<<<dim3(ceil_div(most, 32), n), 32, 0, ctx->stream>>>(one, d_jobs, lanes, buf);
   post_launch(ctx, "rho_kernel");
   // CTAs per problem, as long as all problems fit the chip together: as many midpoints at once as
   // there is room for, then 4 to 16 CTAs per midpoint (one CTA per problem takes its midpoints one by
