@@ -19,6 +19,7 @@
 #include "cheb.cuh"
 #include "model.cuh"
 #include "sk.cuh"
+#include "sums.cuh"
 
 namespace tbk {
 
@@ -62,32 +63,50 @@ sddmm_one(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __res
   if (lane == 0) Gacc[k] += w * v;
 }
 
-// v[32] FP32 lane values -> lane e holds the lane sum of entry e as hi + lo (to ~2^-47): a butterfly
-// whose additions keep their rounding errors (TwoSum).  FP64 additions take 64 cycles of an SM quarter.
-__device__ __forceinline__ void butterfly32_pair(float (&v)[32], int lane, float& hi, float& lo) {
-  float e[16];
+__device__ __forceinline__ float2 shfl_xor2(float2 v, int off) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, off), __shfl_xor_sync(0xffffffffu, v.y, off));
+}
+// Lane values of 2 N entries, (2 p, 2 p + 1) in v[p] -> the lanes' sum of entry e in each lane with e in its lowest
+// bits: a butterfly reduce-scatter, each addition with its rounding errors.  FP64 additions take 64 cycles of an
+// SM quarter.  EXACT: two floats hold each value, the third is zero.
+template <bool EXACT = false, int N>
+__device__ __forceinline__ double butterfly_sum3(Sum3 (&v)[N], int lane) {
 #pragma unroll
-  for (int off = 16, n = 32; off >= 1; off >>= 1, n >>= 1) {
+  for (int n = N / 2; n >= 1; n >>= 1) {
+    const int off = 2 * n;
     const bool up = (lane & off) != 0;
 #pragma unroll
-    for (int k = 0; k < n / 2; ++k) {
-      const float a = up ? v[k + n / 2] : v[k];
-      const float b = __shfl_xor_sync(0xffffffffu, up ? v[k] : v[k + n / 2], off);
-      float c = 0.f;
-      if (n < 32) c = (up ? e[k + n / 2] : e[k]) + __shfl_xor_sync(0xffffffffu, up ? e[k] : e[k + n / 2], off);
-      const float t = __fadd_rn(a, b);
-      const float z = __fsub_rn(t, a);
-      const float err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
-      v[k] = t;
-      e[k] = n < 32 ? __fadd_rn(c, err) : err;
+    for (int p = 0; p < n; ++p) {
+      const Sum3 give = up ? v[p] : v[p + n];
+      if (up) v[p] = v[p + n];
+      sum3_add(v[p], {shfl_xor2(give.h, off), shfl_xor2(give.m, off),
+                      EXACT && n == N / 2 ? make_float2(0.f, 0.f) : shfl_xor2(give.l, off)});
     }
   }
-  hi = v[0];
-  lo = e[0];
+  const bool odd = (lane & 1) != 0;
+  auto mine = [&](float2 u) { return make_float2(odd ? u.y : u.x, 0.f); };
+  auto other = [&](float2 u) { return make_float2(__shfl_xor_sync(0xffffffffu, odd ? u.x : u.y, 1), 0.f); };
+  Sum3 t = {mine(v[0].h), mine(v[0].m), mine(v[0].l)};
+  sum3_add(t, {other(v[0].h), other(v[0].m), other(v[0].l)});
+  return sum3_value(t.h.x, t.m.x, t.l.x);
+}
+// The same of 32 entries in floats: after one exchange two floats hold each sum exactly.
+__device__ __forceinline__ double butterfly32_sum3(const float2 (&v)[16], int lane) {
+  Sum3 t[8];
+  const bool up = (lane & 16) != 0;
+#pragma unroll
+  for (int p = 0; p < 8; ++p) {
+    t[p].h = up ? v[p + 8] : v[p];
+    two_sum(t[p].h, t[p].m, shfl_xor2(up ? v[p] : v[p + 8], 16));
+    t[p].l = make_float2(0.f, 0.f);
+  }
+  return butterfly_sum3<true>(t, lane);
 }
 
 // FP32 9x9 blocks: a warp takes three rows of a block, a lane probes lane, lane + 32, ... with 27 sums,
-// the next 32 probes loaded ahead.  333 atoms x 100 probes: 18 us against 233 for one warp per block that
+// the next 32 probes loaded ahead.  The lanes' sums are kept in three floats: in two, 47 bits for the 53 of an FP64
+// sum, the calls below are 7 % faster at 1,000 atoms x 100 probes and 2 % at 333 x 384.  333 atoms x 100 probes:
+// 18 us (of two floats) against 233 for one warp per block that
 // loaded as it went and added 81 FP64 butterflies (26 with all 81 sums in a warp, 12 warps per SM; 28 to
 // 32 with a thread per entry and the tiles in shared memory, whose bandwidth then binds).
 __global__ void __launch_bounds__(128, 5)
@@ -127,11 +146,11 @@ sddmm_rows32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __
     fetch(p + 64, yv, xv);
     add(yn, xn);
   }
-  float v[32], hi, lo;
+  float2 v[16];
 #pragma unroll
-  for (int e = 0; e < 32; ++e) v[e] = e < 27 ? acc[e] : 0.f;
-  butterfly32_pair(v, lane, hi, lo);
-  if (lane < 27) atomicAdd(Gacc + (int64_t)k * 81 + 27 * g + lane, w * ((double)hi + (double)lo));
+  for (int p = 0; p < 16; ++p) v[p] = make_float2(p < 14 ? acc[2 * p] : 0.f, p < 13 ? acc[2 * p + 1] : 0.f);
+  const double sum = butterfly32_sum3(v, lane);
+  if (lane < 27) atomicAdd(Gacc + (int64_t)k * 81 + 27 * g + lane, w * sum);
 }
 
 constexpr int OUT_STEPS = 64;  // steps per launch at most
@@ -140,17 +159,12 @@ struct OuterPanels {
   const float* x[OUT_STEPS];  // ybar_{k+1} (or b_{k+1})
 };
 
-// hi + lo += a, the rounding error of the addition kept in lo.
-__device__ __forceinline__ void pair_add(float& hi, float& lo, float a) {
-  const float t = __fadd_rn(hi, a), z = __fsub_rn(t, hi);
-  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(a, z)));
-  hi = t;
-}
-
 // The same for several steps after them, as long as their panels stay in L2: a lane adds its 27 sums of each
-// step to pairs (7 operations an entry where the butterfly takes 14), and one butterfly per launch adds the
-// pairs of the lanes.  A CTA is one block, so that its three warps find x in L1.  333 atoms x 100 probes: 14.6
-// us a step against 18; the loads' latency (12 warps per SM) and 630 instructions a step bind.
+// step to sums of three floats (13 packed operations for two entries), and one butterfly per launch adds those of
+// the lanes.  A CTA is one block, so that its three warps find x in L1.  The loads' latency (12 warps per SM) and
+// about 600 instructions a step bind; 168 registers are the limit, so that loads go 64 probes ahead (128: spills) and
+// row offsets are formed on the way.  A whole call, us per order, 333 atoms x 100 probes: 32.8 (31.8 with sums of
+// two floats, 37.1 with loads 128 ahead); launch by launch 34.0.
 __global__ void __launch_bounds__(96, 4)
 sddmm_steps32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t nnzb,
               const __grid_constant__ OuterPanels wp, int nt, int last_is_y0, int s, double* __restrict__ Gacc) {
@@ -161,14 +175,11 @@ sddmm_steps32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* _
   const int k = (int)(gw / 3), g = (int)(gw - 3 * (int64_t)k);
   const int b = __ldg(col + k), a = row_of_block(row_ptr, n_atoms, k, lane);
   // byte offsets of the rows (panels of a window are a few MB), so that a load needs no 64-bit arithmetic
-  uint32_t oy[3], ox[9];
+  const uint32_t oy = 4u * ((9u * a + 3u * g) * s + lane), ox = 4u * (9u * b * s + lane), row = 4u * s;
+  float acc[27], yv[2][3], xv[2][9];  // 64 probes ahead: with 128, spills take more than the latency
+  Sum3 sum[16];
 #pragma unroll
-  for (int i = 0; i < 3; ++i) oy[i] = 4u * ((9u * a + 3u * g + i) * s + lane);
-#pragma unroll
-  for (int l = 0; l < 9; ++l) ox[l] = 4u * ((9u * b + l) * s + lane);
-  float acc[27], hi[32], lo[32], yv[4][3], xv[4][9];  // 128 probes ahead
-#pragma unroll
-  for (int e = 0; e < 32; ++e) hi[e] = lo[e] = 0.f;
+  for (int p = 0; p < 16; ++p) sum[p].h = sum[p].m = sum[p].l = make_float2(0.f, 0.f);
   // probes p0 + 32 c + lane of step t; past the last probe zeros, which leave the sums as they are
   auto fetch = [&](int t, int p0, int c) {
     const char* Y = reinterpret_cast<const char*>(wp.y[t] + p0) + 128 * c;
@@ -176,28 +187,28 @@ sddmm_steps32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* _
     auto at = [](const char* p, uint32_t o) { return __ldg(reinterpret_cast<const float*>(p + o)); };
     if (p0 + 32 * c + 32 <= s) {
 #pragma unroll
-      for (int i = 0; i < 3; ++i) yv[c][i] = at(Y, oy[i]);
+      for (int i = 0; i < 3; ++i) yv[c][i] = at(Y, oy + i * row);
 #pragma unroll
-      for (int l = 0; l < 9; ++l) xv[c][l] = at(X, ox[l]);
+      for (int l = 0; l < 9; ++l) xv[c][l] = at(X, ox + l * row);
     } else {
       const bool in = p0 + 32 * c + lane < s;
 #pragma unroll
-      for (int i = 0; i < 3; ++i) yv[c][i] = in ? at(Y, oy[i]) : 0.f;
+      for (int i = 0; i < 3; ++i) yv[c][i] = in ? at(Y, oy + i * row) : 0.f;
 #pragma unroll
-      for (int l = 0; l < 9; ++l) xv[c][l] = in ? at(X, ox[l]) : 0.f;
+      for (int l = 0; l < 9; ++l) xv[c][l] = in ? at(X, ox + l * row) : 0.f;
     }
   };
 #pragma unroll
-  for (int c = 0; c < 4; ++c)
+  for (int c = 0; c < 2; ++c)
     if (32 * c < s) fetch(0, 0, c);
   for (int t = 0; t < nt; ++t) {
 #pragma unroll
     for (int e = 0; e < 27; ++e) acc[e] = 0.f;
-    for (int p0 = 0; p0 < s; p0 += 128) {
-      const bool more = p0 + 128 < s;
-      const int tn = more ? t : t + 1, pn = more ? p0 + 128 : 0;
+    for (int p0 = 0; p0 < s; p0 += 64) {
+      const bool more = p0 + 64 < s;
+      const int tn = more ? t : t + 1, pn = more ? p0 + 64 : 0;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
+      for (int c = 0; c < 2; ++c) {
         if (p0 + 32 * c < s)
 #pragma unroll
           for (int i = 0; i < 3; ++i)
@@ -206,25 +217,16 @@ sddmm_steps32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* _
         if (tn < nt && pn + 32 * c < s) fetch(tn, pn, c);
       }
     }
-    // the weight 2 is exact at any point: pairs hold half of what the launch adds, and y_0 enters with half
-    const float w = last_is_y0 && t == nt - 1 ? 0.5f : 1.f;
+    // the weight 2 is exact at any point: the sums hold half of what the launch adds, and y_0 enters with half
+    if (last_is_y0 && t == nt - 1) {
 #pragma unroll
-    for (int e = 0; e < 27; ++e) pair_add(hi[e], lo[e], w * acc[e]);
-  }
-  // lane e: the lanes' sum of entry e
-#pragma unroll
-  for (int off = 16, n = 32; off >= 1; off >>= 1, n >>= 1) {
-    const bool up = (lane & off) != 0;
-#pragma unroll
-    for (int e = 0; e < n / 2; ++e) {
-      const float x = __shfl_xor_sync(0xffffffffu, up ? hi[e] : hi[e + n / 2], off);
-      const float c = __shfl_xor_sync(0xffffffffu, up ? lo[e] : lo[e + n / 2], off);
-      hi[e] = up ? hi[e + n / 2] : hi[e];
-      lo[e] = __fadd_rn(up ? lo[e + n / 2] : lo[e], c);
-      pair_add(hi[e], lo[e], x);
+      for (int e = 0; e < 27; ++e) acc[e] *= 0.5f;
     }
+#pragma unroll
+    for (int p = 0; p < 14; ++p) sum3_add(sum[p], make_float2(acc[2 * p], p < 13 ? acc[2 * p + 1] : 0.f));
   }
-  if (lane < 27) atomicAdd(Gacc + (int64_t)k * 81 + 27 * g + lane, 2.0 * ((double)hi[0] + (double)lo[0]));
+  const double v = butterfly_sum3(sum, lane);
+  if (lane < 27) atomicAdd(Gacc + (int64_t)k * 81 + 27 * g + lane, 2.0 * v);
 }
 
 // FP64 9x9 blocks: a warp takes a block, 27 of its lanes three entries each over all probes (no sums
