@@ -5,6 +5,7 @@
 
 #include "bulk.cuh"
 #include "cheb.cuh"
+#include "sums.cuh"
 
 namespace tbk {
 
@@ -661,7 +662,9 @@ cheb_step_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
       sd = __ldg(batch.seed + cl);
       rloc = (int64_t)9 * (a - __ldg(batch.atom0 + cl));
     }
-    float cs0 = 0.f, cc0 = 0.f, cs1 = 0.f, cc1 = 0.f;  // the task's compensated partial sums
+    // the task's partial sums, compensated; of narrow tasks in three floats, as good as the plain kernel's FP64 sums
+    float cs0 = 0.f, cc0 = 0.f, cs1 = 0.f, cc1 = 0.f;
+    Sum3 cs = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
       const int64_t row = (int64_t)9 * a + i;
@@ -696,13 +699,17 @@ cheb_step_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
           q0 = fmaf(yo[v], xin[v], q0);
           q1 = fmaf(yo[v], yo[v], q1);
         }
-        two_sum_acc(cs0, cc0, q0);
-        two_sum_acc(cs1, cc1, q1);
+        if constexpr (NARROW) {
+          sum3_add(cs, make_float2(q0, q1));
+        } else {
+          two_sum_acc(cs0, cc0, q0);
+          two_sum_acc(cs1, cc1, q1);
+        }
       }
     }
     if (partials) {
-      sum0 += (double)cs0 + (double)cc0;
-      sum1 += (double)cs1 + (double)cc1;
+      sum0 += NARROW ? sum3_value(cs.h.x, cs.m.x, cs.l.x) : (double)cs0 + (double)cc0;
+      sum1 += NARROW ? sum3_value(cs.h.y, cs.m.y, cs.l.y) : (double)cs1 + (double)cc1;
     }
     if (per_task && partials) {
       for (int o = 16; o > 0; o >>= 1) {
@@ -854,7 +861,8 @@ cheb_step_lane(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
   const int pl = 32 * warp + lane;  // this lane's probe in the chunk
   // items of the epilogue: row irow[j], probes 4 igrp .. 4 igrp + 3 of the warp's 32
   const int igrp = lane & 7, irow = lane >> 3;  // item j: row irow + 4 j, j < 3
-  float cs0 = 0.f, cc0 = 0.f, cs1 = 0.f, cc1 = 0.f;  // compensated partial sums
+  // partial sums of all tasks of the CTA, in three floats: as good as the FP64 sums of the plain kernel
+  Sum3 cs = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
   int st = 0, ph = 0;
   bool ok = true;
   for (int task = blockIdx.x; task < n_tasks && ok; task += gridDim.x) {
@@ -948,14 +956,14 @@ cheb_step_lane(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
           q0 = fmaf(yo[v], xin[v], q0);
           q1 = fmaf(yo[v], yo[v], q1);
         }
-        two_sum_acc(cs0, cc0, q0);
-        two_sum_acc(cs1, cc1, q1);
+        sum3_add(cs, make_float2(q0, q1));
       }
     }
     __syncwarp();  // the buffer is free again
   }
   if (!ok) atomicOr(err, 2);
-  if (!ADJ && partials) step_partials(partials, (double)cs0 + (double)cc0, (double)cs1 + (double)cc1, warp, lane, nw);
+  if (!ADJ && partials)
+    step_partials(partials, sum3_value(cs.h.x, cs.m.x, cs.l.x), sum3_value(cs.h.y, cs.m.y, cs.l.y), warp, lane, nw);
 }
 
 // ---- FP64 step by rows -------------------------------------------------------------------------------
