@@ -130,6 +130,10 @@ int tbk_test_stall_next_step(tbk_ctx* ctx);
    up after 2 s, the adjoint call returns TBK_ERR_TIMEOUT, and the context stays usable.  Host-side
    only. */
 int tbk_test_stall_next_adjoint(tbk_ctx* ctx);
+/* Test of the launch geometry: n_ctas (host) receives the CTAs of a recurrence step of tbk_chebyshev_probe_moments
+   with these arguments.  Of H the sizes are read; nothing is launched.  Host-side only. */
+int tbk_test_step_grid(tbk_ctx* ctx, const tbk_bsr* H, int32_t n_probes, int32_t order, int32_t flags,
+                       int32_t* n_ctas);
 
 /* tbk_autotune: time, on this operator (9x9 blocks, mixed precision) with n_probes a multiple
    of 128, the probe chunk (128, 256 or 512 probes) per task of the TMA-fed recurrence step and

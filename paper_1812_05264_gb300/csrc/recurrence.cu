@@ -1122,13 +1122,17 @@ static Occ& occ_cache(int dev) {
   return o[dev < 0 || dev >= 64 ? 0 : dev];
 }
 
-template <typename T, int B>
-static dim3 simple_block(int s) {
-  constexpr int VEC = Vec16<T>::N;
-  const int lanes_needed = (s + VEC - 1) / VEC;
+// Block of the plain kernel: `vec` probes per lane, rows in y.
+static dim3 simple_block(int s, int vec) {
+  const int lanes_needed = (s + vec - 1) / vec;
   int lanes = 1;  // a power of two, so that every warp of the CTA is complete
   while (lanes < lanes_needed && lanes < STEP_THREADS) lanes <<= 1;
   return dim3(lanes, STEP_THREADS / lanes);
+}
+static int64_t simple_tasks(const HOp& op, int s) {
+  const int vec = op.prec == TBK_MIXED ? Vec16<float>::N : Vec16<double>::N;
+  const dim3 b = simple_block(s, vec);
+  return (int64_t)ceil_div(op.n_atoms, b.y) * ceil_div(s, b.x * vec);
 }
 
 bool tc_eligible(const HOp& op, int s);
@@ -1189,18 +1193,22 @@ static bool dense_bulk(const tbk_ctx* ctx, const HOp& op, int s, int cw) {
 
 int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s, int K, bool resident) {
   const Occ& o = occupancies(ctx);
-  // every kernel loops over its tasks and none waits on another CTA, so any grid will do; the
-  // tensor-core step and the plain kernel run on the resident one (CTAs that set up their TMEM once; fewer tasks)
+  // every kernel loops over its tasks and none waits on another CTA, so any grid will do
+  const int cw = chosen_cw(ctx, op, s, 0);
+  if (resident) {
+    // the tensor-core step (CTAs that set up their TMEM once) and the plain kernel, as many as fit
+    const int64_t held = (int64_t)(cw && o.bulk[cw] > 0 ? o.bulk[cw] : o.simple) * ctx->num_sms;
+    return (int)std::min(held, std::max(simple_tasks(op, s), cw ? (int64_t)op.n_atoms * (s / 128) : 0));
+  }
   if (use_rows64(op))
     return (int)std::min<int64_t>((fp64_units(op, s, fp64_rows(ctx, op, s)) + 3) / 4, 4 * ctx->num_sms);
   if (use_lane(op, s))
     return (int)std::min<int64_t>((int64_t)op.n_atoms * ((s + 511) / 512), (int64_t)std::max(1, o.lane[lane_class(s)]) * ctx->num_sms);
-  const int cw = chosen_cw(ctx, op, s, 0);
   const bool narrow = op.prec == TBK_MIXED && op.B == 9 && s < 128;
+  if (!cw && !narrow) return (int)std::min((int64_t)o.simple * ctx->num_sms, simple_tasks(op, s));
   const int fed = cw && dense_bulk(ctx, op, s, cw) ? o.dense : (cw ? o.bulk[cw] : 0);
   const int per_sm = narrow && o.bulk[1] > 0 ? o.bulk[1] : (fed > 0 ? fed : o.simple);
   const int64_t tasks = cw ? (int64_t)op.n_atoms * (s / (128 * cw)) : op.n_atoms, held = (int64_t)per_sm * ctx->num_sms;
-  if (resident || (!cw && !narrow)) return (int)std::max<int64_t>(1, std::min(held, tasks));
   // at most 256 MB of partial sums
   return (int)std::min<int64_t>(task_grid(tasks, held), std::max<int64_t>(held, ((int64_t)1 << 24) / std::max(1, K)));
 }
@@ -1217,7 +1225,7 @@ static StepSources<T> sources(const StepArgs& a) {
 
 template <typename T, int B>
 static void launch_simple(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
-  const dim3 blk = simple_block<T, B>(a.s);
+  const dim3 blk = simple_block(a.s, Vec16<T>::N);
   const T* hv = (const T*)op.hv;
   if (a.cur_is_probe)
     cheb_step_kernel<T, B, true><<<G, blk, 0, ctx->stream>>>(
@@ -1787,5 +1795,23 @@ extern "C" int tbk_chebyshev_probe_moments(tbk_ctx* ctx, const tbk_bsr* H, doubl
   double* mom = moments;
   if (!mom) mom = (double*)scratch(ctx, WS_COEF, sizeof(double) * (size_t)std::max(1, order));
   moments_sweep(ctx, H, emin, emax, probe_seed, n_probes, order, flags, mom, per_probe);
+  TBK_API_END
+}
+
+extern "C" int tbk_test_step_grid(tbk_ctx* ctx, const tbk_bsr* H, int32_t n_probes, int32_t order, int32_t flags,
+                                  int32_t* n_ctas) {
+  TBK_API_BEGIN
+  TBK_CHECK_ARG(ctx != nullptr && H != nullptr && n_ctas != nullptr, "NULL argument");
+  TBK_CHECK_ARG(H->n_orb == 1 || H->n_orb == 9, "n_orb must be 1 or 9");
+  TBK_CHECK_ARG(H->n_atoms >= 1 && order >= 1 && n_probes >= 4 && n_probes % 4 == 0, "bad size");
+  DeviceGuard dg(ctx);
+  HOp op;
+  op.B = H->n_orb;
+  op.prec = (flags & TBK_FP64) ? TBK_FP64 : TBK_MIXED;
+  op.n_atoms = H->n_atoms;
+  op.n_rows = (int64_t)H->n_atoms * H->n_orb;
+  op.nnzb = H->nnzb;
+  *n_ctas = step_grid_ctas(ctx, op, n_probes, (flags & TBK_MOMENTS_DIRECT) ? order - 1 : order / 2,
+                           (flags & (TBK_TENSOR_CORES | TBK_PLAIN_KERNEL)) != 0);
   TBK_API_END
 }
