@@ -134,7 +134,9 @@ struct StepSources {
   T c[3];
 };
 
-template <typename T, int B, bool PROBE_IN>
+// SRC: with the further own-row terms.  Where none is asked for, the tests for them alone made FP64 steps of 1x1
+// blocks, whose rows are short, 20 % slower (10,648 sites x 512 probes 138 -> 166 us).
+template <typename T, int B, bool PROBE_IN, bool SRC>
 __global__ void __launch_bounds__(STEP_THREADS)
 cheb_step_kernel(const int n_atoms, const int32_t* __restrict__ row_ptr,
                  const int32_t* __restrict__ col, const T* __restrict__ hv,
@@ -223,14 +225,16 @@ cheb_step_kernel(const int n_atoms, const int32_t* __restrict__ row_ptr,
 #pragma unroll
           for (int v = 0; v < VEC; ++v) yo[v] -= t[v];
         }
+        if constexpr (SRC) {
 #pragma unroll
-        for (int e = 0; e < 3; ++e)
-          if (src.p[e]) {
-            T t[VEC];
-            ldg16(src.p[e] + off, t);
+          for (int e = 0; e < 3; ++e)
+            if (src.p[e]) {
+              T t[VEC];
+              ldg16(src.p[e] + off, t);
 #pragma unroll
-            for (int v = 0; v < VEC; ++v) yo[v] = fma(src.c[e], t[v], yo[v]);
-          }
+              for (int v = 0; v < VEC; ++v) yo[v] = fma(src.c[e], t[v], yo[v]);
+            }
+        }
         st16(yout + off, yo);
         if (partials) {
           T xin[VEC];
@@ -1053,7 +1057,7 @@ cheb_step_fp64(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
 template <typename T, int B, bool P>
 static int occupancy_simple() {
   int n = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cheb_step_kernel<T, B, P>, STEP_THREADS, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cheb_step_kernel<T, B, P, false>, STEP_THREADS, 0);
   return n > 0 ? n : 1;
 }
 
@@ -1227,14 +1231,16 @@ template <typename T, int B>
 static void launch_simple(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
   const dim3 blk = simple_block(a.s, Vec16<T>::N);
   const T* hv = (const T*)op.hv;
-  if (a.cur_is_probe)
-    cheb_step_kernel<T, B, true><<<G, blk, 0, ctx->stream>>>(
-        op.n_atoms, op.row_ptr, op.col, hv, (const T*)a.yin, (const T*)a.yprev, (T*)a.yout, (T)a.alpha,
-        (T)a.c_r, a.seed, a.s, a.direct, sources<T>(a), a.partials);
-  else
-    cheb_step_kernel<T, B, false><<<G, blk, 0, ctx->stream>>>(
-        op.n_atoms, op.row_ptr, op.col, hv, (const T*)a.yin, (const T*)a.yprev, (T*)a.yout, (T)a.alpha,
-        (T)a.c_r, a.seed, a.s, a.direct, sources<T>(a), a.partials);
+  auto go = [&](auto kernel) {
+    kernel<<<G, blk, 0, ctx->stream>>>(op.n_atoms, op.row_ptr, op.col, hv, (const T*)a.yin, (const T*)a.yprev, (T*)a.yout,
+                                       (T)a.alpha, (T)a.c_r, a.seed, a.s, a.direct, sources<T>(a), a.partials);
+  };
+  if (a.src[0] || a.src[1] || a.src[2]) {
+    // the FP64 adjoint of 1x1 operators; other kernels take the other ones
+    TBK_CHECK_ARG((sizeof(T) == 8 && B == 1), "a plain step with further own-row terms");
+    if constexpr (sizeof(T) == 8 && B == 1) go(cheb_step_kernel<T, B, false, true>);
+  } else if (a.cur_is_probe) go(cheb_step_kernel<T, B, true, false>);
+  else go(cheb_step_kernel<T, B, false, false>);
   post_launch(ctx, "cheb_step_kernel");
 }
 
