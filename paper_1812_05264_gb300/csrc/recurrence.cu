@@ -2,6 +2,7 @@
 // partial sums (Sec. II.B.1 Eq. poly_PQ with S = I; Sec. II.C.2 random approximation).
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 
 #include "bulk.cuh"
 #include "cheb.cuh"
@@ -1121,11 +1122,6 @@ struct Occ {
   int simple = 0, bulk[5] = {0, 0, 0, 0, 0}, dense = 0, lane[3] = {0, 0, 0};
 };
 
-static Occ& occ_cache(int dev) {
-  static Occ o[64];
-  return o[dev < 0 || dev >= 64 ? 0 : dev];
-}
-
 // Block of the plain kernel: `vec` probes per lane, rows in y.
 static dim3 simple_block(int s, int vec) {
   const int lanes_needed = (s + vec - 1) / vec;
@@ -1145,9 +1141,14 @@ void launch_step_tc(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G);
 
 static int lane_class(int s);
 
-static Occ& occupancies(tbk_ctx* ctx) {
-  Occ& o = occ_cache(ctx->device);
-  if (!o.simple) {
+// CTAs per SM of the step kernels on the context's device; the first call also sets their shared-memory limits.
+// Nobody sees a device's numbers before all of them are there: contexts of several threads may come at once.
+static const Occ& occupancies(const tbk_ctx* ctx) {
+  static Occ occ[64];
+  static std::once_flag once[64];
+  const int dev = ctx->device < 0 || ctx->device >= 64 ? 0 : ctx->device;
+  std::call_once(once[dev], [&] {
+    Occ& o = occ[dev];
     int m = 1 << 30;
     m = std::min(m, std::min(occupancy_simple<float, 9, false>(), occupancy_simple<float, 9, true>()));
     m = std::min(m, std::min(occupancy_simple<float, 1, false>(), occupancy_simple<float, 1, true>()));
@@ -1161,8 +1162,8 @@ static Occ& occupancies(tbk_ctx* ctx) {
     o.lane[0] = occupancy_lane<4>();
     o.lane[1] = occupancy_lane<8>();
     o.lane[2] = occupancy_lane<16>();
-  }
-  return o;
+  });
+  return occ[dev];
 }
 
 // FP32 steps that the one-probe-per-lane kernel takes: few tiles for the chip, or a width between 128
@@ -1324,9 +1325,9 @@ void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
     return;
   }
   const int cw = chosen_cw(ctx, op, a.s, a.per_task);
-  if (cw && !a.cur_is_probe && a.err && !a.force_simple && occ_cache(ctx->device).bulk[cw] > 0) {
+  if (cw && !a.cur_is_probe && a.err && !a.force_simple && occupancies(ctx).bulk[cw] > 0) {
     if (cw == 4) launch_bulk<4>(ctx, op, a, G);
-    else if (cw == 2 && dense_bulk(ctx, op, a.s, cw) && occ_cache(ctx->device).dense > 0) launch_bulk<2, true>(ctx, op, a, G);
+    else if (cw == 2 && dense_bulk(ctx, op, a.s, cw) && occupancies(ctx).dense > 0) launch_bulk<2, true>(ctx, op, a, G);
     else if (cw == 2) launch_bulk<2>(ctx, op, a, G);
     else launch_self<false>(ctx, op, a, G);
     return;
