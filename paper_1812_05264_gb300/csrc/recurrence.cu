@@ -1512,6 +1512,7 @@ __global__ void probe_moments_finish(const double* __restrict__ dots, int K, int
 constexpr int SWEEP_THREADS = 512;
 constexpr int64_t SWEEP_ROWS = 11000;                   // two panels in shared memory
 constexpr size_t SWEEP_PARTIALS = (size_t)256 << 20;    // bytes of partial sums
+constexpr int64_t SWEEP_SMEM = 220 << 10;
 
 __device__ __forceinline__ void store_cluster(double* p, int rank, double x) {
   uint32_t a;
@@ -1523,8 +1524,8 @@ __device__ __forceinline__ void cluster_barrier() {
 }
 
 // probe_panel: y_0, or NULL for the +-1 probes of the seed.  partials: two per warp and step.  cap: blocks of
-// the operator that fit in shared memory beside the panels (the cluster's barrier drops what L1 holds, so
-// blocks left in global memory come from L2 in every step; a share of the rows with more blocks does that).
+// the operator that fit in shared memory beside the panels; rows of a CTA's share beyond them stay in global memory
+// and come from L2 in every step (the cluster's barrier drops what L1 holds), a lane walking its own row.
 __global__ void __launch_bounds__(SWEEP_THREADS)
 moments_sweep_b1(int n, int C, int cap, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                  const double* __restrict__ hv, const double* __restrict__ probe_panel, uint64_t seed, int s, int K,
@@ -1541,8 +1542,8 @@ moments_sweep_b1(int n, int C, int cap, const int32_t* __restrict__ row_ptr, con
     ysm[i] = probe_panel ? probe_panel[(int64_t)i * s + probe] : (double)tbk_probe_sign(seed, i, probe);
   const int k0 = __ldg(row_ptr + r0), nz = __ldg(row_ptr + r0 + rows) - k0;
   for (int i = threadIdx.x; i <= rows; i += blockDim.x) rp[i] = __ldg(row_ptr + r0 + i) - k0;
-  const bool staged = nz <= cap;
-  for (int k = threadIdx.x; k < nz && staged; k += blockDim.x) {
+  const int staged = min(nz, cap);
+  for (int k = threadIdx.x; k < staged; k += blockDim.x) {
     hs[k] = __ldg(hv + k0 + k);
     cs[k] = __ldg(col + k0 + k);
   }
@@ -1554,7 +1555,7 @@ moments_sweep_b1(int n, int C, int cap, const int32_t* __restrict__ row_ptr, con
     for (int i = threadIdx.x; i < rows; i += blockDim.x) {
       double acc = 0.0;
       const int k1 = rp[i + 1];
-      if (staged) {
+      if (k1 <= staged) {
 #pragma unroll 4
         for (int k = rp[i]; k < k1; ++k) acc = fma(hs[k], in[cs[k]], acc);
       } else {
@@ -1588,9 +1589,22 @@ static int sweep_partials(const tbk_ctx* ctx, const HOp& op, int s) {
   return s * sweep_cluster(ctx, s) * sweep_warps(ctx, op, s);
 }
 
+// Blocks that fit beside the panels and the row pointers.
+static int64_t sweep_room(const HOp& op, int C) {
+  return (SWEEP_SMEM - 16 * op.n_rows - 4 * (op.n_rows / C + 2)) / 12 - 1;
+}
+
+// Short rows always (us a step, sweep against a launch each: 10,648 sites of 7 blocks x 4 probes 6.4 / 7.1, x 512 126 /
+// 138, although their blocks do not fit); longer ones where the blocks fit in shared memory (2,744 sites x 32 probes, 17
+// blocks a row 5.8 / 10.3, 23 blocks, beyond it, 20.4 / 12.4; 5,832 x 512 of 143 blocks 4,599 / 744) and the chip is
+// not full of FMAs anyway (216 sites x 512 probes, 36 blocks 17.5 / 18.6, 47 blocks 23.5 / 22.7; 1,000 x 512, 16
+// blocks 28.4 / 26.8).
 static bool use_sweep(const tbk_ctx* ctx, const HOp& op, int s, int K, int direct, const void* per_probe, int flags) {
-  return op.B == 1 && op.prec == TBK_FP64 && K >= 1 && !direct && !per_probe && !(flags & TBK_PLAIN_KERNEL) &&
-         op.n_rows <= SWEEP_ROWS && s <= 512 && 16 * (size_t)K * sweep_partials(ctx, op, s) <= SWEEP_PARTIALS;
+  if (op.B != 1 || op.prec != TBK_FP64 || K < 1 || direct || per_probe || (flags & TBK_PLAIN_KERNEL) ||
+      op.n_rows > SWEEP_ROWS || s > 512 || 16 * (size_t)K * sweep_partials(ctx, op, s) > SWEEP_PARTIALS)
+    return false;
+  const int C = sweep_cluster(ctx, s);
+  return op.nnzb <= 8 * op.n_rows || (op.nnzb <= C * sweep_room(op, C) && s * op.nnzb <= (int64_t)30000 * ctx->num_sms);
 }
 
 static void launch_sweep(tbk_ctx* ctx, const HOp& op, const void* probe_panel, uint64_t seed, int s, int K,
@@ -1598,10 +1612,9 @@ static void launch_sweep(tbk_ctx* ctx, const HOp& op, const void* probe_panel, u
   KernelTimerScope timer(ctx, TBK_KERNEL_STEP);
   const int C = sweep_cluster(ctx, s), n = (int)op.n_rows;
   // panels, row pointers, and a quarter more blocks than the average share
-  const int64_t fix = 16 * (int64_t)n + 4 * (n / C + 2), most = 220 << 10;
-  const int cap = (int)std::max<int64_t>(0, std::min((most - fix) / 12 - 1, op.nnzb / C * 5 / 4 + 32)) & ~1;
-  const size_t smem = fix + 12 * (size_t)cap;
-  TBK_CUDA(cudaFuncSetAttribute(moments_sweep_b1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+  const int cap = (int)std::max<int64_t>(0, std::min(sweep_room(op, C), op.nnzb / C * 5 / 4 + 32)) & ~1;
+  const size_t smem = 16 * (size_t)n + 4 * (n / C + 2) + 12 * (size_t)cap;
+  TBK_CUDA(cudaFuncSetAttribute(moments_sweep_b1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SWEEP_SMEM));
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(s * C);
   cfg.blockDim = dim3(32 * sweep_warps(ctx, op, s));

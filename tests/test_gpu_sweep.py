@@ -1,0 +1,50 @@
+"""FP64 moments of 1x1 operators with longer rows than the lattice's: all steps in one launch where the rule says
+so, some or all blocks of a share in shared memory, against a launch per step."""
+import pytest
+
+import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def _operator(ctx, size, r, ragged=False):
+    import torch
+    from paper_1812_05264_gb300 import api
+    g0 = torch.Generator().manual_seed(3)
+    pos = torch.as_tensor(wl.sc_disorder(L=size).positions, dtype=torch.float64)
+    if ragged:  # the last eighth of the sites closer together: their rows hold most of the blocks
+        pos[-len(pos) // 8:] *= 0.4
+    pos = pos.cuda()
+    g = api.build_neighbors(ctx, pos, r)
+    rows = torch.repeat_interleave(torch.arange(len(pos)), (g.row_ptr[1:] - g.row_ptr[:-1]).cpu())
+    cols = g.col.cpu().long()
+    # a symmetric value per pair, small beside the bounds of -9 .. 9
+    lo, hi = torch.minimum(rows, cols), torch.maximum(rows, cols)
+    val = (0.02 * torch.cos((lo * 7919 + hi * 104729).double()) + 2.0 * (lo == hi) * torch.rand(1, generator=g0).double())
+    return api.BSR(g, 1, val.reshape(-1, 1, 1).cuda())
+
+
+# FP64 rounding of the sums: 1e-12 of mu_0.  Blocks that fit with room, to the last, in part (ragged rows), and not
+@pytest.mark.parametrize("size,r,s,ragged", [(6, 2.5, 4, False), (6, 3.5, 4, False), (10, 2.5, 32, False),
+                                             (10, 3.0, 32, False), (10, 1.5, 512, False), (14, 1.5, 32, False),
+                                             (14, 1.8, 32, False), (18, 2.0, 4, False), (10, 2.0, 32, True),
+                                             (14, 1.2, 8, True), (22, 1.0, 64, True)])
+def test_moments_equal_the_steps(size, r, s, ragged):
+    from paper_1812_05264_gb300 import api
+    ctx = api.Context()
+    H = _operator(ctx, size, r, ragged)
+    got = api.chebyshev_moments(ctx, H, -9.0, 9.0, 5, s, 21, fp64=True)
+    ref = api.chebyshev_moments(ctx, H, -9.0, 9.0, 5, s, 21, fp64=True, plain=True)
+    assert (got - ref).abs().max().item() <= 1e-12 * size ** 3
+
+
+# launches of a call: one for all steps, or one each (11) and what prepares and finishes them
+@pytest.mark.parametrize("size,r,s,one", [(10, 1.0, 32, True), (22, 1.0, 512, True), (10, 2.5, 32, True),
+                                          (18, 2.0, 4, False), (14, 1.8, 32, False), (10, 1.5, 512, False)])
+def test_one_launch_where_the_blocks_fit(size, r, s, one):
+    from paper_1812_05264_gb300 import api
+    ctx = api.Context()
+    H = _operator(ctx, size, r)
+    n0 = ctx.launches
+    api.chebyshev_moments(ctx, H, -9.0, 9.0, 5, s, 23, fp64=True)
+    assert (ctx.launches - n0 < 8) == one
