@@ -473,10 +473,11 @@ int tbk_rational_density(tbk_ctx* ctx, const tbk_bsr* H, const tbk_model* model,
    memory while they run (latency-bounded loops where an allocation may block on the device,
    embedders whose device memory is budgeted by a framework that owns every allocation, drivers
    that forbid allocation between set-up and shutdown).  It computes exactly what
-   tbk_chebyshev_moments computes, with the same kernels, but takes all of its scratch from one
-   static device array of 64 MiB (TBK_NOALLOC_SCRATCH_BYTES) that is part of the library and
-   stays reserved on every GPU that loads the library until the process exits.  The call
-   allocates nothing: no cudaMalloc, cudaFree or allocating library routine.
+   tbk_chebyshev_moments computes, with the same kernels and the same bits (but where the array has
+   no room for the partial sums of a single step: those are then fewer, and grouped otherwise),
+   but takes all of its scratch from one static device array of 64 MiB (TBK_NOALLOC_SCRATCH_BYTES)
+   that is part of the library and stays reserved on every GPU that loads the library until the
+   process exits.  The call allocates nothing: no cudaMalloc, cudaFree or allocating library routine.
    - Arguments, layout, ownership and errors are those of tbk_chebyshev_moments; in addition a
      problem whose scratch (mapped H, two panels, per-step partial sums) exceeds the static size
      fails with TBK_ERR_ARG and a message giving the bytes it would need.

@@ -102,10 +102,17 @@ bool lane_adjoint_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a);
 // panel = c * r (probe block) for all rows.
 void launch_scaled_probe(tbk_ctx* ctx, const HOp& op, void* panel, double c, uint64_t seed, int s);
 
+// All steps of a small 1x1 operator in one launch: its CTAs, each with two partial sums a step, or 0 where it does not
+// apply; flags as in tbk_chebyshev_moments.
+int sweep_ctas(const tbk_ctx* ctx, const HOp& op, int s, int K, int direct, bool per_probe, int flags);
+void launch_sweep(tbk_ctx* ctx, const HOp& op, const void* probe_panel, uint64_t seed, int s, int K, double* partials);
+
 // Allocation-free building blocks: bytes of the mapped operator, building it into caller
-// memory, and the per-step partial-sum reduction into moments (flag bit 1 = spectrum error).
+// memory, the sums of `steps` steps' partial sums, and the moments from the sums of all K (of their partial sums
+// where given; flag bit 1 = spectrum error).
 size_t mapped_h_bytes(const tbk_bsr* H, int prec);
 HOp prepare_hop_into(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, int prec, void* dst, int* err);
+void launch_partial_sums(tbk_ctx* ctx, const double* partials, int nctas, int steps, double* sums);
 void launch_moment_reduction(tbk_ctx* ctx, const double* partials, int nctas, int K, int order, int s,
                              int64_t n_rows, int direct, double* sums, double* moments, int* flag);
 

@@ -1,4 +1,4 @@
-// tbk_chebyshev_moments_noalloc: the Chebyshev moments (same kernels and results as
+// tbk_chebyshev_moments_noalloc: the Chebyshev moments (same kernels and, to the bit, results as
 // tbk_chebyshev_moments) with every piece of device scratch taken from one fixed array that is
 // part of the library image, so that the call itself never allocates device memory.
 //
@@ -7,6 +7,7 @@
 // embedders whose device memory is budgeted up front by a framework that owns all allocations,
 // and drivers that forbid allocation between set-up and shutdown.  They still provide H and the
 // output buffer; only the library's own scratch moves into the static array.
+#include <algorithm>
 #include <mutex>
 
 #include "cheb.cuh"
@@ -88,26 +89,31 @@ extern "C" int tbk_chebyshev_moments_noalloc(tbk_ctx* ctx, const tbk_bsr* H, dou
   shape.n_atoms = H->n_atoms;
   shape.n_rows = n_rows;    // the grid follows any tuned choice for this shape, as the steps do
   shape.nnzb = H->nnzb;
-  int nctas = step_grid_ctas(ctx, shape, s, K, (flags & TBK_PLAIN_KERNEL) != 0);
+  const int sweep = sweep_ctas(ctx, shape, s, K, direct, false, flags);  // all steps in one launch, no panels
+  int nctas = sweep ? sweep : step_grid_ctas(ctx, shape, s, K, (flags & TBK_PLAIN_KERNEL) != 0);
+  int chunk = std::max(1, K);  // steps whose partial sums are kept before they are added
   // layout: flag | sums | partials | mapped H | panel A | panel B, each 256-byte aligned
   const size_t o_flag = 0;
   const size_t o_sums = o_flag + 256;
   const size_t o_part = o_sums + align256(sizeof(double) * 2 * (size_t)std::max(1, K) + 64);
   size_t o_hhat, o_pa, o_pb, need;
   auto place = [&]() {
-    o_hhat = o_part + align256(sizeof(double) * 2 * (size_t)std::max(1, K) * nctas);
+    o_hhat = o_part + align256(sizeof(double) * 2 * (size_t)chunk * nctas);
     o_pa = o_hhat + align256(mapped_h_bytes(H, prec));
-    o_pb = o_pa + (K >= 1 ? align256(panel) : 0);
-    need = o_pb + (K >= 2 ? align256(panel) : 0);
+    o_pb = o_pa + (K >= 1 && !sweep ? align256(panel) : 0);
+    need = o_pb + (K >= 2 && !sweep ? align256(panel) : 0);
   };
   place();
-  if (need > kStaticScratchBytes) {
-    nctas = step_grid_ctas(ctx, shape, s, K, true);
+  if (need > kStaticScratchBytes && !sweep) {
+    // partial sums of as many steps as there is room for
+    const size_t other = need - (o_hhat - o_part);
+    const size_t room = other < kStaticScratchBytes ? (kStaticScratchBytes - other) / (sizeof(double) * 2 * nctas) : 0;
+    chunk = (int)std::max<size_t>(1, std::min<size_t>(room, chunk));
     place();
-  }
-  if (need > kStaticScratchBytes && nctas > ctx->num_sms) {
-    nctas = ctx->num_sms;  // fewer CTAs leave fewer partial sums
-    place();
+    if (need > kStaticScratchBytes && nctas > ctx->num_sms) {
+      nctas = ctx->num_sms;  // not even of one: fewer CTAs leave fewer (and group them otherwise)
+      place();
+    }
   }
   if (need > kStaticScratchBytes)
     throw Error(TBK_ERR_ARG, "tbk_chebyshev_moments_noalloc: this problem needs " +
@@ -117,18 +123,23 @@ extern "C" int tbk_chebyshev_moments_noalloc(tbk_ctx* ctx, const tbk_bsr* H, dou
   int* flag = (int*)(base + o_flag);
   double* sums = (double*)(base + o_sums);
   double* partials = (double*)(base + o_part);
-  void* A = K >= 1 ? (void*)(base + o_pa) : nullptr;
-  void* Bp = K >= 2 ? (void*)(base + o_pb) : nullptr;
+  void* A = K >= 1 && !sweep ? (void*)(base + o_pa) : nullptr;
+  void* Bp = K >= 2 && !sweep ? (void*)(base + o_pb) : nullptr;
   // the array keeps the previous call's contents: the error flag must start at zero
   TBK_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), ctx->stream));
   HOp op = prepare_hop_into(ctx, H, emin, emax, prec, base + o_hhat, flag);
   void *cur = nullptr, *prev = nullptr;
-  for (int j = 1; j <= K; ++j) {
+  if (sweep) {
+    launch_sweep(ctx, op, nullptr, probe_seed, s, K, partials);
+    launch_partial_sums(ctx, partials, nctas, K, sums);
+  }
+  for (int j = 1; j <= K && !sweep; ++j) {
     StepArgs a;
     a.seed = probe_seed;
     a.s = s;
     a.direct = direct;
-    a.partials = partials + (size_t)(j - 1) * nctas * 2;
+    const int at = (j - 1) % chunk;
+    a.partials = partials + (size_t)at * nctas * 2;
     a.err = flag;
     a.force_simple = (flags & TBK_PLAIN_KERNEL) ? 1 : 0;
     a.grid = nctas;
@@ -154,8 +165,9 @@ extern "C" int tbk_chebyshev_moments_noalloc(tbk_ctx* ctx, const tbk_bsr* H, dou
       std::swap(cur, prev);
     }
     launch_step(ctx, op, a);
+    if (at + 1 == chunk || j == K) launch_partial_sums(ctx, partials, nctas, at + 1, sums + 2 * (size_t)(j - 1 - at));
   }
-  launch_moment_reduction(ctx, partials, nctas, K, order, s, op.n_rows, direct, sums, moments, flag);
+  launch_moment_reduction(ctx, nullptr, nctas, K, order, s, op.n_rows, direct, sums, moments, flag);
   int hflag = 0;
   TBK_CUDA(cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   sync(ctx);

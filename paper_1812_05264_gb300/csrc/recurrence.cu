@@ -1507,12 +1507,13 @@ __global__ void probe_moments_finish(const double* __restrict__ dots, int K, int
 // every CTA of the cluster, and a step ends with the cluster's barrier.  Rows are summed in the order of the
 // step kernel.  A warp's FP64 instruction takes an SM 19 cycles: 10 per row and probe are the bound (0.6 us a
 // step at 1,000 sites and 32 probes), then the chain of a row and the barrier.  Microseconds per step,
-// a launch each -> so: 216 sites x 32 probes 6.2 -> 1.4, 1,000 x 32 8.2 -> 1.9, 1,000 x 512 22.5 -> 17.3,
-// 2,744 x 64 12.4 -> 5.3, 5,832 x 64 18.6 -> 10.3, 10,648 x 4 8.2 -> 6.5, 10,648 x 512 166 -> 126.
+// a launch each -> so: 216 sites x 32 probes 6.2 -> 1.4, 1,000 x 32 8.2 -> 1.7, 1,000 x 512 18.9 -> 16.6,
+// 2,744 x 64 10.3 -> 5.3, 5,832 x 64 16.4 -> 10.0, 10,648 x 4 7.1 -> 6.2, 10,648 x 512 138 -> 125.
 constexpr int SWEEP_THREADS = 512;
 constexpr int64_t SWEEP_ROWS = 11000;                   // two panels in shared memory
-constexpr size_t SWEEP_PARTIALS = (size_t)256 << 20;    // bytes of partial sums
-constexpr int64_t SWEEP_SMEM = 220 << 10;
+constexpr size_t SWEEP_PARTIALS = (size_t)56 << 20;     // bytes of partial sums: fit tbk_chebyshev_moments_noalloc's scratch
+constexpr int SWEEP_FLUSH = 16;                         // steps whose sums wait in shared memory
+constexpr int64_t SWEEP_SMEM = 220 << 10;               // beside them; with 4 KB more L1 is a tenth slower at 10,648 sites
 
 __device__ __forceinline__ void store_cluster(double* p, int rank, double x) {
   uint32_t a;
@@ -1523,7 +1524,7 @@ __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// probe_panel: y_0, or NULL for the +-1 probes of the seed.  partials: two per warp and step.  cap: blocks of
+// probe_panel: y_0, or NULL for the +-1 probes of the seed.  partials: two per CTA and step.  cap: blocks of
 // the operator that fit in shared memory beside the panels; rows of a CTA's share beyond them stay in global memory
 // and come from L2 in every step (the cluster's barrier drops what L1 holds), a lane walking its own row.
 __global__ void __launch_bounds__(SWEEP_THREADS)
@@ -1533,8 +1534,8 @@ moments_sweep_b1(int n, int C, int cap, const int32_t* __restrict__ row_ptr, con
   extern __shared__ double ysm[];
   const int rank = blockIdx.x % C, probe = blockIdx.x / C;
   const int r0 = (int)((int64_t)n * rank / C), rows = (int)((int64_t)n * (rank + 1) / C) - r0;
-  const int lane = threadIdx.x & 31, warps = blockDim.x / 32, n_part = gridDim.x * warps;
-  double* part = partials + 2 * ((int64_t)blockIdx.x * warps + (threadIdx.x >> 5));
+  const int lane = threadIdx.x & 31, warps = blockDim.x / 32;
+  __shared__ double sums[SWEEP_FLUSH][2][SWEEP_THREADS / 32];  // of each warp
   double* hs = ysm + 2 * n;
   int* cs = reinterpret_cast<int*>(hs + cap);
   int* rp = cs + cap;
@@ -1570,8 +1571,30 @@ moments_sweep_b1(int n, int C, int cap, const int32_t* __restrict__ row_ptr, con
     double a = lane < 16 ? s0 : s1;
     a += __shfl_xor_sync(0xffffffffu, lane < 16 ? s1 : s0, 16);
     for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if ((lane & 15) == 0) part[2 * (int64_t)(j - 1) * n_part + (lane >> 4)] = a;
+    if ((lane & 15) == 0) sums[(j - 1) % SWEEP_FLUSH][lane >> 4][threadIdx.x >> 5] = a;
     cluster_barrier();
+    if (j % SWEEP_FLUSH == 0 || j == K) {
+      // the warps' sums of the last steps: eight threads add the (at most 16) of one
+      const int j0 = (j - 1) / SWEEP_FLUSH * SWEEP_FLUSH;
+      for (int e = threadIdx.x / 8; e < 2 * SWEEP_FLUSH; e += blockDim.x / 8) {
+        const int w = threadIdx.x % 8;
+        const bool has = j0 + e / 2 < j;
+        double t = has && w < warps ? sums[e / 2][e & 1][w] : 0.0, err = 0.0;
+        auto add = [&](double b) {  // t + b, its rounding error (TwoSum) to err
+          const double u = t + b, z = u - t;
+          err += (t - (u - z)) + (b - z);
+          t = u;
+        };
+        if (has && w + 8 < warps) add(sums[e / 2][e & 1][w + 8]);
+        for (int o = 4; o > 0; o >>= 1) {
+          const double b = __shfl_xor_sync(0xffffffffu, t, o);
+          err += __shfl_xor_sync(0xffffffffu, err, o);
+          add(b);
+        }
+        if (has && w == 0) partials[2 * ((int64_t)(j0 + e / 2) * gridDim.x + blockIdx.x) + (e & 1)] = t + err;
+      }
+      __syncthreads();
+    }
   }
 }
 
@@ -1585,9 +1608,7 @@ static int sweep_warps(const tbk_ctx* ctx, const HOp& op, int s) {
   return std::min(SWEEP_THREADS / 32, ceil_div(op.n_rows, 32 * sweep_cluster(ctx, s)));
 }
 
-static int sweep_partials(const tbk_ctx* ctx, const HOp& op, int s) {
-  return s * sweep_cluster(ctx, s) * sweep_warps(ctx, op, s);
-}
+static int sweep_partials(const tbk_ctx* ctx, int s) { return s * sweep_cluster(ctx, s); }
 
 // Blocks that fit beside the panels and the row pointers.
 static int64_t sweep_room(const HOp& op, int C) {
@@ -1599,15 +1620,16 @@ static int64_t sweep_room(const HOp& op, int C) {
 // blocks a row 5.8 / 10.3, 23 blocks, beyond it, 20.4 / 12.4; 5,832 x 512 of 143 blocks 4,599 / 744) and the chip is
 // not full of FMAs anyway (216 sites x 512 probes, 36 blocks 17.5 / 18.6, 47 blocks 23.5 / 22.7; 1,000 x 512, 16
 // blocks 28.4 / 26.8).
-static bool use_sweep(const tbk_ctx* ctx, const HOp& op, int s, int K, int direct, const void* per_probe, int flags) {
+int sweep_ctas(const tbk_ctx* ctx, const HOp& op, int s, int K, int direct, bool per_probe, int flags) {
   if (op.B != 1 || op.prec != TBK_FP64 || K < 1 || direct || per_probe || (flags & TBK_PLAIN_KERNEL) ||
-      op.n_rows > SWEEP_ROWS || s > 512 || 16 * (size_t)K * sweep_partials(ctx, op, s) > SWEEP_PARTIALS)
-    return false;
+      op.n_rows > SWEEP_ROWS || s > 512 || 16 * (size_t)K * sweep_partials(ctx, s) > SWEEP_PARTIALS)
+    return 0;
   const int C = sweep_cluster(ctx, s);
-  return op.nnzb <= 8 * op.n_rows || (op.nnzb <= C * sweep_room(op, C) && s * op.nnzb <= (int64_t)30000 * ctx->num_sms);
+  const bool fits = op.nnzb <= C * sweep_room(op, C), small = s * op.nnzb <= (int64_t)30000 * ctx->num_sms;
+  return op.nnzb <= 8 * op.n_rows || (fits && small) ? sweep_partials(ctx, s) : 0;
 }
 
-static void launch_sweep(tbk_ctx* ctx, const HOp& op, const void* probe_panel, uint64_t seed, int s, int K,
+void launch_sweep(tbk_ctx* ctx, const HOp& op, const void* probe_panel, uint64_t seed, int s, int K,
                          double* partials) {
   KernelTimerScope timer(ctx, TBK_KERNEL_STEP);
   const int C = sweep_cluster(ctx, s), n = (int)op.n_rows;
@@ -1672,12 +1694,14 @@ HOp prepare_hop_into(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, i
   return op;
 }
 
+void launch_partial_sums(tbk_ctx* ctx, const double* partials, int nctas, int steps, double* sums) {
+  reduce_partials<<<steps, 256, 0, ctx->stream>>>(partials, nctas, sums);
+  post_launch(ctx, "reduce_partials");
+}
+
 void launch_moment_reduction(tbk_ctx* ctx, const double* partials, int nctas, int K, int order, int s,
                              int64_t n_rows, int direct, double* sums, double* moments, int* flag) {
-  if (K >= 1) {
-    reduce_partials<<<K, 256, 0, ctx->stream>>>(partials, nctas, sums);
-    post_launch(ctx, "reduce_partials");
-  }
+  if (K >= 1 && partials) launch_partial_sums(ctx, partials, nctas, K, sums);
   finish_moments<<<1, 256, 0, ctx->stream>>>(sums, K, order, s, n_rows, direct, moments, flag);
   post_launch(ctx, "finish_moments");
 }
@@ -1708,8 +1732,8 @@ void moments_sweep(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, uin
   const size_t esz = prec == TBK_MIXED ? 4 : 8;
   const size_t panel = (size_t)op.n_rows * s * esz;
   const int K = direct ? order - 1 : order / 2;   // steps: largest moment index 2K >= order - 1
-  const bool sweep = use_sweep(ctx, op, s, K, direct, per_probe, flags);
-  const int nctas = sweep ? sweep_partials(ctx, op, s)
+  const int sweep = sweep_ctas(ctx, op, s, K, direct, per_probe != nullptr, flags);
+  const int nctas = sweep ? sweep
                           : step_grid_ctas(ctx, op, s, K, (flags & (TBK_TENSOR_CORES | TBK_PLAIN_KERNEL)) != 0);
   double* partials = (double*)scratch(ctx, WS_PARTIALS, sizeof(double) * 2 * (size_t)std::max(1, K) * nctas);
   double* sums = (double*)scratch(ctx, WS_MISC, sizeof(double) * 2 * (size_t)std::max(1, K) + 64);
@@ -1771,12 +1795,7 @@ void moments_sweep(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, uin
       post_launch(ctx, "probe_dots_reduce");
     }
   }
-  if (K >= 1) {
-    reduce_partials<<<K, 256, 0, ctx->stream>>>(partials, nctas, sums);
-    post_launch(ctx, "reduce_partials");
-  }
-  finish_moments<<<1, 256, 0, ctx->stream>>>(sums, K, order, nrm, op.n_rows, direct, moments, flag);
-  post_launch(ctx, "finish_moments");
+  launch_moment_reduction(ctx, partials, nctas, K, order, nrm, op.n_rows, direct, sums, moments, flag);
   if (per_probe) {
     const int64_t n = (int64_t)order * s;
     probe_moments_finish<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, ctx->stream>>>(
