@@ -15,6 +15,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "adjoint_plan.cuh"
 #include "bulk.cuh"
 #include "cheb.cuh"
 #include "model.cuh"
@@ -578,8 +579,6 @@ clenshaw_sddmm_bulk(const int n_atoms, const int32_t* __restrict__ row_ptr,
 //
 // Gacc_ab += w sum_{t < nw} sum_probes y_{k_t}[a] ybar_{k_t + 1}[b]^T for every stored block (a, b).
 // Summing nw steps before the cross-lane reduction spreads its cost over nw block products.
-
-constexpr int SDW = 4;  // steps per window
 
 struct WindowPanels {
   const float* y[SDW];  // y_{k_t} panels (n_rows x s)
@@ -1558,28 +1557,21 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
   const size_t panel = (size_t)op.n_rows * s * esz;
   size_t budget = max_panel_bytes > 0 ? (size_t)max_panel_bytes : panel_budget(ctx, WS_CHECKPOINTS);
   const int npan = K;  // y_1 .. y_K
-  // ybar_j lives in ring slot j mod NB: the two of the recurrence, plus the window's SDW panels
-  // when the outer products are summed over windows of steps; a batch also keeps the probe panel
+  AdjointPlan plan;
+  plan.npan = plan.seg = npan;
+  plan.panel = panel;
+  plan.windowed = windowed;
+  plan.batch = bt != nullptr;
   if (defer > 0) {
     // as many ybar panels as fit beside the all-stored plan
     const int64_t room = (int64_t)(budget / panel) - (npan + 2) - 2;
-    defer = room < 0 ? 0 : (int)std::min<int64_t>(std::min(defer, K), room + 1);
+    plan.defer = room < 0 ? 0 : (int)std::min<int64_t>(std::min(defer, K), room + 1);
   }
-  const int NB = windowed ? SDW + 2 : (defer > 1 ? defer + 1 : 2);
-  const int NX = NB + (bt ? 1 : 0);
-  int seg = std::max(1, npan);
-  auto seg_plan = [&]() {
-    // segments of a multiple of SDW steps, so that windows never straddle a segment
-    const int r = std::max(2, (int)std::ceil(std::sqrt(2.0 * npan)));
-    return ((r + SDW - 1) / SDW) * SDW;
-  };
   // A batch's step t runs on the clusters with K_c >= t, a prefix of the merged rows, so its
   // all-stored plan can keep every y_j compactly: panel j holds the rows of the clusters still
   // running at step j - 1 (backward step j - 1 reads y_j on those rows, with a zero coefficient
   // for the clusters that stop there).  poff: byte offsets of P(0 .. npan) and E = y_{npan+1}.
-  bool prefix = false;
   std::vector<size_t> poff;
-  size_t prefix_tail = 0;
   if (bt) {
     const size_t row_bytes = (size_t)op.B * s * esz;
     poff.resize((size_t)npan + 2);
@@ -1589,36 +1581,28 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
       o += (size_t)active(std::max(i - 1, 0)) * row_bytes;
       o = (o + 255) & ~(size_t)255;
     }
-    prefix_tail = o;
-    prefix = o + (size_t)NX * panel <= budget;
+    if (o + (size_t)plan.nx() * panel <= budget) plan.prefix_tail = o;
   }
-  if (!prefix && (size_t)(npan + 2 + NX) * panel > budget && npan > 2) {
-    seg = seg_plan();
-    const size_t need = (size_t)(2 * ((npan + seg - 1) / seg) + seg + 2 + NX) * panel;
-    if (need > budget)
+  if (!plan.prefix_tail && plan.bytes() > budget && npan > 2) {
+    plan.segment();
+    if (plan.bytes() > budget)
       throw Error(TBK_ERR_OOM, "panel scratch budget of " + std::to_string(budget) +
-                                   " bytes is below the checkpoint plan's " + std::to_string(need));
+                                   " bytes is below the checkpoint plan's " + std::to_string(plan.bytes()));
   }
-  int nseg = (npan + seg - 1) / seg;
-  // P(0 .. seg): segment panels (P(i) = y_{t0 - 1 + i}); checkpoints (y_{t0-2}, y_{t0-1}); E = y_{t1+1};
-  // NB ybar panels; the probe panel of a batch
-  auto plan_bytes = [&]() {
-    if (prefix) return prefix_tail + (size_t)NX * panel;
-    return panel * ((size_t)seg + 1 + (nseg <= 1 ? 0 : 2 * (size_t)nseg) + 1 + NX);
-  };
   char* base = nullptr;
-  try {
-    base = (char*)scratch(ctx, WS_CHECKPOINTS, plan_bytes());
-  } catch (const Error& e) {
-    // the device could not map the all-stored plan after all: replay segments instead
-    if (e.code != TBK_ERR_OOM || nseg > 1 || npan <= 2) throw;
-    prefix = false;
-    seg = seg_plan();
-    nseg = (npan + seg - 1) / seg;
-    base = (char*)scratch(ctx, WS_CHECKPOINTS, plan_bytes());
+  while (!base) {
+    try {
+      base = (char*)scratch(ctx, WS_CHECKPOINTS, plan.bytes());
+    } catch (const Error& e) {
+      // the device could not map the plan after all: a smaller one
+      if (e.code != TBK_ERR_OOM || !plan.shrink()) throw;
+    }
   }
-  const bool all_stored = nseg <= 1;
-  const size_t n_seg_pan = (size_t)seg + 1, n_ckpt = all_stored ? 0 : 2 * (size_t)nseg;
+  const bool prefix = plan.prefix_tail > 0, all_stored = plan.nseg() <= 1;
+  const size_t prefix_tail = plan.prefix_tail;
+  const int NB = plan.nb(), seg = plan.seg, nseg = plan.nseg();
+  const size_t n_seg_pan = (size_t)seg + 1, n_ckpt = plan.n_ckpt();
+  defer = plan.defer;
   // P(0 .. npan + 1) of the prefix plan at poff, the full-size panels after them
   auto P = [&](size_t i) -> void* {
     if (!prefix) return base + i * panel;
@@ -1681,7 +1665,6 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
       }
     }
   }
-  if (!all_stored) defer = 0;  // the replay reuses the panels that waiting outer products read
   OuterPanels wait{};
   int n_wait = 0;
   int k = K;
@@ -1899,8 +1882,17 @@ extern "C" int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_
     int defer = all_stored && !plain && npan > 0 ? general_deferred_steps(op, s) : 0;
     defer = (int)std::max<int64_t>(0, std::min<int64_t>(std::min(defer, p - 1), (int64_t)(budget / panel) - (npan + 2)));
     if (defer < 8) defer = 0;
-    const size_t n_ring = defer ? (size_t)defer + 1 : 2;
-    char* base = (char*)scratch(ctx, WS_CHECKPOINTS, panel * (n_seg_pan + n_ckpt + n_ring));
+    size_t n_ring = defer ? (size_t)defer + 1 : 2;
+    char* base = nullptr;
+    try {
+      base = (char*)scratch(ctx, WS_CHECKPOINTS, panel * (n_seg_pan + n_ckpt + n_ring));
+    } catch (const Error& e) {
+      // the device could not map that after all: with two b panels
+      if (e.code != TBK_ERR_OOM || !defer) throw;
+      defer = 0;
+      n_ring = 2;
+      base = (char*)scratch(ctx, WS_CHECKPOINTS, panel * (n_seg_pan + n_ckpt + n_ring));
+    }
     auto P = [&](size_t i) { return (void*)(base + i * panel); };
     auto CK = [&](int sg, int which) { return P(n_seg_pan + 2 * (size_t)sg + which); };
     auto ring = [&](int i) { return P(n_seg_pan + n_ckpt + (size_t)((i + (int)n_ring) % (int)n_ring)); };
