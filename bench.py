@@ -273,6 +273,65 @@ SMS, FP32_LANES, SM_MAX_MHZ = 152, 128, 2070.0
 L2_BYTES = 126 * 2 ** 20
 
 
+def family_work(sched, p, launches, steps, panel, entries, esz, n_probes, n_orb, fp64, chunk):
+    """Algorithmic bytes and flops (2 per FMA) of each kernel family over `steps` timed steps, the kernels that ran and
+    their profile: {family: (bytes, flops, kernel, profile or None, source)}, and the block products (H times a
+    panel) of a step.  launches: bracketed launches per family; panel: bytes of a panel; entries: stored entries
+    of H.  From the steps of the algorithm: an adjoint may take several launches for one step or one for several."""
+    K = p // 2
+    hb, gb, blk = entries * esz, entries * 16, 2 * entries * n_probes   # H^, G read and written, one product
+    doubled = fp64 or (n_orb == 9 and n_probes in (128, 256, 512))
+    if fp64 or not doubled:
+        sched = "fused"                                       # the only one
+    n_back = max(0, (K if doubled else p - 1) - 1)            # adjoint steps
+    pairs = K if doubled else max(0, p - 1)                   # outer products y_j ybar_{j+1}^T, j = 0 too
+    # ybar_k = g_k + 2 H^ ybar_{k+1} - ybar_{k+2}: reads ybar_{k+1}, ybar_{k+2}, y_k, y_{k-1}, y_{k+1} (general form:
+    # b_{j+1}, b_{j+2}), the H^ blocks, writes ybar_k
+    own = n_back * ((6 if doubled else 3) * panel + hb)
+    after = launches["backward"] / steps - n_back             # launches of outer products after their steps
+    if sched != "fused":
+        # (the tensor-core schedule leaves that of y_0 to a launch of this family)
+        back = (own + after * (2 * panel + gb), (n_back + after) * blk)
+        name, prof = ("clenshaw_self" if n_probes == 128 else "clenshaw_sddmm_bulk"), None
+    elif doubled and not fp64 and n_probes == 512:
+        # and G += 2 y_k ybar_{k+1}^T from the same tiles; that of y_0 in a launch of its own
+        back = (own + 2 * panel + pairs * gb, (n_back + pairs) * blk)
+        name, prof = "clenshaw_sddmm_bulk", "clenshaw_sddmm_bulk_fcc10000.md"
+    else:
+        back = (own + pairs * 2 * panel + after * gb, (n_back + pairs) * blk)
+        if fp64:
+            name = "cheb_step_fp64 + sddmm_rows64" if n_orb == 9 else "cheb_step_kernel + sddmm_one"
+        elif n_probes in (128, 256):
+            name = ("clenshaw_self + outer_blocks", "clenshaw_sddmm_bulk + outer_rows")[n_probes == 256]
+        else:
+            name = "cheb_step_lane or cheb_step_self + sddmm_steps32 or sddmm_rows32"
+        prof = None
+    if fp64:
+        step_k = "cheb_step_fp64" if n_orb == 9 else "cheb_step_kernel"
+    elif n_probes % 128:
+        step_k = "cheb_step_lane or cheb_step_self"
+    else:
+        # 128-probe tasks take the self-fed kernels
+        step_k = "cheb_step_self" if chunk == 128 or n_probes == 128 else "cheb_step_bulk"
+    n_step = launches["step"]
+    n_win = (K - 1 + 3) // 4 + 1 if K >= 1 else 0
+    if sched == "tensor":
+        # one pair per launch, the accumulator read and written by each
+        n = launches["window"]
+        window = (n * (2 * panel + gb), n * blk, "sddmm_tc", None, "tc_sddmm.cu")
+    else:
+        # G += sum_j y_j ybar_{j+1}^T: both panels of every pair, the accumulator once per window
+        window = (steps * (K * 2 * panel + n_win * gb), steps * K * blk, "sddmm_window_g", None, "adjoint.cu")
+    alg = {
+        # y_{k+1} = 2 H^ y_k - y_{k-1}: reads y_k, y_{k-1}, the H^ blocks, writes y_{k+1}
+        "step": (n_step * (3 * panel + hb), n_step * blk, step_k,
+                 "cheb_step_bulk_fcc10000.md" if step_k == "cheb_step_bulk" else None, "recurrence.cu"),
+        "backward": (steps * back[0], steps * back[1], name, prof, "adjoint.cu"),
+        "window": window,
+    }
+    return alg, n_step / steps + n_back
+
+
 def run_ours(args, rank, world):
     import torch
     from paper_1812_05264_gb300 import build as _build
@@ -376,44 +435,16 @@ def run_ours(args, rank, world):
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     B2 = wk.n_orb ** 2
     alu = 1.25 if fp64 else SMS * FP32_LANES * 2 * SM_MAX_MHZ * 1e6 / 1e12
-    K = p // 2
-    nwin = (K - 1 + 3) // 4 + 1 if K >= 1 else 0
-    # algorithmic bytes and flops (2 per FMA) of each family over the timed steps
-    hb, blk = nnzb * B2 * esz, 2 * nnzb * B2 * wk.n_probes
     sched = args.adjoint if args.adjoint != "auto" else (tuned[1] if tuned else "fused")
-    windowed = sched == "windowed"
     tensor = sched == "tensor"
-    # the kernels that ran: 128-probe tasks take the self-fed kernels; the profiles under
-    # profiles/ are of the TMA-fed step and the fused adjoint step
-    chunk = tuned[0] if tuned else wk.n_probes
-    step_k = "cheb_step_self" if chunk == 128 or wk.n_probes == 128 else "cheb_step_bulk"
-    bwd_k = "clenshaw_self" if sched != "fused" and wk.n_probes == 128 else "clenshaw_sddmm_bulk"
-    alone = sched != "fused"     # the backward step without its outer products
-    alg = {
-        # y_{k+1} = 2 H^ y_k - y_{k-1}: reads y_k, y_{k-1}, the H^ blocks, writes y_{k+1}
-        "step": (lambda n: n * (3 * panel + hb), lambda n: n * blk, step_k,
-                 "cheb_step_bulk_fcc10000.md" if step_k == "cheb_step_bulk" else None, "recurrence.cu"),
-        # ybar_k = g_k + 2 H^ ybar_{k+1} - ybar_{k+2}: reads ybar_{k+1}, ybar_{k+2}, y_k, y_{k-1},
-        # y_{k+1}, the H^ blocks, writes ybar_k; fused: and G += 2 y_k ybar_{k+1}^T (the same
-        # tiles, as many FMAs again, the FP64 accumulator read and written once)
-        "backward": (lambda n: n * (6 * panel + hb + (0 if alone else nnzb * B2 * 16)),
-                     lambda n: n * blk * (1 if alone else 2), bwd_k,
-                     None if alone else "clenshaw_sddmm_bulk_fcc10000.md", "adjoint.cu"),
-        # windowed: G += sum_j y_j ybar_{j+1}^T (j = 0 .. K-1, K pairs a step): reads both panels
-        # of every pair, reads and writes the FP64 accumulator once per window; tensor: one pair
-        # per launch (K - 1 a step), the accumulator read and written every launch
-        "window": ((lambda n: n * (2 * panel + nnzb * B2 * 16)) if tensor else
-                   (lambda n: args.steps * (K * 2 * panel + nwin * nnzb * B2 * 16)),
-                   (lambda n: n * blk) if tensor else (lambda n: args.steps * K * blk),
-                   "sddmm_tc" if tensor else "sddmm_window_g", None,
-                   "tc_sddmm.cu" if tensor else "adjoint.cu"),
-    }
+    alg, n_products = family_work(sched, p, {f: n for f, (_, n) in fam.items()}, args.steps, panel, nnzb * B2, esz,
+                                  wk.n_probes, wk.n_orb, fp64, tuned[0] if tuned else wk.n_probes)
     kernels = {}
     for f, (tms, nl) in fam.items():
         if nl == 0:
             continue
-        byf, flf, kname, prof, src = alg[f]
-        by, fl = byf(nl) / args.steps, flf(nl) / args.steps
+        by, fl, kname, prof, src = alg[f]
+        by, fl = by / args.steps, fl / args.steps
         sec = tms / 1e3 / args.steps
         t_mem, t_alu = by / (hbm * 1e9), fl / (alu * 1e12)
         if f == "window" and tensor:
@@ -441,8 +472,6 @@ def run_ours(args, rank, world):
         kernels[f] = r
     dom = max(kernels, key=lambda f: kernels[f]["share_of_step"])
     roof = dict(kernels[dom])
-    # (the fused schedule's y_0 launch is an outer product only)
-    n_products = (fam["step"][1] + fam["backward"][1]) / args.steps - (0 if windowed else 1)
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",

@@ -150,8 +150,12 @@ int tbk_autotune(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, int32
 /* Kernel families that tbk_kernel_timer can bracket with CUDA events. */
 #define TBK_KERNEL_NONE 0
 #define TBK_KERNEL_STEP 1     /* one recurrence step y_{k+1} = 2 H^ y_k - y_{k-1} (Eq. cheb_rec) */
-#define TBK_KERNEL_BACKWARD 2 /* one adjoint step ybar_k = g_k + 2 H^ ybar_{k+1} - ybar_{k+2} */
-#define TBK_KERNEL_WINDOW 3   /* the sampled outer products sum y_j ybar_{j+1}^T of a few steps */
+#define TBK_KERNEL_BACKWARD 2 /* one adjoint step ybar_k = g_k + 2 H^ ybar_{k+1} - ybar_{k+2}, with its outer
+                                 products; where these run in launches of their own after one or more steps
+                                 (every precision and probe count but 512 in mixed precision), those too, so
+                                 that launches are not steps */
+#define TBK_KERNEL_WINDOW 3   /* the sampled outer products sum y_j ybar_{j+1}^T of a few steps, with
+                                 TBK_WINDOWED or TBK_TC_OUTER */
 /* Select the kernel families whose launches on ctx's stream are from now on bracketed by pairs
    of CUDA events: mask = sum of (1 << TBK_KERNEL_*) (0 switches timing off); earlier pairs are
    forgotten.  Launches captured into CUDA graphs are not bracketed.  Host-side only. */

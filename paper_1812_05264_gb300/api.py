@@ -45,8 +45,9 @@ class Context:
 
     def time_kernels(self, *families: str):
         """Bracket every launch of the named kernel families ("step": one recurrence step,
-        "backward": one adjoint step, "window": the outer products of a window of steps) with CUDA
-        events on this context's stream; no names switches timing off.  Read with kernel_time()."""
+        "backward": one adjoint step or its outer products where they run after it, "window": the outer
+        products of the windowed and tensor-core schedules) with CUDA events on this context's stream; no
+        names switches timing off.  Read with kernel_time()."""
         mask = 0
         for f in families:
             mask |= 1 << self._FAMILIES[f]

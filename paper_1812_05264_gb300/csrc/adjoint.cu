@@ -1386,6 +1386,7 @@ static int general_deferred_steps(const HOp& op, int s) {
 
 static void launch_sddmm_steps(tbk_ctx* ctx, const HOp& op, const OuterPanels& wp, int nt, int last_is_y0, int s,
                                double* Gacc) {
+  KernelTimerScope timer(ctx, TBK_KERNEL_BACKWARD);
   launch_pdl(ctx, sddmm_steps32, (unsigned)op.nnzb, 96, 0, op.n_atoms, op.row_ptr, op.col, op.nnzb, wp, nt,
              last_is_y0, s, Gacc);
   post_launch(ctx, "sddmm_steps32");
@@ -1714,9 +1715,13 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
       }
       if (f64) {
         // G += 2 y_k ybar_{k+1}^T (y_0 ybar_1^T last), then ybar_k = g_k + 2 H^ ybar_{k+1} - ybar_{k+2}
-        launch_sddmm(ctx, o, Y(k), YB(k + 1), s, k ? 2.0 : 1.0, Gacc);
+        {
+          KernelTimerScope timer(ctx, TBK_KERNEL_BACKWARD);
+          launch_sddmm(ctx, o, Y(k), YB(k + 1), s, k ? 2.0 : 1.0, Gacc);
+        }
         if (k == 0) continue;
         StepArgs a;
+        a.family = TBK_KERNEL_BACKWARD;
         a.seed = probe_seed;
         a.s = s;
         a.yin = YB(k + 1);
@@ -1966,10 +1971,12 @@ extern "C" int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_
               n_wait = 0;
             }
           } else {
+            KernelTimerScope timer(ctx, TBK_KERNEL_BACKWARD);
             launch_sddmm(ctx, op, yj, ring(ib), s, j == 0 ? 1.0 : 2.0, Gacc);
           }
           if (j >= 1) {
             StepArgs a;
+            a.family = TBK_KERNEL_BACKWARD;
             a.seed = probe_seed;
             a.s = s;
             a.yin = ring(ib);

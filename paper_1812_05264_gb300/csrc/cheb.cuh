@@ -78,6 +78,7 @@ struct StepArgs {
   int per_task = 0;
   int use_tc = 0;           // tensor-core (tcgen05) step where it applies
   int grid = 0;             // CTAs of the launch (0: step_grid_ctas; with partials: their number per step)
+  int family = TBK_KERNEL_STEP;  // what the kernel timer books the launch as
   int adjoint = 0;          // lane kernel: src[0] is added before y_prev, src[1] and src[2] after; no sums
 };
 // Consumer warps of the TMA-fed step kernel for this operator and probe count (0 = not used).

@@ -1303,7 +1303,7 @@ static void launch_fp64(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
 }
 
 void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
-  KernelTimerScope timer(ctx, TBK_KERNEL_STEP);
+  KernelTimerScope timer(ctx, a.family);
   const int G = a.grid > 0 ? a.grid : step_grid_ctas(ctx, op, a.s, 0, a.force_simple || a.use_tc);
   if (a.use_tc && !a.cur_is_probe && a.err && !a.force_simple && !a.batch.atom_cl && !a.per_task &&
       tc_eligible(op, a.s)) {
