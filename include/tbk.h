@@ -125,11 +125,14 @@ int64_t tbk_launch_count(tbk_ctx* ctx);
    and the call that launched it returns TBK_ERR_TIMEOUT.  Nothing faults; the context stays
    usable and the next calls compute normally.  Host-side only. */
 int tbk_test_stall_next_step(tbk_ctx* ctx);
-/* The same test for the fused adjoint step (the TMA-fed Clenshaw step with the sampled outer
-   products): the next such launch on ctx gets a producer that copies nothing; its consumers give
-   up after 2 s, the adjoint call returns TBK_ERR_TIMEOUT, and the context stays usable.  Host-side
-   only. */
+/* The same test for the adjoint step: the next TMA-fed one on ctx, with the sampled outer products
+   fused into it or alone, gets a producer that copies nothing; its consumers give up after 2 s, the
+   adjoint call returns TBK_ERR_TIMEOUT, and the context stays usable.  The FP64 and the plain
+   adjoint have no such launch.  Host-side only. */
 int tbk_test_stall_next_adjoint(tbk_ctx* ctx);
+/* And for the outer products after the adjoint steps at 256 probes, whose panels are copied tile by tile.
+   Host-side only. */
+int tbk_test_stall_next_outer(tbk_ctx* ctx);
 /* Test of the launch geometry: n_ctas (host) receives the CTAs of a recurrence step of tbk_chebyshev_probe_moments
    with these arguments.  Of H the sizes are read; nothing is launched.  Host-side only. */
 int tbk_test_step_grid(tbk_ctx* ctx, const tbk_bsr* H, int32_t n_probes, int32_t order, int32_t flags,

@@ -74,6 +74,7 @@ SIGNATURES = {
     "tbk_destroy": [_P],
     "tbk_test_stall_next_step": [_P],
     "tbk_test_stall_next_adjoint": [_P],
+    "tbk_test_stall_next_outer": [_P],
     "tbk_test_step_grid": [_P, C.POINTER(tbk_bsr), _I, _I, _I, C.POINTER(_I)],
     "tbk_autotune": [_P, C.POINTER(tbk_bsr), _D, _D, _I, C.POINTER(_I)],
     "tbk_kernel_timer": [_P, _I],

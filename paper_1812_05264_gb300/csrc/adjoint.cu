@@ -857,7 +857,7 @@ template <int NW>
 __global__ void __launch_bounds__(32 * NW, 12 / NW)
 outer_rows(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
             const __grid_constant__ OuterPanels wp, const int nt, const int last_is_y0, double* __restrict__ Gacc,
-            int* __restrict__ err) {
+            int* __restrict__ err, const int stall) {
   constexpr int NC = 2, S = 128 * NC, XB = 9 * S * 4;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bars[4];
@@ -875,7 +875,9 @@ outer_rows(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t
   // tiles y_t[a] of the CTA's rows and steps, in order: number it in buffer it & 1
   const int rows = (n_atoms - blockIdx.x + gridDim.x - 1) / gridDim.x;
   const int n_tiles = rows * nt;
+  // (stall: a test of the bounded waits; nothing is copied, the warps give up and report)
   auto issue = [&](int it) {
+    if (stall) return;
     const int a = blockIdx.x + (it / nt) * gridDim.x;
     const uint32_t bar = full + 8 * (it & 1);
     mbar_expect_tx(bar, XB);
@@ -951,7 +953,7 @@ outer_rows(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t
   if (!ok) {
     if (lane == 0) atomicOr(err, 2);
     // let the copies in flight land before the CTA exits
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0 && !stall)
       for (int j = it; j < it + 2 && j < n_tiles; ++j) mbar_wait(full + 8 * (j & 1), (j >> 1) & 1);
   }
 }
@@ -976,7 +978,7 @@ clenshaw_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int3
               const float* __restrict__ hv, const float* __restrict__ bin, const float* bprev, float* bout,
               const float* __restrict__ ypan, const float4 cf, const uint64_t seed, const int s,
               int* __restrict__ err, const BatchRows batch, const float4* __restrict__ cf_cl,
-              const float* __restrict__ ym1, const float* __restrict__ yp1, const int y_first) {
+              const float* __restrict__ ym1, const float* __restrict__ yp1, const int y_first, const int stall) {
   using C = ClenSelfCfg<R>;
   extern __shared__ __align__(128) unsigned char smem[];
   const uint32_t bar0 = smem_u32(smem + R * C::SB);
@@ -1009,8 +1011,9 @@ clenshaw_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int3
       if (p_nb + n_extra > 0) break;
     }
   };
+  // (stall: a test of the bounded waits; nothing is copied, the warp gives up and reports)
   auto issue_next = [&]() {
-    if (p_a >= n_atoms) return;
+    if (stall || p_a >= n_atoms) return;
     const bool own = p_q >= p_nb;
     const int b = own ? p_a : __ldg(col + p_k0 + p_q);
     const float* src = (own ? extra_src[p_q - p_nb] : bin) + (int64_t)9 * b * s;
@@ -1295,7 +1298,8 @@ void launch_fused(tbk_ctx* ctx, const HOp& op, const void* bin, const void* bpre
     const int G = task_grid(op.n_atoms, (int64_t)occ * ctx->num_sms);
     launch_pdl(ctx, clenshaw_self<CLEN_SELF_R>, G, 32, C::SMEM, op.n_atoms, op.row_ptr, op.col, (const float*)op.hv,
                (const float*)bin, (const float*)bprev, (float*)bout, (const float*)ypan, cf, seed, s, err, batch, cf_cl,
-               (const float*)ym1, (const float*)yp1, y_first);
+               (const float*)ym1, (const float*)yp1, y_first, ctx->stall_next_adjoint);
+    ctx->stall_next_adjoint = 0;
     post_launch(ctx, "clenshaw_self");
   }
 }
@@ -1320,6 +1324,7 @@ static void launch_adjoint_step(tbk_ctx* ctx, const HOp& op, const void* bin, vo
   a.csrc[2] = yp1 ? cf.w : 0.0;
   a.err = err;
   a.adjoint = 1;
+  a.family = TBK_KERNEL_BACKWARD;
   if (lane_adjoint_step(ctx, op, a)) return;
   launch_fused(ctx, op, bin, bprev, bout, ypan, cf, seed, s, 0.0, nullptr, err, BatchRows(), nullptr, ym1, yp1, 1);
 }
@@ -1337,7 +1342,8 @@ static void launch_outer_rows(tbk_ctx* ctx, const HOp& op, const OuterPanels& wp
     TBK_CHECK_ARG(occ > 0, "outer-product kernel does not fit on this device");
   }
   launch_pdl(ctx, outer_rows<NW>, task_grid(op.n_atoms, (int64_t)occ * ctx->num_sms), 32 * NW, SMEM, op.n_atoms, op.row_ptr,
-             op.col, wp, nt, last_is_y0, Gacc, err);
+             op.col, wp, nt, last_is_y0, Gacc, err, ctx->stall_next_outer);
+  ctx->stall_next_outer = 0;
 }
 
 static void launch_outer(tbk_ctx* ctx, const HOp& op, const OuterPanels& wp, int nt, int last_is_y0, int s,

@@ -54,7 +54,8 @@ struct tbk_ctx {
   void* pinned = nullptr;        // small pinned host buffer for scalar read-back
   size_t pinned_bytes = 0;
   int stall_next_step = 0;       // test hook: the next TMA-fed step's producer issues no copies
-  int stall_next_adjoint = 0;    // test hook: the next fused adjoint step's producer issues no copies
+  int stall_next_adjoint = 0;    // test hook: the same of the next TMA-fed adjoint step, fused or alone
+  int stall_next_outer = 0;      // test hook: the same of the next outer_rows launch
   struct Tuned {                 // tbk_autotune's choices, per operator shape and probe count
     int64_t n_rows, nnzb;
     int s, cw, windowed;        // windowed: the outer-product schedule (0 fused, 1 windowed, 2 tensor cores)

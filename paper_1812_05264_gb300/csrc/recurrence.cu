@@ -1245,14 +1245,21 @@ static void launch_simple(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G)
   post_launch(ctx, "cheb_step_kernel");
 }
 
+// The test hook that a TMA-fed step answers to, taken.
+static int take_stall(tbk_ctx* ctx, const StepArgs& a) {
+  int& hook = a.family == TBK_KERNEL_BACKWARD ? ctx->stall_next_adjoint : ctx->stall_next_step;
+  const int stall = hook;
+  hook = 0;
+  return stall;
+}
+
 template <int CW, bool DENSE = false>
 static void launch_bulk(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
   using C = BulkCfg<CW, BULK_D>;
   launch_pdl(ctx, cheb_step_bulk<CW, BULK_D, DENSE>, G, C::THREADS, C::SMEM,
                op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)a.yin, (const float*)a.yprev,
                (float*)a.yout, (float)a.alpha, (float)a.c_r, a.seed, a.s, a.direct, a.partials, a.err, a.batch,
-               a.per_task, ctx->stall_next_step);
-  ctx->stall_next_step = 0;
+               a.per_task, take_stall(ctx, a));
   post_launch(ctx, "cheb_step_bulk");
 }
 
@@ -1262,8 +1269,7 @@ static void launch_self(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
   launch_pdl(ctx, cheb_step_self<SELF_R, NARROW>, G, 32, C::SMEM,
                op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)a.yin, (const float*)a.yprev,
                (float*)a.yout, (float)a.alpha, (float)a.c_r, a.seed, a.s, a.direct, a.partials, a.err, a.batch,
-               a.per_task, ctx->stall_next_step);
-  ctx->stall_next_step = 0;
+               a.per_task, take_stall(ctx, a));
   post_launch(ctx, "cheb_step_self");
 }
 
@@ -1273,8 +1279,7 @@ static void launch_lane_nw(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G
   launch_pdl(ctx, a.adjoint ? cheb_step_lane<NW, true> : cheb_step_lane<NW, false>, G, 32 * (nw + 1), LaneCfg<NW>::SMEM,
              op.n_atoms, op.row_ptr, op.col, (const float*)op.hv, (const float*)a.yin, (const float*)a.yprev,
              (float*)a.yout, (float)a.alpha, (float)a.c_r, a.seed, a.s, a.direct, sources<float>(a), a.partials, a.err,
-             ctx->stall_next_step);
-  ctx->stall_next_step = 0;
+             take_stall(ctx, a));
   post_launch(ctx, "cheb_step_lane");
 }
 
