@@ -1771,7 +1771,7 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
                      (k >= 2 || r_panel) ? Y(k - 1) : nullptr, Y(k + 1), 0);
         // G += 2 y_k ybar_{k+1}^T on the pattern, on the tensor cores
         if (tensor) launch_tc_sddmm(ctx, o, Y(k), YB(k + 1), s, 2.0, Gacc, err);
-        if (windowed && (k - 1) % SDW == 0) {
+        if (windowed && (k - 1) % SDW == 0 && k < K) {
           // G += 2 y_j ybar_{j+1}^T on the pattern for the window j = k .. min(k + SDW, K) - 1
           WindowPanels wp{};
           const int nw = std::min(SDW, K - k);
