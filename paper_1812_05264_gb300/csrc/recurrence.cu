@@ -1136,7 +1136,6 @@ static int64_t simple_tasks(const HOp& op, int s) {
 }
 
 bool tc_eligible(const HOp& op, int s);
-int tc_grid(tbk_ctx* ctx);
 void launch_step_tc(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G);
 
 static int lane_class(int s);

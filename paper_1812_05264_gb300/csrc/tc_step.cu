@@ -314,8 +314,6 @@ bool tc_eligible(const HOp& op, int s) {
   return op.prec == TBK_MIXED && op.B == 9 && s % 128 == 0 && tc_occupancy() > 0;
 }
 
-int tc_grid(tbk_ctx* ctx) { return std::max(1, tc_occupancy()) * ctx->num_sms; }
-
 void launch_step_tc(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
   using C = TcCfg<TC_GROUP, TC_D>;
   cheb_step_tc<TC_GROUP, TC_D><<<G, C::THREADS, C::SMEM, ctx->stream>>>(
