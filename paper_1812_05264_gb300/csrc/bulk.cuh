@@ -162,4 +162,17 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& c, float q) {
   c = __fadd_rn(c, err);
 }
 
+// ---- thread-block clusters -----------------------------------------------------------------------
+
+// Store x at the same shared-memory place in CTA `rank` of the cluster.
+__device__ __forceinline__ void store_cluster(double* p, int rank, double x) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(x) : "memory");
+}
+// Barrier of the cluster's threads; what they stored before is visible after.
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 }  // namespace tbk

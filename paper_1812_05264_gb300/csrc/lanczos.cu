@@ -6,6 +6,7 @@
 #include <cmath>
 #include <vector>
 
+#include "bulk.cuh"
 #include "common.cuh"
 
 namespace tbk {
@@ -261,16 +262,6 @@ __global__ void lz_transpose(int64_t n, const double* __restrict__ H, double* __
 // in shared memory there the same).
 constexpr int LZ_CL_UNITS = 128;
 
-__device__ __forceinline__ void lz_cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Store x at the same shared-memory place in CTA `rank` of the cluster.
-__device__ __forceinline__ void lz_store_remote(double* p, int rank, double x) {
-  uint32_t a;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(x) : "memory");
-}
-
 template <int B, int CL>
 __global__ void __launch_bounds__(32 * LZ_CL_UNITS / CL)
 lz_run_cluster(int n_atoms, int cap, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
@@ -288,12 +279,12 @@ lz_run_cluster(int n_atoms, int cap, const int32_t* __restrict__ row_ptr, const 
   int* cs = reinterpret_cast<int*>(lz_smem + (int64_t)cap * B * T) + threadIdx.x;
   for (int i = threadIdx.x; i < n; i += blockDim.x) vs[i] = (double)tbk_probe_sign(seed, i, 0) / sqrt((double)n);
   for (int i = threadIdx.x; i < 2 * LZ_CL_UNITS; i += blockDim.x) part[0][i] = 0.0;
-  lz_cluster_barrier();
+  cluster_barrier();
   // the sum of the units' values d, in every thread
   auto total = [&](int set, double d) {
     d = lz_warp_sum(d);
-    if (u < units && lane < CL) lz_store_remote(&part[set][u], lane, d);
-    lz_cluster_barrier();
+    if (u < units && lane < CL) store_cluster(&part[set][u], lane, d);
+    cluster_barrier();
     double s = 0.0;
     if (lane < nb) {
       const double* p = part[set] + 8 * lane;
@@ -336,10 +327,10 @@ lz_run_cluster(int n_atoms, int cap, const int32_t* __restrict__ row_ptr, const 
     vprev = v;
     v = has && bj > 0.0 ? x / bj : 0.0;
     if (has)
-      for (int r = 0; r < CL; ++r) lz_store_remote(vs + row, r, v);
-    lz_cluster_barrier();
+      for (int r = 0; r < CL; ++r) store_cluster(vs + row, r, v);
+    cluster_barrier();
   }
-  lz_cluster_barrier();  // no CTA leaves while another may still write to it
+  cluster_barrier();  // no CTA leaves while another may still write to it
 }
 
 template <int B, bool TR, bool PF>

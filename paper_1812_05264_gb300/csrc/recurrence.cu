@@ -1519,15 +1519,6 @@ constexpr size_t SWEEP_PARTIALS = (size_t)56 << 20;     // bytes of partial sums
 constexpr int SWEEP_FLUSH = 16;                         // steps whose sums wait in shared memory
 constexpr int64_t SWEEP_SMEM = 220 << 10;               // beside them; with 4 KB more L1 is a tenth slower at 10,648 sites
 
-__device__ __forceinline__ void store_cluster(double* p, int rank, double x) {
-  uint32_t a;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(x) : "memory");
-}
-__device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // probe_panel: y_0, or NULL for the +-1 probes of the seed.  partials: two per CTA and step.  cap: blocks of
 // the operator that fit in shared memory beside the panels; rows of a CTA's share beyond them stay in global memory
 // and come from L2 in every step (the cluster's barrier drops what L1 holds), a lane walking its own row.
