@@ -1381,13 +1381,13 @@ void launch_sddmm(tbk_ctx* ctx, const HOp& op, const void* y, const void* x, int
 }
 
 // Steps of the general adjoint whose outer products run together (0: after each step), as many as stay in
-// half of L2.  us per order of a whole call, after each step -> 16 together: 147 atoms x 36 probes 21.6 ->
+// 3/8 of L2.  us per order of a whole call, after each step -> 16 together: 147 atoms x 36 probes 21.6 ->
 // 19.5, 333 x 36 29.0 -> 25.3, 2,000 x 64 131 -> 107, 4,000 x 64 250 -> 202; 55 x 100 19.8 -> 18.8, 333 x 100
 // 34.0 -> 32.4, 700 x 100 61.2 -> 60.3, 1,000 x 100 78.0 -> 78.6, 333 x 124 34.3 -> 33.4.  Beyond, the butterfly
 // is a small part and the registers of the sums cost warps: 147 x 200 27.2 -> 28.2, 333 x 384 69.7 -> 95.8.
-static int general_deferred_steps(const HOp& op, int s) {
-  if (op.prec != TBK_MIXED || op.B != 9 || s > (op.n_atoms <= 500 ? 128 : 64)) return 0;
-  return (int)std::min<int64_t>(16, ((int64_t)48 << 20) / (2 * op.n_rows * s * 4));
+static int general_deferred_steps(const tbk_ctx* ctx, const HOp& op, int s) {
+  if (op.prec != TBK_MIXED || op.B != 9 || s > (10 * (int64_t)op.n_atoms <= 33 * (int64_t)ctx->num_sms ? 128 : 64)) return 0;
+  return (int)std::min<int64_t>(16, ctx->l2_bytes * 3 / 8 / (2 * op.n_rows * s * 4));
 }
 
 static void launch_sddmm_steps(tbk_ctx* ctx, const HOp& op, const OuterPanels& wp, int nt, int last_is_y0, int s,
@@ -1501,14 +1501,14 @@ __global__ void ybar_init(int64_t n, T ca, const T* __restrict__ yk, T cb, const
 }
 
 // Steps whose outer products run together after them (0: fused into each step).  Up to 64, as long as
-// their panels stay within half of L2, where the next kernel finds them; at 128 probes at least 8, since
+// their panels stay within 3/8 of L2, where the next kernel finds them; at 128 probes at least 8, since
 // one warp per block then also saves the additions to Gacc.  us per step pair (forward and backward), fused
 // and 1 / 2 / 4 / 8 steps: 2,000 atoms x 128 probes 120, 94 / 84 / 81 / 78; 10,000 x 128 584, 465 / 402 /
 // 375 / 365; 2,000 x 256 160, 141 / 140 / 140 / 139; 10,000 x 256 750, 704 / 704 / 707 / 710; at 512
 // probes 500 atoms 66.2 / 65.7, 1,000 atoms 119.1 / 119.4, 10,000 atoms 1147 / 1148.
-static int deferred_steps(const HOp& op, int s) {
+static int deferred_steps(const tbk_ctx* ctx, const HOp& op, int s) {
   if (s == 512) return 0;
-  const int64_t fit = ((int64_t)48 << 20) / (2 * op.n_rows * s * 4);
+  const int64_t fit = ctx->l2_bytes * 3 / 8 / (2 * op.n_rows * s * 4);
   return (int)std::max<int64_t>(s == 128 ? 8 : 1, std::min<int64_t>(OUT_STEPS, fit));
 }
 
@@ -1525,7 +1525,7 @@ void adjoint_doubling(tbk_ctx* ctx, const HOp& op, uint64_t probe_seed, int s, i
   const size_t esz = f64 ? 8 : 4;
   const bool windowed = sched == 1 && !f64;
   // fused schedule: steps whose outer products run after them in one launch (0: inside each step)
-  int defer = sched == 0 && !f64 && !bt ? deferred_steps(op, s) : 0;
+  int defer = sched == 0 && !f64 && !bt ? deferred_steps(ctx, op, s) : 0;
   // outer products on the tensor cores after each backward step, where that kernel applies
   const bool tensor = sched == 2 && !bt && !f64 && tc_sddmm_eligible(ctx, op, s, tc_sddmm_max_row(ctx, op));
   // a stored probe block y_0 (single system): read wherever the probe enters
@@ -1890,7 +1890,7 @@ extern "C" int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_
     const size_t n_seg_pan = (size_t)seg + 1;
     const size_t n_ckpt = all_stored ? 0 : 2 * (size_t)nseg;
     // b panels in a ring: two, or those of the steps whose outer products wait, as far as they fit
-    int defer = all_stored && !plain && npan > 0 ? general_deferred_steps(op, s) : 0;
+    int defer = all_stored && !plain && npan > 0 ? general_deferred_steps(ctx, op, s) : 0;
     defer = (int)std::max<int64_t>(0, std::min<int64_t>(std::min(defer, p - 1), (int64_t)(budget / panel) - (npan + 2)));
     if (defer < 8) defer = 0;
     size_t n_ring = defer ? (size_t)defer + 1 : 2;

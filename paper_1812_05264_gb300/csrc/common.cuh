@@ -48,6 +48,7 @@ struct tbk_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
   int num_sms = 0;
+  int64_t l2_bytes = 0;
   int64_t launches = 0;
   void* slot_ptr[tbk::WS_NSLOTS] = {};
   size_t slot_bytes[tbk::WS_NSLOTS] = {};

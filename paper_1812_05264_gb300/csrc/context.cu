@@ -132,6 +132,9 @@ int tbk_create(tbk_ctx** out, int device, void* stream) {
   cudaGetDevice(&prev);
   cudaSetDevice(device);
   cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
+  int l2 = 0;
+  cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, device);
+  c->l2_bytes = l2;
   if (prev >= 0) cudaSetDevice(prev);
   *out = c;
   TBK_API_END

@@ -1165,15 +1165,14 @@ static const Occ& occupancies(const tbk_ctx* ctx) {
   return occ[dev];
 }
 
-// FP32 steps that the one-probe-per-lane kernel takes: few tiles for the chip, or a width between 128
-// and 512 that is no multiple of 128 (whose tiles the other kernels would fetch row by row: 1,000 atoms
-// x 196 probes 71 us a step against 33).  Measured us a step, lane against self-fed kernel at 128 probes:
-// 147 atoms 8.3 (16.0), 333 atoms 9.6 (15.9), 700 atoms 16.4 (16.6); against cheb_step_bulk at 256: 147
-// atoms 10.1 (9.5).
-static bool use_lane(const HOp& op, int s) {
+// FP32 steps that the one-probe-per-lane kernel takes: up to 17 warps' work per SM, or any width beyond 128
+// that is no multiple of 128 (whose tiles the other kernels would fetch row by row: 1,000 atoms x 196 probes 71 us a
+// step against 33).  Measured us a step on 152 SMs, lane against self-fed kernel at 128 probes: 147 atoms 8.3
+// (16.0), 333 atoms 9.6 (15.9), 700 atoms 16.4 (16.6); against cheb_step_bulk at 256: 147 atoms 10.1 (9.5).
+static bool use_lane(const tbk_ctx* ctx, const HOp& op, int s) {
   if (op.prec != TBK_MIXED || op.B != 9) return false;
   if (s > 128) return s % 128 != 0;
-  return (int64_t)op.n_atoms * ((s + 31) / 32) <= 2600;
+  return (int64_t)op.n_atoms * ((s + 31) / 32) <= 17 * (int64_t)ctx->num_sms;
 }
 // FP64 9x9 steps run by rows at every size.
 static bool use_rows64(const HOp& op) { return op.prec == TBK_FP64 && op.B == 9; }
@@ -1206,7 +1205,7 @@ int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s, int K, bool resident) {
   }
   if (use_rows64(op))
     return (int)std::min<int64_t>((fp64_units(op, s, fp64_rows(ctx, op, s)) + 3) / 4, 4 * ctx->num_sms);
-  if (use_lane(op, s))
+  if (use_lane(ctx, op, s))
     return (int)std::min<int64_t>((int64_t)op.n_atoms * ((s + 511) / 512), (int64_t)std::max(1, o.lane[lane_class(s)]) * ctx->num_sms);
   const bool narrow = op.prec == TBK_MIXED && op.B == 9 && s < 128;
   if (!cw && !narrow) return (int)std::min((int64_t)o.simple * ctx->num_sms, simple_tasks(op, s));
@@ -1292,7 +1291,7 @@ static void launch_lane(tbk_ctx* ctx, const HOp& op, const StepArgs& a, int G) {
 }
 
 bool lane_adjoint_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
-  if (!use_lane(op, a.s)) return false;
+  if (!use_lane(ctx, op, a.s)) return false;
   KernelTimerScope timer(ctx, TBK_KERNEL_BACKWARD);
   launch_lane(ctx, op, a, step_grid_ctas(ctx, op, a.s));
   return true;
@@ -1320,7 +1319,7 @@ void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
     else launch_fp64<1>(ctx, op, a, G);
     return;
   }
-  if (fed && !a.per_task && use_lane(op, a.s)) {
+  if (fed && !a.per_task && use_lane(ctx, op, a.s)) {
     launch_lane(ctx, op, a, G);
     return;
   }
