@@ -46,7 +46,8 @@ typedef enum {
 } tbk_status;
 
 /* Precision / algorithm flags of the recurrence. */
-#define TBK_MIXED 0            /* FP32 panels and FP32 mapped H, FP64 moment sums (default) */
+#define TBK_MIXED 0            /* FP32 panels and FP32 mapped H (default); moment sums in FP64, within a thread in
+                                  unevaluated sums of two or three FP32 numbers */
 #define TBK_FP64 1             /* FP64 panels and FP64 mapped H throughout */
 #define TBK_MOMENTS_DIRECT 2   /* mu_k = <r, y_k> for every k instead of the doubling identity */
 #define TBK_PLAIN_KERNEL 4     /* use the plain load/FMA step kernel instead of the TMA-fed one */
@@ -292,7 +293,7 @@ int tbk_fermi_level(tbk_ctx* ctx, const double* moments, int32_t order, double e
      G = dOmega^/dH = (2/W)(1/s) sum_i sum_{j<order-1} y_ij x_ij^T on the pattern of H,
      y_ij = C_j(H^) r_i,  x_ij = (2 - delta_j0) sum_{k>j} d_k beta_k U_{k-j-1}(H^) r_i,
    returned symmetrised, G_ab <- (G_ab + G_ba^T)/2.  In mixed precision with 9x9 blocks and
-   n_probes 128, 256 or 512 the same gradient is taken through the doubled moments
+   n_probes 128, 256 or 512, and in FP64, but not with TBK_PLAIN_KERNEL, the same gradient is taken through the doubled moments
    mu_2k = 2<y_k, y_k>/s - mu_0, mu_2k-1 = 2<y_k, y_k-1>/s - mu_1, which needs y_j only up to
    j = order/2.  The panels y_j are recomputed from checkpoints when they do not fit in
    max_panel_bytes of scratch (0 = what the device has free, less a reserve).
@@ -309,8 +310,8 @@ int tbk_density_and_forces(tbk_ctx* ctx, const tbk_bsr* H, const tbk_model* mode
 
 /* tbk_energies_and_forces: tbk_chebyshev_moments + tbk_fermi_level + tbk_density_and_forces in
    one call, for the same results.  In mixed precision with 9x9 blocks and n_probes 128, 256 or
-   512 the forward sweep of the adjoint produces the moments as it goes, so no separate moment
-   pass runs.  moments: device, order doubles, or NULL.  observables: host, 4 doubles {mu, Omega,
+   512, and in FP64 unless G and forces are both NULL, but not with TBK_PLAIN_KERNEL, the forward
+   sweep of the adjoint produces the moments as it goes, so no separate moment pass runs.  moments: device, order doubles, or NULL.  observables: host, 4 doubles {mu, Omega,
    E, N}.  G, forces as in tbk_density_and_forces (either may be NULL).  flags: TBK_MIXED or
    TBK_FP64, optionally | TBK_PLAIN_KERNEL | TBK_WINDOWED | TBK_FUSED_ADJOINT | TBK_TC_OUTER.
    Synchronises the stream. */

@@ -68,8 +68,8 @@ __device__ __forceinline__ float2 shfl_xor2(float2 v, int off) {
   return make_float2(__shfl_xor_sync(0xffffffffu, v.x, off), __shfl_xor_sync(0xffffffffu, v.y, off));
 }
 // Lane values of 2 N entries, (2 p, 2 p + 1) in v[p] -> the lanes' sum of entry e in each lane with e in its lowest
-// bits: a butterfly reduce-scatter, each addition with its rounding errors.  FP64 additions take 64 cycles of an
-// SM quarter.  EXACT: two floats hold each value, the third is zero.
+// bits: a butterfly reduce-scatter, each addition with its rounding errors.  A warp's FP64 addition takes the
+// SM about 19 cycles.  EXACT: two floats hold each value, the third is zero.
 template <bool EXACT = false, int N>
 __device__ __forceinline__ double butterfly_sum3(Sum3 (&v)[N], int lane) {
 #pragma unroll
@@ -160,7 +160,7 @@ struct OuterPanels {
   const float* x[OUT_STEPS];  // ybar_{k+1} (or b_{k+1})
 };
 
-// The same for several steps after them, as long as their panels stay in L2: a lane adds its 27 sums of each
+// The same for several steps after them: a lane adds its 27 sums of each
 // step to sums of three floats (13 packed operations for two entries), and one butterfly per launch adds those of
 // the lanes.  A CTA is one block, so that its three warps find x in L1.  The loads' latency (12 warps per SM) and
 // about 600 instructions a step bind; 168 registers are the limit, so that loads go 64 probes ahead (128: spills) and
@@ -175,7 +175,7 @@ sddmm_steps32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* _
   if (gw >= 3 * nnzb) return;
   const int k = (int)(gw / 3), g = (int)(gw - 3 * (int64_t)k);
   const int b = __ldg(col + k), a = row_of_block(row_ptr, n_atoms, k, lane);
-  // byte offsets of the rows (panels of a window are a few MB), so that a load needs no 64-bit arithmetic
+  // byte offsets of the rows (panels are below 4 GB), so that a load needs no 64-bit arithmetic
   const uint32_t oy = 4u * ((9u * a + 3u * g) * s + lane), ox = 4u * (9u * b * s + lane), row = 4u * s;
   float acc[27], yv[2][3], xv[2][9];  // 64 probes ahead: with 128, spills take more than the latency
   Sum3 sum[16];
@@ -1155,8 +1155,8 @@ __device__ __forceinline__ double mi(double d, double L) { return L > 0.0 ? d - 
 
 // tq[k] = <G_ab, dH_ab/dd> - <G_ba, dH_ba/dd>, d = R_b - R_a, for every off-diagonal block k = (a, b) whose
 // transpose is stored, else 0 (SK model).  Since H_ba(-d) = H_ab(d)^T this is <G_ab + G_ba^T, dH_ab/dd>, and
-// the transpose's value is its negative: one evaluation per pair.  The FP64 units (a warp instruction takes an
-// SM quarter 64 cycles) bind; forward-mode derivatives of all entries of every block by a thread that walks
+// the transpose's value is its negative: one evaluation per pair.  The FP64 units (an SM takes about 19
+// cycles for a warp's instruction) bind; forward-mode derivatives of all entries of every block by a thread that walks
 // its own 648 bytes took 928 us at 10,000 atoms and 372 at 1,000 and 147; this 200, 58 and 29.
 // A warp takes `rows` block rows, lists their pairs a < b, and stages G_ab + G_ba^T of 32 of them at a time
 // (a stride of 81 doubles: no bank conflicts) for one thread each.
@@ -1380,14 +1380,16 @@ void launch_sddmm(tbk_ctx* ctx, const HOp& op, const void* y, const void* x, int
   post_launch(ctx, "sddmm");
 }
 
-// Steps of the general adjoint whose outer products run together (0: after each step), as many as stay in
-// 3/8 of L2.  us per order of a whole call, after each step -> 16 together: 147 atoms x 36 probes 21.6 ->
-// 19.5, 333 x 36 29.0 -> 25.3, 2,000 x 64 131 -> 107, 4,000 x 64 250 -> 202; 55 x 100 19.8 -> 18.8, 333 x 100
-// 34.0 -> 32.4, 700 x 100 61.2 -> 60.3, 1,000 x 100 78.0 -> 78.6, 333 x 124 34.3 -> 33.4.  Beyond, the butterfly
-// is a small part and the registers of the sums cost warps: 147 x 200 27.2 -> 28.2, 333 x 384 69.7 -> 95.8.
+// Steps of the general adjoint whose outer products run together (0: after each step).  us per order of a whole call,
+// after each step -> 16 together: 147 atoms x 36 probes 21.4 -> 18.8, 333 x 36 30.3 -> 25.6, 2,500 x 36 172 -> 141, 10,000
+// x 36 659 -> 542, x 64 679 -> 548; 55 x 100 18.8 -> 17.6, 333 x 100 35.1 -> 32.8, 700 x 100 64.8 -> 61.6, 1,000 x 100
+// 83.8 -> 80.6, 4,000 x 100 299 -> 293, 10,000 x 100 743 -> 753, x 124 752 -> 809; 333 x 124 35.5 -> 34.2.  Beyond 128
+// probes the butterfly is a small part and the registers of the sums cost warps: 147 x 200 29.5 -> 31.0, 333 x 384
+// 70.6 -> 98.4.  The kernel's row offsets have 32 bits.
 static int general_deferred_steps(const tbk_ctx* ctx, const HOp& op, int s) {
-  if (op.prec != TBK_MIXED || op.B != 9 || s > (10 * (int64_t)op.n_atoms <= 33 * (int64_t)ctx->num_sms ? 128 : 64)) return 0;
-  return (int)std::min<int64_t>(16, ctx->l2_bytes * 3 / 8 / (2 * op.n_rows * s * 4));
+  const bool few = 10 * (int64_t)op.n_atoms <= 66 * (int64_t)ctx->num_sms;
+  if (op.prec != TBK_MIXED || op.B != 9 || s > (few ? 128 : 64) || 4 * op.n_rows * s >= (int64_t)1 << 32) return 0;
+  return 16;
 }
 
 static void launch_sddmm_steps(tbk_ctx* ctx, const HOp& op, const OuterPanels& wp, int nt, int last_is_y0, int s,

@@ -122,8 +122,8 @@ __host__ __device__ inline int rho_lanes(int M, int lanes) {
 // (cos(k (pi - t)) = (-1)^k cos(k t): half the terms of two separate sums).  S lanes share the sums of
 // two pairs of nodes, lane r takes k = r, r + S, ..., one parity per lane, each sum compensated, and so
 // are the sums of the lanes.  The compensated chain
-// is four dependent FP64 operations of ~85 cycles a term, at 1/64 of the FP32 rate: one thread per
-// node took 432 us at p = 2476 by latency alone; S lanes cut the chain until the issue rate binds.  Two pairs
+// is four dependent FP64 operations a term, 64 cycles each (an SM takes about 19 for a warp's when all four
+// quarters are at them): one thread per node took 432 us at p = 2476 by latency alone; S lanes cut the chain until the issue rate binds.  Two pairs
 // per lane: two chains in flight, and after the first exchange between lanes each has one pair to add.
 __global__ void __launch_bounds__(32)
 rho_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int lanes, double* __restrict__ buf) {
@@ -210,7 +210,7 @@ __device__ __forceinline__ double count_occupation(double e, double mu, double i
 // bisection's; one barrier for `depth` halvings.  N(mu) is summed as FERMI_LANES strided chains and
 // a tree over them whatever the launch, and the observables over fixed runs of nodes, so that the results of a
 // problem do not depend on the launch.  Latency binds: an FP64 operation
-// takes ~85 cycles and an occupation ~40 of them (45 halvings one after the other in one CTA: 0.65 ms
+// takes 64 cycles or more and an occupation ~40 of them (45 halvings one after the other in one CTA: 0.65 ms
 // at M = 504, 9.2 ms at M = 9904; this form 0.084 and 0.119 ms, of which the sums over 32 parts and the
 // decisions were 0.02 and 0.05 more with every warp of every CTA at them).
 __global__ void __launch_bounds__(FERMI_THREADS)

@@ -78,7 +78,7 @@ __global__ void lz_start(int64_t n, uint64_t seed, double* __restrict__ v) {
 // of all FP64 issue at 10,000 atoms).  The sums keep one order: rows in groups of 256, a tree per
 // group, 256 strided chains of groups, a tree; that of lz_reduce_block.
 //
-// An FP64 operation takes ~85 cycles here and a row of 19 blocks is a chain of 171: ~7 us a step,
+// An FP64 operation takes 64 cycles and a row of 19 blocks is a chain of 171: 5.3 us a step,
 // while five launches a step took 57 us on 147 atoms (41 us of it in the product, whose rows sat on
 // 6 SMs) and 66 us on 10,000 atoms, where the FP64 issue rate allows 27.  Now 23 us a step on 1,000
 // atoms and 47 us on 10,000.
@@ -259,7 +259,8 @@ __global__ void lz_transpose(int64_t n, const double* __restrict__ H, double* __
 // square root, division and barriers.  147 atoms: 21.9 us a step over the grid,
 // 15.5 with 8 CTAs, 11.7 with 16 (where the device takes such clusters).  With 16: 340 atoms 14.1, 455 atoms
 // 17.4; the grid takes 21.1 at 456 atoms and 22.6 at 1,000, most of it its barriers (with H and the gathered v
-// in shared memory there the same).
+// in shared memory there the same).  Longer rows do not turn it: cluster / grid at 147 atoms 38 / 53 with 44 blocks a
+// row, 68 / 90 with 79; at 455 atoms 48 / 57 with 53 and 101 / 117 with 108.
 constexpr int LZ_CL_UNITS = 128;
 
 template <int B, int CL>

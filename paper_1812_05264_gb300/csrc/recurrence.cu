@@ -46,7 +46,7 @@ __device__ __forceinline__ void st16(T* p, const T* x) {
 // ---- H^ in the padded kernel layout --------------------------------------------------------
 
 // One warp per block row, element by element (lanes over a block's 81 or, for 1 x 1 blocks, over the row):
-// reads are coalesced and the FP64 product and conversion, the two that bind (an SM quarter takes 64
+// reads are coalesced and the FP64 product and conversion, the two that bind (an SM takes about 19
 // cycles for a warp's), run for stored elements only.  One thread per block: 34 us at 1,000 atoms, 188 at
 // 10,000; so 18 and 99.
 constexpr int MAP_THREADS = 128;
@@ -538,9 +538,9 @@ cheb_step_bulk(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
 // R tiles in flight and, as soon as the warp has finished with a stage, refills it with the tile
 // R positions ahead in the CTA's tile sequence (its tasks' neighbour tiles, then the y_prev tile
 // of each task).  With 128 probes a task is quickly done, so a CTA that spends half its warps
-// and registers on a producer limits how many consumers an SM holds.  The last chunk of a probe
-// count that is no multiple of 128 is narrower: its rows are copied as far as they go, and the
-// lanes past the end compute on what the ring holds and store nothing.
+// and registers on a producer limits how many consumers an SM holds.  NARROW: fewer than 128 probes, one
+// narrower task a row (its tile is one contiguous copy); the lanes past the end compute on what the ring holds
+// and store nothing.  Wider counts that are no multiple of 128 take the lane kernel.
 template <int R>
 struct SelfCfg {
   static constexpr int P = 128;
@@ -974,11 +974,12 @@ cheb_step_lane(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
 // ---- FP64 step by rows -------------------------------------------------------------------------------
 //
 // A warp takes 32 probes of ROWS (3 or 1) of the 9 rows of an atom, on its own, with the next block and
-// tile loaded a block ahead.  Each quarter of an SM issues an FP64 FMA in 64 cycles, so nothing but the
+// tile loaded a block ahead.  A warp's FP64 FMA takes 64 cycles, and the SM about 19 for each when all four
+// quarters issue them, so nothing but the
 // even spread of the FMAs over the quarters counts; a warp of a third or a ninth of a row spreads them
 // to within a few per cent (a row per three-warp CTA leaves every fourth quarter idle).  Narrow panels
-// put several row groups into a warp.  200 atoms x 64 probes: 37 us a step against 125 with the plain
-// kernel on 50 SMs (the FP64 rate alone allows 24), 2,000 x 128: 635 against 716.
+// put several row groups into a warp.  200 atoms x 64 probes: 36 us a step against 125 with the plain
+// kernel on 50 SMs, 2,000 x 128: 636 against 716, which is 18.4 cycles an FMA; at that rate 200 x 64 takes 27.
 template <int ROWS>
 __global__ void __launch_bounds__(128)
 cheb_step_fp64(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
