@@ -91,17 +91,27 @@ __device__ __forceinline__ double butterfly_sum3(Sum3 (&v)[N], int lane) {
   sum3_add(t, {other(v[0].h), other(v[0].m), other(v[0].l)});
   return sum3_value(t.h.x, t.m.x, t.l.x);
 }
-// The same of 32 entries in floats: after one exchange two floats hold each sum exactly.
-__device__ __forceinline__ double butterfly32_sum3(const float2 (&v)[16], int lane) {
-  Sum3 t[8];
-  const bool up = (lane & 16) != 0;
+// The lanes' sum of entry `lane` of 27, through a 27 x 33 buffer of the warp: a lane adds the 32 values of its entry in
+// a tree, two halves packed.  The butterfly's exchanges and selections take a third more instructions.
+__device__ __forceinline__ double transposed_sum3(const float (&v)[27], float (*buf)[33], int lane) {
 #pragma unroll
-  for (int p = 0; p < 8; ++p) {
-    t[p].h = up ? v[p + 8] : v[p];
-    two_sum(t[p].h, t[p].m, shfl_xor2(up ? v[p] : v[p + 8], 16));
-    t[p].l = make_float2(0.f, 0.f);
+  for (int e = 0; e < 27; ++e) buf[e][lane] = v[e];
+  __syncwarp();
+  const float* mine = buf[min(lane, 26)];
+  Sum3 t[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    t[j].h = make_float2(mine[j], mine[j + 16]);
+    two_sum(t[j].h, t[j].m, make_float2(mine[j + 8], mine[j + 24]));
+    t[j].l = make_float2(0.f, 0.f);
   }
-  return butterfly_sum3<true>(t, lane);
+#pragma unroll
+  for (int n = 4; n >= 1; n >>= 1)
+#pragma unroll
+    for (int j = 0; j < n; ++j) sum3_add(t[j], t[j + n]);
+  Sum3 r = {make_float2(t[0].h.x, 0.f), make_float2(t[0].m.x, 0.f), make_float2(t[0].l.x, 0.f)};
+  sum3_add(r, {make_float2(t[0].h.y, 0.f), make_float2(t[0].m.y, 0.f), make_float2(t[0].l.y, 0.f)});
+  return sum3_value(r.h.x, r.m.x, r.l.x);
 }
 
 // FP32 9x9 blocks: a warp takes three rows of a block, a lane probes lane, lane + 32, ... with 27 sums,
@@ -110,10 +120,11 @@ __device__ __forceinline__ double butterfly32_sum3(const float2 (&v)[16], int la
 // 18 us (of two floats) against 233 for one warp per block that
 // loaded as it went and added 81 FP64 butterflies (26 with all 81 sums in a warp, 12 warps per SM; 28 to
 // 32 with a thread per entry and the tiles in shared memory, whose bandwidth then binds).
-__global__ void __launch_bounds__(128, 5)
+__global__ void __launch_bounds__(128, 7)
 sddmm_rows32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t nnzb,
              const float* __restrict__ y, const float* __restrict__ x, int s, double w,
              double* __restrict__ Gacc) {
+  __shared__ float buf[4][27][33];
   pdl_wait();
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -147,10 +158,7 @@ sddmm_rows32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __
     fetch(p + 64, yv, xv);
     add(yn, xn);
   }
-  float2 v[16];
-#pragma unroll
-  for (int p = 0; p < 16; ++p) v[p] = make_float2(p < 14 ? acc[2 * p] : 0.f, p < 13 ? acc[2 * p + 1] : 0.f);
-  const double sum = butterfly32_sum3(v, lane);
+  const double sum = transposed_sum3(acc, buf[threadIdx.x >> 5], lane);
   if (lane < 27) atomicAdd(Gacc + (int64_t)k * 81 + 27 * g + lane, w * sum);
 }
 

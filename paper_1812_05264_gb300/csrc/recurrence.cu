@@ -532,6 +532,14 @@ cheb_step_bulk(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
   }
 }
 
+// The lanes' sums of s0, in lanes 0..15, and of s1, in lanes 16..31: half the FP64 instructions of two butterflies.
+__device__ __forceinline__ double lanes_sum2(double s0, double s1, int lane) {
+  double a = lane < 16 ? s0 : s1;
+  a += __shfl_xor_sync(0xffffffffu, lane < 16 ? s1 : s0, 16);
+  for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
+}
+
 // ---- self-fed step for 128-probe tasks ---------------------------------------------------------
 //
 // The same step as cheb_step_bulk<1, D> with one warp per CTA and no producer warp: lane 0 keeps
@@ -717,14 +725,8 @@ cheb_step_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
       sum1 += NARROW ? sum3_value(cs.h.y, cs.m.y, cs.l.y) : (double)cs1 + (double)cc1;
     }
     if (per_task && partials) {
-      for (int o = 16; o > 0; o >>= 1) {
-        sum0 += __shfl_xor_sync(0xffffffffu, sum0, o);
-        sum1 += __shfl_xor_sync(0xffffffffu, sum1, o);
-      }
-      if (lane == 0) {
-        partials[2 * (int64_t)a] = sum0;
-        partials[2 * (int64_t)a + 1] = sum1;
-      }
+      const double t = lanes_sum2(sum0, sum1, lane);
+      if ((lane & 15) == 0) partials[2 * (int64_t)a + (lane >> 4)] = t;
       sum0 = sum1 = 0.0;
     }
   }
@@ -737,14 +739,8 @@ cheb_step_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
     return;
   }
   if (partials && !per_task) {
-    for (int o = 16; o > 0; o >>= 1) {
-      sum0 += __shfl_xor_sync(0xffffffffu, sum0, o);
-      sum1 += __shfl_xor_sync(0xffffffffu, sum1, o);
-    }
-    if (lane == 0) {
-      partials[2 * blockIdx.x] = sum0;
-      partials[2 * blockIdx.x + 1] = sum1;
-    }
+    const double t = lanes_sum2(sum0, sum1, lane);
+    if ((lane & 15) == 0) partials[2 * blockIdx.x + (lane >> 4)] = t;
   }
 }
 
@@ -753,23 +749,13 @@ cheb_step_self(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
 __device__ __forceinline__ void step_partials(double* __restrict__ partials, double sum0, double sum1, int warp,
                                               int lane, int nw) {
   __shared__ double red[2][32];
-  for (int o = 16; o > 0; o >>= 1) {
-    sum0 += __shfl_xor_sync(0xffffffffu, sum0, o);
-    sum1 += __shfl_xor_sync(0xffffffffu, sum1, o);
-  }
-  if (lane == 0) {
-    red[0][warp] = sum0;
-    red[1][warp] = sum1;
-  }
+  const double a = lanes_sum2(sum0, sum1, lane);
+  if ((lane & 15) == 0) red[lane >> 4][warp] = a;
   asm volatile("bar.sync 1, %0;" ::"r"(32 * nw) : "memory");
-  if (threadIdx.x == 0) {
-    double a0 = 0.0, a1 = 0.0;
-    for (int w = 0; w < nw; ++w) {
-      a0 += red[0][w];
-      a1 += red[1][w];
-    }
-    partials[2 * blockIdx.x] = a0;
-    partials[2 * blockIdx.x + 1] = a1;
+  if (threadIdx.x < 2) {
+    double t = 0.0;
+    for (int w = 0; w < nw; ++w) t += red[threadIdx.x][w];
+    partials[2 * blockIdx.x + threadIdx.x] = t;
   }
 }
 
@@ -796,9 +782,11 @@ struct LaneCfg {
 };
 
 // ADJ: a step of the adjoint, with the further terms of `src` added in the fused adjoint kernel's order
-// (y_k before y_prev, the others after) and no moment sums.
+// (y_k before y_prev, the others after) and no moment sums.  The other form asks for the CTAs per SM
+// that shared memory gives: without the number the compiler took 80 registers and fetched less ahead (147 atoms x
+// 200 probes 9.3 -> 10.6 us); with it the adjoint's, which needs 124, lost a tenth.
 template <int NW, bool ADJ>
-__global__ void __launch_bounds__(32 * (NW + 1))
+__global__ void __launch_bounds__(32 * (NW + 1), ADJ ? 0 : (NW == 4 ? 4 : (NW == 8 ? 2 : 1)))
 cheb_step_lane(const int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                const float* __restrict__ hv, const float* __restrict__ yin, const float* yprev, float* yout,
                const float alpha, const float c_r, const uint64_t seed, const int s, const int direct,
@@ -1562,10 +1550,7 @@ moments_sweep_b1(int n, int C, int cap, const int32_t* __restrict__ row_ptr, con
       s0 = fma(y, in[r0 + i], s0);
       s1 = fma(y, y, s1);
     }
-    // lanes 0..15 sum s0, lanes 16..31 s1
-    double a = lane < 16 ? s0 : s1;
-    a += __shfl_xor_sync(0xffffffffu, lane < 16 ? s1 : s0, 16);
-    for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    const double a = lanes_sum2(s0, s1, lane);
     if ((lane & 15) == 0) sums[(j - 1) % SWEEP_FLUSH][lane >> 4][threadIdx.x >> 5] = a;
     cluster_barrier();
     if (j % SWEEP_FLUSH == 0 || j == K) {
