@@ -69,8 +69,8 @@ __device__ __forceinline__ float2 shfl_xor2(float2 v, int off) {
 }
 // Lane values of 2 N entries, (2 p, 2 p + 1) in v[p] -> the lanes' sum of entry e in each lane with e in its lowest
 // bits: a butterfly reduce-scatter, each addition with its rounding errors.  A warp's FP64 addition takes the
-// SM about 19 cycles.  EXACT: two floats hold each value, the third is zero.
-template <bool EXACT = false, int N>
+// SM about 19 cycles.
+template <int N>
 __device__ __forceinline__ double butterfly_sum3(Sum3 (&v)[N], int lane) {
 #pragma unroll
   for (int n = N / 2; n >= 1; n >>= 1) {
@@ -80,8 +80,7 @@ __device__ __forceinline__ double butterfly_sum3(Sum3 (&v)[N], int lane) {
     for (int p = 0; p < n; ++p) {
       const Sum3 give = up ? v[p] : v[p + n];
       if (up) v[p] = v[p + n];
-      sum3_add(v[p], {shfl_xor2(give.h, off), shfl_xor2(give.m, off),
-                      EXACT && n == N / 2 ? make_float2(0.f, 0.f) : shfl_xor2(give.l, off)});
+      sum3_add(v[p], {shfl_xor2(give.h, off), shfl_xor2(give.m, off), shfl_xor2(give.l, off)});
     }
   }
   const bool odd = (lane & 1) != 0;
@@ -92,7 +91,7 @@ __device__ __forceinline__ double butterfly_sum3(Sum3 (&v)[N], int lane) {
   return sum3_value(t.h.x, t.m.x, t.l.x);
 }
 // The lanes' sum of entry `lane` of 27, through a 27 x 33 buffer of the warp: a lane adds the 32 values of its entry in
-// a tree, two halves packed.  The butterfly's exchanges and selections take a third more instructions.
+// a tree, two halves packed, without a butterfly's exchanges and selections.
 __device__ __forceinline__ double transposed_sum3(const float (&v)[27], float (*buf)[33], int lane) {
 #pragma unroll
   for (int e = 0; e < 27; ++e) buf[e][lane] = v[e];
@@ -115,11 +114,12 @@ __device__ __forceinline__ double transposed_sum3(const float (&v)[27], float (*
 }
 
 // FP32 9x9 blocks: a warp takes three rows of a block, a lane probes lane, lane + 32, ... with 27 sums,
-// the next 32 probes loaded ahead.  The lanes' sums are kept in three floats: in two, 47 bits for the 53 of an FP64
-// sum, the calls below are 7 % faster at 1,000 atoms x 100 probes and 2 % at 333 x 384.  333 atoms x 100 probes:
-// 18 us (of two floats) against 233 for one warp per block that
+// the next 32 probes loaded ahead.  The lanes' sums have no fewer bits than FP64 ones.  333 atoms x 100 probes:
+// 18 us against 233 for one warp per block that
 // loaded as it went and added 81 FP64 butterflies (26 with all 81 sums in a warp, 12 warps per SM; 28 to
-// 32 with a thread per entry and the tiles in shared memory, whose bandwidth then binds).
+// 32 with a thread per entry and the tiles in shared memory, whose bandwidth then binds).  A whole call at 10,000
+// x 100, us per order: 683 (674 with sums of two floats and a butterfly, 744 with those of three; six CTAs per SM
+// 694, eight 791).
 __global__ void __launch_bounds__(128, 7)
 sddmm_rows32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t nnzb,
              const float* __restrict__ y, const float* __restrict__ x, int s, double w,
@@ -173,7 +173,7 @@ struct OuterPanels {
 // the lanes.  A CTA is one block, so that its three warps find x in L1.  The loads' latency (12 warps per SM) and
 // about 600 instructions a step bind; 168 registers are the limit, so that loads go 64 probes ahead (128: spills) and
 // row offsets are formed on the way.  A whole call, us per order, 333 atoms x 100 probes: 32.8 (31.8 with sums of
-// two floats, 37.1 with loads 128 ahead); launch by launch 34.0.
+// two floats, 37.1 with loads 128 ahead).
 __global__ void __launch_bounds__(96, 4)
 sddmm_steps32(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int64_t nnzb,
               const __grid_constant__ OuterPanels wp, int nt, int last_is_y0, int s, double* __restrict__ Gacc) {
@@ -1389,14 +1389,14 @@ void launch_sddmm(tbk_ctx* ctx, const HOp& op, const void* y, const void* x, int
 }
 
 // Steps of the general adjoint whose outer products run together (0: after each step).  us per order of a whole call,
-// after each step -> 16 together: 147 atoms x 36 probes 21.4 -> 18.8, 333 x 36 30.3 -> 25.6, 2,500 x 36 172 -> 141, 10,000
-// x 36 659 -> 542, x 64 679 -> 548; 55 x 100 18.8 -> 17.6, 333 x 100 35.1 -> 32.8, 700 x 100 64.8 -> 61.6, 1,000 x 100
-// 83.8 -> 80.6, 4,000 x 100 299 -> 293, 10,000 x 100 743 -> 753, x 124 752 -> 809; 333 x 124 35.5 -> 34.2.  Beyond 128
-// probes the butterfly is a small part and the registers of the sums cost warps: 147 x 200 29.5 -> 31.0, 333 x 384
-// 70.6 -> 98.4.  The kernel's row offsets have 32 bits.
+// after each step -> 16 together: 147 atoms x 36 probes 20.8 -> 18.8, 333 x 36 28.4 -> 25.6, 2,500 x 36 156 -> 141, 10,000
+// x 36 594 -> 544, x 64 602 -> 551, 4,000 x 68 270 -> 252; 55 x 100 18.9 -> 17.8, 333 x 100 33.2 -> 32.8, 333 x 124 33.4
+// -> 34.1, 700 x 100 61.3 -> 61.8, 4,000 x 100 276 -> 294, 10,000 x 124 689 -> 813; 147 x 200 26.0 -> 28.2, 333 x 384
+// 68.7 -> 98.1: with more probes the lanes' sums are a smaller part, and the registers of the kept ones cost warps.
+// The kernel's row offsets have 32 bits.
 static int general_deferred_steps(const tbk_ctx* ctx, const HOp& op, int s) {
-  const bool few = 10 * (int64_t)op.n_atoms <= 66 * (int64_t)ctx->num_sms;
-  if (op.prec != TBK_MIXED || op.B != 9 || s > (few ? 128 : 64) || 4 * op.n_rows * s >= (int64_t)1 << 32) return 0;
+  const bool few = 10 * (int64_t)op.n_atoms <= 33 * (int64_t)ctx->num_sms;
+  if (op.prec != TBK_MIXED || op.B != 9 || s > (few ? 128 : 96) || 4 * op.n_rows * s >= (int64_t)1 << 32) return 0;
   return 16;
 }
 

@@ -142,7 +142,7 @@ rho_kernel(const FermiJob one, const FermiJob* __restrict__ jobs, int lanes, dou
     step[q] = S * odd % period;
     m[q] = r * odd % period;
   }
-#pragma unroll 4
+#pragma unroll 2
   for (int k = r; k < p; k += S) {
     const double w = __ldg(b.w + k);
 #pragma unroll

@@ -95,8 +95,9 @@ def test_general_deferred_outer_products(n_atoms, s, order):
     assert (G0 - G1).abs().max().item() <= 1e-10 * G0.abs().max().item()
 
 
-# The same where 16 steps run together whatever the size (up to 64 probes) and at the line for wider ones (1,003 atoms on
+# The same where 16 steps run together whatever the size (up to 96 probes) and at the line for wider ones (501 atoms on
 # 152 SMs).
-@pytest.mark.parametrize("n_atoms,s,order", [(1003, 68, 22), (1004, 68, 22), (4000, 64, 20), (9000, 12, 19)])
+@pytest.mark.parametrize("n_atoms,s,order", [(501, 100, 22), (502, 100, 22), (1003, 96, 22), (4000, 64, 20),
+                                             (9000, 12, 19)])
 def test_general_deferred_outer_products_of_large_panels(n_atoms, s, order):
     test_general_deferred_outer_products(n_atoms, s, order)
