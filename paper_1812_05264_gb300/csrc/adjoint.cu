@@ -799,8 +799,9 @@ sddmm_window_g(const int n_atoms, const int32_t* __restrict__ row_ptr, const int
 // a butterfly over the lanes, FP64 over the steps), so the result has its bits.  A warp holds all 81 sums
 // of a block: 18 16-byte reads serve 324 FMAs where the fused kernel's three rows per warp read 12 for
 // 108.  The next 128 probes (or the next step or block) of x come into each register as the rows are done
-// with it: 8/9 of the FMAs cover their latency.  12 warps per SM of 168 registers; what binds is the
-// latency that these leave and, at 128 probes, the butterfly (372 of 775 instructions a block and step).
+// with it: 8/9 of the FMAs cover their latency.  16 warps per SM of 121 registers at 128 probes, 12 of 168 at
+// 256; what binds is the latency that these leave (issue 64 to 66 % busy, L1 54 to 60 %) and, at 128 probes, the
+// butterfly (372 of 775 instructions a block and step).
 // us per backward step with its outer products, fused -> a step kernel and these: 147 atoms x 128 probes
 // 31 -> 11, 1,000 x 128 61 -> 30, 10,000 x 128 488 -> 263, 147 x 256 27 -> 15, 1,000 x 256 66 -> 58, 10,000
 // x 256 548 -> 510.  At 512 probes both take the same (823 -> 836 at 10,000 atoms) and the fused kernel stays.
