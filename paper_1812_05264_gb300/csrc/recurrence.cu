@@ -1163,8 +1163,13 @@ static bool use_lane(const tbk_ctx* ctx, const HOp& op, int s) {
   if (s > 128) return s % 128 != 0;
   return (int64_t)op.n_atoms * ((s + 31) / 32) <= 17 * (int64_t)ctx->num_sms;
 }
-// FP64 9x9 steps run by rows at every size.
-static bool use_rows64(const HOp& op) { return op.prec == TBK_FP64 && op.B == 9; }
+// FP64 9x9 steps by rows: while the plain kernel's tasks take fewer than two rounds of its CTAs.  Beyond, its tiles of
+// several rows and probes read less.  us a step, rows / plain: 1,000 atoms x 128 probes (0.8 rounds) 315 / 370, 3,000 x
+// 64 (1.2) 500 / 541, 7,000 x 32 (1.4) 633 / 650; 10,000 x 32 (2.1) 911 / 886, 5,832 full rows x 64 (2.4) 1,102 /
+// 1,040, 1,000 x 512 (3.3) 1,237 / 1,253, 10,000 x 128 (8) 3,408 / 3,274, x 512 (33) 13,609 / 12,834.
+static bool use_rows64(const tbk_ctx* ctx, const HOp& op, int s) {
+  return op.prec == TBK_FP64 && op.B == 9 && simple_tasks(op, s) < 2 * (int64_t)occupancies(ctx).simple * ctx->num_sms;
+}
 
 // Warps of an FP64 step by rows, and the rows a warp takes: one where three would leave SM quarters idle.
 static int64_t fp64_units(const HOp& op, int s, int rows) {
@@ -1192,7 +1197,7 @@ int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s, int K, bool resident) {
     const int64_t held = (int64_t)(cw && o.bulk[cw] > 0 ? o.bulk[cw] : o.simple) * ctx->num_sms;
     return (int)std::min(held, std::max(simple_tasks(op, s), cw ? (int64_t)op.n_atoms * (s / 128) : 0));
   }
-  if (use_rows64(op))
+  if (use_rows64(ctx, op, s))
     return (int)std::min<int64_t>((fp64_units(op, s, fp64_rows(ctx, op, s)) + 3) / 4, 4 * ctx->num_sms);
   if (use_lane(ctx, op, s))
     return (int)std::min<int64_t>((int64_t)op.n_atoms * ((s + 511) / 512), (int64_t)std::max(1, o.lane[lane_class(s)]) * ctx->num_sms);
@@ -1303,7 +1308,8 @@ void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
     return;
   }
   const bool fed = !a.cur_is_probe && a.err && !a.force_simple && op.B == 9;  // a panel by bulk copies
-  if (fed && use_rows64(op)) {
+  // (with an adjoint's own-row terms at every size: the plain kernel has none for 9x9 blocks)
+  if (fed && op.prec == TBK_FP64 && (use_rows64(ctx, op, a.s) || a.src[0] || a.src[1] || a.src[2])) {
     if (fp64_rows(ctx, op, a.s) == 3) launch_fp64<3>(ctx, op, a, G);
     else launch_fp64<1>(ctx, op, a, G);
     return;

@@ -41,3 +41,29 @@ def test_nine_orbitals(n_atoms, s, order, flags):
     import torch
     a, b = _both(wl.fcc_cu(n_atoms, kT=0.5, n_probes=s, jitter=0.05), s, order, flags)
     assert torch.equal(a, b)
+
+
+# FP64 around the line between the step by rows and the plain one (two rounds of 608 CTAs on 152 SMs), against the
+# plain kernel to FP64 rounding of a sum of n s terms
+@pytest.mark.parametrize("n_atoms,s", [(607, 260), (608, 260), (700, 512)])
+def test_fp64_steps_around_the_line(n_atoms, s):
+    import torch
+    a, b = _both(wl.fcc_cu(n_atoms, kT=0.5, n_probes=s, jitter=0.05), s, 13, 1)
+    assert torch.equal(a, b)
+    p, _ = _both(wl.fcc_cu(n_atoms, kT=0.5, n_probes=s, jitter=0.05), s, 13, 1 + 4)
+    assert (a - p).abs().max().item() <= 1e-13 * 9 * n_atoms
+
+
+def test_fp64_gradient_of_a_large_panel_has_the_steps_terms():
+    """1,300 x 256 in FP64: plain forward steps, backward steps by rows; the gradient against mixed precision."""
+    import torch
+    from paper_1812_05264_gb300 import api
+    wk = wl.fcc_cu(1300, kT=0.5, n_probes=256, jitter=0.05)
+    ctx = api.Context()
+    pos = torch.as_tensor(wk.positions, dtype=torch.float64, device="cuda")
+    H = api.assemble_H(ctx, api.Model.from_workload(wk, "cuda"), pos, api.build_neighbors(ctx, pos, wk.cutoff))
+    lo, hi = api.spectral_bounds(ctx, H)
+    args = (ctx, H, None, None, None, lo, hi, 3, 256, 20, 6.0, 0.5)
+    G, _ = api.density_and_forces(*args, fp64=True, want_forces=False)
+    Gm, _ = api.density_and_forces(*args, want_forces=False)
+    assert (G - Gm).abs().max().item() <= 2e-5 * G.abs().max().item()
