@@ -100,6 +100,8 @@ inline int task_grid(int64_t tasks, int64_t held) {
 void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a);
 // An adjoint step (a.adjoint) on the kernel for small operators; false where that does not apply.
 bool lane_adjoint_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a);
+// Whether a sweep of more than one step writes its probe block once, into the panel that its second step overwrites.
+bool probe_panel_pays(const HOp& op);
 // panel = c * r (probe block) for all rows.
 void launch_scaled_probe(tbk_ctx* ctx, const HOp& op, void* panel, double c, uint64_t seed, int s);
 

@@ -128,7 +128,7 @@ extern "C" int tbk_chebyshev_moments_noalloc(tbk_ctx* ctx, const tbk_bsr* H, dou
   // the array keeps the previous call's contents: the error flag must start at zero
   TBK_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), ctx->stream));
   HOp op = prepare_hop_into(ctx, H, emin, emax, prec, base + o_hhat, flag);
-  void *cur = nullptr, *prev = nullptr;
+  void *cur = nullptr, *prev = nullptr, *y0 = probe_panel_pays(op) ? Bp : nullptr;
   if (sweep) {
     launch_sweep(ctx, op, nullptr, probe_seed, s, K, partials);
     launch_partial_sums(ctx, partials, nctas, K, sums);
@@ -144,16 +144,16 @@ extern "C" int tbk_chebyshev_moments_noalloc(tbk_ctx* ctx, const tbk_bsr* H, dou
     a.force_simple = (flags & TBK_PLAIN_KERNEL) ? 1 : 0;
     a.grid = nctas;
     if (j == 1) {
-      if (Bp) launch_scaled_probe(ctx, op, Bp, 1.0, probe_seed, s);  // y_0, until y_2 takes its place
-      a.yin = Bp;
-      a.cur_is_probe = Bp ? 0 : 1;
+      if (y0) launch_scaled_probe(ctx, op, y0, 1.0, probe_seed, s);  // until y_2 takes its place
+      a.yin = y0;
+      a.cur_is_probe = y0 ? 0 : 1;
       a.alpha = 1.0;
       a.yout = A;
       cur = A;
     } else if (j == 2) {
       a.yin = A;
       a.alpha = 2.0;
-      a.yprev = Bp;
+      if (y0) a.yprev = y0; else a.c_r = -1.0;
       a.yout = Bp;
       prev = A;
       cur = Bp;

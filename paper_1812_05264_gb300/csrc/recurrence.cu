@@ -1337,32 +1337,34 @@ void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
   }
 }
 
-// A thread writes four probes of a row (16-byte stores), a warp 128.
+// A thread writes four probes of a row (16-byte stores), neighbouring threads neighbouring ones, over the rows' ends: a
+// warp per row left most of its lanes idle on narrow panels.
 template <typename T>
 __global__ void __launch_bounds__(256)
-scaled_probe_kernel(int64_t n_rows, int s, double c, uint64_t seed, T* __restrict__ out) {
-  const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (row >= n_rows) return;
-  for (int p = 4 * (threadIdx.x & 31); p < s; p += 128) {
-    T v[4];
+scaled_probe_kernel(int64_t n_items, int groups, double c, uint64_t seed, T* __restrict__ out) {
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= n_items) return;
+  const int64_t row = n_items <= 0xffffffffll ? (int64_t)((uint32_t)i / (uint32_t)groups) : i / groups;
+  const int p = 4 * (int)(i - row * groups);
+  T v[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = (T)(c * (double)tbk_probe_sign(seed, row, p + j));
-    T* o = out + row * s + p;
-    if constexpr (sizeof(T) == 4) {
-      st16(o, v);
-    } else {
-      st16(o, v);
-      st16(o + 2, v + 2);
-    }
+  for (int j = 0; j < 4; ++j) v[j] = (T)(c * (double)tbk_probe_sign(seed, row, p + j));
+  T* o = out + 4 * i;
+  if constexpr (sizeof(T) == 4) {
+    st16(o, v);
+  } else {
+    st16(o, v);
+    st16(o + 2, v + 2);
   }
 }
 
 void launch_scaled_probe(tbk_ctx* ctx, const HOp& op, void* panel, double c, uint64_t seed, int s) {
-  const int grid = ceil_div(op.n_rows, 8);
+  const int64_t n = op.n_rows * (s / 4);
+  const unsigned grid = (unsigned)((n + 255) / 256);
   if (op.prec == TBK_MIXED)
-    scaled_probe_kernel<float><<<grid, 256, 0, ctx->stream>>>(op.n_rows, s, c, seed, (float*)panel);
+    scaled_probe_kernel<float><<<grid, 256, 0, ctx->stream>>>(n, s / 4, c, seed, (float*)panel);
   else
-    scaled_probe_kernel<double><<<grid, 256, 0, ctx->stream>>>(op.n_rows, s, c, seed, (double*)panel);
+    scaled_probe_kernel<double><<<grid, 256, 0, ctx->stream>>>(n, s / 4, c, seed, (double*)panel);
   post_launch(ctx, "scaled_probe_kernel");
 }
 
@@ -1641,6 +1643,12 @@ void launch_sweep(tbk_ctx* ctx, const HOp& op, const void* probe_panel, uint64_t
 
 // ---- building blocks that allocate nothing (for the static-scratch entry point) --------------
 
+// 9x9 blocks: a step on a panel takes a third of the time of one that regenerates every neighbour's probes.  1x1: the
+// FP64 arithmetic hides the regeneration (us of seven steps, regenerated / from a panel: 17,576 sites x 16 probes 113 /
+// 119, 216,000 x 128 of 168 blocks a row 32,472 / 32,505); FP32 from about eight blocks a row (216,000 x 128 of 7 blocks
+// 1,004 / 1,006, 18 blocks 1,622 / 1,390, 77 blocks 4,812 / 3,318; 17,576 x 16 of 7 blocks 94 / 100).
+bool probe_panel_pays(const HOp& op) { return op.B == 9 || (op.prec == TBK_MIXED && op.nnzb > 8 * op.n_rows); }
+
 size_t mapped_h_bytes(const tbk_bsr* H, int prec) {
   const int bs = H->n_orb == 9 ? (prec == TBK_MIXED ? Layout<float, 9>::BS : Layout<double, 9>::BS) : 1;
   return (size_t)H->nnzb * bs * (prec == TBK_MIXED ? 4 : 8);
@@ -1733,6 +1741,8 @@ void moments_sweep(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, uin
   double* pd_dots = per_probe ? (double*)scratch(ctx, WS_SEGMENT, sizeof(double) * 2 * (size_t)std::max(1, K) * s)
                               : nullptr;
   void *cur = nullptr, *prev = nullptr;
+  // y_0: the given panel, or one written into the second step's, or (NULL) regenerated by the first two steps
+  void* y0 = probe_panel ? const_cast<void*>(probe_panel) : (probe_panel_pays(op) ? Bp : nullptr);
   for (int j = 1; j <= K && !sweep; ++j) {
     StepArgs a;
     a.seed = probe_seed;
@@ -1744,18 +1754,17 @@ void moments_sweep(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, uin
     a.use_tc = (flags & TBK_TENSOR_CORES) ? 1 : 0;
     a.grid = nctas;
     if (j == 1) {
-      // a further step follows: its panel holds the probe block until then (a step on a panel takes a
-      // third of the time of one that regenerates every neighbour's probes)
-      if (!probe_panel && Bp) launch_scaled_probe(ctx, op, Bp, 1.0, probe_seed, s);
-      a.yin = probe_panel ? probe_panel : Bp;
-      a.cur_is_probe = a.yin ? 0 : 1;
+      // a further step follows: its panel holds the probe block until then
+      if (y0 && !probe_panel) launch_scaled_probe(ctx, op, y0, 1.0, probe_seed, s);
+      a.yin = y0;
+      a.cur_is_probe = y0 ? 0 : 1;
       a.alpha = 1.0;
       a.yout = A;
       cur = A;
     } else if (j == 2) {
       a.yin = A;
       a.alpha = 2.0;
-      a.yprev = probe_panel ? const_cast<void*>(probe_panel) : Bp;
+      if (y0) a.yprev = y0; else a.c_r = -1.0;
       a.yout = Bp;
       prev = A;
       cur = Bp;

@@ -48,3 +48,26 @@ def test_one_launch_where_the_blocks_fit(size, r, s, one):
     n0 = ctx.launches
     api.chebyshev_moments(ctx, H, -9.0, 9.0, 5, s, 23, fp64=True)
     assert (ctx.launches - n0 < 8) == one
+
+
+# The first two steps from a probe panel (FP32 rows of more than eight blocks) or from regenerated probes: the same
+# values, so with one operator's values on a shorter and a longer pattern (zeros appended) the same moments.
+@pytest.mark.parametrize("fp64", [False, True])
+@pytest.mark.parametrize("direct", [False, True])
+def test_first_steps_of_one_orbital_operators(fp64, direct):
+    import torch
+    from paper_1812_05264_gb300 import api
+    ctx = api.Context()
+    short, wide = _operator(ctx, 9, 1.0), _operator(ctx, 9, 1.5)
+    pos = torch.as_tensor(wl.sc_disorder(L=9).positions, dtype=torch.float64).cuda()
+    rows = torch.repeat_interleave(torch.arange(729, device="cuda"), wide.graph.row_ptr.diff().long())
+    near = (pos[rows] - pos[wide.graph.col.long()]).norm(dim=1) <= 1.0 + 1e-9
+    val = torch.zeros_like(wide.val)
+    val[near] = short.val
+    wide = api.BSR(wide.graph, 1, val)
+    assert short.graph.nnzb <= 8 * 729 < wide.graph.nnzb
+    args = (-9.0, 9.0, 5, 516, 13, fp64, direct)
+    m0, p0 = api.chebyshev_probe_moments(ctx, short, *args)
+    m1, p1 = api.chebyshev_probe_moments(ctx, wide, *args)
+    assert torch.equal(p0, p1)
+    assert (m0 - m1).abs().max().item() <= 1e-12 * 729
