@@ -45,23 +45,28 @@ __device__ __forceinline__ void st16(T* p, const T* x) {
 
 // ---- H^ in the padded kernel layout --------------------------------------------------------
 
-// One warp per block row, element by element (lanes over a block's 81 or, for 1 x 1 blocks, over the row):
+// One warp per block row, element by element (lanes over a block's 81; 1 x 1 blocks: eight lanes over the row, whose
+// seven blocks leave most of a warp idle):
 // reads are coalesced and the FP64 product and conversion, the two that bind (an SM takes about 19
 // cycles for a warp's), run for stored elements only.  One thread per block: 34 us at 1,000 atoms, 188 at
 // 10,000; so 18 and 99.
 constexpr int MAP_THREADS = 128;
+template <int B>
+constexpr int map_lanes() { return B == 1 ? 8 : 32; }
+static int map_grid(const HOp& op) { return ceil_div(op.n_atoms, MAP_THREADS / (op.B == 1 ? map_lanes<1>() : map_lanes<9>())); }
 
 template <typename T, int B>
 __global__ void __launch_bounds__(MAP_THREADS)
 map_h_kernel(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
              const double* __restrict__ H, double shift, double inv_half_w, T* __restrict__ out, int* __restrict__ err) {
   constexpr int RS = Layout<T, B>::RS, BS = Layout<T, B>::BS;
-  const int a = blockIdx.x * (MAP_THREADS / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  constexpr int L = map_lanes<B>();
+  const int a = blockIdx.x * (MAP_THREADS / L) + threadIdx.x / L, lane = threadIdx.x % L;
   if (a >= n_atoms) return;
   bool has_diag = false;
   const int k1 = row_ptr[a + 1];
   if constexpr (B == 1) {
-    for (int k = row_ptr[a] + lane; k < k1; k += 32) {
+    for (int k = row_ptr[a] + lane; k < k1; k += L) {
       const bool diag = col[k] == a;
       has_diag |= diag;
       double v = H[k];
@@ -86,7 +91,8 @@ map_h_kernel(int n_atoms, const int32_t* __restrict__ row_ptr, const int32_t* __
       if (lane < B * (RS - B)) o[lane / (RS - B) * RS + B + lane % (RS - B)] = T(0);
     }
   }
-  if (!__any_sync(0xffffffffu, has_diag) && lane == 0) atomicOr(err, ERR_NO_DIAGONAL);
+  const unsigned row_mask = L == 32 ? 0xffffffffu : ((1u << L) - 1) << (threadIdx.x & 31 & ~(L - 1));
+  if (!__any_sync(row_mask, has_diag) && lane == 0) atomicOr(err, ERR_NO_DIAGONAL);
 }
 
 HOp prepare_hop(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, int prec, Slot slot, int* err) {
@@ -106,7 +112,7 @@ HOp prepare_hop(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, int pr
   op.row_ptr = H->row_ptr;
   op.col = H->col;
   const double shift = 0.5 * (emax + emin), inv = 2.0 / (emax - emin);
-  const int blk = MAP_THREADS, grid = ceil_div(op.n_atoms, MAP_THREADS / 32);
+  const int blk = MAP_THREADS, grid = map_grid(op);
 #define TBK_MAP(TT, BB)                                                                        \
   {                                                                                            \
     TT* out = (TT*)scratch(ctx, slot, sizeof(TT) * (size_t)op.nnzb * Layout<TT, BB>::BS);      \
@@ -1672,7 +1678,7 @@ HOp prepare_hop_into(tbk_ctx* ctx, const tbk_bsr* H, double emin, double emax, i
   op.col = H->col;
   op.hv = dst;
   const double shift = 0.5 * (emax + emin), inv = 2.0 / (emax - emin);
-  const int blk = MAP_THREADS, grid = ceil_div(op.n_atoms, MAP_THREADS / 32);
+  const int blk = MAP_THREADS, grid = map_grid(op);
   if (prec == TBK_MIXED) {
     if (op.B == 9)
       map_h_kernel<float, 9><<<grid, blk, 0, ctx->stream>>>(op.n_atoms, op.row_ptr, op.col, H->val, shift, inv, (float*)dst, err);

@@ -71,3 +71,22 @@ def test_first_steps_of_one_orbital_operators(fp64, direct):
     m1, p1 = api.chebyshev_probe_moments(ctx, wide, *args)
     assert torch.equal(p0, p1)
     assert (m0 - m1).abs().max().item() <= 1e-12 * 729
+
+
+# A row without its diagonal entry is found wherever it lies among the rows that share a warp, in the last one too
+@pytest.mark.parametrize("row", [0, 1, 2, 3, 7, 124])
+@pytest.mark.parametrize("fp64", [False, True])
+def test_one_orbital_row_without_its_diagonal_is_rejected(row, fp64):
+    import torch
+    from paper_1812_05264_gb300 import _lib as L, api
+    ctx = api.Context()
+    H = _operator(ctx, 5, 1.0)
+    api.chebyshev_moments(ctx, H, -9.0, 9.0, 5, 8, 9, fp64=fp64)
+    rows = torch.repeat_interleave(torch.arange(125, device="cuda"), H.graph.row_ptr.diff().long())
+    keep = ~((rows == row) & (H.graph.col == row))
+    rp = H.graph.row_ptr.clone()
+    rp[row + 1:] -= 1
+    bad = api.BSR(api.Graph(125, H.graph.nnzb - 1, rp, H.graph.col[keep].contiguous()), 1, H.val[keep].contiguous())
+    with pytest.raises(L.TbkError) as e:
+        api.chebyshev_moments(ctx, bad, -9.0, 9.0, 5, 8, 9, fp64=fp64)
+    assert e.value.code == L.TBK_ERR_ARG and "diagonal" in str(e.value)
