@@ -1169,6 +1169,12 @@ static bool use_lane(const tbk_ctx* ctx, const HOp& op, int s) {
   if (s > 128) return s % 128 != 0;
   return (int64_t)op.n_atoms * ((s + 31) / 32) <= 17 * (int64_t)ctx->num_sms;
 }
+// The self-fed kernel with narrow tasks, where there is too much for the lane kernel: a warp per row whatever the
+// probes, so that it loses to the plain kernel's several rows per warp on many rows of few.  us a step, narrow / plain:
+// 4,000 atoms x 16 probes 40 / 55, 6,000 x 16 58 / 53, 10,000 x 16 93 / 54, x 20 93 / 98, 20,000 x 8 182 / 117, x 32 182 / 232.
+static bool use_narrow(const tbk_ctx* ctx, const HOp& op, int s) {
+  return op.prec == TBK_MIXED && op.B == 9 && s < 128 && (s > 16 || op.n_atoms <= 36 * ctx->num_sms);
+}
 // FP64 9x9 steps by rows: while the plain kernel's tasks take fewer than two rounds of its CTAs.  Beyond, its tiles of
 // several rows and probes read less.  us a step, rows / plain: 1,000 atoms x 128 probes (0.8 rounds) 315 / 370, 3,000 x
 // 64 (1.2) 500 / 541, 7,000 x 32 (1.4) 633 / 650; 10,000 x 32 (2.1) 911 / 886, 5,832 full rows x 64 (2.4) 1,102 /
@@ -1207,7 +1213,7 @@ int step_grid_ctas(tbk_ctx* ctx, const HOp& op, int s, int K, bool resident) {
     return (int)std::min<int64_t>((fp64_units(op, s, fp64_rows(ctx, op, s)) + 3) / 4, 4 * ctx->num_sms);
   if (use_lane(ctx, op, s))
     return (int)std::min<int64_t>((int64_t)op.n_atoms * ((s + 511) / 512), (int64_t)std::max(1, o.lane[lane_class(s)]) * ctx->num_sms);
-  const bool narrow = op.prec == TBK_MIXED && op.B == 9 && s < 128;
+  const bool narrow = use_narrow(ctx, op, s);
   if (!cw && !narrow) return (int)std::min((int64_t)o.simple * ctx->num_sms, simple_tasks(op, s));
   const int fed = cw && dense_bulk(ctx, op, s, cw) ? o.dense : (cw ? o.bulk[cw] : 0);
   const int per_sm = narrow && o.bulk[1] > 0 ? o.bulk[1] : (fed > 0 ? fed : o.simple);
@@ -1324,7 +1330,7 @@ void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
     launch_lane(ctx, op, a, G);
     return;
   }
-  if (fed && op.prec == TBK_MIXED && a.s < 128) {
+  if (fed && use_narrow(ctx, op, a.s)) {
     launch_self<true>(ctx, op, a, G);
     return;
   }
