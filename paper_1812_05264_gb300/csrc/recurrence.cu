@@ -1353,14 +1353,14 @@ void launch_step(tbk_ctx* ctx, const HOp& op, const StepArgs& a) {
 // warp per row left most of its lanes idle on narrow panels.
 template <typename T>
 __global__ void __launch_bounds__(256)
-scaled_probe_kernel(int64_t n_items, int groups, double c, uint64_t seed, T* __restrict__ out) {
+scaled_probe_kernel(int64_t n_items, int groups, T c, uint64_t seed, T* __restrict__ out) {
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= n_items) return;
   const int64_t row = n_items <= 0xffffffffll ? (int64_t)((uint32_t)i / (uint32_t)groups) : i / groups;
   const int p = 4 * (int)(i - row * groups);
   T v[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) v[j] = (T)(c * (double)tbk_probe_sign(seed, row, p + j));
+  for (int j = 0; j < 4; ++j) v[j] = tbk_probe_sign(seed, row, p + j) < 0.f ? -c : c;
   T* o = out + 4 * i;
   if constexpr (sizeof(T) == 4) {
     st16(o, v);
@@ -1374,7 +1374,7 @@ void launch_scaled_probe(tbk_ctx* ctx, const HOp& op, void* panel, double c, uin
   const int64_t n = op.n_rows * (s / 4);
   const unsigned grid = (unsigned)((n + 255) / 256);
   if (op.prec == TBK_MIXED)
-    scaled_probe_kernel<float><<<grid, 256, 0, ctx->stream>>>(n, s / 4, c, seed, (float*)panel);
+    scaled_probe_kernel<float><<<grid, 256, 0, ctx->stream>>>(n, s / 4, (float)c, seed, (float*)panel);
   else
     scaled_probe_kernel<double><<<grid, 256, 0, ctx->stream>>>(n, s / 4, c, seed, (double*)panel);
   post_launch(ctx, "scaled_probe_kernel");
